@@ -110,6 +110,35 @@ void launch_split_blocks(long long R, int n, int RB, int ld, int k0, const doubl
 void launch_pack_complex(int nw, int n, const float* C, long long ldc, int splits, long long split_stride,
                          const double* add, double2* out, long long ldo, cudaStream_t st);
 
+// tc_dgemm.cu: FP64 products on the BF16 tensor cores (exact-integer split).
+// An operand: the digit slices [8][rows][dg_k_padded(K)] of its rows and their
+// exponents [rows]; batch entry z starts at row z * batch_rows (0: shared). A
+// complex operand has two rows (real, imaginary part) per complex row.
+struct DgOperand {
+    const void* s = nullptr;
+    const int* e = nullptr;
+    int rows = 0;
+    int batch_rows = 0;
+};
+// C[z c_batch + n c_n + m c_m] = mul sum_k A_z[m][k] B_z[n][k], m < Mr rows of
+// A, n < Nc complex rows of B; acc (optional, same layout) += C. With splits >
+// 1 (batch must be 1) the contraction is divided and split z writes its part at
+// z c_batch, for dg_sum_splits.
+struct DgOut {
+    int Mr = 0, Nc = 0, batch = 1, splits = 1;
+    double2* C = nullptr;
+    long long c_batch = 0, c_n = 0, c_m = 1;
+    double2* acc = nullptr;
+    double mul = 1.0;
+};
+int dg_k_padded(int K);
+size_t dg_row_bytes(int K);              // slices and exponent of one real row
+int dg_splits(int Mr, int K);
+void dg_slice_real(long long R, int K, const double* src, long long ld, void* S, int* ex, cudaStream_t st);
+void dg_slice_complex(long long R, int K, const double2* src, long long ld, void* S, int* ex, cudaStream_t st);
+int dg_gemm(const DgOperand& A, const DgOperand& B, const DgOut& o, int K, unsigned* err, cudaStream_t st);
+void dg_sum_splits(int R, int Cc, int splits, const double2* part, double2* out, long long ldo, cudaStream_t st);
+
 // tc_fepi.cu: the Cholesky contraction of the energy fused with its
 // per-(walker, vector) epilogue (same outputs as tc_gemm_3xtf32 followed by
 // launch_fepi_f32). A: split rows of dG[occ0][virt], part c of walker w at

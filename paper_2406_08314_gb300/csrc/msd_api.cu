@@ -93,6 +93,14 @@ struct Buf {
     size_t bytes = 0;
 };
 
+// Digit slices of a constant real operand of the FP64 contractions
+// (tc_dgemm.cu), built on first use.
+struct DgConst {
+    void* s = nullptr;
+    int* e = nullptr;
+    bool tried = false;
+};
+
 }  // namespace
 
 struct msd_ctx {
@@ -175,6 +183,9 @@ struct msd_ctx {
     std::vector<double> h_corr;   // [M][M]
     double* d_E[2] = {nullptr, nullptr};
     double prop_dt = -1.0;
+    // FP64 contractions on the tensor cores: the half-rotated Cholesky rows per
+    // spin, both spins' rows concatenated, the transposed Cholesky vectors
+    DgConst dg_Lh[2], dg_Lcat, dg_Lt;
 };
 
 namespace {
@@ -280,6 +291,63 @@ int arena_get(msd_ctx* ctx, const char* name, size_t bytes, void** out)
         b.bytes = bytes;
     }
     *out = b.p;
+    return MSD_OK;
+}
+
+void free_dg(DgConst& c)
+{
+    cudaFree(c.s);
+    cudaFree(c.e);
+    c = DgConst{};
+}
+
+// The contraction with a constant [rows][K] operand runs on the tensor cores
+// (tc_dgemm.cu) from this size on: below it the slicing pass and the fixed cost
+// of the persistent kernel outweigh the products. The rule does not look at the
+// number of walkers, so a walker's result does not depend on the chunk it is in.
+bool dg_use(long long rows, long long K) { return K >= 24 && rows * K >= 65536 && rows < (1ll << 27); }
+size_t dg_bytes(long long rows, int K, int complex_rows)
+{
+    return dg_use(rows, K) ? 2 * dg_row_bytes(K) * (size_t)complex_rows : 0;
+}
+
+// C[m][n] = sum_k A[m][k] B[n][k] in FP64: A Mr complex rows (walkers), B the
+// constant real operand [Nc][K] whose slices `cB` keeps. Where the slices' memory
+// cannot be had, the FP64 kernel runs.
+int gemm_zd(msd_ctx* ctx, int Mr, int Nc, int K, const double2* A, long long lda, const double* B, long long ldb,
+            DgConst& cB, double2* C, long long ldc, cudaStream_t st)
+{
+    if (dg_use(Nc, K) && !cB.tried) {
+        cB.tried = true;
+        if (cudaMalloc(&cB.s, dg_row_bytes(K) * (size_t)Nc) != cudaSuccess ||
+            cudaMalloc((void**)&cB.e, sizeof(int) * (size_t)Nc) != cudaSuccess) {
+            cudaGetLastError();
+            free_dg(cB);
+            cB.tried = true;
+        } else {
+            dg_slice_real(Nc, K, B, ldb, cB.s, cB.e, st);
+            CK(cudaStreamSynchronize(st));   // other streams may use the slices next
+        }
+    }
+    if (!dg_use(Nc, K) || !cB.s) {
+        launch_gemm_zd(Mr, Nc, K, A, lda, B, ldb, C, ldc, st);
+        return MSD_OK;
+    }
+    int rc;
+    void *s, *e, *part = C;
+    const int splits = dg_splits(Nc, K);
+    if ((rc = arena_get(ctx, "dg_s", dg_row_bytes(K) * 2 * (size_t)Mr, &s))) return rc;
+    if ((rc = arena_get(ctx, "dg_e", sizeof(int) * 2 * (size_t)Mr, &e))) return rc;
+    if (splits > 1 && (rc = arena_get(ctx, "dg_part", sizeof(double2) * splits * (size_t)Mr * Nc, &part))) return rc;
+    dg_slice_complex(Mr, K, A, lda, s, (int*)e, st);
+    DgOut o;
+    o.Mr = Nc; o.Nc = Mr; o.splits = splits;
+    o.C = (double2*)part;
+    o.c_n = splits > 1 ? Nc : ldc;
+    o.c_batch = (long long)Mr * Nc;
+    if (dg_gemm({cB.s, cB.e, Nc, 0}, {s, (int*)e, 2 * Mr, 0}, o, K, ctx->d_err, st))
+        return fail(ctx, MSD_ERR_CUDA, "FP64 tensor-core contraction launch failed");
+    if (splits > 1) dg_sum_splits(Mr, Nc, splits, (const double2*)part, C, ldc, st);
     return MSD_OK;
 }
 
@@ -539,6 +607,9 @@ void free_mixed(msd_ctx* ctx)
     cudaFree(ctx->d_c0sum);
     ctx->d_c0sum = nullptr;
     ctx->mixed_ready = false;
+    free_dg(ctx->dg_Lh[0]);
+    free_dg(ctx->dg_Lh[1]);
+    free_dg(ctx->dg_Lcat);
     free_exact_ref(ctx);
 }
 
@@ -992,6 +1063,8 @@ size_t fb_bytes_per_walker(msd_ctx* ctx, bool fp32)
         b += sizeof(double2) * (size_t)t.nh * t.np;
     }
     if (fp32) b += sizeof(float) * 2 * 2 * ctx->Kdp + sizeof(float) * 16 * 2 * ctx->n_chol;
+    else if (dg_use(ctx->n_chol, ctx->Kd))
+        b += dg_bytes(ctx->n_chol, (int)ctx->Kd, 1) + sizeof(double2) * dg_splits(ctx->n_chol, (int)ctx->Kd) * ctx->n_chol;
     return b;
 }
 
@@ -1058,9 +1131,10 @@ int fb_chunk(msd_ctx* ctx, Chunk& c, FbWork& f, int w0, int nw, int cap, bool fp
         th.end(st);
     } else {
         th.begin("k_gemm_vbias", st);
-        launch_gemm_zd(nw, ctx->n_chol, (int)ctx->Kd, (const double2*)f.GT, ctx->Kd, ctx->d_Lcat, ctx->Kd, out,
-                       ctx->n_chol, st);
+        rc = gemm_zd(ctx, nw, ctx->n_chol, (int)ctx->Kd, (const double2*)f.GT, ctx->Kd, ctx->d_Lcat, ctx->Kd,
+                     ctx->dg_Lcat, out, ctx->n_chol, st);
         th.end(st);
+        if (rc) return rc;
     }
     CKLAUNCH();
     return MSD_OK;
@@ -1139,7 +1213,13 @@ size_t en_bytes_per_walker(msd_ctx* ctx, bool fp32)
         }
         b += f + a;
     } else {
-        for (int s = 0; s < 2; ++s) b += sizeof(double2) * T1[s].N * (size_t)G * (T1[s].N + T1[s].np);
+        size_t d = 0;
+        for (int s = 0; s < 2; ++s) {
+            const int NC = T1[s].N + T1[s].np;
+            b += sizeof(double2) * T1[s].N * (size_t)G * NC;
+            d = std::max(d, dg_bytes((long long)G * NC, ctx->M, T1[s].N));
+        }
+        b += d;
     }
     return b;
 }
@@ -1252,9 +1332,10 @@ int en_fepi(msd_ctx* ctx, Chunk& c, EnWork& E, int nw, int cap, bool fp32, cudaS
             th.end(st);
         } else {
             th.begin("k_gemm_F", st);
-            launch_gemm_zd(nw * N, G * NC[s], M, c.Gr[s], M, ctx->sp[s].d_Lh, M, (double2*)E.F[s],
-                           (long long)G * NC[s], st);
+            const int g = gemm_zd(ctx, nw * N, G * NC[s], M, c.Gr[s], M, ctx->sp[s].d_Lh, M, ctx->dg_Lh[s],
+                                  (double2*)E.F[s], (long long)G * NC[s], st);
             th.end(st);
+            if (g) return g;
             th.begin("k_fepi", st);
             launch_fepi(T[s], nw, M, G, (double2*)E.F[s], (long long)G * NC[s], c.Gr[s], (double2*)E.v0[s],
                         (double2*)E.xx[s], (double2*)E.La[s], (double2*)E.Xi[s], st);
@@ -1620,6 +1701,7 @@ void free_prop(msd_ctx* ctx)
 {
     cudaFree(ctx->d_Lt);
     ctx->d_Lt = nullptr;
+    free_dg(ctx->dg_Lt);
     for (int s = 0; s < 2; ++s) { cudaFree(ctx->d_E[s]); ctx->d_E[s] = nullptr; }
     ctx->h_corr.clear();
     ctx->prop_dt = -1.0;
@@ -1725,7 +1807,7 @@ int propagate(msd_ctx* ctx, int n_w, double* phi_a, double* phi_b, double* weigh
     launch_prop_coef(n_w, G, dt, x, (const double2*)vb, (double2*)cf, (double2*)ex, st);
     th.end(st);
     // B(x - xbar) on walker chunks: V, half steps, Taylor series
-    const size_t per = sizeof(double2) * ((size_t)M * M + 3 * (size_t)M * Nm);
+    const size_t per = sizeof(double2) * ((size_t)M * M + 3 * (size_t)M * Nm) + dg_bytes((long long)M * M, G, 1);
     const int cap = (int)std::max<size_t>(1, std::min<size_t>((size_t)n_w, ctx->ws_limit / 2 / per));
     void *V, *t0, *t1, *ac;
     if ((rc = arena_get(ctx, "pr_V", sizeof(double2) * (size_t)cap * M * M, &V))) return rc;
@@ -1735,9 +1817,10 @@ int propagate(msd_ctx* ctx, int n_w, double* phi_a, double* phi_b, double* weigh
     for (int w0 = 0; w0 < n_w; w0 += cap) {
         const int nw = std::min(cap, n_w - w0);
         th.begin("k_gemm_V", st);
-        launch_gemm_zd(nw, M * M, G, (const double2*)cf + (size_t)w0 * G, G, ctx->d_Lt, G, (double2*)V,
-                       (long long)M * M, st);
+        rc = gemm_zd(ctx, nw, M * M, G, (const double2*)cf + (size_t)w0 * G, G, ctx->d_Lt, G, ctx->dg_Lt, (double2*)V,
+                     (long long)M * M, st);
         th.end(st);
+        if (rc) return rc;
         for (int s = 0; s < 2; ++s) {
             const int N = ctx->n[s];
             double2* phi = (double2*)(s ? phi_b : phi_a) + (size_t)w0 * M * N;
