@@ -121,21 +121,32 @@ struct DgOperand {
     int batch_rows = 0;
 };
 // C[z c_batch + n c_n + m c_m] = mul sum_k A_z[m][k] B_z[n][k], m < Mr rows of
-// A, n < Nc complex rows of B; acc (optional, same layout) += C. With splits >
-// 1 (batch must be 1) the contraction is divided and split z writes its part at
-// z c_batch, for dg_sum_splits.
+// A, n < Nc complex rows of B; acc (optional, same layout) = acc_in + C. With
+// splits > 1 (batch must be 1) the contraction is divided and split z writes its
+// part at z c_batch, for dg_sum_splits. gx >= 0: the rows of A and B stack gx
+// alpha and gy beta entries, and the (alpha, alpha), (beta, beta) and (alpha,
+// beta) blocks go to K[0], K[2], K[1] ([batch][rows][columns] each) instead of C.
 struct DgOut {
     int Mr = 0, Nc = 0, batch = 1, splits = 1;
     double2* C = nullptr;
     long long c_batch = 0, c_n = 0, c_m = 1;
     double2* acc = nullptr;
+    const double2* acc_in = nullptr;
     double mul = 1.0;
+    int gx = -1, gy = 0;
+    double2* K[3] = {nullptr, nullptr, nullptr};
 };
 int dg_k_padded(int K);
 size_t dg_row_bytes(int K);              // slices and exponent of one real row
 int dg_splits(int Mr, int K);
 void dg_slice_real(long long R, int K, const double* src, long long ld, void* S, int* ex, cudaStream_t st);
 void dg_slice_complex(long long R, int K, const double2* src, long long ld, void* S, int* ex, cudaStream_t st);
+// Columns of src[z][k][c] (k < K, c < nc) as the operand rows z rows + row0 + c:
+// mode 0 a left operand (Sa, length 2 K) and the matching complex right operand
+// (Sb, two rows each), mode 1 the right operand alone, mode 2 the two parts as
+// plain rows of length K (Sb).
+void dg_slice_columns(int mode, int K, int nc, int batch, const double2* src, long long ld, long long src_batch,
+                      int row0, int rows, void* Sa, int* ea, void* Sb, int* eb, cudaStream_t st);
 int dg_gemm(const DgOperand& A, const DgOperand& B, const DgOut& o, int K, unsigned* err, cudaStream_t st);
 void dg_sum_splits(int R, int Cc, int splits, const double2* part, double2* out, long long ldo, cudaStream_t st);
 

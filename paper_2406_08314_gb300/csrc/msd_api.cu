@@ -185,7 +185,8 @@ struct msd_ctx {
     double prop_dt = -1.0;
     // FP64 contractions on the tensor cores: the half-rotated Cholesky rows per
     // spin, both spins' rows concatenated, the transposed Cholesky vectors
-    DgConst dg_Lh[2], dg_Lcat, dg_Lt;
+    // and exp(-dt h'/2)
+    DgConst dg_Lh[2], dg_Lcat, dg_Lt, dg_E[2];
 };
 
 namespace {
@@ -311,25 +312,31 @@ size_t dg_bytes(long long rows, int K, int complex_rows)
     return dg_use(rows, K) ? 2 * dg_row_bytes(K) * (size_t)complex_rows : 0;
 }
 
+// Slices of a constant real [rows][K] operand on first use; false where their
+// memory cannot be had (the FP64 kernels run then).
+bool dg_ready(DgConst& c, long long rows, int K, const double* src, long long ld, cudaStream_t st)
+{
+    if (!c.tried) {
+        c.tried = true;
+        if (cudaMalloc(&c.s, dg_row_bytes(K) * (size_t)rows) != cudaSuccess ||
+            cudaMalloc((void**)&c.e, sizeof(int) * (size_t)rows) != cudaSuccess) {
+            cudaGetLastError();
+            free_dg(c);
+            c.tried = true;
+        } else {
+            dg_slice_real(rows, K, src, ld, c.s, c.e, st);
+            cudaStreamSynchronize(st);   // other streams may use the slices next
+        }
+    }
+    return c.s != nullptr;
+}
+
 // C[m][n] = sum_k A[m][k] B[n][k] in FP64: A Mr complex rows (walkers), B the
-// constant real operand [Nc][K] whose slices `cB` keeps. Where the slices' memory
-// cannot be had, the FP64 kernel runs.
+// constant real operand [Nc][K] whose slices `cB` keeps.
 int gemm_zd(msd_ctx* ctx, int Mr, int Nc, int K, const double2* A, long long lda, const double* B, long long ldb,
             DgConst& cB, double2* C, long long ldc, cudaStream_t st)
 {
-    if (dg_use(Nc, K) && !cB.tried) {
-        cB.tried = true;
-        if (cudaMalloc(&cB.s, dg_row_bytes(K) * (size_t)Nc) != cudaSuccess ||
-            cudaMalloc((void**)&cB.e, sizeof(int) * (size_t)Nc) != cudaSuccess) {
-            cudaGetLastError();
-            free_dg(cB);
-            cB.tried = true;
-        } else {
-            dg_slice_real(Nc, K, B, ldb, cB.s, cB.e, st);
-            CK(cudaStreamSynchronize(st));   // other streams may use the slices next
-        }
-    }
-    if (!dg_use(Nc, K) || !cB.s) {
+    if (!dg_use(Nc, K) || !dg_ready(cB, Nc, K, B, ldb, st)) {
         launch_gemm_zd(Mr, Nc, K, A, lda, B, ldb, C, ldc, st);
         return MSD_OK;
     }
@@ -348,6 +355,37 @@ int gemm_zd(msd_ctx* ctx, int Mr, int Nc, int K, const double2* A, long long lda
     if (dg_gemm({cB.s, cB.e, Nc, 0}, {s, (int*)e, 2 * Mr, 0}, o, K, ctx->d_err, st))
         return fail(ctx, MSD_ERR_CUDA, "FP64 tensor-core contraction launch failed");
     if (splits > 1) dg_sum_splits(Mr, Nc, splits, (const double2*)part, C, ldc, st);
+    return MSD_OK;
+}
+
+// The FP64 Gram matrices of a walker, (Xa + Xb)^2 products of length n_chol, run
+// on the tensor cores from this size on (as dg_use: by shape only).
+bool dg_gram_use(int Xa, int Xb, int G) { return (long long)(Xa + Xb) * (Xa + Xb) * G >= 262144; }
+size_t dg_gram_bytes(int Xa, int Xb, int G)
+{
+    return dg_gram_use(Xa, Xb, G) ? 3 * (size_t)(Xa + Xb) * dg_row_bytes(2 * G) : 0;
+}
+
+// K_aa, K_bb, K_ab of nw walkers from the Lambda rows [w][g][x] of both spins.
+int dg_gram(msd_ctx* ctx, int nw, int Xa, int Xb, const double2* La, const double2* Lb, double2* Kaa, double2* Kbb,
+            double2* Kab, cudaStream_t st)
+{
+    const int G = ctx->n_chol, X = Xa + Xb;
+    const long long rows = (long long)nw * X;
+    int rc;
+    void *sa, *ea, *sb, *eb;
+    if ((rc = arena_get(ctx, "dg_s", dg_row_bytes(2 * G) * 2 * rows, &sb))) return rc;
+    if ((rc = arena_get(ctx, "dg_e", sizeof(int) * 2 * rows, &eb))) return rc;
+    if ((rc = arena_get(ctx, "dg_sa", dg_row_bytes(2 * G) * rows, &sa))) return rc;
+    if ((rc = arena_get(ctx, "dg_ea", sizeof(int) * rows, &ea))) return rc;
+    dg_slice_columns(0, G, Xa, nw, La, Xa, (long long)G * Xa, 0, X, sa, (int*)ea, sb, (int*)eb, st);
+    dg_slice_columns(0, G, Xb, nw, Lb, Xb, (long long)G * Xb, Xa, X, sa, (int*)ea, sb, (int*)eb, st);
+    DgOut o;
+    o.Mr = o.Nc = X; o.batch = nw;
+    o.gx = Xa; o.gy = Xb;
+    o.K[0] = Kaa; o.K[1] = Kab; o.K[2] = Kbb;
+    if (dg_gemm({sa, (int*)ea, (int)rows, X}, {sb, (int*)eb, (int)(2 * rows), 2 * X}, o, 2 * G, ctx->d_err, st))
+        return fail(ctx, MSD_ERR_CUDA, "FP64 tensor-core Gram launch failed");
     return MSD_OK;
 }
 
@@ -1219,7 +1257,7 @@ size_t en_bytes_per_walker(msd_ctx* ctx, bool fp32)
             b += sizeof(double2) * T1[s].N * (size_t)G * NC;
             d = std::max(d, dg_bytes((long long)G * NC, ctx->M, T1[s].N));
         }
-        b += d;
+        b += std::max(d, dg_gram_bytes(X[0], X[1], G));
     }
     return b;
 }
@@ -1413,6 +1451,10 @@ int en_rest(msd_ctx* ctx, Chunk& c, EnWork& E, int nw, int cap, bool fp32, cudaS
         } else {
             launch_gram_f32(nw, G, jobs, 3, st);
         }
+    } else if (dg_gram_use(X[0], X[1], G)) {
+        const int g = dg_gram(ctx, nw, X[0], X[1], (double2*)E.La[0], (double2*)E.La[1], (double2*)E.Kaa,
+                              (double2*)E.Kbb, (double2*)E.Kab, st);
+        if (g) return g;
     } else {
         launch_gram(nw, X[0], X[0], G, (double2*)E.La[0], (double2*)E.La[0], E.Kaa, false, st);
         launch_gram(nw, X[1], X[1], G, (double2*)E.La[1], (double2*)E.La[1], E.Kbb, false, st);
@@ -1702,7 +1744,7 @@ void free_prop(msd_ctx* ctx)
     cudaFree(ctx->d_Lt);
     ctx->d_Lt = nullptr;
     free_dg(ctx->dg_Lt);
-    for (int s = 0; s < 2; ++s) { cudaFree(ctx->d_E[s]); ctx->d_E[s] = nullptr; }
+    for (int s = 0; s < 2; ++s) { cudaFree(ctx->d_E[s]); ctx->d_E[s] = nullptr; free_dg(ctx->dg_E[s]); }
     ctx->h_corr.clear();
     ctx->prop_dt = -1.0;
 }
@@ -1771,10 +1813,57 @@ int prepare_prop(msd_ctx* ctx, double dt, cudaStream_t st)
                 a[e] = -0.5 * dt * (ctx->h_h1[(size_t)s * M * M + e] - 0.5 * ctx->h_corr[e]);
             int rc = upload(ctx, &ctx->d_E[s], expm_host(a, M));
             if (rc) return rc;
+            free_dg(ctx->dg_E[s]);
         }
         ctx->prop_dt = dt;
     }
     return MSD_OK;
+}
+
+// The propagator's products run on the tensor cores from this orbital count on:
+// a walker's V is one 128-row tile of the 2 M long contraction, mostly padding
+// below it.
+bool dg_apply_use(int M) { return M >= 32; }
+
+// E T_n(V) E phi of nw walkers on the tensor cores, both spins in one product
+// per Taylor term: cur, nxt, acc [nw][M][Na + Nb].
+int apply_tc(msd_ctx* ctx, int nw, const double2* V, double2* const phi[2], double2* cur, double2* nxt, double2* acc,
+             int order, cudaStream_t st)
+{
+    const int M = ctx->M, Nt = ctx->n[0] + ctx->n[1];
+    const long long mn = (long long)M * Nt;
+    int rc;
+    void *sa, *ea, *sb, *eb;
+    if ((rc = arena_get(ctx, "dg_s", dg_row_bytes(2 * M) * 2 * (size_t)Nt * nw, &sb))) return rc;
+    if ((rc = arena_get(ctx, "dg_e", sizeof(int) * 2 * (size_t)Nt * nw, &eb))) return rc;
+    if ((rc = arena_get(ctx, "dg_sa", dg_row_bytes(2 * M) * (size_t)M * nw, &sa))) return rc;
+    if ((rc = arena_get(ctx, "dg_ea", sizeof(int) * (size_t)M * nw, &ea))) return rc;
+    auto half = [&](const double2* src, long long lds, long long src_batch, int s, double2* dst, long long ldd,
+                    long long dst_batch) {
+        const int N = ctx->n[s];
+        dg_slice_columns(2, M, N, nw, src, lds, src_batch, 0, N, nullptr, nullptr, sb, (int*)eb, st);
+        DgOut o;
+        o.Mr = M; o.Nc = N; o.batch = nw;
+        o.C = dst; o.c_batch = dst_batch; o.c_n = 1; o.c_m = ldd;
+        return dg_gemm({ctx->dg_E[s].s, ctx->dg_E[s].e, M, 0}, {sb, (int*)eb, 2 * N * nw, 2 * N}, o, M, ctx->d_err, st);
+    };
+    int g = 0;
+    for (int s = 0; s < 2 && !g; ++s)
+        g = half(phi[s], ctx->n[s], (long long)M * ctx->n[s], s, cur + (s ? ctx->n[0] : 0), Nt, mn);
+    dg_slice_real((long long)nw * M, 2 * M, (const double*)V, 2 * M, sa, (int*)ea, st);
+    for (int k = 1; k <= order && !g; ++k) {
+        dg_slice_columns(1, M, Nt, nw, cur, Nt, mn, 0, Nt, nullptr, nullptr, sb, (int*)eb, st);
+        DgOut o;
+        o.Mr = M; o.Nc = Nt; o.batch = nw;
+        o.C = nxt; o.c_batch = mn; o.c_n = 1; o.c_m = Nt;
+        o.acc = acc; o.acc_in = k == 1 ? cur : acc;
+        o.mul = 1.0 / k;
+        g = dg_gemm({sa, (int*)ea, nw * M, M}, {sb, (int*)eb, 2 * Nt * nw, 2 * Nt}, o, 2 * M, ctx->d_err, st);
+        std::swap(cur, nxt);
+    }
+    for (int s = 0; s < 2 && !g; ++s)
+        g = half(acc + (s ? ctx->n[0] : 0), Nt, mn, s, phi[s], ctx->n[s], (long long)M * ctx->n[s]);
+    return g ? fail(ctx, MSD_ERR_CUDA, "propagator tensor-core launch failed") : MSD_OK;
 }
 
 int propagate(msd_ctx* ctx, int n_w, double* phi_a, double* phi_b, double* weights, const double* x, double dt,
@@ -1807,13 +1896,17 @@ int propagate(msd_ctx* ctx, int n_w, double* phi_a, double* phi_b, double* weigh
     launch_prop_coef(n_w, G, dt, x, (const double2*)vb, (double2*)cf, (double2*)ex, st);
     th.end(st);
     // B(x - xbar) on walker chunks: V, half steps, Taylor series
-    const size_t per = sizeof(double2) * ((size_t)M * M + 3 * (size_t)M * Nm) + dg_bytes((long long)M * M, G, 1);
+    bool tc = dg_apply_use(M);
+    for (int s = 0; s < 2 && tc; ++s) tc = dg_ready(ctx->dg_E[s], M, M, ctx->d_E[s], M, st);
+    const int Nt = ctx->n[0] + ctx->n[1], Nw = tc ? Nt : Nm;   // columns of the work arrays
+    const size_t per = sizeof(double2) * ((size_t)M * M + 3 * (size_t)M * Nw) +
+                       std::max(dg_bytes((long long)M * M, G, 1), tc ? dg_row_bytes(2 * M) * (M + 2 * (size_t)Nt) : 0);
     const int cap = (int)std::max<size_t>(1, std::min<size_t>((size_t)n_w, ctx->ws_limit / 2 / per));
     void *V, *t0, *t1, *ac;
     if ((rc = arena_get(ctx, "pr_V", sizeof(double2) * (size_t)cap * M * M, &V))) return rc;
-    if ((rc = arena_get(ctx, "pr_t0", sizeof(double2) * (size_t)cap * M * Nm, &t0))) return rc;
-    if ((rc = arena_get(ctx, "pr_t1", sizeof(double2) * (size_t)cap * M * Nm, &t1))) return rc;
-    if ((rc = arena_get(ctx, "pr_acc", sizeof(double2) * (size_t)cap * M * Nm, &ac))) return rc;
+    if ((rc = arena_get(ctx, "pr_t0", sizeof(double2) * (size_t)cap * M * Nw, &t0))) return rc;
+    if ((rc = arena_get(ctx, "pr_t1", sizeof(double2) * (size_t)cap * M * Nw, &t1))) return rc;
+    if ((rc = arena_get(ctx, "pr_acc", sizeof(double2) * (size_t)cap * M * Nw, &ac))) return rc;
     for (int w0 = 0; w0 < n_w; w0 += cap) {
         const int nw = std::min(cap, n_w - w0);
         th.begin("k_gemm_V", st);
@@ -1821,6 +1914,15 @@ int propagate(msd_ctx* ctx, int n_w, double* phi_a, double* phi_b, double* weigh
                      (long long)M * M, st);
         th.end(st);
         if (rc) return rc;
+        if (tc) {
+            double2* const phi[2] = {(double2*)phi_a + (size_t)w0 * M * ctx->n[0], (double2*)phi_b + (size_t)w0 * M * ctx->n[1]};
+            th.begin("k_apply_rows", st);
+            rc = apply_tc(ctx, nw, (const double2*)V, phi, (double2*)t0, (double2*)t1, (double2*)ac, order, st);
+            th.end(st);
+            if (rc) return rc;
+            CKLAUNCH();
+            continue;
+        }
         for (int s = 0; s < 2; ++s) {
             const int N = ctx->n[s];
             double2* phi = (double2*)(s ? phi_b : phi_a) + (size_t)w0 * M * N;

@@ -76,8 +76,13 @@ struct DgArgs {
     const int* eb;           // [b_rows]
     double2* C;              // C[z c_batch + n c_n + m c_m], z = batch entry or split
     long long c_batch, c_n, c_m;
-    double2* acc;            // optional, same layout: acc += C
+    double2* acc;            // optional, same layout: acc = acc_in + C
+    const double2* acc_in;
     double mul;              // C = mul (A B)
+    // Gram form (gx >= 0): rows and columns stack gx alpha and gy beta entries;
+    // the (alpha, alpha), (alpha, beta) and (beta, beta) blocks go to K[0..2]
+    int gx, gy;
+    double2* K[3];
     unsigned* err;
 };
 
@@ -136,6 +141,13 @@ __device__ __forceinline__ DgTile dg_tile(const DgArgs& a, int t)
     return {(g * DG_GROUP + r % gm) * DG_BM, (r / gm) * DG_BN, z};
 }
 
+// Tiles of the Gram form that hold only the (beta, alpha) block, which nobody
+// reads.
+__device__ __forceinline__ bool dg_skip(const DgArgs& a, const DgTile& t)
+{
+    return a.gx >= 0 && t.m0 >= a.gx && t.n0 + DG_BN <= 2 * a.gx;
+}
+
 __global__ void __launch_bounds__(DG_THREADS, 1)
 k_tc_dgemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb,
            const __grid_constant__ DgArgs a)
@@ -179,6 +191,7 @@ k_tc_dgemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUten
             bool ok = true;
             for (int t = blockIdx.x; t < ntile && ok; t += gridDim.x) {
                 const DgTile q = dg_tile(a, t);
+                if (dg_skip(a, q)) continue;
                 const int bz = a.splits > 1 ? 0 : q.z, ke = kend(q.z);
                 const int ra = bz * a.a_batch + q.m0, rb = bz * a.b_batch + q.n0;
                 for (int kb = kbeg(q.z); kb < ke; ++kb, ++it) {
@@ -205,7 +218,9 @@ k_tc_dgemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUten
             bool ok = true;
             int it = 0, unit = 0;   // unit: one chunk of one tile, one use of the accumulators
             for (int t = blockIdx.x; t < ntile && ok; t += gridDim.x) {
-                const int z = dg_tile(a, t).z, k1 = kend(z);
+                const DgTile tl = dg_tile(a, t);
+                if (dg_skip(a, tl)) continue;
+                const int z = tl.z, k1 = kend(z);
                 for (int c0 = kbeg(z); c0 < k1 && ok; c0 += DG_CHUNK, ++unit) {
                     const int c1 = min(k1, c0 + DG_CHUNK);
                     for (int kb = c0; kb < c1; ++kb, ++it) {
@@ -258,6 +273,7 @@ k_tc_dgemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUten
         int unit = 0;
         for (int t = blockIdx.x; t < ntile && ok; t += gridDim.x) {
             const DgTile tl = dg_tile(a, t);
+            if (dg_skip(a, tl)) continue;
             long long hi[DG_HALF], lo[DG_HALF];
 #pragma unroll
             for (int i = 0; i < DG_HALF; ++i) hi[i] = lo[i] = 0;
@@ -301,10 +317,20 @@ k_tc_dgemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUten
                         double2 v = make_double2(dg_value(hi[i], lo[i], ea + ebp[n2]),
                                                  dg_value(hi[i + 1], lo[i + 1], ea + ebp[n2 + 1]));
                         if (a.mul != 1.0) v = make_double2(v.x * a.mul, v.y * a.mul);
+                        if (a.gx >= 0) {
+                            const int X = a.gx, Y = a.gy;
+                            if (n >= X) {
+                                if (m < X) a.K[1][((size_t)tl.z * X + m) * Y + n - X] = v;
+                                else a.K[2][((size_t)tl.z * Y + m - X) * Y + n - X] = v;
+                            } else if (m < X) {
+                                a.K[0][((size_t)tl.z * X + m) * X + n] = v;
+                            }
+                            continue;
+                        }
                         const long long o = o0 + (long long)n * a.c_n;
                         a.C[o] = v;
                         if (a.acc) {
-                            const double2 p = a.acc[o];
+                            const double2 p = a.acc_in[o];
                             a.acc[o] = make_double2(p.x + v.x, p.y + v.y);
                         }
                     }
@@ -342,13 +368,13 @@ __device__ __forceinline__ long long dg_fixed(double x, int e)
     return b < 0 ? -m : m;
 }
 
-// The eight digits of eight fixed-point values, as BF16: out[i * stride] holds
-// digit i (most significant first) of the eight.
-__device__ __forceinline__ void dg_store8(long long* q, __nv_bfloat16* out, size_t stride)
+// The eight digits of eight fixed-point values as BF16: u[i] packs digit i (most
+// significant first) of the eight.
+__device__ __forceinline__ void dg_digits8(long long* q, uint4* u)
 {
 #pragma unroll
     for (int i = DG_S - 1; i >= 0; --i) {
-        uint32_t u[4];
+        uint32_t w[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             uint32_t h[2];
@@ -365,10 +391,19 @@ __device__ __forceinline__ void dg_store8(long long* q, __nv_bfloat16* out, size
                 // d as a float through the integer part of 1.5 2^23 + d
                 h[k] = __float_as_uint(__uint_as_float(0x4b400000u + (uint32_t)d) - 12582912.f);
             }
-            u[j] = __byte_perm(h[0], h[1], 0x7632);
+            w[j] = __byte_perm(h[0], h[1], 0x7632);
         }
-        *reinterpret_cast<uint4*>(out + (size_t)i * stride) = make_uint4(u[0], u[1], u[2], u[3]);
+        u[i] = make_uint4(w[0], w[1], w[2], w[3]);
     }
+}
+
+// ... stored at out[i * stride].
+__device__ __forceinline__ void dg_store8(long long* q, __nv_bfloat16* out, size_t stride)
+{
+    uint4 u[DG_S];
+    dg_digits8(q, u);
+#pragma unroll
+    for (int i = 0; i < DG_S; ++i) *reinterpret_cast<uint4*>(out + (size_t)i * stride) = u[i];
 }
 
 __device__ __forceinline__ unsigned dg_mag(double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; }
@@ -427,6 +462,95 @@ k_dg_rows(long long R, int K, int Kp, const double* __restrict__ src, long long 
     }
 }
 
+// Columns of a complex matrix src[z][k][c] (row stride ld, batch stride
+// src_batch) as operand rows, one per column, batch entry z's rows from z *
+// rows + row0 on. MODE 0 writes the row of a left operand, k' = 2 k + part
+// (re, im interleaved), to Sa and the two rows of a right operand that make the
+// real and the imaginary part of its complex product with such a row,
+// (re, -im) and (im, re), to Sb; MODE 1 only the latter; MODE 2 the real and the
+// imaginary part as plain rows (for a real left operand) to Sb. All rows of a
+// column share its exponent. One block per 16 columns: a pass for the
+// exponents, then tiles of 64 k staged in shared memory, so that reads run
+// along c and the 16-byte digit stores along k.
+template <int MODE>
+__global__ void __launch_bounds__(256)
+k_dg_cols(int K, int Kp, int nc, const double2* __restrict__ src, long long ld, long long src_batch, int row0, int rows,
+          __nv_bfloat16* __restrict__ Sa, int* __restrict__ ea, size_t stride_a, __nv_bfloat16* __restrict__ Sb,
+          int* __restrict__ eb, size_t stride_b)
+{
+    constexpr int TK = MODE == 2 ? 128 : 64;   // k per staged tile
+    __shared__ double2 tile[TK][17];
+    __shared__ unsigned top[16][17];
+    __shared__ int ex[16];
+    const int z = blockIdx.y, c0 = blockIdx.x * 16, t = threadIdx.x, cl = t & 15, kl = t >> 4;
+    const double2* s = src + (size_t)z * src_batch;
+    unsigned mx = 0;
+    if (c0 + cl < nc)
+        for (int k = kl; k < K; k += 16) {
+            const double2 v = s[(size_t)k * ld + c0 + cl];
+            mx = max(mx, max(dg_mag(v.x), dg_mag(v.y)));
+        }
+    top[kl][cl] = mx;
+    __syncthreads();
+    if (t < 16) {
+        for (int i = 1; i < 16; ++i) mx = max(mx, top[i][t]);
+        ex[t] = dg_exponent(mx);
+        if (c0 + t < nc) {
+            const size_t r = (size_t)z * rows + row0 + c0 + t;
+            if (MODE == 0) ea[r] = ex[t];
+            eb[2 * r] = eb[2 * r + 1] = ex[t];
+        }
+    }
+    __syncthreads();
+    // an item is 8 consecutive elements of an operand row: 4 complex k (modes 0,
+    // 1) or 8 k of one part (mode 2)
+    const int ci = t >> 4, gi = t & 15, e = ex[ci];
+    const size_t r = (size_t)z * rows + row0 + c0 + ci;
+    const int Kk = MODE == 2 ? Kp : Kp / 2;
+    for (int k0 = 0; k0 < Kk; k0 += TK) {
+        for (int kk = kl; kk < TK; kk += 16)
+            tile[kk][cl] = (k0 + kk < K && c0 + cl < nc) ? s[(size_t)(k0 + kk) * ld + c0 + cl] : make_double2(0, 0);
+        __syncthreads();
+        if (c0 + ci < nc) {
+            if (MODE == 2) {
+                const int kb = gi * 8;
+                if (k0 + kb < Kp)
+                    for (int part = 0; part < 2; ++part) {
+                        long long q[8];
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) q[j] = dg_fixed(part ? tile[kb + j][ci].y : tile[kb + j][ci].x, e);
+                        dg_store8(q, Sb + (2 * r + part) * Kp + k0 + kb, stride_b);
+                    }
+            } else {
+                const int kb = gi * 4;
+                if (2 * (k0 + kb) < Kp) {
+                    long long q[8];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        q[2 * j] = dg_fixed(tile[kb + j][ci].x, e);
+                        q[2 * j + 1] = dg_fixed(tile[kb + j][ci].y, e);
+                    }
+                    const size_t o = (size_t)2 * (k0 + kb);
+                    uint4 u[DG_S];
+                    dg_digits8(q, u);
+#pragma unroll
+                    for (int i = 0; i < DG_S; ++i) {
+                        if (MODE == 0) *reinterpret_cast<uint4*>(Sa + i * stride_a + r * Kp + o) = u[i];
+                        // (re, -im): the sign of the odd digits; (im, re): halves swapped
+                        __nv_bfloat16* b = Sb + i * stride_b + 2 * r * Kp + o;
+                        *reinterpret_cast<uint4*>(b) = make_uint4(u[i].x ^ 0x80000000u, u[i].y ^ 0x80000000u,
+                                                                  u[i].z ^ 0x80000000u, u[i].w ^ 0x80000000u);
+                        *reinterpret_cast<uint4*>(b + Kp) =
+                            make_uint4(__byte_perm(u[i].x, 0, 0x1032), __byte_perm(u[i].y, 0, 0x1032),
+                                       __byte_perm(u[i].z, 0, 0x1032), __byte_perm(u[i].w, 0, 0x1032));
+                    }
+                }
+            }
+        }
+        __syncthreads();
+    }
+}
+
 // out[r ldo + c] = sum over splits of part[split][r][c], in split order.
 __global__ void k_dg_sum(int R, int Cc, int splits, const double2* __restrict__ part, double2* __restrict__ out,
                          long long ldo)
@@ -456,6 +580,20 @@ void dg_slice_complex(long long R, int K, const double2* src, long long ld, void
     const int Kp = dg_k_padded(K);
     k_dg_rows<true><<<(unsigned)((R + 7) / 8), 256, 0, st>>>(R, K, Kp, (const double*)src, ld, (__nv_bfloat16*)S, ex,
                                                              (size_t)2 * R * Kp);
+    msd_note_launch();
+}
+
+void dg_slice_columns(int mode, int K, int nc, int batch, const double2* src, long long ld, long long src_batch,
+                      int row0, int rows, void* Sa, int* ea, void* Sb, int* eb, cudaStream_t st)
+{
+    if (nc <= 0 || batch <= 0) return;
+    const int Kp = dg_k_padded(mode == 2 ? K : 2 * K);
+    const size_t sa = (size_t)batch * rows * Kp, sb = 2 * sa;
+    const dim3 grid((nc + 15) / 16, batch);
+    __nv_bfloat16 *a = (__nv_bfloat16*)Sa, *b = (__nv_bfloat16*)Sb;
+    if (mode == 0) k_dg_cols<0><<<grid, 256, 0, st>>>(K, Kp, nc, src, ld, src_batch, row0, rows, a, ea, sa, b, eb, sb);
+    else if (mode == 1) k_dg_cols<1><<<grid, 256, 0, st>>>(K, Kp, nc, src, ld, src_batch, row0, rows, a, ea, sa, b, eb, sb);
+    else k_dg_cols<2><<<grid, 256, 0, st>>>(K, Kp, nc, src, ld, src_batch, row0, rows, a, ea, sa, b, eb, sb);
     msd_note_launch();
 }
 
@@ -489,7 +627,9 @@ int dg_gemm(const DgOperand& A, const DgOperand& B, const DgOut& o, int K, unsig
     a.batch = o.batch;
     a.ea = A.e; a.eb = B.e;
     a.C = o.C; a.c_batch = o.c_batch; a.c_n = o.c_n; a.c_m = o.c_m;
-    a.acc = o.acc; a.mul = o.mul; a.err = err;
+    a.acc = o.acc; a.acc_in = o.acc_in; a.mul = o.mul; a.err = err;
+    a.gx = o.gx; a.gy = o.gy;
+    for (int i = 0; i < 3; ++i) a.K[i] = o.K[i];
     const long long tiles = (long long)a.mt * a.nt * a.batch * a.splits;
     if (tiles <= 0) return 0;
     if (tiles > 0x7fffffffll) return -1;
