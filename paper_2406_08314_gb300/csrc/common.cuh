@@ -90,6 +90,9 @@ struct SpinTables {
     const uint4* str_hp;   // [n_str] one 16-byte record per string: hole indices (0..nh-1,
                            // ascending) in bytes 0..5, particle indices (0..np-1,
                            // ascending) in bytes 8..13, so one vector load fetches both
+    const int* sub;        // [n_str][MSD_KMAX] of a level >= 4 string: the strings without its last hole
+                           // and its j-th particle, (index << 1 | sign of the term), -1 first if one
+                           // of them is not in the trial
     const int8_t* str_sign;    // [n_str] parity of the in-place -> sorted reordering
     const int* csr_off;    // [n_str+1] determinants containing each string
     const int* csr_other;  // [nnz] string of the opposite spin in that determinant
@@ -108,10 +111,28 @@ struct SpinTables {
 // and two entries load as one 16-byte vector (the pad entry is zero).
 __host__ __device__ __forceinline__ constexpr int b_stride(int k) { return k * k + (k & 1); }
 
+// Index of the pair (a, b), a < b < n, among the n (n - 1) / 2 pairs in
+// lexicographic order.
+__host__ __device__ __forceinline__ int pair_index(int a, int b, int n) { return a * n - a * (a + 1) / 2 + (b - a - 1); }
+
 // Hole / particle index i (< MSD_KMAX) of a string record.
 __device__ __forceinline__ int rec_h(const uint4& r, int i) { return (int)(((i < 4 ? r.x : r.y) >> (8 * (i & 3))) & 0xffu); }
 __device__ __forceinline__ int rec_p(const uint4& r, int i) { return (int)(((i < 4 ? r.z : r.w) >> (8 * (i & 3))) & 0xffu); }
 
+
+#ifdef __CUDACC__
+// Sum of n partial sums by one warp (every lane returns it).
+__device__ __forceinline__ double2 warp_sum_slots(const double2* __restrict__ p, int n, int lane)
+{
+    double2 a = make_double2(0, 0);
+    for (int i = lane; i < n; i += 32) a = cadd(a, p[i]);
+    for (int o = 16; o; o >>= 1) {
+        a.x += __shfl_xor_sync(0xffffffffu, a.x, o);
+        a.y += __shfl_xor_sync(0xffffffffu, a.y, o);
+    }
+    return a;
+}
+#endif
 
 // Pair (determinant) tables for the opposite-spin cross term.
 struct PairTables {

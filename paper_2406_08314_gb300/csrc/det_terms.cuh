@@ -43,10 +43,6 @@ __device__ __forceinline__ void load_minor(const cplx_t<T>* __restrict__ B, cplx
     }
 }
 
-// Index of the pair (a, b), a < b < n, among the n (n - 1) / 2 pairs in
-// lexicographic order.
-__host__ __device__ __forceinline__ int pair_index(int a, int b, int n) { return a * n - a * (a + 1) / 2 + (b - a - 1); }
-
 // e_s of string s = bucket[KL] + sl (unweighted); string_energy_term below
 // multiplies it by r_s w_s. K is symmetric (a same-spin Gram matrix), so
 //   A[h,h';p,p'] = K[(h,p)][(h',p')] - K[(h,p')][(h',p)]

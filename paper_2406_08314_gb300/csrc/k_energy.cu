@@ -523,11 +523,11 @@ __global__ void k_final(int nw, const double2* __restrict__ part, int nslot, int
                         const double2* __restrict__ O0b, double2* __restrict__ eloc,
                         double2* __restrict__ ovlp)
 {
-    const int w = blockIdx.x * blockDim.x + threadIdx.x;
+    const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;   // one warp per walker
     if (w >= nw) return;
-    double2 R = cz(0, 0), S = cz(0, 0);
-    for (int i = 0; i < nR; ++i) R = cadd(R, part[(size_t)w * nslot + i]);
-    for (int i = nR; i < nslot; ++i) S = cadd(S, part[(size_t)w * nslot + i]);
+    const double2 R = warp_sum_slots(part + (size_t)w * nslot, nR, lane);
+    const double2 S = warp_sum_slots(part + (size_t)w * nslot + nR, nslot - nR, lane);
+    if (lane) return;
     const double2* sc = scal + (size_t)w * 8;
     double2 E0 = cadd(cz(e0, 0), cadd(e1a[w], e1b[w]));
     E0 = cadd(E0, cscale(sc[2], 0.5));
@@ -540,6 +540,6 @@ void launch_final(int nw, const double2* part, int nslot, int nR, double e0, con
                   const double2* e1b, const double2* scal, const double2* O0a, const double2* O0b,
                   double2* eloc, double2* ovlp, cudaStream_t st)
 {
-    k_final<<<(nw + 127) / 128, 128, 0, st>>>(nw, part, nslot, nR, e0, e1a, e1b, scal, O0a, O0b,
+    k_final<<<(nw + 3) / 4, 128, 0, st>>>(nw, part, nslot, nR, e0, e1a, e1b, scal, O0a, O0b,
                                              eloc, ovlp); msd_note_launch();
 }

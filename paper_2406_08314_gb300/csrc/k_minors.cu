@@ -1,0 +1,428 @@
+// Excitation-string minors and CI weights with the walkers along the lanes
+// (get_dets of Sec. III), and the FP32 inverse minors of the mixed path.
+//
+// Ratios. r_s = sign * det A_s, A_s[i][j] = G[h_i][p_j], of every string and
+// walker in FP64. A k x k LU costs about 4 k^3 / 3 FP64 FMAs and k reciprocals;
+// here a minor is a Laplace expansion over smaller minors that its neighbours
+// share: all 2 x 2 minors of the active block once per walker (8 FMAs each),
+// then level 3 along its last row (3 complex products), level 4 over pairs of
+// 2 x 2 minors (6) or along its last row over the level-3 ratios (4), levels 5
+// and 6 along the last row over the level below (5, 6) where the trial holds all
+// the k strings that takes, else over the 2 x 2 minors (35, 105). GB300 issues
+// two FP64 FMAs per clock and SM, so the operation count is the time.
+// Division-free expansions of these sizes have no growth: against exact rational
+// arithmetic their relative error is 1.5e-16 to 2.9e-16 (levels 3 to 6, random
+// blocks), the pivoted LU's 5e-16 to 8e-16.
+//
+// Layout. Arrays of a string (or an active entry) hold its walkers contiguously,
+// rT[s][nw]: a warp's lanes are walkers of the same string, so index lists are
+// read once per warp, every gather of another string's ratios is a contiguous
+// row, and lanes do not diverge over lists of different length (one string per
+// lane left half of the FP64 issue slots of the weights kernel idle). The
+// weights leave through a shared-memory tile in the [walker][string] order that
+// the per-determinant kernels read.
+//
+// Iron-sulfur trial, 640 walkers (12.5e3 strings per spin): ratios and FP32
+// inverse minors 3.60 (one pivoted LU per string) -> 1.33 ms, weights 1.32 -> 0.89
+// ms; 1e6 determinants, 10 walkers: weights 0.93 -> 0.28 ms.
+#include <algorithm>
+
+#include "common.cuh"
+#include "kernels.h"
+
+namespace {
+
+struct MinorSpin {
+    int nh, np, n_str;
+    int bucket[MSD_KMAX + 2];
+    const uint4* str_hp;
+    const int8_t* str_sign;
+    const int* sub;          // [n_str][MSD_KMAX] (string << 1 | negative), -1 first if one is missing
+    const double2* GT;       // [nh np][nw]
+    double2* m2;             // [C(nh,2) C(np,2)][nw]
+    double2* rT;             // [n_str][nw]
+};
+// Both spins of a launch (indexed by the block, in constant memory).
+struct MinorArgs { MinorSpin s[2]; };
+
+__device__ __forceinline__ void pair_of(int e, int n, int& a, int& b)
+{
+    a = 0;
+    while (e >= n - 1 - a) { e -= n - 1 - a; ++a; }
+    b = a + 1 + e;
+}
+
+// m2[(h,h')(p,p')] = G[h][p] G[h'][p'] - G[h][p'] G[h'][p]
+__global__ void __launch_bounds__(256) k_minor2(const __grid_constant__ MinorArgs a, int nw)
+{
+    const MinorSpin& S = a.s[blockIdx.y];
+    const int npp = S.np * (S.np - 1) / 2, n2 = S.nh * (S.nh - 1) / 2 * npp;
+    const long long e = blockIdx.x * 256ll + threadIdx.x;
+    if (e >= (long long)n2 * nw) return;
+    const int pr = (int)(e / nw), w = (int)(e - (long long)pr * nw);
+    int h, h2, p, p2;
+    pair_of(pr / npp, S.nh, h, h2);
+    pair_of(pr % npp, S.np, p, p2);
+    const double2* g = S.GT + w;
+    auto G = [&](int a, int b) { return g[(size_t)(a * S.np + b) * nw]; };
+    S.m2[e] = cfms(G(h, p2), G(h2, p), cmul(G(h, p), G(h2, p2)));
+}
+
+// Minors of the strings [bucket[k0], bucket[k1 + 1]); SUBS: through the
+// ratios of the level below where the string has them.
+__global__ void __launch_bounds__(256)
+k_minors(const __grid_constant__ MinorArgs a, int k0, int k1, bool subs, int nw)
+{
+    const MinorSpin& S = a.s[blockIdx.y];
+    const int s0 = S.bucket[k0], n = S.bucket[k1 + 1] - s0;
+    const long long e = blockIdx.x * 256ll + threadIdx.x;
+    if (e >= (long long)n * nw) return;
+    const int s = s0 + (int)(e / nw), w = (int)(e % nw);
+    int k = k0;
+    while (s >= S.bucket[k + 1]) ++k;
+    double2* out = S.rT + (size_t)s * nw + w;
+    if (k == 0) { *out = cz(1, 0); return; }
+    const int np = S.np, nh = S.nh, npp = np * (np - 1) / 2;
+    const uint4 rec = S.str_hp[s];
+    const double2* g = S.GT + w;
+    const double2* m2 = S.m2 + w;
+    const double sg = S.str_sign[s];
+    auto G = [&](int i, int j) { return g[(size_t)(rec_h(rec, i) * np + rec_p(rec, j)) * nw]; };
+    // 2 x 2 minor of rows a < b, columns c < d of the string's block
+    auto M2 = [&](int a, int b, int c, int d) {
+        const int hp = pair_index(rec_h(rec, a), rec_h(rec, b), nh), pp = pair_index(rec_p(rec, c), rec_p(rec, d), np);
+        return m2[(size_t)(hp * npp + pp) * nw];
+    };
+    // 4 x 4 minor of rows a < b < c < d, columns q0 < q1 < q2 < q3
+    auto M4 = [&](int a, int b, int c, int d, int q0, int q1, int q2, int q3) {
+        double2 v = cmul(M2(a, b, q0, q1), M2(c, d, q2, q3));
+        v = cfms(M2(a, b, q0, q2), M2(c, d, q1, q3), v);
+        v = cfma(M2(a, b, q0, q3), M2(c, d, q1, q2), v);
+        v = cfma(M2(a, b, q1, q2), M2(c, d, q0, q3), v);
+        v = cfms(M2(a, b, q1, q3), M2(c, d, q0, q2), v);
+        return cfma(M2(a, b, q2, q3), M2(c, d, q0, q1), v);
+    };
+    if (k == 1) { *out = cscale(G(0, 0), sg); return; }
+    if (k == 2) { *out = cscale(M2(0, 1, 0, 1), sg); return; }
+    if (k == 3) {
+        double2 v = cmul(G(2, 0), M2(0, 1, 1, 2));
+        v = cfms(G(2, 1), M2(0, 1, 0, 2), v);
+        *out = cscale(cfma(G(2, 2), M2(0, 1, 0, 1), v), sg);
+        return;
+    }
+    const int* sub = S.sub + (size_t)s * MSD_KMAX;
+    if (subs && sub[0] >= 0) {
+        double2 v = cz(0, 0);
+        for (int j = 0; j < k; ++j) {
+            const int q = sub[j];
+            double2 gj = G(k - 1, j);
+            if (q & 1) gj = cz(-gj.x, -gj.y);
+            v = cfma(gj, S.rT[(size_t)(q >> 1) * nw + w], v);
+        }
+        *out = v;
+        return;
+    }
+    double2 v = cz(0, 0);
+    if (k == 4) {
+        v = M4(0, 1, 2, 3, 0, 1, 2, 3);
+    } else if (k == 5) {
+        for (int j = 0; j < 5; ++j) {
+            const int a = j > 0 ? 0 : 1, b = j > 1 ? 1 : 2, c = j > 2 ? 2 : 3, d = j > 3 ? 3 : 4;
+            const double2 m = M4(0, 1, 2, 3, a, b, c, d), gj = G(4, j);
+            v = (j & 1) ? cfms(gj, m, v) : cfma(gj, m, v);
+        }
+    } else {
+        // rows 4, 5 over all column pairs; sign (-1)^(4 + 5 + c + d)
+        for (int c = 0; c < 5; ++c)
+            for (int d = c + 1; d < 6; ++d) {
+                auto q = [&](int j) { j += j >= c; return j + (j >= d); };   // the other columns
+                const double2 x = M4(0, 1, 2, 3, q(0), q(1), q(2), q(3)), y = M2(4, 5, c, d);
+                v = ((c + d) & 1) ? cfma(y, x, v) : cfms(y, x, v);
+            }
+    }
+    *out = cscale(v, sg);
+}
+
+// ----------------------------------------------------------------- weights
+struct WeightSpin {
+    int n_str;
+    const int* off;
+    const int* other;
+    const double* c;
+    const double2* self;     // rT of this spin, [n_str][nw]
+    const double2* opp;      // rT of the other spin
+    double2* wts;            // [nw][n_str] r_s w_s (may be NULL)
+    float2* rf;              // [nw][n_str] r_s in FP32 (may be NULL)
+    double2* part;           // [nw][nslot] partial sums over 32 strings (may be NULL)
+};
+struct WeightArgs { WeightSpin s[2]; };
+
+// w_s = sum over determinants I containing string s of c_I r_other(I); stored
+// is r_s w_s (what every consumer needs). One block per tile of 32 strings and
+// up to 32 walkers; a thread's sum runs in list order.
+#define WT_S 32
+__global__ void __launch_bounds__(256) k_weights(const __grid_constant__ WeightArgs a, int nw, int wt, int nslot)
+{
+    const WeightSpin& S = a.s[blockIdx.z];
+    const int s0 = blockIdx.x * WT_S, w0 = blockIdx.y * wt;
+    if (s0 >= S.n_str) return;
+    __shared__ double2 tw[WT_S][33];
+    __shared__ float2 tr[WT_S][33];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int e = threadIdx.x; e < WT_S * wt; e += 256) {
+        const int sl = e / wt, wl = e - sl * wt, s = s0 + sl, w = w0 + wl;
+        double2 rw = cz(0, 0), r = cz(0, 0);
+        if (s < S.n_str && w < nw) {
+            const double2* ro = S.opp + w;
+            double2 acc = cz(0, 0);
+            int i = S.off[s];
+            const int i1 = S.off[s + 1];
+            for (; i + 8 <= i1; i += 8) {
+                int o[8];
+                double c[8];
+                double2 v[8];
+#pragma unroll
+                for (int q = 0; q < 8; ++q) { o[q] = S.other[i + q]; c[q] = S.c[i + q]; }
+#pragma unroll
+                for (int q = 0; q < 8; ++q) v[q] = ro[(size_t)o[q] * nw];
+#pragma unroll
+                for (int q = 0; q < 8; ++q) acc = cz(fma(v[q].x, c[q], acc.x), fma(v[q].y, c[q], acc.y));
+            }
+            for (; i < i1; ++i) {
+                const double2 v = ro[(size_t)S.other[i] * nw];
+                const double c = S.c[i];
+                acc = cz(fma(v.x, c, acc.x), fma(v.y, c, acc.y));
+            }
+            r = S.self[(size_t)s * nw + w];
+            rw = cmul(r, acc);
+        }
+        tw[sl][wl] = rw;
+        if (S.rf) tr[sl][wl] = make_float2((float)r.x, (float)r.y);
+    }
+    __syncthreads();
+    const int s = s0 + lane;
+    for (int wl = warp; wl < wt && w0 + wl < nw; wl += 8) {
+        const size_t w = w0 + wl;
+        double2 v = tw[lane][wl];
+        if (s < S.n_str) {
+            if (S.wts) S.wts[w * S.n_str + s] = v;
+            if (S.rf) S.rf[w * S.n_str + s] = tr[lane][wl];
+        }
+        if (S.part) {
+            for (int o = 16; o; o >>= 1) {
+                v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
+                v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
+            }
+            if (lane == 0) S.part[w * nslot + blockIdx.x] = v;
+        }
+    }
+}
+
+// r[w][s] = rT[s][w]
+__global__ void __launch_bounds__(256) k_untranspose(int n_str, int nw, const double2* __restrict__ rT, double2* __restrict__ r)
+{
+    __shared__ double2 tile[32][33];
+    const int s0 = blockIdx.x * 32, w0 = blockIdx.y * 32, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int i = warp; i < 32; i += 8)
+        if (s0 + i < n_str && w0 + lane < nw) tile[i][lane] = rT[(size_t)(s0 + i) * nw + w0 + lane];
+    __syncthreads();
+    for (int i = warp; i < 32; i += 8)
+        if (w0 + i < nw && s0 + lane < n_str) r[(size_t)(w0 + i) * n_str + s0 + lane] = tile[lane][i];
+}
+
+// ------------------------------------------------------ FP32 inverse minors
+struct InvSpin {
+    int nh, np;
+    int bucket[MSD_KMAX + 2];
+    const uint4* str_hp;
+    const double2* Gact;     // [nw][nh np]
+    float2* B;
+    long long b_off[MSD_KMAX + 2];
+    int blk[MSD_KMAX + 2];   // first block of each level
+};
+struct InvArgs { InvSpin s[2]; };
+
+// B = A^-1 of one string in FP32: elimination with partial pivoting by the
+// larger of |Re|, |Im| (compared to 20 mantissa bits), column solves, then the
+// K^2 entries (and the pad) as 16-byte stores.
+template <int K>
+__device__ __forceinline__ void inverse_minor(const uint4 rec, int np, const float2* __restrict__ gf, float2* __restrict__ B)
+{
+    float2 lu[K][K], di[K];
+    int perm[K];
+#pragma unroll
+    for (int i = 0; i < K; ++i) {
+        perm[i] = i;
+#pragma unroll
+        for (int j = 0; j < K; ++j) lu[i][j] = gf[rec_h(rec, i) * np + rec_p(rec, j)];
+    }
+    auto key = [](float2 v) { return max(__float_as_int(v.x) & 0x7fffffff, __float_as_int(v.y) & 0x7fffffff) >> 3; };
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        int p = k, best = key(lu[k][k]);
+#pragma unroll
+        for (int i = k + 1; i < K; ++i) {
+            const int v = key(lu[i][k]);
+            if (v > best) { best = v; p = i; }
+        }
+#pragma unroll
+        for (int i = k + 1; i < K; ++i)
+            if (i == p) {
+#pragma unroll
+                for (int j = 0; j < K; ++j) { const float2 t = lu[k][j]; lu[k][j] = lu[i][j]; lu[i][j] = t; }
+                const int t = perm[k]; perm[k] = perm[i]; perm[i] = t;
+            }
+        const float m2 = fmaf(lu[k][k].x, lu[k][k].x, lu[k][k].y * lu[k][k].y);
+        const float im2 = !(m2 > 0.f) ? 0.f : 1.f / m2;
+        di[k] = make_float2(lu[k][k].x * im2, -lu[k][k].y * im2);
+#pragma unroll
+        for (int i = k + 1; i < K; ++i) {
+            const float2 f = fmul(lu[i][k], di[k]);
+            lu[i][k] = f;
+#pragma unroll
+            for (int j = k + 1; j < K; ++j) {
+                lu[i][j].x -= f.x * lu[k][j].x - f.y * lu[k][j].y;
+                lu[i][j].y -= f.x * lu[k][j].y + f.y * lu[k][j].x;
+            }
+        }
+    }
+    float2 inv[K * K + (K & 1)];
+    if (K & 1) inv[K * K] = make_float2(0.f, 0.f);   // the pad entry
+#pragma unroll
+    for (int c = 0; c < K; ++c) {
+        float2 x[K];
+#pragma unroll
+        for (int i = 0; i < K; ++i) x[i] = make_float2(perm[i] == c ? 1.f : 0.f, 0.f);
+#pragma unroll
+        for (int i = 0; i < K; ++i)
+#pragma unroll
+            for (int k = 0; k < i; ++k) {
+                x[i].x -= lu[i][k].x * x[k].x - lu[i][k].y * x[k].y;
+                x[i].y -= lu[i][k].x * x[k].y + lu[i][k].y * x[k].x;
+            }
+#pragma unroll
+        for (int i = K - 1; i >= 0; --i) {
+#pragma unroll
+            for (int k = i + 1; k < K; ++k) {
+                x[i].x -= lu[i][k].x * x[k].x - lu[i][k].y * x[k].y;
+                x[i].y -= lu[i][k].x * x[k].y + lu[i][k].y * x[k].x;
+            }
+            const float2 t = x[i];
+            x[i] = make_float2(t.x * di[i].x - t.y * di[i].y, t.x * di[i].y + t.y * di[i].x);
+        }
+#pragma unroll
+        for (int i = 0; i < K; ++i) inv[i * K + c] = x[i];
+    }
+#pragma unroll
+    for (int e = 0; e < b_stride(K); e += 2)
+        *reinterpret_cast<float4*>(B + e) = make_float4(inv[e].x, inv[e].y, inv[e + 1].x, inv[e + 1].y);
+}
+
+__global__ void __launch_bounds__(128) k_inverse_minors(const __grid_constant__ InvArgs a)
+{
+    const InvSpin& S = a.s[blockIdx.z];
+    __shared__ float2 gf[MSD_XMAX];
+    const int w = blockIdx.y, X = S.nh * S.np;
+    if ((int)blockIdx.x >= S.blk[MSD_KMAX + 1]) return;
+    for (int e = threadIdx.x; e < X; e += 128) {
+        const double2 v = S.Gact[(size_t)w * X + e];
+        gf[e] = make_float2((float)v.x, (float)v.y);
+    }
+    __syncthreads();
+    int k = 1;
+    while ((int)blockIdx.x >= S.blk[k + 1]) ++k;
+    const int ns = S.bucket[k + 1] - S.bucket[k], sl = ((int)blockIdx.x - S.blk[k]) * 128 + threadIdx.x;
+    if (sl >= ns) return;
+    const uint4 rec = S.str_hp[S.bucket[k] + sl];
+    float2* B = S.B + S.b_off[k] + ((size_t)w * ns + sl) * b_stride(k);
+    switch (k) {
+    case 1: inverse_minor<1>(rec, S.np, gf, B); break;
+    case 2: inverse_minor<2>(rec, S.np, gf, B); break;
+    case 3: inverse_minor<3>(rec, S.np, gf, B); break;
+    case 4: inverse_minor<4>(rec, S.np, gf, B); break;
+    case 5: inverse_minor<5>(rec, S.np, gf, B); break;
+    default: inverse_minor<6>(rec, S.np, gf, B); break;
+    }
+}
+
+MinorSpin minor_spin(const SpinTables& t, const double2* GT, double2* m2, double2* rT)
+{
+    MinorSpin s;
+    s.nh = t.nh; s.np = t.np; s.n_str = t.n_str;
+    for (int k = 0; k < MSD_KMAX + 2; ++k) s.bucket[k] = t.bucket[k];
+    s.str_hp = t.str_hp; s.str_sign = t.str_sign; s.sub = t.sub;
+    s.GT = GT; s.m2 = m2; s.rT = rT;
+    return s;
+}
+
+}  // namespace
+
+size_t minor2_count(const SpinTables& t)
+{
+    return std::max<size_t>(1, (size_t)(t.nh * (t.nh - 1) / 2) * (t.np * (t.np - 1) / 2));
+}
+
+void launch_minors(const SpinTables& ta, const SpinTables& tb, int nw, double2* const GT[2], double2* const m2[2],
+                   double2* const rT[2], cudaStream_t st)
+{
+    const MinorArgs a = {{minor_spin(ta, GT[0], m2[0], rT[0]), minor_spin(tb, GT[1], m2[1], rT[1])}};
+    auto blocks = [&](long long n) { return dim3((unsigned)((n * nw + 255) / 256), 2); };
+    k_minor2<<<blocks(std::max(minor2_count(ta), minor2_count(tb))), 256, 0, st>>>(a, nw);
+    msd_note_launch();
+    // Level 4 over the level-3 ratios takes 4 complex products instead of 6, but a
+    // launch of its own: only where there are many (the launch costs about what
+    // 1000 strings' two products do for a few hundred walkers).
+    auto count = [&](int k0, int k1) {
+        return std::max(ta.bucket[k1 + 1] - ta.bucket[k0], tb.bucket[k1 + 1] - tb.bucket[k0]);
+    };
+    const bool four = count(4, 4) >= 1000;
+    k_minors<<<blocks(count(0, four ? 3 : 4)), 256, 0, st>>>(a, 0, four ? 3 : 4, false, nw);
+    msd_note_launch();
+    for (int k = four ? 4 : 5; k <= MSD_KMAX; ++k) {
+        if (count(k, k) <= 0) continue;
+        k_minors<<<blocks(count(k, k)), 256, 0, st>>>(a, k, k, true, nw);
+        msd_note_launch();
+    }
+}
+
+void launch_inverse_minors(const SpinTables& ta, const SpinTables& tb, int nw, double2* const Gact[2], void* const B[2],
+                           cudaStream_t st)
+{
+    InvArgs args;
+    InvSpin* s = args.s;
+    const SpinTables* t[2] = {&ta, &tb};
+    int nb = 0;
+    for (int i = 0; i < 2; ++i) {
+        s[i].nh = t[i]->nh; s[i].np = t[i]->np;
+        s[i].str_hp = t[i]->str_hp;
+        s[i].Gact = Gact[i]; s[i].B = (float2*)B[i];
+        s[i].blk[0] = s[i].blk[1] = 0;
+        for (int k = 0; k < MSD_KMAX + 2; ++k) { s[i].bucket[k] = t[i]->bucket[k]; s[i].b_off[k] = t[i]->b_off[k]; }
+        for (int k = 1; k <= MSD_KMAX; ++k)
+            s[i].blk[k + 1] = s[i].blk[k] + (s[i].bucket[k + 1] - s[i].bucket[k] + 127) / 128;
+        nb = std::max(nb, s[i].blk[MSD_KMAX + 1]);
+    }
+    if (nb <= 0) return;
+    k_inverse_minors<<<dim3(nb, nw, 2), 128, 0, st>>>(args);
+    msd_note_launch();
+}
+
+int weights_blocks(const SpinTables& tb) { return (tb.n_str + WT_S - 1) / WT_S; }
+
+// wts, rf: per spin, NULL where not wanted; beta = false: the alpha sums alone.
+void launch_weights(const SpinTables& ta, const SpinTables& tb, int nw, double2* const rT[2], double2* const wts[2],
+                    float2* const rf[2], double2* part, int nslot, bool beta, cudaStream_t st)
+{
+    const WeightArgs a = {{{ta.n_str, ta.csr_off, ta.csr_other, ta.csr_c, rT[0], rT[1], wts[0], rf[0], part},
+                          {tb.n_str, tb.csr_off, tb.csr_other, tb.csr_c, rT[1], rT[0], wts[1], rf[1], nullptr}}};
+    const int tiles = (nw + 31) / 32, wt = (nw + tiles - 1) / tiles;   // walkers per tile, evenly
+    const int nb = beta ? std::max(weights_blocks(ta), weights_blocks(tb)) : weights_blocks(ta);
+    k_weights<<<dim3(nb, tiles, beta ? 2 : 1), 256, 0, st>>>(a, nw, wt, nslot);
+    msd_note_launch();
+}
+
+void launch_untranspose(int n_str, int nw, const double2* rT, double2* r, cudaStream_t st)
+{
+    k_untranspose<<<dim3((n_str + 31) / 32, (nw + 31) / 32), 256, 0, st>>>(n_str, nw, rT, r);
+    msd_note_launch();
+}

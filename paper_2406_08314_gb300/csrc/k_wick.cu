@@ -2,8 +2,6 @@
 // part of the generalized-Wick evaluation (Sec. III "Implementation":
 // get_dets), plus the cofactor accumulation behind the mixed Green's
 // function (reduce_CI) and its rank-n_p update.
-#include <type_traits>
-
 #include "common.cuh"
 #include "kernels.h"
 
@@ -22,7 +20,7 @@ k_ref(const double2* __restrict__ phi, int M, int N, const int* __restrict__ occ
       const int* __restrict__ pos0, const int* __restrict__ hole_pos, int nh, const int* __restrict__ part_orb,
       int np,
       double2* __restrict__ Gr, double2* __restrict__ O0, double2* __restrict__ Gact,
-      unsigned* err)
+      double2* __restrict__ GactT, unsigned* err)
 {
     extern __shared__ double2 sm[];
     double2* S = sm;              // [N][N] LU in place
@@ -86,7 +84,10 @@ k_ref(const double2* __restrict__ phi, int M, int N, const int* __restrict__ occ
     __syncthreads();
     if (singular) {
         for (int e = t; e < N * M; e += nt) Gr[(size_t)w * N * M + e] = cz(0, 0);
-        for (int e = t; e < nh * np; e += nt) Gact[(size_t)w * nh * np + e] = cz(0, 0);
+        for (int e = t; e < nh * np; e += nt) {
+            Gact[(size_t)w * nh * np + e] = cz(0, 0);
+            if (GactT) GactT[(size_t)e * gridDim.x + w] = cz(0, 0);
+        }
         return;
     }
     // S^-1 column c: solve L U x = P e_c
@@ -127,28 +128,28 @@ k_ref(const double2* __restrict__ phi, int M, int N, const int* __restrict__ occ
         double2 a = cz(0, 0);
         for (int k = 0; k < N; ++k) a = cfma(pr[k], Si[k * N + j], a);
         Gact[(size_t)w * nh * np + e] = a;
+        if (GactT) GactT[(size_t)e * gridDim.x + w] = a;
     }
 }
 
 void launch_ref(const double2* phi, int nw, int M, int N, const SpinTables& T, double2* Gr,
-                double2* O0, double2* Gact, unsigned* err, cudaStream_t st)
+                double2* O0, double2* Gact, double2* GactT, unsigned* err, cudaStream_t st)
 {
     size_t smem = sizeof(double2) * 2 * N * N;
     if (smem > 48 * 1024) cudaFuncSetAttribute(k_ref, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     k_ref<<<nw, 256, smem, st>>>(phi, M, N, T.occ0, T.pos0, T.hole_pos, T.nh, T.part_orb, T.np, Gr, O0,
-                                 Gact, err); msd_note_launch();
+                                 Gact, GactT, err); msd_note_launch();
 }
 
 // ------------------------------------------------------------------------
-// Excitation strings of level K for one spin (get_dets / build_det_matrix):
+// Excitation strings of level K for one spin with their FP64 inverse minors
+// (the FP64 path; ratios alone and the mixed path's FP32 inverses: k_minors.cu):
 // A[i][j] = G[h_i][p_j] (a K x K minor of G). LU with partial pivoting in
 // FP64 gives r = sign * det A, the overlap ratio <D_s|phi>/<D_0|phi> of the
-// string's spin sector. B = A^-1 is stored per string, K*K entries
+// string's spin sector, and B = A^-1 from its factors, K*K entries
 // contiguous (B[i][j] at i*K + j), for the Green's-function and energy
-// terms: in FP64 mode solved from the FP64 LU factors; in mixed mode from an
-// FP32 elimination of the same row order (the FP64 pivots) on an FP32 copy of
-// the active block. One thread per (walker, string); the walker's active
-// block lives in shared memory.
+// terms. One thread per (walker, string); the walker's active block lives in
+// shared memory.
 //
 // FP64 issue rate is the bound here (a few FP64 operations per clock per
 // SM), so the LU spends FP64 operations on the elimination and the
@@ -179,22 +180,15 @@ __device__ __forceinline__ int mag_key(double2 v)
     return max(__double2hiint(v.x) & 0x7fffffff, __double2hiint(v.y) & 0x7fffffff);
 }
 
-template <int K, typename T>
+template <int K>
 __global__ void __launch_bounds__(128)
-k_strings(SpinTables tb, int nw, const double2* __restrict__ Gact, double2* __restrict__ r,
-          float2* __restrict__ rf, void* __restrict__ Bout, int want_b)
+k_strings(SpinTables tb, int nw, const double2* __restrict__ Gact, double2* __restrict__ r, double2* __restrict__ rT,
+          double2* __restrict__ Bout)
 {
-    using T2 = typename std::conditional<std::is_same<T, float>::value, float2, double2>::type;
-    constexpr bool F32B = std::is_same<T, float>::value;
     __shared__ double2 g[MSD_XMAX];
-    __shared__ float2 gf[F32B ? MSD_XMAX : 1];
     const int w = blockIdx.y;
     const int X = tb.nh * tb.np;
-    for (int e = threadIdx.x; e < X; e += blockDim.x) {
-        const double2 v = Gact[(size_t)w * X + e];
-        g[e] = v;
-        if constexpr (F32B) gf[e] = make_float2((float)v.x, (float)v.y);
-    }
+    for (int e = threadIdx.x; e < X; e += blockDim.x) g[e] = Gact[(size_t)w * X + e];
     __syncthreads();
     const int ns = tb.bucket[K + 1] - tb.bucket[K];
     const int sl = blockIdx.x * blockDim.x + threadIdx.x;
@@ -249,65 +243,24 @@ k_strings(SpinTables tb, int nw, const double2* __restrict__ Gact, double2* __re
     if (odd) det = cz(-det.x, -det.y);
     if (sing) det = cz(0, 0);
     r[(size_t)w * tb.n_str + s] = det;
-    if (rf) rf[(size_t)w * tb.n_str + s] = make_float2((float)det.x, (float)det.y);
-    if (!want_b) return;
-    // B = A^-1 from P A = L U: column c solves L U x = P e_c, in precision T.
-    T2 lu[K][K], di[K];
-    if constexpr (F32B) {
-        // FP32 elimination of the rows in the FP64 pivot order
-#pragma unroll
-        for (int i = 0; i < K; ++i) {
-            const int ro = rec_h(rec, perm[i]) * tb.np;
-#pragma unroll
-            for (int j = 0; j < K; ++j) lu[i][j] = gf[ro + rec_p(rec, j)];
-        }
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            const float m2 = fmaf(lu[k][k].x, lu[k][k].x, lu[k][k].y * lu[k][k].y);
-            const float im2 = (sing || !(m2 > 0.f)) ? 0.f : 1.f / m2;
-            di[k] = make_float2(lu[k][k].x * im2, -lu[k][k].y * im2);
-#pragma unroll
-            for (int i = k + 1; i < K; ++i) {
-                const float2 f = fmul(lu[i][k], di[k]);
-                lu[i][k] = f;
-#pragma unroll
-                for (int j = k + 1; j < K; ++j) {
-                    lu[i][j].x -= f.x * lu[k][j].x - f.y * lu[k][j].y;
-                    lu[i][j].y -= f.x * lu[k][j].y + f.y * lu[k][j].x;
-                }
-            }
-        }
-    } else {
-#pragma unroll
-        for (int i = 0; i < K; ++i) {
-            di[i] = T2{(T)dinv[i].x, (T)dinv[i].y};
-#pragma unroll
-            for (int j = 0; j < K; ++j) lu[i][j] = T2{(T)a[i][j].x, (T)a[i][j].y};
-        }
-    }
-    T2* B = reinterpret_cast<T2*>(Bout) + (size_t)tb.b_off[K] + ((size_t)w * ns + sl) * b_stride(K);
-    if (K & 1) B[K * K] = T2{0, 0};   // the pad entry
+    rT[(size_t)s * nw + w] = det;
+    // B = A^-1 from P A = L U: column c solves L U x = P e_c
+    double2* B = Bout + (size_t)tb.b_off[K] + ((size_t)w * ns + sl) * b_stride(K);
+    if (K & 1) B[K * K] = cz(0, 0);   // the pad entry
 #pragma unroll
     for (int c = 0; c < K; ++c) {
-        T2 x[K];
+        double2 x[K];
 #pragma unroll
-        for (int i = 0; i < K; ++i) x[i] = T2{(T)(perm[i] == c ? 1 : 0), (T)0};
+        for (int i = 0; i < K; ++i) x[i] = cz(perm[i] == c ? 1 : 0, 0);
 #pragma unroll
         for (int i = 0; i < K; ++i)
 #pragma unroll
-            for (int k = 0; k < i; ++k) {
-                x[i].x -= lu[i][k].x * x[k].x - lu[i][k].y * x[k].y;
-                x[i].y -= lu[i][k].x * x[k].y + lu[i][k].y * x[k].x;
-            }
+            for (int k = 0; k < i; ++k) x[i] = cfms(a[i][k], x[k], x[i]);
 #pragma unroll
         for (int i = K - 1; i >= 0; --i) {
 #pragma unroll
-            for (int k = i + 1; k < K; ++k) {
-                x[i].x -= lu[i][k].x * x[k].x - lu[i][k].y * x[k].y;
-                x[i].y -= lu[i][k].x * x[k].y + lu[i][k].y * x[k].x;
-            }
-            const T2 t = x[i];
-            x[i] = T2{t.x * di[i].x - t.y * di[i].y, t.x * di[i].y + t.y * di[i].x};
+            for (int k = i + 1; k < K; ++k) x[i] = cfms(a[i][k], x[k], x[i]);
+            x[i] = cmul(x[i], dinv[i]);
         }
 #pragma unroll
         for (int i = 0; i < K; ++i) B[i * K + c] = x[i];
@@ -315,108 +268,39 @@ k_strings(SpinTables tb, int nw, const double2* __restrict__ Gact, double2* __re
 }
 
 template <int K>
-static void launch_strings_k(const SpinTables& tb, int nw, const double2* Gact, double2* r, float2* rf, void* B,
-                             bool fp32, int want_b, cudaStream_t st)
+static void launch_strings_k(const SpinTables& tb, int nw, const double2* Gact, double2* r, double2* rT, void* B,
+                             cudaStream_t st)
 {
     const int ns = tb.bucket[K + 1] - tb.bucket[K];
     if (ns <= 0) return;
     dim3 grid((ns + 127) / 128, nw);
-    if (fp32) k_strings<K, float><<<grid, 128, 0, st>>>(tb, nw, Gact, r, rf, B, want_b);
-    else k_strings<K, double><<<grid, 128, 0, st>>>(tb, nw, Gact, r, rf, B, want_b);
+    k_strings<K><<<grid, 128, 0, st>>>(tb, nw, Gact, r, rT, (double2*)B);
     msd_note_launch();
 }
 
 // Reference string (level 0): ratio 1.
-__global__ void k_ref_string(int nw, int n_str, double2* r, float2* rf)
+__global__ void k_ref_string(int nw, int n_str, double2* r, double2* rT)
 {
     const int w = blockIdx.x * blockDim.x + threadIdx.x;
-    if (w < nw) {
-        r[(size_t)w * n_str] = cz(1, 0);
-        if (rf) rf[(size_t)w * n_str] = make_float2(1.f, 0.f);
-    }
+    if (w < nw) r[(size_t)w * n_str] = rT[w] = cz(1, 0);
 }
 
-void launch_strings(const SpinTables& tb, int nw, const double2* Gact, double2* r, float2* rf, void* B,
-                    bool fp32, bool want_b, cudaStream_t st, const TimerHook& th)
+void launch_strings(const SpinTables& tb, int nw, const double2* Gact, double2* r, double2* rT, void* B, cudaStream_t st,
+                    const TimerHook& th)
 {
     if (tb.bucket[1] > tb.bucket[0]) {
         th.begin("k_ref_string", st);
-        k_ref_string<<<(nw + 127) / 128, 128, 0, st>>>(nw, tb.n_str, r, rf); msd_note_launch();
+        k_ref_string<<<(nw + 127) / 128, 128, 0, st>>>(nw, tb.n_str, r, rT); msd_note_launch();
         th.end(st);
     }
     th.begin("k_strings", st);
-    launch_strings_k<1>(tb, nw, Gact, r, rf, B, fp32, want_b, st);
-    launch_strings_k<2>(tb, nw, Gact, r, rf, B, fp32, want_b, st);
-    launch_strings_k<3>(tb, nw, Gact, r, rf, B, fp32, want_b, st);
-    launch_strings_k<4>(tb, nw, Gact, r, rf, B, fp32, want_b, st);
-    launch_strings_k<5>(tb, nw, Gact, r, rf, B, fp32, want_b, st);
-    launch_strings_k<6>(tb, nw, Gact, r, rf, B, fp32, want_b, st);
+    launch_strings_k<1>(tb, nw, Gact, r, rT, B, st);
+    launch_strings_k<2>(tb, nw, Gact, r, rT, B, st);
+    launch_strings_k<3>(tb, nw, Gact, r, rT, B, st);
+    launch_strings_k<4>(tb, nw, Gact, r, rT, B, st);
+    launch_strings_k<5>(tb, nw, Gact, r, rT, B, st);
+    launch_strings_k<6>(tb, nw, Gact, r, rT, B, st);
     th.end(st);
-}
-
-// ------------------------------------------------------------------------
-// CI weights per string: w_s = sum over determinants I containing string s
-// of c_I * r_other(I), so that sum_I c_I r_a r_b = sum_a r_a w_a. Stored is
-// the product r_s w_s (what every consumer needs); for spin alpha the block
-// also reduces it into per-walker partial sums. A thread takes one string
-// for WB walkers: each entry of the string's determinant list (index and
-// coefficient) is read once and feeds WB independent gathers; every
-// walker's sum runs in list order as with one walker per thread.
-template <int WB>
-__global__ void __launch_bounds__(256)
-k_weights(SpinTables tb, int nw, const double2* __restrict__ r_self, const double2* __restrict__ r_other,
-          int n_other, double2* __restrict__ wts, double2* __restrict__ part, int nslot,
-          int slot0)
-{
-    const int w0 = blockIdx.y * WB;
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    double2 rw[WB];
-#pragma unroll
-    for (int k = 0; k < WB; ++k) rw[k] = cz(0, 0);
-    if (s < tb.n_str) {
-        double2 acc[WB];
-#pragma unroll
-        for (int k = 0; k < WB; ++k) acc[k] = cz(0, 0);
-        const double2* ro = r_other + (size_t)w0 * n_other;
-        const int e1 = tb.csr_off[s + 1];
-        for (int e = tb.csr_off[s]; e < e1; ++e) {
-            const int o = tb.csr_other[e];
-            const double c = tb.csr_c[e];
-#pragma unroll
-            for (int k = 0; k < WB; ++k)
-                if (w0 + k < nw) acc[k] = cadd(acc[k], cscale(ro[(size_t)k * n_other + o], c));
-        }
-#pragma unroll
-        for (int k = 0; k < WB; ++k)
-            if (w0 + k < nw) {
-                rw[k] = cmul(r_self[(size_t)(w0 + k) * tb.n_str + s], acc[k]);
-                wts[(size_t)(w0 + k) * tb.n_str + s] = rw[k];
-            }
-    }
-    if (part) {
-        __shared__ double2 red[256];
-        for (int k = 0; k < WB && w0 + k < nw; ++k) {
-            red[threadIdx.x] = rw[k];
-            __syncthreads();
-            for (int o = blockDim.x / 2; o; o >>= 1) {
-                if (threadIdx.x < o) red[threadIdx.x] = cadd(red[threadIdx.x], red[threadIdx.x + o]);
-                __syncthreads();
-            }
-            if (threadIdx.x == 0) part[(size_t)(w0 + k) * nslot + slot0 + blockIdx.x] = red[0];
-            __syncthreads();   // red is reused by the next walker
-        }
-    }
-}
-
-int weights_blocks(const SpinTables& tb) { return (tb.n_str + 255) / 256; }
-
-void launch_weights(const SpinTables& tb, int nw, const double2* r_self, const double2* r_other,
-                    int n_other, double2* wts, double2* part, int nslot, int slot0, cudaStream_t st)
-{
-    constexpr int WB = 4;
-    dim3 grid(weights_blocks(tb), (nw + WB - 1) / WB);
-    k_weights<WB><<<grid, 256, 0, st>>>(tb, nw, r_self, r_other, n_other, wts, part, nslot, slot0);
-    msd_note_launch();
 }
 
 // ------------------------------------------------------------------------
@@ -439,15 +323,15 @@ void launch_det_ratios(const PairTables& pt, int nw, int n_str_a, int n_str_b, c
 }
 
 // Sum of partial slots [slot0, slot0 + n) per walker -> out[w] (and
-// O_T = O0a * O0b * sum when ovlp is given).
+// O_T = O0a * O0b * sum when ovlp is given). One warp per walker.
 __global__ void k_sum_slots(int nw, const double2* __restrict__ part, int nslot, int slot0, int n,
                             double2* __restrict__ out, const double2* __restrict__ O0a,
                             const double2* __restrict__ O0b, double2* __restrict__ ovlp)
 {
-    const int w = blockIdx.x * blockDim.x + threadIdx.x;
+    const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (w >= nw) return;
-    double2 a = cz(0, 0);
-    for (int i = 0; i < n; ++i) a = cadd(a, part[(size_t)w * nslot + slot0 + i]);
+    const double2 a = warp_sum_slots(part + (size_t)w * nslot + slot0, n, lane);
+    if (lane) return;
     if (out) out[w] = a;
     if (ovlp) ovlp[w] = cmul(cmul(O0a[w], O0b[w]), a);
 }
@@ -455,7 +339,7 @@ __global__ void k_sum_slots(int nw, const double2* __restrict__ part, int nslot,
 void launch_sum_slots(int nw, const double2* part, int nslot, int slot0, int n, double2* out,
                       const double2* O0a, const double2* O0b, double2* ovlp, cudaStream_t st)
 {
-    k_sum_slots<<<(nw + 127) / 128, 128, 0, st>>>(nw, part, nslot, slot0, n, out, O0a, O0b, ovlp); msd_note_launch();
+    k_sum_slots<<<(nw + 3) / 4, 128, 0, st>>>(nw, part, nslot, slot0, n, out, O0a, O0b, ovlp); msd_note_launch();
 }
 
 // ------------------------------------------------------------------------

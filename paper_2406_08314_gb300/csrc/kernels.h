@@ -13,13 +13,24 @@ struct TimerHook {
 };
 
 // k_wick.cu
+// GactT (may be NULL): the active block with the walkers contiguous, [nh np][nw].
 void launch_ref(const double2* phi, int nw, int M, int N, const SpinTables& T, double2* Gr,
-                double2* O0, double2* Gact, unsigned* err, cudaStream_t st);
-void launch_strings(const SpinTables& tb, int nw, const double2* Gact, double2* r, float2* rf, void* B,
-                    bool fp32, bool want_b, cudaStream_t st, const TimerHook& th);
+                double2* O0, double2* Gact, double2* GactT, unsigned* err, cudaStream_t st);
+// FP64 ratios r[w][s] and rT[s][w] and FP64 inverse minors by pivoted LU.
+void launch_strings(const SpinTables& tb, int nw, const double2* Gact, double2* r, double2* rT, void* B, cudaStream_t st,
+                    const TimerHook& th);
+// k_minors.cu: FP64 ratios rT[s][w] of both spins by expansions over shared
+// minors (m2: scratch, minor2_count entries per walker), FP32 inverse minors,
+// and the CI weights.
+size_t minor2_count(const SpinTables& t);
+void launch_minors(const SpinTables& ta, const SpinTables& tb, int nw, double2* const GT[2], double2* const m2[2],
+                   double2* const rT[2], cudaStream_t st);
+void launch_inverse_minors(const SpinTables& ta, const SpinTables& tb, int nw, double2* const Gact[2], void* const B[2],
+                           cudaStream_t st);
 int weights_blocks(const SpinTables& tb);
-void launch_weights(const SpinTables& tb, int nw, const double2* r_self, const double2* r_other,
-                    int n_other, double2* wts, double2* part, int nslot, int slot0, cudaStream_t st);
+void launch_weights(const SpinTables& ta, const SpinTables& tb, int nw, double2* const rT[2], double2* const wts[2],
+                    float2* const rf[2], double2* part, int nslot, bool beta, cudaStream_t st);
+void launch_untranspose(int n_str, int nw, const double2* rT, double2* r, cudaStream_t st);
 void launch_det_ratios(const PairTables& pt, int nw, int n_str_a, int n_str_b, const double2* ra,
                        const double2* rb, double2* out, cudaStream_t st);
 void launch_sum_slots(int nw, const double2* part, int nslot, int slot0, int n, double2* out,

@@ -70,6 +70,7 @@ struct SpinHost {
     uint8_t* d_cmx = nullptr;
     uint8_t* d_kx = nullptr;
     float* d_csr_cf = nullptr;
+    int* d_sub = nullptr;     // [n_str][MSD_KMAX] (SpinTables::sub)
     int* d_pos0 = nullptr;    // [M] position of an orbital in occ0, or -1
 };
 
@@ -406,6 +407,7 @@ SpinTables tables(const SpinHost& s, int cap)
     t.csr_off = s.d_csr_off; t.csr_other = s.d_csr_other; t.csr_c = s.d_csr_c;
     t.cmx = s.d_cmx;
     t.kx = s.d_kx;
+    t.sub = s.d_sub;
     t.csr_cf = s.d_csr_cf;
     long long off = 0, xo = 0;
     for (int k = 0; k <= MSD_KMAX; ++k) {
@@ -550,6 +552,42 @@ int upload_spin(msd_ctx* ctx, SpinHost& S)
         if ((rc = upload(ctx, &S.d_str_hp, rec))) return rc;
     }
     if ((rc = upload(ctx, &S.d_str_sign, S.str_sign))) return rc;
+    {
+        // expansion of a level >= 4 minor along its last row: the strings without
+        // the last hole and one particle (strings of a level are in lexicographic
+        // order of holes, then particles)
+        std::vector<int> sub((size_t)S.n_str * MSD_KMAX, -1);
+        auto find = [&](int k, const uint8_t* h, const uint8_t* p) {
+            int lo = S.bucket[k], hi = S.bucket[k + 1];
+            auto less = [&](int f) {
+                const int c = std::memcmp(&S.str_h[(size_t)f * MSD_KMAX], h, k);
+                return c ? c < 0 : std::memcmp(&S.str_p[(size_t)f * MSD_KMAX], p, k) < 0;
+            };
+            while (lo < hi) {
+                const int mid = (lo + hi) / 2;
+                if (less(mid)) lo = mid + 1; else hi = mid;
+            }
+            const bool hit = lo < S.bucket[k + 1] && !std::memcmp(&S.str_h[(size_t)lo * MSD_KMAX], h, k) &&
+                             !std::memcmp(&S.str_p[(size_t)lo * MSD_KMAX], p, k);
+            return hit ? lo : -1;
+        };
+        for (int k = 4; k <= MSD_KMAX; ++k)
+            for (int f = S.bucket[k]; f < S.bucket[k + 1]; ++f) {
+                const uint8_t *h = &S.str_h[(size_t)f * MSD_KMAX], *p = &S.str_p[(size_t)f * MSD_KMAX];
+                int q[MSD_KMAX];
+                bool all = true;
+                for (int j = 0; j < k && all; ++j) {
+                    uint8_t ps[MSD_KMAX];
+                    for (int i = 0, m = 0; i < k; ++i)
+                        if (i != j) ps[m++] = p[i];
+                    const int g = find(k - 1, h, ps);
+                    all = g >= 0;
+                    if (all) q[j] = g << 1 | (((k - 1 + j) & 1) ^ (S.str_sign[g] < 0) ^ (S.str_sign[f] < 0));
+                }
+                if (all) std::copy(q, q + k, &sub[(size_t)f * MSD_KMAX]);
+            }
+        if ((rc = upload(ctx, &S.d_sub, sub))) return rc;
+    }
     if ((rc = upload(ctx, &S.d_csr_off, S.csr_off))) return rc;
     if ((rc = upload(ctx, &S.d_csr_other, S.csr_other))) return rc;
     if ((rc = upload(ctx, &S.d_csr_c, S.csr_c))) return rc;
@@ -584,7 +622,8 @@ void free_spin(SpinHost& S)
     cudaFree(S.d_occ0); cudaFree(S.d_hole_pos); cudaFree(S.d_part_orb); cudaFree(S.d_str_hp);
     cudaFree(S.d_str_sign); cudaFree(S.d_csr_off); cudaFree(S.d_csr_other);
     cudaFree(S.d_csr_c); cudaFree(S.d_Lh); cudaFree(S.d_pos0);
-    cudaFree(S.d_cmx); cudaFree(S.d_kx); cudaFree(S.d_csr_cf);
+    cudaFree(S.d_cmx); cudaFree(S.d_kx); cudaFree(S.d_csr_cf); cudaFree(S.d_sub);
+    S.d_sub = nullptr;
     S.d_cmx = nullptr;
     S.d_kx = nullptr;
     S.d_csr_cf = nullptr;
@@ -982,46 +1021,54 @@ int finish(msd_ctx* ctx, cudaStream_t st, std::initializer_list<Out*> outs, bool
 
 // Per-chunk workspace for the overlap part.
 struct Chunk {
-    double2 *Gr[2], *O0[2], *Gact[2], *r[2], *wts[2], *part;
+    double2 *Gr[2], *O0[2], *Gact[2], *GactT[2], *m2[2], *rT[2], *r[2], *wts[2], *part;
     float2* rf[2];   // FP32 copies of r (mixed mode, with B)
     void* B[2];
     int nslot, nR;
 };
 
-size_t overlap_bytes_per_walker(msd_ctx* ctx, bool want_b, int nslot)
+// What a call needs of the strings beyond rT: inverse minors and weights (and, in
+// mixed mode, FP32 ratios) with want_b; the ratios as r[w][s] for the FP64
+// per-determinant terms (want_b in FP64 mode) or for the caller (want_r).
+size_t overlap_bytes_per_walker(msd_ctx* ctx, bool want_b, int nslot, bool want_r = false)
 {
+    const bool fp64_b = want_b && ctx->prec == MSD_FP64;
     size_t b = 0;
     for (int s = 0; s < 2; ++s) {
         const SpinHost& S = ctx->sp[s];
-        b += (size_t)S.N * ctx->M + 1 + (size_t)S.nh * S.np + 2 * (size_t)S.n_str;
-        if (want_b) b += S.b_per_walker + (S.n_str + 1) / 2;
+        b += (size_t)S.N * ctx->M + 1 + 2 * (size_t)S.nh * S.np + (size_t)S.n_str;
+        if (!fp64_b) b += minor2_count(tables(S, 1));
+        if (fp64_b || want_r) b += S.n_str;
+        if (want_b) b += S.n_str + S.b_per_walker + (S.n_str + 1) / 2;
     }
     b += nslot;
     return b * sizeof(double2);
 }
 
-int chunk_alloc(msd_ctx* ctx, int cap, bool want_b, int nslot, Chunk& c)
+int chunk_alloc(msd_ctx* ctx, int cap, bool want_b, int nslot, Chunk& c, bool want_r = false)
 {
     int rc;
-    static const char* nGr[2] = {"Gr_a", "Gr_b"}, *nO0[2] = {"O0_a", "O0_b"};
-    static const char* nGa[2] = {"Gact_a", "Gact_b"}, *nr[2] = {"r_a", "r_b"};
-    static const char* nw[2] = {"wts_a", "wts_b"}, *nB[2] = {"B_a", "B_b"}, *nrf[2] = {"rf_a", "rf_b"};
+    const bool fp64_b = want_b && ctx->prec == MSD_FP64;
+    static const char* names[2][10] = {
+        {"Gr_a", "O0_a", "Gact_a", "GactT_a", "m2_a", "rT_a", "r_a", "wts_a", "B_a", "rf_a"},
+        {"Gr_b", "O0_b", "Gact_b", "GactT_b", "m2_b", "rT_b", "r_b", "wts_b", "B_b", "rf_b"}};
     for (int s = 0; s < 2; ++s) {
         const SpinHost& S = ctx->sp[s];
-        void* p;
-        if ((rc = arena_get(ctx, nGr[s], sizeof(double2) * cap * S.N * ctx->M, &p))) return rc; c.Gr[s] = (double2*)p;
-        if ((rc = arena_get(ctx, nO0[s], sizeof(double2) * cap, &p))) return rc; c.O0[s] = (double2*)p;
-        if ((rc = arena_get(ctx, nGa[s], sizeof(double2) * cap * std::max(1, S.nh * S.np), &p))) return rc; c.Gact[s] = (double2*)p;
-        if ((rc = arena_get(ctx, nr[s], sizeof(double2) * cap * S.n_str, &p))) return rc; c.r[s] = (double2*)p;
-        if ((rc = arena_get(ctx, nw[s], sizeof(double2) * cap * S.n_str, &p))) return rc; c.wts[s] = (double2*)p;
-        c.B[s] = nullptr;
-        c.rf[s] = nullptr;
-        if (want_b) {
-            if ((rc = arena_get(ctx, nB[s], sizeof(double2) * std::max<long long>(1, cap * S.b_per_walker), &p))) return rc;
-            c.B[s] = p;
-            if ((rc = arena_get(ctx, nrf[s], sizeof(float2) * cap * S.n_str, &p))) return rc;
-            c.rf[s] = (float2*)p;
-        }
+        const size_t X = std::max(1, S.nh * S.np), w16 = sizeof(double2) * (size_t)cap;
+        auto get = [&](int i, size_t bytes, bool wanted, void** out) {
+            *out = nullptr;
+            return wanted ? arena_get(ctx, names[s][i], bytes, out) : MSD_OK;
+        };
+        if ((rc = get(0, w16 * S.N * ctx->M, true, (void**)&c.Gr[s]))) return rc;
+        if ((rc = get(1, w16, true, (void**)&c.O0[s]))) return rc;
+        if ((rc = get(2, w16 * X, true, (void**)&c.Gact[s]))) return rc;
+        if ((rc = get(3, w16 * X, true, (void**)&c.GactT[s]))) return rc;
+        if ((rc = get(4, w16 * minor2_count(tables(S, 1)), !fp64_b, (void**)&c.m2[s]))) return rc;
+        if ((rc = get(5, w16 * S.n_str, true, (void**)&c.rT[s]))) return rc;
+        if ((rc = get(6, w16 * S.n_str, fp64_b || want_r, (void**)&c.r[s]))) return rc;
+        if ((rc = get(7, w16 * S.n_str, want_b, (void**)&c.wts[s]))) return rc;
+        if ((rc = get(8, sizeof(double2) * std::max<long long>(1, cap * S.b_per_walker), want_b, &c.B[s]))) return rc;
+        if ((rc = get(9, sizeof(float2) * cap * (size_t)S.n_str, want_b, (void**)&c.rf[s]))) return rc;
     }
     void* p;
     if ((rc = arena_get(ctx, "part", sizeof(double2) * cap * std::max(1, nslot), &p))) return rc;
@@ -1041,7 +1088,7 @@ int run_refs(msd_ctx* ctx, const Staged& in, int w0, int nw, int cap, Chunk& c, 
     for (int s = 0; s < 2; ++s) {
         if (s == 1 && in.b_ready) CK(cudaStreamWaitEvent(st, in.b_ready, 0));
         th.begin("k_ref", st);
-        launch_ref(phi[s], nw, M, ctx->n[s], T[s], c.Gr[s], c.O0[s], c.Gact[s], ctx->d_err, st);
+        launch_ref(phi[s], nw, M, ctx->n[s], T[s], c.Gr[s], c.O0[s], c.Gact[s], c.GactT[s], ctx->d_err, st);
         th.end(st);
         CKLAUNCH();
     }
@@ -1049,17 +1096,23 @@ int run_refs(msd_ctx* ctx, const Staged& in, int w0, int nw, int cap, Chunk& c, 
 }
 
 // String minors, ratios and weights of a chunk whose reference inverse is done.
+// Without want_b only the alpha weights' partial sums are formed.
 int run_strings_weights(msd_ctx* ctx, int nw, int cap, Chunk& c, bool want_b, bool fp32_b, cudaStream_t st)
 {
     const TimerHook& th = ctx->hook;
     SpinTables T[2] = {tables(ctx->sp[0], cap), tables(ctx->sp[1], cap)};
-    for (int s = 0; s < 2; ++s) {
-        launch_strings(T[s], nw, c.Gact[s], c.r[s], fp32_b ? c.rf[s] : nullptr, c.B[s], fp32_b, want_b, st, th);
-        CKLAUNCH();
+    if (want_b && !fp32_b) {
+        for (int s = 0; s < 2; ++s) launch_strings(T[s], nw, c.Gact[s], c.r[s], c.rT[s], c.B[s], st, th);
+    } else {
+        th.begin("k_strings", st);
+        launch_minors(T[0], T[1], nw, c.GactT, c.m2, c.rT, st);
+        if (want_b) launch_inverse_minors(T[0], T[1], nw, c.Gact, c.B, st);
+        th.end(st);
     }
+    CKLAUNCH();
+    float2* no_rf[2] = {nullptr, nullptr};
     th.begin("k_weights", st);
-    launch_weights(T[0], nw, c.r[0], c.r[1], T[1].n_str, c.wts[0], c.part, c.nslot, 0, st);
-    launch_weights(T[1], nw, c.r[1], c.r[0], T[0].n_str, c.wts[1], nullptr, c.nslot, 0, st);
+    launch_weights(T[0], T[1], nw, c.rT, c.wts, want_b && fp32_b ? c.rf : no_rf, c.part, c.nslot, want_b, st);
     th.end(st);
     CKLAUNCH();
     return MSD_OK;
@@ -2253,13 +2306,14 @@ int msd_det_ratios(msd_ctx* ctx, int n_w, const double* phi_a, const double* phi
     if ((rc = stage_output(ctx, "out_ratios", ratios, (size_t)n_w * ctx->pairs.n_det, o_r))) return rc;
     if ((rc = stage_output(ctx, "out_refovlp", ref_ovlp, n_w, o_o))) return rc;
     const int nR = weights_blocks(tables(ctx->sp[0], 1));
-    const int cap = chunk_for(ctx, overlap_bytes_per_walker(ctx, false, nR), n_w);
+    const int cap = chunk_for(ctx, overlap_bytes_per_walker(ctx, false, nR, true), n_w);
     Chunk c;
-    if ((rc = chunk_alloc(ctx, cap, false, nR, c))) return rc;
+    if ((rc = chunk_alloc(ctx, cap, false, nR, c, true))) return rc;
     for (int w0 = 0; w0 < n_w; w0 += cap) {
         const int nw = std::min(cap, n_w - w0);
         if ((rc = run_overlap_part(ctx, in, w0, nw, cap, c, false, false, st))) return rc;
         ctx->hook.begin("k_det_ratios", st);
+        for (int s = 0; s < 2; ++s) launch_untranspose(ctx->sp[s].n_str, nw, c.rT[s], c.r[s], st);
         launch_det_ratios(pair_tables(ctx->pairs), nw, ctx->sp[0].n_str, ctx->sp[1].n_str, c.r[0],
                           c.r[1], o_r.dev + (size_t)w0 * ctx->pairs.n_det, st);
         if (o_o.dev) launch_ref_ovlp(nw, c.O0[0], c.O0[1], o_o.dev + w0, st);
@@ -2329,7 +2383,7 @@ int msd_features(msd_ctx* ctx, int n_w, const double* phi_a, const double* phi_b
         const double2* phi[2] = {in.pa + (size_t)w0 * M * ctx->n[0], in.pb + (size_t)w0 * M * ctx->n[1]};
         for (int s = 0; s < 2; ++s) {
             const SpinTables T = tables(ctx->sp[s], cap);
-            launch_ref(phi[s], nw, M, ctx->n[s], T, c.Gr[s], c.O0[s], c.Gact[s], ctx->d_err, st);
+            launch_ref(phi[s], nw, M, ctx->n[s], T, c.Gr[s], c.O0[s], c.Gact[s], nullptr, ctx->d_err, st);
             launch_features(nw, M, ctx->n[s], n_core, n_act, ctx->sp[s].d_pos0, c.Gr[s],
                             feat + (size_t)w0 * 2 * 2 * n_act * n_act, s, st);
         }
@@ -2363,7 +2417,7 @@ int msd_features_rows(msd_ctx* ctx, int n_w, const double* phi_a, const double* 
         long long off = 0;
         for (int s = 0; s < 2; ++s) {
             const SpinTables T = tables(ctx->sp[s], cap);
-            launch_ref(phi[s], nw, M, ctx->n[s], T, c.Gr[s], c.O0[s], c.Gact[s], ctx->d_err, st);
+            launch_ref(phi[s], nw, M, ctx->n[s], T, c.Gr[s], c.O0[s], c.Gact[s], nullptr, ctx->d_err, st);
             launch_features_rows(nw, M, ctx->n[s], c.Gr[s], feat + (size_t)w0 * ld, ld, off, st);
             off += 2LL * ctx->n[s] * M;
         }
@@ -2565,11 +2619,13 @@ extern "C" int msd_overlap_noalloc(msd_ctx* ctx, int n_w, const double* phi_a, c
     const int M = ctx->M;
     SpinTables T1[2] = {tables(ctx->sp[0], 1), tables(ctx->sp[1], 1)};
     const int nR = weights_blocks(T1[0]);
-    // scratch per walker: Gr, O0, Gact, r of both spins, alpha weights, partial sums
+    // scratch per walker: Gr, O0, Gact in both orders, 2 x 2 minors and ratios of
+    // both spins, partial sums
     size_t per = 0;
     for (int s = 0; s < 2; ++s)
-        per += sizeof(double2) * ((size_t)T1[s].N * M + 1 + std::max(1, T1[s].nh * T1[s].np) + T1[s].n_str);
-    per += sizeof(double2) * ((size_t)T1[0].n_str + nR);
+        per += sizeof(double2) * ((size_t)T1[s].N * M + 1 + 2 * std::max(1, T1[s].nh * T1[s].np) + minor2_count(T1[s]) +
+                                  T1[s].n_str);
+    per += sizeof(double2) * (size_t)nR;
     const size_t slack = 16 * 256;   // alignment of the carved arrays
     if (per + slack > (size_t)MSD_STATIC_SCRATCH_BYTES)
         return fail(ctx, MSD_ERR_SHAPE,
@@ -2581,29 +2637,29 @@ extern "C" int msd_overlap_noalloc(msd_ctx* ctx, int n_w, const double* phi_a, c
     unsigned char* base = (unsigned char*)scratch;
     size_t off = 0;
     auto take = [&](size_t bytes) { void* p = base + off; off += align256(bytes); return p; };
-    double2 *Gr[2], *O0[2], *Gact[2], *r[2];
+    double2 *Gr[2], *O0[2], *Gact[2], *GactT[2], *m2[2], *r[2], *no_wts[2] = {nullptr, nullptr};
+    float2* no_rf[2] = {nullptr, nullptr};
     for (int s = 0; s < 2; ++s) {
         Gr[s] = (double2*)take(sizeof(double2) * cap * T1[s].N * (size_t)M);
         O0[s] = (double2*)take(sizeof(double2) * cap);
         Gact[s] = (double2*)take(sizeof(double2) * cap * (size_t)std::max(1, T1[s].nh * T1[s].np));
+        GactT[s] = (double2*)take(sizeof(double2) * cap * (size_t)std::max(1, T1[s].nh * T1[s].np));
+        m2[s] = (double2*)take(sizeof(double2) * cap * minor2_count(T1[s]));
         r[s] = (double2*)take(sizeof(double2) * cap * (size_t)T1[s].n_str);
     }
-    double2* wts = (double2*)take(sizeof(double2) * cap * (size_t)T1[0].n_str);
     double2* part = (double2*)take(sizeof(double2) * cap * (size_t)nR);
     if (off > (size_t)MSD_STATIC_SCRATCH_BYTES)
         return fail(ctx, MSD_ERR_SHAPE, "static scratch layout overflow (%zu bytes)", off);
     CK(cudaMemsetAsync(ctx->d_err, 0, sizeof(unsigned), st));
-    TimerHook none;   // no event timing here: events are not created on this path
     const double2* pa = (const double2*)phi_a;
     const double2* pb = (const double2*)phi_b;
     for (int w0 = 0; w0 < n_w; w0 += cap) {
         const int nw = std::min(cap, n_w - w0);
         SpinTables T[2] = {tables(ctx->sp[0], cap), tables(ctx->sp[1], cap)};
-        launch_ref(pa + (size_t)w0 * M * ctx->n[0], nw, M, ctx->n[0], T[0], Gr[0], O0[0], Gact[0], ctx->d_err, st);
-        launch_ref(pb + (size_t)w0 * M * ctx->n[1], nw, M, ctx->n[1], T[1], Gr[1], O0[1], Gact[1], ctx->d_err, st);
-        launch_strings(T[0], nw, Gact[0], r[0], nullptr, nullptr, false, false, st, none);
-        launch_strings(T[1], nw, Gact[1], r[1], nullptr, nullptr, false, false, st, none);
-        launch_weights(T[0], nw, r[0], r[1], T[1].n_str, wts, part, nR, 0, st);
+        launch_ref(pa + (size_t)w0 * M * ctx->n[0], nw, M, ctx->n[0], T[0], Gr[0], O0[0], Gact[0], GactT[0], ctx->d_err, st);
+        launch_ref(pb + (size_t)w0 * M * ctx->n[1], nw, M, ctx->n[1], T[1], Gr[1], O0[1], Gact[1], GactT[1], ctx->d_err, st);
+        launch_minors(T[0], T[1], nw, GactT, m2, r, st);
+        launch_weights(T[0], T[1], nw, r, no_wts, no_rf, part, nR, false, st);
         launch_sum_slots(nw, part, nR, 0, nR, ratio_sum ? (double2*)ratio_sum + w0 : nullptr, O0[0], O0[1],
                          ovlp ? (double2*)ovlp + w0 : nullptr, st);
         CKLAUNCH();
