@@ -7,32 +7,58 @@
 
 // ------------------------------------------------------------------------
 // Reference determinant per (walker, spin): S = D0^dag phi = phi[occ0, :]
-// (Sec. II A overlap of two determinants). LU with partial pivoting in
-// FP64 gives O0 = det S and S^-1; then
+// (Sec. II A overlap of two determinants). Gauss-Jordan elimination with partial
+// pivoting (by the larger of |Re|, |Im|) in FP64 gives O0 = det S and S^-1; then
 //   Gr[j][r]  = (phi S^-1)[r][j] = G[occ0_j][r]   (G = G0^T, G0 = Theta D0^dag)
 //               (rows r in occ0 of phi are S itself, so there Gr is exactly
 //               the identity and is written, not computed)
 //   Gact[h][p] = G[H_h][P_p]                       (active hole x particle block)
-// One block per walker. A walker whose |det S| falls below 1e-14 times the
-// product of the column norms of S is flagged singular.
-__global__ void __launch_bounds__(256)
-k_ref(const double2* __restrict__ phi, int M, int N, const int* __restrict__ occ0,
-      const int* __restrict__ pos0, const int* __restrict__ hole_pos, int nh, const int* __restrict__ part_orb,
-      int np,
-      double2* __restrict__ Gr, double2* __restrict__ O0, double2* __restrict__ Gact,
-      double2* __restrict__ GactT, unsigned* err)
+// One block per (walker, spin). A walker whose |det S| falls below 1e-14 times
+// the product of the column norms of S is flagged singular.
+//
+// All N^2 entries of a step are independent (an LU followed by column solves left
+// one thread per column with a serial chain: 35 us for a 5 x 5 block, and two
+// thirds of the inversion's FP64 operations on one warp). The product with phi,
+// (M - N) N^2 complex FMAs and most of the FP64 work at larger N, runs on the
+// tensor cores from ref_dg_use on (S^-1 then goes out to Sinv), else here.
+// Measured, both spins: N = 5, 16 walkers 70 -> 21 us; iron-sulfur (N = 30, M = 160)
+// 640 walkers 1.95 -> 1.15 ms, 64 walkers 0.81 -> 0.24 ms; copper-oxo (N = 16, M =
+// 108) 640 walkers 0.73 -> 0.46 ms.
+struct RefIn {
+    const double2* phi;     // [nw][M][N]
+    int N, nh, np;
+    const int *occ0, *pos0, *hole_pos, *part_orb;
+    double2 *Gr, *O0;
+    double2 *Gact, *GactT;  // [nw][nh np], [nh np][nw] (either may be NULL)
+    double2* Sinv;          // [nw][N][N], or NULL: form Gr and the active block here
+};
+struct RefArgs { RefIn s[2]; };
+
+__device__ __forceinline__ double recip_nr(double m);
+__device__ __forceinline__ int mag_key(double2 v);
+
+__device__ __forceinline__ double2 crecip(double2 z)
 {
-    extern __shared__ double2 sm[];
-    double2* S = sm;              // [N][N] LU in place
-    double2* Si = S + N * N;      // [N][N] inverse
-    __shared__ int piv[MSD_NMAX];
+    const double m2 = fma(z.x, z.x, z.y * z.y);
+    if (!(m2 > 1e-280 && m2 < 1e280)) return cdiv(cz(1, 0), z);
+    const double i = recip_nr(m2);
+    return cz(z.x * i, -z.y * i);
+}
+
+__global__ void __launch_bounds__(256)
+k_ref(const __grid_constant__ RefArgs args, int M, unsigned* err)
+{
+    extern __shared__ double2 S[];   // [N][N], overwritten by its inverse (columns permuted)
+    __shared__ double2 prow[MSD_NMAX], pcol[MSD_NMAX], pinv;
+    __shared__ int piv[MSD_NMAX], col[MSD_NMAX];
     __shared__ double cn[MSD_NMAX];
     __shared__ int singular;
-    const int w = blockIdx.x;
+    const RefIn& R = args.s[blockIdx.y];
+    const int w = blockIdx.x, nw = gridDim.x, N = R.N;
     const int t = threadIdx.x, nt = blockDim.x;
-    const double2* ph = phi + (size_t)w * M * N;
+    const double2* ph = R.phi + (size_t)w * M * N;
 
-    for (int e = t; e < N * N; e += nt) S[e] = ph[(size_t)occ0[e / N] * N + e % N];
+    for (int e = t; e < N * N; e += nt) S[e] = ph[(size_t)R.occ0[e / N] * N + e % N];
     if (t == 0) singular = 0;
     __syncthreads();
     for (int j = t; j < N; j += nt) {
@@ -40,105 +66,150 @@ k_ref(const double2* __restrict__ phi, int M, int N, const int* __restrict__ occ
         for (int i = 0; i < N; ++i) a += S[i * N + j].x * S[i * N + j].x + S[i * N + j].y * S[i * N + j].y;
         cn[j] = sqrt(a);
     }
+    double2 det = cz(1, 0);   // thread 0
     for (int k = 0; k < N; ++k) {
         if (t < 32) {
-            double best = -1; int bi = k;
+            int best = -1, bi = k;
             for (int i = k + t; i < N; i += 32) {
-                double v = S[i * N + k].x * S[i * N + k].x + S[i * N + k].y * S[i * N + k].y;
+                const int v = mag_key(S[i * N + k]);
                 if (v > best) { best = v; bi = i; }
             }
-            for (int o = 16; o; o >>= 1) {
-                double ob = __shfl_down_sync(0xffffffffu, best, o);
-                int oi = __shfl_down_sync(0xffffffffu, bi, o);
-                if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
+            const int top = __reduce_max_sync(0xffffffffu, best);
+            bi = __reduce_min_sync(0xffffffffu, best == top ? bi : 0x7fffffff);
+            if (t == 0) {
+                const double2 p = S[bi * N + k];
+                piv[k] = bi;
+                if (p.x == 0.0 && p.y == 0.0) singular = 1;
+                det = cmul(det, p);
+                if (bi != k) det = cz(-det.x, -det.y);
+                pinv = crecip(p);
             }
-            if (t == 0) { piv[k] = bi; if (best == 0.0) singular = 1; }
         }
         __syncthreads();
         if (singular) break;
         const int p = piv[k];
-        if (p != k)
-            for (int j = t; j < N; j += nt) { double2 a = S[k * N + j]; S[k * N + j] = S[p * N + j]; S[p * N + j] = a; }
-        __syncthreads();
-        for (int i = k + 1 + t; i < N; i += nt) S[i * N + k] = cdiv(S[i * N + k], S[k * N + k]);
-        __syncthreads();
-        const int m = N - k - 1;
-        for (int e = t; e < m * m; e += nt) {
-            int i = k + 1 + e / m, j = k + 1 + e % m;
-            S[i * N + j] = cfms(S[i * N + k], S[k * N + j], S[i * N + j]);
+        const double2 pi = pinv;
+        // row p to the pivot place, scaled; row k to row p; column k set aside
+        for (int j = t; j < N; j += nt) {
+            const double2 a = S[p * N + j];
+            prow[j] = j == k ? pi : cmul(a, pi);
+            pcol[j] = j == p ? S[k * N + k] : S[j * N + k];
         }
         __syncthreads();
+        for (int e = t; e < N * N; e += nt) {
+            const int i = e / N, j = e - i * N;
+            if (i == k) continue;
+            const double2 f = pcol[i];
+            const double2 a = j == k ? cz(0, 0) : i == p ? S[k * N + j] : S[e];
+            S[e] = cfms(f, prow[j], a);
+        }
+        __syncthreads();
+        for (int j = t; j < N; j += nt) S[k * N + j] = prow[j];
+        // the pivot search below reads rows > k of column k + 1 only
+        if (t < 32) __syncwarp();
     }
-    __shared__ double2 det;
     if (t == 0) {
-        double2 d = cz(1, 0);
         double nrm = 1;
         if (!singular) {
-            for (int k = 0; k < N; ++k) { d = cmul(d, S[k * N + k]); if (piv[k] != k) d = cz(-d.x, -d.y); nrm *= cn[k]; }
-            if (!(sqrt(d.x * d.x + d.y * d.y) > 1e-14 * nrm)) singular = 1;
+            for (int k = 0; k < N; ++k) { nrm *= cn[k]; col[k] = k; }
+            if (!(sqrt(det.x * det.x + det.y * det.y) > 1e-14 * nrm)) singular = 1;
+            // the row exchanges, undone as column exchanges in reverse order
+            for (int k = N - 1; k >= 0; --k) { const int c = col[k]; col[k] = col[piv[k]]; col[piv[k]] = c; }
         }
-        if (singular) { d = cz(0, 0); atomicOr(err, MSD_DEV_ERR_SINGULAR); }
-        det = d;
-        O0[w] = d;
+        if (singular) { det = cz(0, 0); atomicOr(err, MSD_DEV_ERR_SINGULAR); }
+        R.O0[w] = det;
     }
     __syncthreads();
-    if (singular) {
-        for (int e = t; e < N * M; e += nt) Gr[(size_t)w * N * M + e] = cz(0, 0);
-        for (int e = t; e < nh * np; e += nt) {
-            Gact[(size_t)w * nh * np + e] = cz(0, 0);
-            if (GactT) GactT[(size_t)e * gridDim.x + w] = cz(0, 0);
-        }
+    const int nh = R.nh, np = R.np;
+    double2* gr = R.Gr + (size_t)w * N * M;
+    if (R.Sinv) {
+        double2* out = R.Sinv + (size_t)w * N * N;
+        for (int e = t; e < N * N; e += nt) out[e] = singular ? cz(0, 0) : S[e - e % N + col[e % N]];
         return;
     }
-    // S^-1 column c: solve L U x = P e_c
-    for (int c = t; c < N; c += nt) {
-        double2 x[MSD_NMAX];
-        for (int i = 0; i < N; ++i) x[i] = cz(i == c ? 1 : 0, 0);
-        for (int k = 0; k < N; ++k) { int p = piv[k]; if (p != k) { double2 a = x[k]; x[k] = x[p]; x[p] = a; } }
-        for (int i = 0; i < N; ++i)
-            for (int k = 0; k < i; ++k) x[i] = cfms(S[i * N + k], x[k], x[i]);
-        for (int i = N - 1; i >= 0; --i) {
-            for (int k = i + 1; k < N; ++k) x[i] = cfms(S[i * N + k], x[k], x[i]);
-            x[i] = cdiv(x[i], S[i * N + i]);
-        }
-        for (int i = 0; i < N; ++i) Si[i * N + c] = x[i];
-    }
-    __syncthreads();
-    double2* gr = Gr + (size_t)w * N * M;
-    // lanes over the columns j (S^-1 row reads contiguous, the phi element a
-    // broadcast), warps over the rows r
-    const int JW = N <= 32 ? 32 : 64;
-    for (int e = t; e < M * JW; e += nt) {
-        const int r = e / JW, j = e - r * JW;
-        if (j >= N) continue;
-        const int q = pos0[r];
-        if (q >= 0) {
-            gr[(size_t)j * M + r] = cz(q == j ? 1.0 : 0.0, 0.0);
-            continue;
-        }
-        const double2* pr = ph + (size_t)r * N;
+    for (int e = t; e < M * N; e += nt) {
+        const int r = e / N, j = e - r * N, q = R.pos0[r];
         double2 a = cz(0, 0);
-        for (int k = 0; k < N; ++k) a = cfma(pr[k], Si[k * N + j], a);
+        if (!singular) {
+            if (q >= 0) {
+                a = cz(q == j ? 1.0 : 0.0, 0.0);
+            } else {
+                const double2* pr = ph + (size_t)r * N;
+                const int c = col[j];
+                for (int k = 0; k < N; ++k) a = cfma(pr[k], S[k * N + c], a);
+            }
+        }
         gr[(size_t)j * M + r] = a;
     }
+    __syncthreads();
     for (int e = t; e < nh * np; e += nt) {
-        const int h = e / np, p = e % np;
-        const double2* pr = ph + (size_t)part_orb[p] * N;
-        const int j = hole_pos[h];
-        double2 a = cz(0, 0);
-        for (int k = 0; k < N; ++k) a = cfma(pr[k], Si[k * N + j], a);
-        Gact[(size_t)w * nh * np + e] = a;
-        if (GactT) GactT[(size_t)e * gridDim.x + w] = a;
+        const double2 a = gr[(size_t)R.hole_pos[e / np] * M + R.part_orb[e % np]];
+        if (R.Gact) R.Gact[(size_t)w * nh * np + e] = a;
+        if (R.GactT) R.GactT[(size_t)e * nw + w] = a;
     }
 }
 
-void launch_ref(const double2* phi, int nw, int M, int N, const SpinTables& T, double2* Gr,
-                double2* O0, double2* Gact, double2* GactT, unsigned* err, cudaStream_t st)
+// The active block from the rows of G, in both orders (walkers contiguous in
+// GactT), for blockIdx.y of two spins.
+__global__ void __launch_bounds__(256) k_gact(const __grid_constant__ RefArgs args, int M, int nw)
 {
-    size_t smem = sizeof(double2) * 2 * N * N;
-    if (smem > 48 * 1024) cudaFuncSetAttribute(k_ref, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_ref<<<nw, 256, smem, st>>>(phi, M, N, T.occ0, T.pos0, T.hole_pos, T.nh, T.part_orb, T.np, Gr, O0,
-                                 Gact, GactT, err); msd_note_launch();
+    const RefIn& R = args.s[blockIdx.y];
+    const int X = R.nh * R.np;
+    const long long e = blockIdx.x * 256ll + threadIdx.x;
+    if (e >= (long long)X * nw) return;
+    const int x = (int)(e / nw), w = (int)(e - (long long)x * nw);
+    const double2 a = R.Gr[((size_t)w * R.N + R.hole_pos[x / R.np]) * M + R.part_orb[x % R.np]];
+    if (R.Gact) R.Gact[(size_t)w * X + x] = a;
+    if (R.GactT) R.GactT[e] = a;
+}
+
+// The product with phi runs on the tensor cores from this many complex FMAs per
+// walker on: below, its three launches take longer than the FP64 units (16e3
+// complex FMAs are about 17 us of one SM's).
+bool ref_dg_use(int M, int N) { return (long long)(M - N) * N * N >= 16384; }
+size_t ref_dg_bytes(int M, int N)
+{
+    return ref_dg_use(M, N) ? sizeof(double2) * (size_t)N * N + dg_row_bytes(2 * N) * (M + 2 * (size_t)N) : 0;
+}
+
+int launch_refs(const RefSpinIn* in, int n_spin, int nw, int M, unsigned* err, cudaStream_t st)
+{
+    RefArgs a;
+    int Nmax = 1, X = 0;
+    bool dg = false;
+    for (int s = 0; s < n_spin; ++s) {
+        const SpinTables& T = *in[s].T;
+        a.s[s] = RefIn{in[s].phi, T.N, T.nh, T.np, T.occ0, T.pos0, T.hole_pos, T.part_orb, in[s].Gr, in[s].O0, in[s].Gact,
+                       in[s].GactT, in[s].Sinv};
+        Nmax = Nmax > T.N ? Nmax : T.N;
+        X = X > T.nh * T.np ? X : T.nh * T.np;
+        dg = dg || in[s].Sinv;
+    }
+    const size_t smem = sizeof(double2) * Nmax * Nmax;
+    if (smem > 40 * 1024) cudaFuncSetAttribute(k_ref, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // a block's step updates N^2 entries: no more warps than it has work for
+    const int threads = Nmax <= 8 ? 64 : Nmax <= 16 ? 128 : 256;
+    k_ref<<<dim3(nw, n_spin), threads, smem, st>>>(a, M, err);
+    msd_note_launch();
+    if (!dg) return 0;
+    for (int s = 0; s < n_spin; ++s) {
+        if (!in[s].Sinv) continue;
+        const int N = in[s].T->N;
+        dg_slice_real((long long)nw * M, 2 * N, (const double*)in[s].phi, 2 * N, in[s].sa, in[s].ea, st);
+        dg_slice_columns(1, N, N, nw, in[s].Sinv, N, (long long)N * N, 0, N, nullptr, nullptr, in[s].sb, in[s].eb, st);
+        DgOut o;
+        o.Mr = M; o.Nc = N; o.batch = nw;
+        o.C = in[s].Gr; o.c_batch = (long long)N * M; o.c_n = M; o.c_m = 1;
+        o.eye = in[s].T->pos0;
+        if (dg_gemm({in[s].sa, in[s].ea, nw * M, M}, {in[s].sb, in[s].eb, 2 * N * nw, 2 * N}, o, 2 * N, err, st)) return -1;
+    }
+    if (X > 0 && (in[0].Gact || in[0].GactT)) {
+        // spins whose product ran in k_ref have their block already; writing it
+        // again is the same values
+        k_gact<<<dim3((unsigned)(((long long)X * nw + 255) / 256), n_spin), 256, 0, st>>>(a, M, nw);
+        msd_note_launch();
+    }
+    return 0;
 }
 
 // ------------------------------------------------------------------------

@@ -13,9 +13,21 @@ struct TimerHook {
 };
 
 // k_wick.cu
-// GactT (may be NULL): the active block with the walkers contiguous, [nh np][nw].
-void launch_ref(const double2* phi, int nw, int M, int N, const SpinTables& T, double2* Gr,
-                double2* O0, double2* Gact, double2* GactT, unsigned* err, cudaStream_t st);
+// Reference inverse of one spin: inputs, outputs and, where ref_dg_use, the
+// scratch of the tensor-core product (Sinv [nw][N][N]; sa, ea: M rows, sb, eb: 2 N
+// rows of dg_row_bytes(2 N) per walker; all NULL otherwise). GactT: the active
+// block with the walkers contiguous, [nh np][nw].
+struct RefSpinIn {
+    const SpinTables* T = nullptr;
+    const double2* phi = nullptr;
+    double2 *Gr = nullptr, *O0 = nullptr, *Gact = nullptr, *GactT = nullptr;
+    double2* Sinv = nullptr;
+    void *sa = nullptr, *sb = nullptr;
+    int *ea = nullptr, *eb = nullptr;
+};
+bool ref_dg_use(int M, int N);
+size_t ref_dg_bytes(int M, int N);   // that scratch per walker (0 if unused)
+int launch_refs(const RefSpinIn* in, int n_spin, int nw, int M, unsigned* err, cudaStream_t st);
 // FP64 ratios r[w][s] and rT[s][w] and FP64 inverse minors by pivoted LU.
 void launch_strings(const SpinTables& tb, int nw, const double2* Gact, double2* r, double2* rT, void* B, cudaStream_t st,
                     const TimerHook& th);
@@ -137,6 +149,7 @@ struct DgOperand {
 // part at z c_batch, for dg_sum_splits. gx >= 0: the rows of A and B stack gx
 // alpha and gy beta entries, and the (alpha, alpha), (beta, beta) and (alpha,
 // beta) blocks go to K[0], K[2], K[1] ([batch][rows][columns] each) instead of C.
+// eye [Mr]: rows m with eye[m] >= 0 are written as unit vectors (1 at n = eye[m]).
 struct DgOut {
     int Mr = 0, Nc = 0, batch = 1, splits = 1;
     double2* C = nullptr;
@@ -146,6 +159,7 @@ struct DgOut {
     double mul = 1.0;
     int gx = -1, gy = 0;
     double2* K[3] = {nullptr, nullptr, nullptr};
+    const int* eye = nullptr;
 };
 int dg_k_padded(int K);
 size_t dg_row_bytes(int K);              // slices and exponent of one real row

@@ -1037,6 +1037,7 @@ size_t overlap_bytes_per_walker(msd_ctx* ctx, bool want_b, int nslot, bool want_
     for (int s = 0; s < 2; ++s) {
         const SpinHost& S = ctx->sp[s];
         b += (size_t)S.N * ctx->M + 1 + 2 * (size_t)S.nh * S.np + (size_t)S.n_str;
+        b += ref_dg_bytes(ctx->M, S.N) / sizeof(double2) + 1;
         if (!fp64_b) b += minor2_count(tables(S, 1));
         if (fp64_b || want_r) b += S.n_str;
         if (want_b) b += S.n_str + S.b_per_walker + (S.n_str + 1) / 2;
@@ -1078,20 +1079,40 @@ int chunk_alloc(msd_ctx* ctx, int cap, bool want_b, int nslot, Chunk& c, bool wa
     return MSD_OK;
 }
 
-// Reference inverse of walkers [w0, w0 + nw), both spins.
-int run_refs(msd_ctx* ctx, const Staged& in, int w0, int nw, int cap, Chunk& c, cudaStream_t st)
+// Reference inverse of walkers [w0, w0 + nw), both spins: one launch, or alpha
+// first while host beta walkers are still being copied.
+int run_refs(msd_ctx* ctx, const Staged& in, int w0, int nw, int cap, Chunk& c, cudaStream_t st, bool want_act = true)
 {
     const int M = ctx->M;
     const TimerHook& th = ctx->hook;
-    SpinTables T[2] = {tables(ctx->sp[0], cap), tables(ctx->sp[1], cap)};
-    const double2* phi[2] = {in.pa + (size_t)w0 * M * ctx->n[0], in.pb + (size_t)w0 * M * ctx->n[1]};
+    const SpinTables T[2] = {tables(ctx->sp[0], cap), tables(ctx->sp[1], cap)};
+    RefSpinIn r[2];
+    static const char* names[2][5] = {{"ref_inv_a", "ref_sa_a", "ref_ea_a", "ref_sb_a", "ref_eb_a"},
+                                      {"ref_inv_b", "ref_sa_b", "ref_ea_b", "ref_sb_b", "ref_eb_b"}};
     for (int s = 0; s < 2; ++s) {
-        if (s == 1 && in.b_ready) CK(cudaStreamWaitEvent(st, in.b_ready, 0));
-        th.begin("k_ref", st);
-        launch_ref(phi[s], nw, M, ctx->n[s], T[s], c.Gr[s], c.O0[s], c.Gact[s], c.GactT[s], ctx->d_err, st);
-        th.end(st);
-        CKLAUNCH();
+        const int N = ctx->n[s];
+        r[s].T = &T[s];
+        r[s].phi = (s ? in.pb : in.pa) + (size_t)w0 * M * N;
+        r[s].Gr = c.Gr[s]; r[s].O0 = c.O0[s];
+        if (want_act) { r[s].Gact = c.Gact[s]; r[s].GactT = c.GactT[s]; }
+        if (!ref_dg_use(M, N)) continue;
+        int rc;
+        const size_t rb = dg_row_bytes(2 * N);
+        if ((rc = arena_get(ctx, names[s][0], sizeof(double2) * cap * (size_t)N * N, (void**)&r[s].Sinv))) return rc;
+        if ((rc = arena_get(ctx, names[s][1], rb * cap * (size_t)M, &r[s].sa))) return rc;
+        if ((rc = arena_get(ctx, names[s][2], sizeof(int) * cap * (size_t)M, (void**)&r[s].ea))) return rc;
+        if ((rc = arena_get(ctx, names[s][3], rb * cap * 2 * (size_t)N, &r[s].sb))) return rc;
+        if ((rc = arena_get(ctx, names[s][4], sizeof(int) * cap * 2 * (size_t)N, (void**)&r[s].eb))) return rc;
     }
+    th.begin("k_ref", st);
+    int g = launch_refs(r, in.b_ready ? 1 : 2, nw, M, ctx->d_err, st);
+    if (!g && in.b_ready) {
+        CK(cudaStreamWaitEvent(st, in.b_ready, 0));
+        g = launch_refs(r + 1, 1, nw, M, ctx->d_err, st);
+    }
+    th.end(st);
+    if (g) return fail(ctx, MSD_ERR_CUDA, "reference tensor-core product launch failed");
+    CKLAUNCH();
     return MSD_OK;
 }
 
@@ -2380,10 +2401,8 @@ int msd_features(msd_ctx* ctx, int n_w, const double* phi_a, const double* phi_b
     const int M = ctx->M;
     for (int w0 = 0; w0 < n_w; w0 += cap) {
         const int nw = std::min(cap, n_w - w0);
-        const double2* phi[2] = {in.pa + (size_t)w0 * M * ctx->n[0], in.pb + (size_t)w0 * M * ctx->n[1]};
+        if ((rc = run_refs(ctx, in, w0, nw, cap, c, st, false))) return rc;
         for (int s = 0; s < 2; ++s) {
-            const SpinTables T = tables(ctx->sp[s], cap);
-            launch_ref(phi[s], nw, M, ctx->n[s], T, c.Gr[s], c.O0[s], c.Gact[s], nullptr, ctx->d_err, st);
             launch_features(nw, M, ctx->n[s], n_core, n_act, ctx->sp[s].d_pos0, c.Gr[s],
                             feat + (size_t)w0 * 2 * 2 * n_act * n_act, s, st);
         }
@@ -2413,11 +2432,9 @@ int msd_features_rows(msd_ctx* ctx, int n_w, const double* phi_a, const double* 
     if (ld > need) CK(cudaMemsetAsync(feat, 0, sizeof(float) * (size_t)n_w * ld, st));
     for (int w0 = 0; w0 < n_w; w0 += cap) {
         const int nw = std::min(cap, n_w - w0);
-        const double2* phi[2] = {in.pa + (size_t)w0 * M * ctx->n[0], in.pb + (size_t)w0 * M * ctx->n[1]};
+        if ((rc = run_refs(ctx, in, w0, nw, cap, c, st, false))) return rc;
         long long off = 0;
         for (int s = 0; s < 2; ++s) {
-            const SpinTables T = tables(ctx->sp[s], cap);
-            launch_ref(phi[s], nw, M, ctx->n[s], T, c.Gr[s], c.O0[s], c.Gact[s], nullptr, ctx->d_err, st);
             launch_features_rows(nw, M, ctx->n[s], c.Gr[s], feat + (size_t)w0 * ld, ld, off, st);
             off += 2LL * ctx->n[s] * M;
         }
@@ -2619,11 +2636,11 @@ extern "C" int msd_overlap_noalloc(msd_ctx* ctx, int n_w, const double* phi_a, c
     const int M = ctx->M;
     SpinTables T1[2] = {tables(ctx->sp[0], 1), tables(ctx->sp[1], 1)};
     const int nR = weights_blocks(T1[0]);
-    // scratch per walker: Gr, O0, Gact in both orders, 2 x 2 minors and ratios of
-    // both spins, partial sums
+    // scratch per walker: Gr, O0, active block, 2 x 2 minors and ratios of both
+    // spins, partial sums
     size_t per = 0;
     for (int s = 0; s < 2; ++s)
-        per += sizeof(double2) * ((size_t)T1[s].N * M + 1 + 2 * std::max(1, T1[s].nh * T1[s].np) + minor2_count(T1[s]) +
+        per += sizeof(double2) * ((size_t)T1[s].N * M + 1 + std::max(1, T1[s].nh * T1[s].np) + minor2_count(T1[s]) +
                                   T1[s].n_str);
     per += sizeof(double2) * (size_t)nR;
     const size_t slack = 16 * 256;   // alignment of the carved arrays
@@ -2637,12 +2654,11 @@ extern "C" int msd_overlap_noalloc(msd_ctx* ctx, int n_w, const double* phi_a, c
     unsigned char* base = (unsigned char*)scratch;
     size_t off = 0;
     auto take = [&](size_t bytes) { void* p = base + off; off += align256(bytes); return p; };
-    double2 *Gr[2], *O0[2], *Gact[2], *GactT[2], *m2[2], *r[2], *no_wts[2] = {nullptr, nullptr};
+    double2 *Gr[2], *O0[2], *GactT[2], *m2[2], *r[2], *no_wts[2] = {nullptr, nullptr};
     float2* no_rf[2] = {nullptr, nullptr};
     for (int s = 0; s < 2; ++s) {
         Gr[s] = (double2*)take(sizeof(double2) * cap * T1[s].N * (size_t)M);
         O0[s] = (double2*)take(sizeof(double2) * cap);
-        Gact[s] = (double2*)take(sizeof(double2) * cap * (size_t)std::max(1, T1[s].nh * T1[s].np));
         GactT[s] = (double2*)take(sizeof(double2) * cap * (size_t)std::max(1, T1[s].nh * T1[s].np));
         m2[s] = (double2*)take(sizeof(double2) * cap * minor2_count(T1[s]));
         r[s] = (double2*)take(sizeof(double2) * cap * (size_t)T1[s].n_str);
@@ -2656,8 +2672,13 @@ extern "C" int msd_overlap_noalloc(msd_ctx* ctx, int n_w, const double* phi_a, c
     for (int w0 = 0; w0 < n_w; w0 += cap) {
         const int nw = std::min(cap, n_w - w0);
         SpinTables T[2] = {tables(ctx->sp[0], cap), tables(ctx->sp[1], cap)};
-        launch_ref(pa + (size_t)w0 * M * ctx->n[0], nw, M, ctx->n[0], T[0], Gr[0], O0[0], Gact[0], GactT[0], ctx->d_err, st);
-        launch_ref(pb + (size_t)w0 * M * ctx->n[1], nw, M, ctx->n[1], T[1], Gr[1], O0[1], Gact[1], GactT[1], ctx->d_err, st);
+        RefSpinIn in[2];
+        for (int s = 0; s < 2; ++s) {
+            in[s].T = &T[s];
+            in[s].phi = (s ? pb : pa) + (size_t)w0 * M * ctx->n[s];
+            in[s].Gr = Gr[s]; in[s].O0 = O0[s]; in[s].GactT = GactT[s];
+        }
+        launch_refs(in, 2, nw, M, ctx->d_err, st);
         launch_minors(T[0], T[1], nw, GactT, m2, r, st);
         launch_weights(T[0], T[1], nw, r, no_wts, no_rf, part, nR, false, st);
         launch_sum_slots(nw, part, nR, 0, nR, ratio_sum ? (double2*)ratio_sum + w0 : nullptr, O0[0], O0[1],
