@@ -213,59 +213,72 @@ k_tc_dgemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUten
                 mbar_drain(&full_bar[k % DG_STAGES], (k / DG_STAGES) & 1);
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            // ---------------------------------------------------- MMA issuer
-            constexpr uint32_t idesc = idesc_bf16(DG_BM, DG_BN);
-            bool ok = true;
-            int it = 0, unit = 0;   // unit: one chunk of one tile, one use of the accumulators
-            for (int t = blockIdx.x; t < ntile && ok; t += gridDim.x) {
-                const DgTile tl = dg_tile(a, t);
-                if (dg_skip(a, tl)) continue;
-                const int z = tl.z, k1 = kend(z);
-                for (int c0 = kbeg(z); c0 < k1 && ok; c0 += DG_CHUNK, ++unit) {
-                    const int c1 = min(k1, c0 + DG_CHUNK);
-                    for (int kb = c0; kb < c1; ++kb, ++it) {
-                        const int s = it % DG_STAGES;
-                        if (!mbar_wait(&full_bar[s], (it / DG_STAGES) & 1, wb) || *vfail) { ok = false; break; }
-                        tc_fence_after();
-                        const uint32_t sa = su32(smem + (size_t)s * DG_STAGE);
-                        const uint32_t sb = sa + DG_S * DG_A_SL;
+        // -------------------------------------------------------- MMA issuer
+        // The whole warp runs the loop and one elected thread issues: the
+        // descriptors stay in uniform registers (computed by a single diverged
+        // lane, an MMA of 32 tensor clocks took 90 to issue).
+        constexpr uint32_t idesc = idesc_bf16(DG_BM, DG_BN);
+        const bool leader = elect_one();
+        const uint64_t desc0 = sw64_desc(su32(smem));
+        bool ok = true;
+        int it = 0, unit = 0;   // unit: one chunk of one tile, one use of the accumulators
+        for (int t = blockIdx.x; t < ntile && ok; t += gridDim.x) {
+            const DgTile tl = dg_tile(a, t);
+            if (dg_skip(a, tl)) continue;
+            const int z = tl.z, k1 = kend(z);
+            for (int c0 = kbeg(z); c0 < k1 && ok; c0 += DG_CHUNK, ++unit) {
+                const int c1 = min(k1, c0 + DG_CHUNK);
+                for (int kb = c0; kb < c1; ++kb, ++it) {
+                    const int s = it % DG_STAGES;
+                    const bool got = mbar_wait(&full_bar[s], (it / DG_STAGES) & 1, wb) && !*vfail;
+                    if (!__all_sync(0xffffffffu, got)) { ok = false; break; }
+                    tc_fence_after();
+                    const uint64_t dA = desc0 + (uint64_t)((uint32_t)s * DG_STAGE >> 4);
+                    const uint64_t dB = dA + (uint64_t)(DG_S * DG_A_SL >> 4);
 #pragma unroll
-                        for (int kk = 0; kk < 2; ++kk) {   // 2 x 16 BF16 of K per k-block
-                            uint64_t da[DG_S], db[DG_S];
-#pragma unroll
-                            for (int i = 0; i < DG_S; ++i) {
-                                da[i] = sw64_desc(sa + i * DG_A_SL + kk * 32);
-                                db[i] = sw64_desc(sb + i * DG_B_SL + kk * 32);
-                            }
-                            const bool first = kb == c0 && kk == 0;
+                    for (int kk = 0; kk < 2; ++kk) {   // 2 x 16 BF16 of K per k-block
+                        if (kb == c0 && kk == 0) {
+                            // first use of the accumulators: as the epilogue
+                            // releases them, c ascending
 #pragma unroll
                             for (int c = 0; c < DG_S; ++c) {   // accumulator c: i + j = c (digits from 0)
-                                if (first && unit > 0 && ok) {
-                                    // the epilogue has read this accumulator of the previous unit
-                                    if (!mbar_wait(&tempty[c], (unit - 1) & 1, wb)) ok = false;
+                                if (unit > 0) {
+                                    const bool free_ = mbar_wait(&tempty[c], (unit - 1) & 1, wb);
+                                    ok = __all_sync(0xffffffffu, free_) && ok;
                                     tc_fence_after();
                                 }
-                                if (ok) {
+                                if (ok && leader) {
 #pragma unroll
                                     for (int i = 0; i <= c; ++i)
-                                        mma_bf16(tmem + (uint32_t)(c * DG_BN), da[i], db[c - i], idesc,
-                                                 (first && i == 0) ? 0u : 1u);
+                                        mma_bf16(tmem + (uint32_t)(c * DG_BN), dA + (uint64_t)(i * (DG_A_SL >> 4)),
+                                                 dB + (uint64_t)((c - i) * (DG_B_SL >> 4)), idesc, i == 0 ? 0u : 1u);
                                 }
                             }
+                        } else if (ok && leader) {
+                            // consecutive products go to different accumulators
+#pragma unroll
+                            for (int i = 0; i < DG_S; ++i)
+#pragma unroll
+                                for (int c = DG_S - 1; c >= i; --c)
+                                    mma_bf16(tmem + (uint32_t)(c * DG_BN), dA + (uint64_t)(i * (DG_A_SL >> 4) + kk * 2),
+                                             dB + (uint64_t)((c - i) * (DG_B_SL >> 4) + kk * 2), idesc, 1u);
                         }
-                        if (!ok) break;
-                        mma_commit(&empty_bar[s]);
                     }
+                    __syncwarp();
                     if (!ok) break;
-                    mma_commit(&tfull);
+                    if (leader) mma_commit(&empty_bar[s]);
                 }
+                if (!ok) break;
+                if (leader) mma_commit(&tfull);
             }
+        }
+        if (leader) {
             if (!ok) { *vfail = 1; atomicOr(a.err, MSD_DEV_ERR_TIMEOUT); }
             // every product issued by this thread completes before TMEM is freed
             mma_commit(&drain_bar);
             mbar_drain(&drain_bar, 0);
         }
+        __syncwarp();
     } else {
         // -------------------------------------------------------- epilogue
         const int q = warp & 3, hf = (warp - 2) >> 2;
