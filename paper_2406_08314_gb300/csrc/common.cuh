@@ -121,6 +121,20 @@ __device__ __forceinline__ int rec_p(const uint4& r, int i) { return (int)(((i <
 
 
 #ifdef __CUDACC__
+// x 2^-e as an integer of 56 fractional bits, rounded to nearest (integer
+// operations only: FP64 ones issue at a sixty-fourth of their rate).
+__device__ __forceinline__ long long fixed56(double x, int e)
+{
+    const long long b = __double_as_longlong(x);
+    const int f = (int)((b >> 52) & 0x7ff);
+    long long m = b & 0xfffffffffffffll;
+    if (f) m |= 1ll << 52;
+    const int sh = (f ? f : 1) - 1075 + 56 - e;   // <= 3
+    if (sh >= 0) m <<= min(sh, 3);
+    else m = sh > -56 ? (m + (1ll << (-sh - 1))) >> -sh : 0;
+    return b < 0 ? -m : m;
+}
+
 // Sum of n partial sums by one warp (every lane returns it).
 __device__ __forceinline__ double2 warp_sum_slots(const double2* __restrict__ p, int n, int lane)
 {

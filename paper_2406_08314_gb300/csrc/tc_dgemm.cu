@@ -370,20 +370,6 @@ __device__ __forceinline__ int dg_exponent(unsigned top)
     return f == 0x7ff ? DG_NAN : f - 1022;
 }
 
-// x 2^-e as an integer of 56 fractional bits, rounded to nearest (integer
-// operations only: FP64 ones issue at a sixty-fourth of their rate).
-__device__ __forceinline__ long long dg_fixed(double x, int e)
-{
-    const long long b = __double_as_longlong(x);
-    const int f = (int)((b >> 52) & 0x7ff);
-    long long m = b & 0xfffffffffffffll;
-    if (f) m |= 1ll << 52;
-    const int sh = (f ? f : 1) - 1075 + 56 - e;   // <= 3
-    if (sh >= 0) m <<= min(sh, 3);
-    else m = sh > -56 ? (m + (1ll << (-sh - 1))) >> -sh : 0;
-    return b < 0 ? -m : m;
-}
-
 // The eight digits of eight fixed-point values as BF16: u[i] packs digit i (most
 // significant first) of the eight.
 __device__ __forceinline__ void dg_digits8(long long* q, uint4* u)
@@ -424,58 +410,74 @@ __device__ __forceinline__ void dg_store8(long long* q, __nv_bfloat16* out, size
 
 __device__ __forceinline__ unsigned dg_mag(double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; }
 
-__device__ __forceinline__ unsigned warp_max(unsigned v)
-{
-    for (int o = 16; o; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
-}
-
-// Rows of a row-major matrix, one warp per row: src[r ld + k], real (part 0 of
-// 1) or the two parts of a complex row as rows 2r, 2r + 1.
-template <bool CPLX>
+// Rows of a row-major matrix: src[r ld + k], real, or the two parts of a complex
+// row as rows 2r, 2r + 1. LR lanes per row, each 8 consecutive elements of the
+// row at a time (one 16-byte store per digit).
+template <bool CPLX, int LR>
 __global__ void __launch_bounds__(256)
 k_dg_rows(long long R, int K, int Kp, const double* __restrict__ src, long long ld, __nv_bfloat16* __restrict__ S,
           int* __restrict__ ex, size_t stride)
 {
-    const long long r = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31;
-    if (r >= R) return;
-    const double* p = src + (CPLX ? 2 : 1) * r * ld;
+    const long long r = ((long long)blockIdx.x * 256 + threadIdx.x) / LR;
+    const int lane = threadIdx.x % LR;
+    const bool live = r < R;
+    const double* p = src + (CPLX ? 2 : 1) * (live ? r : 0) * ld;
     unsigned t0 = 0, t1 = 0;
-    if (CPLX) {
-        const double2* p2 = reinterpret_cast<const double2*>(p);
-        for (int k = lane; k < K; k += 32) {
-            const double2 v = p2[k];
-            t0 = max(t0, dg_mag(v.x));
-            t1 = max(t1, dg_mag(v.y));
+    if (live) {
+        if (CPLX) {
+            const double2* p2 = reinterpret_cast<const double2*>(p);
+            for (int k = lane; k < K; k += LR) {
+                const double2 v = p2[k];
+                t0 = max(t0, dg_mag(v.x));
+                t1 = max(t1, dg_mag(v.y));
+            }
+        } else {
+            for (int k = lane; k < K; k += LR) t0 = max(t0, dg_mag(p[k]));
         }
-        t1 = warp_max(t1);
-    } else {
-        for (int k = lane; k < K; k += 32) t0 = max(t0, dg_mag(p[k]));
     }
-    t0 = warp_max(t0);
+#pragma unroll
+    for (int o = LR / 2; o; o >>= 1) {
+        t0 = max(t0, __shfl_xor_sync(0xffffffffu, t0, o));
+        if (CPLX) t1 = max(t1, __shfl_xor_sync(0xffffffffu, t1, o));
+    }
+    if (!live) return;
     const int e0 = dg_exponent(t0), e1 = dg_exponent(t1);
     if (lane == 0) {
         ex[(CPLX ? 2 : 1) * r] = e0;
         if (CPLX) ex[2 * r + 1] = e1;
     }
     __nv_bfloat16* o0 = S + (size_t)((CPLX ? 2 : 1) * r) * Kp;
-    for (int k0 = lane * 8; k0 < Kp; k0 += 256) {
+    for (int k0 = lane * 8; k0 < Kp; k0 += 8 * LR) {
         long long q0[8], q1[8];
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
             const int k = k0 + j;
             if (CPLX) {
                 const double2 v = k < K ? reinterpret_cast<const double2*>(p)[k] : make_double2(0, 0);
-                q0[j] = dg_fixed(v.x, e0);
-                q1[j] = dg_fixed(v.y, e1);
+                q0[j] = fixed56(v.x, e0);
+                q1[j] = fixed56(v.y, e1);
             } else {
-                q0[j] = dg_fixed(k < K ? p[k] : 0.0, e0);
+                q0[j] = fixed56(k < K ? p[k] : 0.0, e0);
             }
         }
         dg_store8(q0, o0 + k0, stride);
         if (CPLX) dg_store8(q1, o0 + Kp + k0, stride);
     }
+}
+
+template <bool CPLX>
+void launch_dg_rows(long long R, int K, const double* src, long long ld, void* S, int* ex, size_t stride, cudaStream_t st)
+{
+    const int Kp = dg_k_padded(K);
+    // lanes per row: as many as have a group of 8 elements to write
+    const int lr = Kp > 128 ? 32 : Kp > 64 ? 16 : Kp > 32 ? 8 : 4;
+    const unsigned grid = (unsigned)((R * lr + 255) / 256);
+    __nv_bfloat16* s = (__nv_bfloat16*)S;
+    if (lr == 32) k_dg_rows<CPLX, 32><<<grid, 256, 0, st>>>(R, K, Kp, src, ld, s, ex, stride);
+    else if (lr == 16) k_dg_rows<CPLX, 16><<<grid, 256, 0, st>>>(R, K, Kp, src, ld, s, ex, stride);
+    else if (lr == 8) k_dg_rows<CPLX, 8><<<grid, 256, 0, st>>>(R, K, Kp, src, ld, s, ex, stride);
+    else k_dg_rows<CPLX, 4><<<grid, 256, 0, st>>>(R, K, Kp, src, ld, s, ex, stride);
+    msd_note_launch();
 }
 
 // Columns of a complex matrix src[z][k][c] (row stride ld, batch stride
@@ -534,7 +536,7 @@ k_dg_cols(int K, int Kp, int nc, const double2* __restrict__ src, long long ld, 
                     for (int part = 0; part < 2; ++part) {
                         long long q[8];
 #pragma unroll
-                        for (int j = 0; j < 8; ++j) q[j] = dg_fixed(part ? tile[kb + j][ci].y : tile[kb + j][ci].x, e);
+                        for (int j = 0; j < 8; ++j) q[j] = fixed56(part ? tile[kb + j][ci].y : tile[kb + j][ci].x, e);
                         dg_store8(q, Sb + (2 * r + part) * Kp + k0 + kb, stride_b);
                     }
             } else {
@@ -543,8 +545,8 @@ k_dg_cols(int K, int Kp, int nc, const double2* __restrict__ src, long long ld, 
                     long long q[8];
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
-                        q[2 * j] = dg_fixed(tile[kb + j][ci].x, e);
-                        q[2 * j + 1] = dg_fixed(tile[kb + j][ci].y, e);
+                        q[2 * j] = fixed56(tile[kb + j][ci].x, e);
+                        q[2 * j + 1] = fixed56(tile[kb + j][ci].y, e);
                     }
                     const size_t o = (size_t)2 * (k0 + kb);
                     uint4 u[DG_S];
@@ -586,17 +588,12 @@ size_t dg_row_bytes(int K) { return (size_t)DG_S * dg_k_padded(K) * sizeof(__nv_
 
 void dg_slice_real(long long R, int K, const double* src, long long ld, void* S, int* ex, cudaStream_t st)
 {
-    const int Kp = dg_k_padded(K);
-    k_dg_rows<false><<<(unsigned)((R + 7) / 8), 256, 0, st>>>(R, K, Kp, src, ld, (__nv_bfloat16*)S, ex, (size_t)R * Kp);
-    msd_note_launch();
+    launch_dg_rows<false>(R, K, src, ld, S, ex, (size_t)R * dg_k_padded(K), st);
 }
 
 void dg_slice_complex(long long R, int K, const double2* src, long long ld, void* S, int* ex, cudaStream_t st)
 {
-    const int Kp = dg_k_padded(K);
-    k_dg_rows<true><<<(unsigned)((R + 7) / 8), 256, 0, st>>>(R, K, Kp, (const double*)src, ld, (__nv_bfloat16*)S, ex,
-                                                             (size_t)2 * R * Kp);
-    msd_note_launch();
+    launch_dg_rows<true>(R, K, (const double*)src, ld, S, ex, (size_t)2 * R * dg_k_padded(K), st);
 }
 
 void dg_slice_columns(int mode, int K, int nc, int batch, const double2* src, long long ld, long long src_batch,

@@ -261,48 +261,48 @@ k_tc_fepi(const __grid_constant__ CUtensorMap ta_hi, const __grid_constant__ CUt
                 mbar_drain(&full_bar[k % FE_STAGES], (k / FE_STAGES) & 1);
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            // ------------------------------------------------ MMA issuer
-            const uint32_t idesc = idesc_tf32(128, a.BNe);
-            int kbg = 0, it = 0;
-            for (int tile = blockIdx.x; tile < a.n_tiles && !*vfail; tile += gridDim.x, ++it) {
-                const int b = it & 1;
-                if (!mbar_wait(&tempty[b], ((it >> 1) & 1) ^ 1, wb)) {
-                    *vfail = 1;
-                    atomicOr(a.err, MSD_DEV_ERR_TIMEOUT);
-                    break;
-                }
+        // ---------------------------------------------------- MMA issuer
+        // (one elected thread of the converged warp: the descriptors stay in
+        // uniform registers)
+        const uint32_t idesc = idesc_tf32(128, a.BNe);
+        const bool leader = elect_one();
+        const uint64_t desc0 = sw64_desc(su32(smem));
+        int kbg = 0, it = 0;
+        bool ok = true;
+        for (int tile = blockIdx.x; tile < a.n_tiles && ok; tile += gridDim.x, ++it) {
+            const int b = it & 1;
+            const bool free_ = mbar_wait(&tempty[b], ((it >> 1) & 1) ^ 1, wb) && !*vfail;
+            if (!__all_sync(0xffffffffu, free_)) { ok = false; break; }
+            tc_fence_after();
+            const uint32_t acc = tmem + (uint32_t)(b * FE_TCOLS);
+            for (int kb = 0; kb < nkb; ++kb, ++kbg) {
+                const int s = kbg % FE_STAGES;
+                const bool got = mbar_wait(&full_bar[s], (kbg / FE_STAGES) & 1, wb) && !*vfail;
+                if (!__all_sync(0xffffffffu, got)) { ok = false; break; }
                 tc_fence_after();
-                const uint32_t acc = tmem + (uint32_t)(b * FE_TCOLS);
-                bool ok = true;
-                for (int kb = 0; kb < nkb; ++kb, ++kbg) {
-                    const int s = kbg % FE_STAGES;
-                    if (!mbar_wait(&full_bar[s], (kbg / FE_STAGES) & 1, wb) || *vfail) { ok = false; break; }
-                    tc_fence_after();
-                    const uint32_t sa = su32(smem + (size_t)s * STAGE_BYTES);
+                if (leader) {
                     const int nk = min(2, (a.K - kb * 16) / 8);
+                    const uint64_t dA = desc0 + (uint64_t)((uint32_t)s * STAGE_BYTES >> 4);
                     for (int kk = 0; kk < nk; ++kk) {   // 2 x 32 bytes of K per k-block
-                        const uint64_t ah = sw64_desc(sa + kk * 32);
-                        const uint64_t al = sw64_desc(sa + FE_A_BYTES + kk * 32);
-                        const uint64_t bh = sw64_desc(sa + 2 * FE_A_BYTES + kk * 32);
-                        const uint64_t bl = sw64_desc(sa + 2 * FE_A_BYTES + B_BYTES + kk * 32);
+                        const uint64_t ah = dA + kk * 2, al = ah + (uint64_t)(FE_A_BYTES >> 4);
+                        const uint64_t bh = al + (uint64_t)(FE_A_BYTES >> 4), bl = bh + (uint64_t)(B_BYTES >> 4);
                         mma_tf32(acc, ah, bh, idesc, (kb | kk) != 0);
                         mma_tf32(acc, ah, bl, idesc, 1u);
                         mma_tf32(acc, al, bh, idesc, 1u);
                     }
                     mma_commit(&empty_bar[s]);
                 }
-                if (!ok) {
-                    *vfail = 1;
-                    atomicOr(a.err, MSD_DEV_ERR_TIMEOUT);
-                    break;
-                }
-                mma_commit(&tfull[b]);
+                __syncwarp();
             }
+            if (ok && leader) mma_commit(&tfull[b]);
+        }
+        if (leader) {
+            if (!ok) { *vfail = 1; atomicOr(a.err, MSD_DEV_ERR_TIMEOUT); }
             // every product issued by this thread completes before TMEM is freed
             mma_commit(&drain_bar);
             mbar_drain(&drain_bar, 0);
         }
+        __syncwarp();
     } else {
         // ---------------------------------------------------- epilogue
         const int et = threadIdx.x - 64, ew = et >> 5;

@@ -103,34 +103,44 @@ k_tc_gemm(const __grid_constant__ CUtensorMap ta_hi, const __grid_constant__ CUt
         // warp may have given up on them)
         for (int kb = issued - STAGES < 0 ? 0 : issued - STAGES; kb < issued; ++kb)
             mbar_drain(&full_bar[kb % STAGES], (kb / STAGES) & 1);
-    } else if (warp == 1 && lane == 0) {
-        // MMA issuer
+    } else if (warp == 1) {
+        // MMA issuer (one elected thread of the converged warp: the descriptors
+        // stay in uniform registers)
         constexpr uint32_t idesc = SPLIT ? idesc_tf32(BM, BN) : idesc_bf16(BM, BN);
+        const bool leader = elect_one();
+        const uint64_t desc0 = sw128_desc(su32(smem));
         for (int kb = 0; kb < nkb; ++kb) {
             const int s = kb % STAGES;
             const uint32_t ph = (kb / STAGES) & 1;
-            if (!mbar_wait(&full_bar[s], ph, wb)) { fail = 1; atomicOr(err, MSD_DEV_ERR_TIMEOUT); break; }
-            tc_fence_after();
-            const uint32_t sa = su32(smem + (size_t)s * Cfg::STAGE_BYTES);
-#pragma unroll
-            for (int kk = 0; kk < 4; ++kk) {   // 4 x 32 bytes of K per k-block
-                const uint64_t ah = sw128_desc(sa + kk * 32);
-                const uint64_t bh = sw128_desc(sa + Cfg::NOPS * Cfg::A_BYTES + kk * 32);
-                if (SPLIT) {
-                    const uint64_t al = sw128_desc(sa + Cfg::A_BYTES + kk * 32);
-                    const uint64_t bl = sw128_desc(sa + 2 * Cfg::A_BYTES + Cfg::B_BYTES + kk * 32);
-                    mma_tf32(tmem, ah, bh, idesc, (kb | kk) != 0);
-                    mma_tf32(tmem, ah, bl, idesc, 1u);
-                    mma_tf32(tmem, al, bh, idesc, 1u);
-                } else {
-                    mma_bf16(tmem, ah, bh, idesc, (kb | kk) != 0);
-                }
+            if (!__all_sync(0xffffffffu, mbar_wait(&full_bar[s], ph, wb))) {
+                if (leader) { fail = 1; atomicOr(err, MSD_DEV_ERR_TIMEOUT); }
+                break;
             }
-            mma_commit(&empty_bar[s]);
+            tc_fence_after();
+            if (leader) {
+                const uint64_t dA = desc0 + (uint64_t)((uint32_t)s * Cfg::STAGE_BYTES >> 4);
+                const uint64_t dB = dA + (uint64_t)(Cfg::NOPS * Cfg::A_BYTES >> 4);
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk) {   // 4 x 32 bytes of K per k-block
+                    const uint64_t ah = dA + kk * 2, bh = dB + kk * 2;
+                    if (SPLIT) {
+                        const uint64_t al = ah + (uint64_t)(Cfg::A_BYTES >> 4), bl = bh + (uint64_t)(Cfg::B_BYTES >> 4);
+                        mma_tf32(tmem, ah, bh, idesc, (kb | kk) != 0);
+                        mma_tf32(tmem, ah, bl, idesc, 1u);
+                        mma_tf32(tmem, al, bh, idesc, 1u);
+                    } else {
+                        mma_bf16(tmem, ah, bh, idesc, (kb | kk) != 0);
+                    }
+                }
+                mma_commit(&empty_bar[s]);
+            }
+            __syncwarp();
         }
-        mma_commit(&done_bar);
-        // every product issued here completes before TMEM may be freed
-        mbar_drain(&done_bar, 0);
+        if (leader) {
+            mma_commit(&done_bar);
+            // every product issued here completes before TMEM may be freed
+            mbar_drain(&done_bar, 0);
+        }
     }
     __syncwarp();
     const bool ok = __all_sync(0xffffffffu, mbar_wait(&done_bar, 0, wb) ? 1 : 0);

@@ -168,48 +168,47 @@ k_tc_ozaki(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUten
                 mbar_drain(&full_bar[k % OZ_STAGES], (k / OZ_STAGES) & 1);
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            // ---------------------------------------------------- MMA issuer
-            constexpr uint32_t idesc = idesc_bf16(OZ_BM, OZ_BN);
-            bool ok = true;
-            for (int ch = 0; ch < nch && ok; ++ch) {
-                // the epilogue has taken the previous chunk out of TMEM
-                if (ch > 0 && !mbar_wait(&tempty, (ch - 1) & 1, wb)) { ok = false; break; }
+        // -------------------------------------------------------- MMA issuer
+        // (the whole warp runs the loop, one elected thread issues, so that the
+        // descriptors stay in uniform registers)
+        constexpr uint32_t idesc = idesc_bf16(OZ_BM, OZ_BN);
+        const bool leader = elect_one();
+        const uint64_t desc0 = sw64_desc(su32(smem));
+        bool ok = true;
+        for (int ch = 0; ch < nch && ok; ++ch) {
+            // the epilogue has taken the previous chunk out of TMEM
+            if (ch > 0 && !__all_sync(0xffffffffu, mbar_wait(&tempty, (ch - 1) & 1, wb))) { ok = false; break; }
+            tc_fence_after();
+            const int kb0 = chunk_begin(ch), kb1 = min(nkt, chunk_begin(ch + 1));
+            for (int kb = kb0; kb < kb1; ++kb) {
+                const int s = kb % OZ_STAGES;
+                const bool got = mbar_wait(&full_bar[s], (kb / OZ_STAGES) & 1, wb) && !*vfail;
+                if (!__all_sync(0xffffffffu, got)) { ok = false; break; }
                 tc_fence_after();
-                const int kb0 = chunk_begin(ch), kb1 = min(nkt, chunk_begin(ch + 1));
-                for (int kb = kb0; kb < kb1; ++kb) {
-                    const int s = kb % OZ_STAGES;
-                    if (!mbar_wait(&full_bar[s], (kb / OZ_STAGES) & 1, wb) || *vfail) { ok = false; break; }
-                    tc_fence_after();
-                    const uint32_t sa = su32(smem + (size_t)s * OZ_STAGE);
-                    const uint32_t sb = sa + OZ_S * OZ_A_SL;
+                const uint64_t dA = desc0 + (uint64_t)((uint32_t)s * OZ_STAGE >> 4);
+                const uint64_t dB = dA + (uint64_t)(OZ_S * OZ_A_SL >> 4);
+                if (leader) {
 #pragma unroll
                     for (int kk = 0; kk < 2; ++kk) {   // 2 x 16 BF16 of K per k-block
-                        uint64_t da[OZ_S], db[OZ_S];
-#pragma unroll
-                        for (int i = 0; i < OZ_S; ++i) {
-                            da[i] = sw64_desc(sa + i * OZ_A_SL + kk * 32);
-                            db[i] = sw64_desc(sb + i * OZ_B_SL + kk * 32);
-                        }
                         const bool first = kb == kb0 && kk == 0;
+                        // i + j = c + 2 shares accumulator c; consecutive products
+                        // go to different accumulators (c's first one has i = 0)
 #pragma unroll
-                        for (int c = 2; c <= OZ_S + 1; ++c) {
-                            bool head = true;
+                        for (int i = 0; i < OZ_S; ++i)
 #pragma unroll
-                            for (int i = 1; i <= OZ_S; ++i) {
-                                const int j = c - i;
-                                if (j < 1 || j > OZ_S) continue;
-                                mma_bf16(tmem + (uint32_t)((c - 2) * OZ_BN), da[i - 1], db[j - 1], idesc,
-                                         (first && head) ? 0u : 1u);
-                                head = false;
-                            }
-                        }
+                            for (int c = OZ_S - 1; c >= i; --c)
+                                mma_bf16(tmem + (uint32_t)(c * OZ_BN), dA + (uint64_t)(i * (OZ_A_SL >> 4) + kk * 2),
+                                         dB + (uint64_t)((c - i) * (OZ_B_SL >> 4) + kk * 2), idesc,
+                                         (first && i == 0) ? 0u : 1u);
                     }
                     mma_commit(&empty_bar[s]);
                 }
-                if (!ok) break;
-                mma_commit(&tfull);
+                __syncwarp();
             }
+            if (!ok) break;
+            if (leader) mma_commit(&tfull);
+        }
+        if (leader) {
             if (!ok) {
                 *vfail = 1;
                 atomicOr(a.err, MSD_DEV_ERR_TIMEOUT);
@@ -218,6 +217,7 @@ k_tc_ozaki(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUten
             mma_commit(&drain_bar);
             mbar_drain(&drain_bar, 0);
         }
+        __syncwarp();
     } else {
         // -------------------------------------------------------- epilogue
         const int q = warp & 3, hf = (warp - 2) >> 2;
@@ -297,16 +297,18 @@ __device__ double block_absmax(double m, double* red)
     return r;
 }
 
-// x 2^-e cut into OZ_S integer slices of OZ_BETA bits (exact in FP64 and BF16).
+// x 2^-e (|x| < 2^e) cut into OZ_S integer slices of OZ_BETA bits, rounded to
+// nearest from the leading one down, in integer arithmetic on 56 fractional bits
+// (in FP64 the pass over the walker rows was bound by the FP64 unit).
 __device__ __forceinline__ void slice_store(double x, int e, __nv_bfloat16* out, size_t slice_stride)
 {
-    double r = ldexp(x, -e);
+    long long q = fixed56(x, e);
 #pragma unroll
     for (int i = 0; i < OZ_S; ++i) {
-        r *= (double)(1 << OZ_BETA);
-        const double ai = rint(r);
-        r -= ai;
-        out[i * slice_stride] = __float2bfloat16_rn((float)ai);
+        const int sh = 56 - OZ_BETA * (i + 1);
+        const long long ai = (q + (1ll << (sh - 1))) >> sh;
+        q -= ai << sh;
+        out[i * slice_stride] = __float2bfloat16_rn((float)(int)ai);
     }
 }
 
