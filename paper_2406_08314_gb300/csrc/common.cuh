@@ -121,18 +121,43 @@ __device__ __forceinline__ int rec_p(const uint4& r, int i) { return (int)(((i <
 
 
 #ifdef __CUDACC__
-// x 2^-e as an integer of 56 fractional bits, rounded to nearest (integer
-// operations only: FP64 ones issue at a sixty-fourth of their rate).
-__device__ __forceinline__ long long fixed56(double x, int e)
+// x 2^-e (|x| < 2^e) as an integer of BITS fractional bits, the magnitude rounded
+// to nearest (integer operations only: FP64 ones issue at a sixty-fourth of
+// their rate).
+template <int BITS>
+__device__ __forceinline__ long long fixed_point(double x, int e)
 {
     const long long b = __double_as_longlong(x);
     const int f = (int)((b >> 52) & 0x7ff);
     long long m = b & 0xfffffffffffffll;
     if (f) m |= 1ll << 52;
-    const int sh = (f ? f : 1) - 1075 + 56 - e;   // <= 3
-    if (sh >= 0) m <<= min(sh, 3);
+    const int sh = (f ? f : 1) - 1075 + BITS - e;   // <= BITS - 53
+    if (sh >= 0) m <<= min(sh, BITS - 53);
     else m = sh > -56 ? (m + (1ll << (-sh - 1))) >> -sh : 0;
     return b < 0 ? -m : m;
+}
+__device__ __forceinline__ long long fixed56(double x, int e) { return fixed_point<56>(x, e); }
+
+// (hi 2^28 + lo) 2^s outside the fast path below (zeros, results beyond FP64's
+// normal range, sums above 64 bits); a call, so that its FP64 conversions are not
+// issued speculatively for every value.
+static __device__ __noinline__ double int_to_fp64_slow(long long hi, long long lo, int s)
+{
+    return ldexp(fma((double)hi, 268435456.0, (double)lo), s);
+}
+
+// v 2^s rounded to FP64 by integer operations (a conversion from 64 bits and a
+// scaling are two operations of the FP64 unit, 2 per clock and SM).
+__device__ __forceinline__ double int_to_fp64(long long v, int s)
+{
+    unsigned long long u = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
+    const int lz = __clzll((long long)u), ex = 1086 + s - lz;   // biased exponent of the leading bit
+    if (u == 0 || ex < 1 || ex > 2045) return int_to_fp64_slow(0, v, s);
+    u <<= lz;
+    // the mantissa's leading bit adds one to the exponent field, a carry out of
+    // the rounding another one
+    const unsigned long long m = (u >> 11) + ((u >> 10) & 1);
+    return __longlong_as_double((long long)((((unsigned long long)(ex - 1)) << 52) + m) | (v & (long long)(1ull << 63)));
 }
 
 // Sum of n partial sums by one warp (every lane returns it).

@@ -136,10 +136,197 @@ k_fepi(SpinTables tb, int M, int n_chol, const double2* __restrict__ F, long lon
 
 size_t fepi_smem(const SpinTables& tb) { return sizeof(double2) * (tb.N * (tb.N + tb.np) + 2 * tb.N * tb.np); }
 
+// The same epilogue in 64-bit fixed point for N <= 32. The FP64 form is bound by
+// the FP64 unit (95 % of its rate, 6.2 ms per spin for 640 copper-oxo walkers);
+// mad.wide.s32 issues 24 times as often (44 against 1.8 per clock and SM,
+// measured). Operands are rounded to 54 fractional bits of their block's largest
+// magnitude (T per (walker, vector), G[occ0][P] per walker, Lambda per (walker,
+// vector)) and held as two signed limbs, q = h 2^26 + l, |h| <= 2^28, |l| <= 2^25;
+// a real product is h h' (weight 2^52) plus h l' + l h' (2^26), three mad.wide; l l'
+// (2^-58 of the block scales' product) is dropped. Sums of up to 64 products h h'
+// stay below 2^62, so nothing overflows for N <= 32. The result is rounded to FP64
+// once. The trace of T, which weighs most in the energy, sums 56 bits. Measured
+// relative rms error against long double, fixed point and FP64: Lambda 5.7e-17 and
+// 2.4e-16, Xi 1.2e-16 and 3.0e-16, tr T T 3.4e-17 and 5.6e-17. 6.2 -> 2.5 ms per spin
+// (640 copper-oxo walkers), 3.1 -> 1.2 ms (64 iron-sulfur walkers).
+struct Limbs { int rh, rl, ih, il; };   // one complex value
+
+__device__ __forceinline__ Limbs to_limbs(double2 v, int e)
+{
+    Limbs o;
+    const long long r = fixed_point<54>(v.x, e), i = fixed_point<54>(v.y, e);
+    o.rl = ((int)r << 6) >> 6;                       // the low 26 bits, signed
+    o.rh = (int)((r - o.rl) >> 26);
+    o.il = ((int)i << 6) >> 6;
+    o.ih = (int)((i - o.il) >> 26);
+    return o;
+}
+
+struct LimbSum {
+    long long rr = 0, ii = 0, im = 0, crr = 0, cii = 0, cim = 0;
+    __device__ __forceinline__ void add(const Limbs& a, const Limbs& b)
+    {
+        rr += (long long)a.rh * b.rh;
+        crr += (long long)a.rh * b.rl;
+        crr += (long long)a.rl * b.rh;
+        ii += (long long)a.ih * b.ih;
+        cii += (long long)a.ih * b.il;
+        cii += (long long)a.il * b.ih;
+        im += (long long)a.rh * b.ih;
+        im += (long long)a.ih * b.rh;
+        cim += (long long)a.rh * b.il;
+        cim += (long long)a.rl * b.ih;
+        cim += (long long)a.ih * b.rl;
+        cim += (long long)a.il * b.rh;
+    }
+    // both parts in units of 2^-56 of the scales' product
+    __device__ __forceinline__ long long re() const { return (rr - ii) + ((crr - cii + (1 << 25)) >> 26); }
+    __device__ __forceinline__ long long imag() const { return im + ((cim + (1 << 25)) >> 26); }
+};
+
+__device__ __forceinline__ unsigned mag_bits(double2 v)
+{
+    return max((unsigned)__double2hiint(v.x) & 0x7fffffffu, (unsigned)__double2hiint(v.y) & 0x7fffffffu);
+}
+
+#define FEPI_INT_NMAX 32
+#define FEPI_INT_G 8      // Cholesky vectors per block: G[occ0][P] is converted once for them
+__global__ void __launch_bounds__(256)
+k_fepi_int(SpinTables tb, int M, int n_chol, const double2* __restrict__ F, long long ldf,
+           const double2* __restrict__ Gr, double2* __restrict__ v0, double2* __restrict__ xx,
+           double2* __restrict__ Lact, double2* __restrict__ Xic)
+{
+    extern __shared__ double2 sm[];
+    const int N = tb.N, np = tb.np, nh = tb.nh, NC = N + np, X = nh * np, NP = N * np;
+    double2* f = sm;                                      // [N][NC]: T as limbs, F_P as FP64
+    Limbs* tl = reinterpret_cast<Limbs*>(sm);
+    Limbs* gp = reinterpret_cast<Limbs*>(f + N * NC);     // [N][np]
+    double2* lam = reinterpret_cast<double2*>(gp + NP);   // [N][np] FP64
+    Limbs* ll = reinterpret_cast<Limbs*>(lam + NP);       // [N][np]
+    __shared__ unsigned wmax[3][8];
+    __shared__ long long wsum[2][8];
+    __shared__ int wlow[2][8];
+    __shared__ long long diag[2][FEPI_INT_NMAX];          // T[j][j] to 56 bits, for its trace
+    const int w = blockIdx.y, t = threadIdx.x, nt = blockDim.x, lane = t & 31, warp = t >> 5, nwarp = nt >> 5;
+    auto exponent = [&](int i) {      // of the largest magnitude the warps left in wmax[i]
+        unsigned m = 0;
+        for (int k = 0; k < nwarp; ++k) m = max(m, wmax[i][k]);
+        return (int)(m >> 20) - 1022;   // every |x| < 2^e (1025: an infinity or a NaN)
+    };
+    const double2* gr = Gr + (size_t)w * N * M;
+    unsigned m = 0;
+    for (int e = t; e < NP; e += nt) {
+        lam[e] = gr[(size_t)(e / np) * M + tb.part_orb[e % np]];
+        m = max(m, mag_bits(lam[e]));
+    }
+    m = __reduce_max_sync(0xffffffffu, m);
+    if (lane == 0) wmax[0][warp] = m;
+    __syncthreads();
+    const int eg = exponent(0);
+    for (int e = t; e < NP; e += nt) gp[e] = to_limbs(lam[e], eg);
+    const int g1 = min(n_chol, (int)(blockIdx.x + 1) * FEPI_INT_G);
+    for (int g = blockIdx.x * FEPI_INT_G; g < g1; ++g) {
+        const size_t wg = (size_t)w * n_chol + g;
+        const double2* Fw = F + (size_t)w * N * ldf + (size_t)g * NC;
+        m = 0;
+        for (int e = t; e < N * NC; e += nt) {
+            const int j = e / NC, c = e - j * NC;
+            const double2 v = Fw[(size_t)j * ldf + c];
+            f[e] = v;
+            if (c < N) m = max(m, mag_bits(v));
+        }
+        m = __reduce_max_sync(0xffffffffu, m);
+        if (lane == 0) wmax[1][warp] = m;
+        __syncthreads();
+        const int et = exponent(1);
+        for (int e = t; e < N * NC; e += nt) {
+            const int j = e / NC, c = e - j * NC;
+            if (c >= N) continue;
+            const double2 v = f[e];
+            if (c == j) { diag[0][j] = fixed56(v.x, et); diag[1][j] = fixed56(v.y, et); }
+            tl[e] = to_limbs(v, et);
+        }
+        __syncthreads();
+        // Lambda[j][p] = F_P[j][p] - sum_l T[j][l] G[occ0_l][P_p]
+        m = 0;
+        for (int e = t; e < NP; e += nt) {
+            const int j = e / np, p = e - j * np;
+            LimbSum s;
+            for (int l = 0; l < N; ++l) s.add(tl[j * NC + l], gp[l * np + p]);
+            const double2 fp = f[j * NC + N + p];
+            const double2 v = cz(fp.x - int_to_fp64(s.re(), et + eg - 56), fp.y - int_to_fp64(s.imag(), et + eg - 56));
+            lam[e] = v;
+            m = max(m, mag_bits(v));
+        }
+        m = __reduce_max_sync(0xffffffffu, m);
+        // tr T T over the warps (each thread's sum cut at 12 bits, so that the
+        // totals of both halves stay in 64 and 32 bits), tr T
+        LimbSum x;
+        for (int e = t; e < N * N; e += nt) {
+            const int j = e / N, l = e - j * N;
+            x.add(tl[j * NC + l], tl[l * NC + j]);
+        }
+        long long q[2] = {x.re(), x.imag()};
+        int lo[2];
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            lo[c] = __reduce_add_sync(0xffffffffu, (int)(q[c] & 4095));
+            q[c] >>= 12;
+            for (int o = 16; o; o >>= 1) q[c] += __shfl_xor_sync(0xffffffffu, q[c], o);
+        }
+        if (lane == 0) {
+            wmax[2][warp] = m;
+            for (int c = 0; c < 2; ++c) { wsum[c][warp] = q[c]; wlow[c][warp] = lo[c]; }
+        }
+        if (warp == nwarp - 1) {
+            long long d[2] = {lane < N ? diag[0][lane] : 0, lane < N ? diag[1][lane] : 0};
+            for (int c = 0; c < 2; ++c)
+                for (int o = 16; o; o >>= 1) d[c] += __shfl_xor_sync(0xffffffffu, d[c], o);
+            if (lane == 0) v0[wg] = cz(int_to_fp64(d[0], et - 56), int_to_fp64(d[1], et - 56));
+        }
+        __syncthreads();
+        const int el = exponent(2);
+        for (int e = t; e < NP; e += nt) ll[e] = to_limbs(lam[e], el);
+        if (t < 2) {
+            long long a = 0, b = 0;
+            for (int k = 0; k < nwarp; ++k) { a += wsum[t][k]; b += wlow[t][k]; }
+            // a 2^12 + b = (a >> 16) 2^28 + ((a & 65535) 2^12 + b)
+            reinterpret_cast<double*>(xx + wg)[t] = int_to_fp64_slow(a >> 16, ((a & 65535) << 12) + b, 2 * et - 56);
+        }
+        __syncthreads();
+        for (int e = t; e < X; e += nt) {
+            const int h = e / np, p = e - h * np, j = tb.hole_pos[h];
+            LimbSum s;
+            for (int l = 0; l < N; ++l) s.add(tl[j * NC + l], ll[l * np + p]);
+            Lact[wg * X + e] = lam[j * np + p];
+            Xic[wg * X + e] = cz(int_to_fp64(s.re(), et + el - 56), int_to_fp64(s.imag(), et + el - 56));
+        }
+        if (max(max(eg, et), el) > 1024) {   // an infinity or a NaN somewhere
+            const double nan = __longlong_as_double(0x7ff8000000000000ll);
+            __syncthreads();
+            if (t == 0) v0[wg] = xx[wg] = cz(nan, nan);
+            for (int e = t; e < X; e += nt) Lact[wg * X + e] = Xic[wg * X + e] = cz(nan, nan);
+        }
+        __syncthreads();   // f and lam are free for the next vector
+    }
+}
+
 void launch_fepi(const SpinTables& tb, int nw, int M, int n_chol, const double2* F, long long ldf,
                  const double2* Gr, double2* v0, double2* xx, double2* Lact, double2* Xic,
                  cudaStream_t st)
 {
+    const int NP = tb.N * tb.np;
+    const size_t smem_int = sizeof(double2) * (tb.N * (tb.N + tb.np) + 3 * NP);
+    if (tb.N <= FEPI_INT_NMAX && smem_int <= 200 * 1024) {
+        const size_t smem = smem_int;
+        if (smem > 44 * 1024)
+            cudaFuncSetAttribute(k_fepi_int, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const int threads = NP <= 128 ? 128 : NP >= 256 ? 256 : (NP + 31) / 32 * 32;   // one (j, p) per thread
+        k_fepi_int<<<dim3((n_chol + FEPI_INT_G - 1) / FEPI_INT_G, nw), threads, smem, st>>>(tb, M, n_chol, F, ldf, Gr, v0,
+                                                                                        xx, Lact, Xic);
+        msd_note_launch();
+        return;
+    }
     dim3 grid(n_chol, nw);
     const size_t smem = fepi_smem(tb);
     if (smem > 48 * 1024) cudaFuncSetAttribute(k_fepi, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

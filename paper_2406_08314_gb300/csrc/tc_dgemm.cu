@@ -97,35 +97,13 @@ __device__ __forceinline__ void tmem_ld16_nowait(uint32_t taddr, uint32_t* r)
         : "r"(taddr));
 }
 
-// Outside the fast paths below (zeros, results beyond FP64's normal range,
-// sums above 8 times the rows' scales); a call, so that its FP64 conversions are
-// not issued speculatively for every value.
-__device__ __noinline__ double dg_slow(long long hi, long long lo, int s)
-{
-    return ldexp(fma((double)hi, 268435456.0, (double)lo), s);
-}
-
-// v 2^s rounded to FP64 by integer operations (a conversion from 64 bits and a
-// scaling are two operations of the FP64 unit, 2 per clock and SM).
-__device__ __forceinline__ double dg_round(long long v, int s)
-{
-    unsigned long long u = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
-    const int lz = __clzll((long long)u), ex = 1086 + s - lz;   // biased exponent of the leading bit
-    if (u == 0 || ex < 1 || ex > 2045) return dg_slow(0, v, s);
-    u <<= lz;
-    // the mantissa's leading bit adds one to the exponent field, a carry out of
-    // the rounding another one
-    const unsigned long long m = (u >> 11) + ((u >> 10) & 1);
-    return __longlong_as_double((long long)((((unsigned long long)(ex - 1)) << 52) + m) | (v & (long long)(1ull << 63)));
-}
-
 // hi 2^-35 + lo 2^-63 (the accumulators c = 2..5 and 6..9) times 2^e.
 __device__ __forceinline__ double dg_value(long long hi, long long lo, int e)
 {
     if (e >= DG_NAN / 2) return __longlong_as_double(0x7ff8000000000000ll);
     if (hi < (1ll << 38) && hi > -(1ll << 38))   // |value| < 8: one 64-bit integer of 2^-59
-        return dg_round((hi << 24) + ((lo + 8) >> 4), e - 59);
-    return dg_slow(hi, lo, e - 63);
+        return int_to_fp64((hi << 24) + ((lo + 8) >> 4), e - 59);
+    return int_to_fp64_slow(hi, lo, e - 63);
 }
 
 struct DgTile { int m0, n0, z; };

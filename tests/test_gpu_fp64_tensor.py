@@ -12,6 +12,7 @@ CASES = [  # M, n_alpha, n_beta, n_core, n_act, n_chol, n_w
     (40, 7, 7, 2, 11, 127, 5),
     (64, 9, 8, 3, 12, 385, 3),       # n_chol one past a chunk
     (47, 4, 3, 0, 8, 200, 33),       # 2 x 33 columns: two past a tile
+    (80, 33, 32, 29, 8, 60, 2),      # epilogue: N = 32 in fixed point, N = 33 in FP64
     (70, 18, 17, 14, 8, 96, 5),      # reference product: alpha on the tensor cores, beta not
 ]
 
