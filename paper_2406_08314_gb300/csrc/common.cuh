@@ -21,6 +21,10 @@ __host__ __device__ __forceinline__ int lam_pitch(int X) { return (X + 15) / 16 
 #define SE_PER_THREAD 4
 #define PC_THREADS 256
 #define PC_PER_THREAD 8
+// The per-determinant terms take one launch for all their levels up to this many
+// blocks per SM (a few resident waves of blocks); above, a launch per level with
+// that level's registers.
+#define ONE_LAUNCH_BLOCKS 6
 
 
 // ---------------------------------------------------------------- complex

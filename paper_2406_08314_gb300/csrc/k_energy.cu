@@ -337,16 +337,24 @@ void launch_fepi(const SpinTables& tb, int nw, int M, int n_chol, const double2*
 // One-body pieces per (walker, spin): e1 = tr(h G), and
 // Lambda_h[(h,p)] = (G hl (I - G))[H_h][P_p] with hl = h, or the matrix the
 // caller gives (linear in it: hl = h + J adds sum_g C_g Lambda_g).
+struct OnebodyArgs {
+    SpinTables t[2];
+    const double *h1[2], *hl[2];
+    const double2* Gr[2];
+    double2 *e1[2], *Lh[2];
+};
 __global__ void __launch_bounds__(128)
-k_onebody(SpinTables tb, int M, const double* __restrict__ h1, const double* __restrict__ hl,
-          const double2* __restrict__ Gr, double2* __restrict__ e1, double2* __restrict__ Lh)
+k_onebody(const __grid_constant__ OnebodyArgs a_, int M)
 {
     extern __shared__ double2 sm[];
+    const int s = blockIdx.y;
+    const SpinTables& tb = a_.t[s];
+    const double *h1 = a_.h1[s], *hl = a_.hl[s];
     const int N = tb.N, np = tb.np, nh = tb.nh, NC = N + np;
     double2* fh = sm;   // [nh][NC]
     __shared__ double2 red[128];
     const int w = blockIdx.x, t = threadIdx.x;
-    const double2* gr = Gr + (size_t)w * N * M;
+    const double2* gr = a_.Gr[s] + (size_t)w * N * M;
     double2 a = cz(0, 0);
     for (int e = t; e < N * M; e += blockDim.x) {
         const int j = e / M, r = e % M;
@@ -366,75 +374,104 @@ k_onebody(SpinTables tb, int M, const double* __restrict__ h1, const double* __r
         if (t < o) red[t] = cadd(red[t], red[t + o]);
         __syncthreads();
     }
-    if (t == 0) e1[w] = red[0];
+    if (t == 0) a_.e1[s][w] = red[0];
     for (int e = t; e < nh * np; e += blockDim.x) {
         const int h = e / np, p = e % np;
         double2 v = fh[h * NC + N + p];
         for (int l = 0; l < N; ++l) v = cfms(fh[h * NC + l], gr[(size_t)l * M + tb.part_orb[p]], v);
-        Lh[(size_t)w * nh * np + e] = v;
+        a_.Lh[s][(size_t)w * nh * np + e] = v;
     }
 }
 
-void launch_onebody(const SpinTables& tb, int nw, int M, const double* h1, const double2* Gr,
-                    double2* e1, double2* Lh, cudaStream_t st, const double* hl)
+void launch_onebody(const SpinTables& ta, const SpinTables& tb, int nw, int M, const double* const h1[2],
+                    const double2* const Gr[2], double2* const e1[2], double2* const Lh[2], cudaStream_t st,
+                    const double* const hl[2])
 {
-    size_t smem = sizeof(double2) * tb.nh * (tb.N + tb.np);
-    if (smem > 48 * 1024) cudaFuncSetAttribute(k_onebody, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_onebody<<<nw, 128, smem, st>>>(tb, M, h1, hl ? hl : h1, Gr, e1, Lh); msd_note_launch();
+    OnebodyArgs a;
+    size_t smem = 0;
+    const SpinTables* T[2] = {&ta, &tb};
+    for (int s = 0; s < 2; ++s) {
+        a.t[s] = *T[s];
+        a.h1[s] = h1[s]; a.hl[s] = hl[s];
+        a.Gr[s] = Gr[s]; a.e1[s] = e1[s]; a.Lh[s] = Lh[s];
+        smem = smem > sizeof(double2) * T[s]->nh * (T[s]->N + T[s]->np) ? smem : sizeof(double2) * T[s]->nh * (T[s]->N + T[s]->np);
+    }
+    if (smem > 44 * 1024) cudaFuncSetAttribute(k_onebody, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    k_onebody<<<dim3(nw, 2), 128, smem, st>>>(a, M); msd_note_launch();
 }
 
 // ------------------------------------------------------------------------
 // Sums over Cholesky vectors per (walker, spin):
 //   Y[x] = Lh[x] + sum_g V0_g Lact_g[x] - sum_g Xic_g[x],  V0_g = v0a_g + v0b_g
 //   scal[w][0 + s] = sum_g xx_g (exchange of G),  scal[w][2] = sum_g V0_g^2
-template <typename TY>
-__global__ void __launch_bounds__(128)
-k_gamma_reduce(int X, int n_chol, int spin, const double2* __restrict__ v0a,
-               const double2* __restrict__ v0b, const double2* __restrict__ xx,
-               const double2* __restrict__ Lact, const double2* __restrict__ Xic,
-               const double2* __restrict__ Lh, TY* __restrict__ Y, double2* __restrict__ scal)
+// One block per (walker, spin): warp k takes the vectors g = k mod 8, lanes over
+// the entries x (contiguous rows); the warps' sums are added in order. (A serial
+// sum over g per entry left 64 walkers with 64 x 75 chains of 1600 dependent FP64
+// operations: 1.05 ms for both iron-sulfur spins.)
+struct GammaArgs {
+    int X[2];
+    const double2 *v0[2], *xx[2], *Lact[2], *Xic[2], *Lh[2];
+    double2* Y[2];
+};
+__global__ void __launch_bounds__(256)
+k_gamma_reduce(const __grid_constant__ GammaArgs a, int n_chol, double2* __restrict__ scal)
 {
-    __shared__ double2 red[2][128];
-    const int w = blockIdx.x, t = threadIdx.x;
+    __shared__ double2 part[8][MSD_XMAX];
+    __shared__ double2 red[2][8];
+    const int w = blockIdx.x, spin = blockIdx.y, t = threadIdx.x, warp = t >> 5, lane = t & 31, X = a.X[spin];
     const size_t base = (size_t)w * n_chol;
-    for (int x = t; x < X; x += blockDim.x) {
-        double2 y = Lh[(size_t)w * X + x];
-        for (int g = 0; g < n_chol; ++g) {
-            const double2 V0 = cadd(v0a[base + g], v0b[base + g]);
-            y = cfma(V0, Lact[(base + g) * X + x], y);
-            y = csub(y, Xic[(base + g) * X + x]);
+    const double2 *va = a.v0[0] + base, *vb = a.v0[1] + base;
+    double2 acc[(MSD_XMAX + 31) / 32];
+#pragma unroll
+    for (int q = 0; q < (MSD_XMAX + 31) / 32; ++q) acc[q] = cz(0, 0);
+    for (int g = warp; g < n_chol; g += 8) {
+        const double2 V0 = cadd(va[g], vb[g]);
+        const double2 *la = a.Lact[spin] + (base + g) * X, *xi = a.Xic[spin] + (base + g) * X;
+#pragma unroll
+        for (int q = 0; q < (MSD_XMAX + 31) / 32; ++q) {
+            const int x = q * 32 + lane;
+            if (q * 32 >= X) break;   // (no FP64 issue slots for empty warps)
+            if (x < X) acc[q] = csub(cfma(V0, la[x], acc[q]), xi[x]);
         }
-        Y[2 * ((size_t)w * X + x)] = (TY)y.x;
-        Y[2 * ((size_t)w * X + x) + 1] = (TY)y.y;
     }
+#pragma unroll
+    for (int q = 0; q < (MSD_XMAX + 31) / 32; ++q)
+        if (q * 32 + lane < X) part[warp][q * 32 + lane] = acc[q];
     double2 s0 = cz(0, 0), s1 = cz(0, 0);
     for (int g = t; g < n_chol; g += blockDim.x) {
-        s0 = cadd(s0, xx[base + g]);
-        const double2 V0 = cadd(v0a[base + g], v0b[base + g]);
+        s0 = cadd(s0, a.xx[spin][base + g]);
+        const double2 V0 = cadd(va[g], vb[g]);
         s1 = cfma(V0, V0, s1);
     }
-    red[0][t] = s0; red[1][t] = s1;
-    __syncthreads();
-    for (int o = 64; o; o >>= 1) {
-        if (t < o) { red[0][t] = cadd(red[0][t], red[0][t + o]); red[1][t] = cadd(red[1][t], red[1][t + o]); }
-        __syncthreads();
+    for (int o = 16; o; o >>= 1) {
+        s0.x += __shfl_xor_sync(0xffffffffu, s0.x, o); s0.y += __shfl_xor_sync(0xffffffffu, s0.y, o);
+        s1.x += __shfl_xor_sync(0xffffffffu, s1.x, o); s1.y += __shfl_xor_sync(0xffffffffu, s1.y, o);
     }
-    if (t == 0) {
-        scal[(size_t)w * 8 + spin] = red[0][0];
-        if (spin == 0) scal[(size_t)w * 8 + 2] = red[1][0];
+    if (lane == 0) { red[0][warp] = s0; red[1][warp] = s1; }
+    __syncthreads();
+    for (int x = t; x < X; x += blockDim.x) {
+        double2 y = a.Lh[spin][(size_t)w * X + x];
+        for (int q = 0; q < 8; ++q) y = cadd(y, part[q][x]);
+        a.Y[spin][(size_t)w * X + x] = y;
+    }
+    if (t < 2) {
+        double2 s = red[t][0];
+        for (int q = 1; q < 8; ++q) s = cadd(s, red[t][q]);
+        if (t == 0) scal[(size_t)w * 8 + spin] = s;
+        else if (spin == 0) scal[(size_t)w * 8 + 2] = s;
     }
 }
 
-void launch_gamma_reduce(int nw, int X, int n_chol, int spin, const double2* v0a, const double2* v0b,
-                         const double2* xx, const double2* Lact, const double2* Xic,
-                         const double2* Lh, void* Y, bool fp32, double2* scal, cudaStream_t st)
+void launch_gamma_reduce(int nw, const int X[2], int n_chol, const double2* const v0[2], const double2* const xx[2],
+                         const double2* const Lact[2], const double2* const Xic[2], const double2* const Lh[2],
+                         double2* const Y[2], double2* scal, cudaStream_t st)
 {
-    if (fp32)
-        k_gamma_reduce<float><<<nw, 128, 0, st>>>(X, n_chol, spin, v0a, v0b, xx, Lact, Xic, Lh,
-                                                  (float*)Y, scal);
-    else
-        k_gamma_reduce<double><<<nw, 128, 0, st>>>(X, n_chol, spin, v0a, v0b, xx, Lact, Xic, Lh,
-                                                   (double*)Y, scal);
+    GammaArgs a;
+    for (int s = 0; s < 2; ++s) {
+        a.X[s] = X[s]; a.v0[s] = v0[s]; a.xx[s] = xx[s]; a.Lact[s] = Lact[s]; a.Xic[s] = Xic[s]; a.Lh[s] = Lh[s];
+        a.Y[s] = Y[s];
+    }
+    k_gamma_reduce<<<dim3(nw, 2), 256, 0, st>>>(a, n_chol, scal);
     msd_note_launch();
 }
 
@@ -499,48 +536,90 @@ void launch_gram(int nw, int Xp, int Xq, int n_chol, const double2* P, const dou
 // antisymmetrized pair table of K (C(nh,2) C(np,2) entries, against X^2 for
 // K) in shared memory; each string then takes C(k,2)^2 gathers of it for
 // (Qc - Qx) / 2 (string_energy_value).
+// Block b of all (spin, level) blocks writes slot slot0 + b. ONLY = 0: one launch
+// for both spins and all levels (a launch per level was most of the time of this
+// term at small sizes, 87 us of 391 for 16 walkers of 100 determinants); ONLY = k: the blocks of level k,
+// with that level's registers (131 for all levels: 1.74 against 1.09 ms at the
+// iron-sulfur size).
+struct SeArgs {
+    SpinTables t[2];
+    const double2* wts[2];
+    const void *B[2], *K[2], *Y[2];
+    int blk[2][MSD_KMAX + 2];   // first block of each (spin, level)
+};
+
 template <int KL, typename T>
-__global__ void __launch_bounds__(SE_THREADS)
-k_string_energy(SpinTables tb, const double2* __restrict__ wts,
-                const void* __restrict__ Bin, const void* __restrict__ Kin, const void* __restrict__ Yin,
-                double2* __restrict__ part, int nslot, int slot0)
+__device__ __forceinline__ double2 string_energy_block(const SpinTables& tb, int w, int blk, const void* B,
+                                                       const cplx_t<T>* as, const cplx_t<T>* ys, const double2* wts)
 {
-    using T2 = typename std::conditional<std::is_same<T, float>::value, float2, double2>::type;
+    const int ns = tb.bucket[KL + 1] - tb.bucket[KL];
+    double2 contrib = cz(0, 0);
+    for (int it = 0; it < SE_PER_THREAD; ++it) {
+        const int sl = blk * (SE_THREADS * SE_PER_THREAD) + it * SE_THREADS + threadIdx.x;
+        if (sl >= ns) break;
+        contrib = cadd(contrib, string_energy_term<KL, T, true>(tb, w, sl, ns, B, as, ys, wts));
+    }
+    return contrib;
+}
+
+template <typename T, int ONLY>
+__global__ void __launch_bounds__(SE_THREADS)
+k_string_energy(const __grid_constant__ SeArgs a, double2* __restrict__ part, int nslot, int slot0)
+{
+    using T2 = cplx_t<T>;
     extern __shared__ __align__(16) unsigned char smraw[];
+    // this block among all (spin, level) blocks
+    int b = blockIdx.x;
+    if (ONLY) {
+        const int na = a.blk[0][ONLY + 1] - a.blk[0][ONLY];
+        b = b < na ? a.blk[0][ONLY] + b : a.blk[1][ONLY] + b - na;
+    }
+    const int s = b >= a.blk[1][1];
+    const SpinTables& tb = a.t[s];
     const int X = tb.nh * tb.np, np = tb.np, nh = tb.nh;
     const int nhp = nh * (nh - 1) / 2, npp = np * (np - 1) / 2;
     T2* as = reinterpret_cast<T2*>(smraw);   // [C(nh,2)][C(np,2)] antisymmetrized pairs of K
     T2* ys = as + nhp * npp;                 // [X]
     __shared__ double2 red[SE_THREADS];
     const int w = blockIdx.y, t = threadIdx.x;
-    const T2* Kw = reinterpret_cast<const T2*>(Kin) + (size_t)w * X * X;
+    int k = ONLY ? ONLY : 1;
+    while (!ONLY && b >= a.blk[s][k + 1]) ++k;
+    const T2* Kw = reinterpret_cast<const T2*>(a.K[s]) + (size_t)w * X * X;
     // A[(h,h')][(p,p')] = K[(h,p)][(h',p')] - K[(h,p')][(h',p)], h < h', p < p'
-    for (int e = t; e < nhp * npp; e += blockDim.x) {
-        int a = e / npp, c = e - a * npp, h = 0, p = 0;
-        while (a >= nh - 1 - h) { a -= nh - 1 - h; ++h; }
+    // (not used by level 1)
+    for (int e = k > 1 ? t : nhp * npp; e < nhp * npp; e += blockDim.x) {
+        int i = e / npp, c = e - i * npp, h = 0, p = 0;
+        while (i >= nh - 1 - h) { i -= nh - 1 - h; ++h; }
         while (c >= np - 1 - p) { c -= np - 1 - p; ++p; }
-        const int h2 = h + 1 + a, p2 = p + 1 + c;
+        const int h2 = h + 1 + i, p2 = p + 1 + c;
         const T2 kc = Kw[(size_t)(h * np + p) * X + h2 * np + p2];
         const T2 kx = Kw[(size_t)(h * np + p2) * X + h2 * np + p];
         as[e] = T2{kc.x - kx.x, kc.y - kx.y};
     }
-    const T2* Yw = reinterpret_cast<const T2*>(Yin) + (size_t)w * X;
+    const T2* Yw = reinterpret_cast<const T2*>(a.Y[s]) + (size_t)w * X;
     for (int e = t; e < X; e += blockDim.x) ys[e] = Yw[e];
     __syncthreads();
-    const int ns = tb.bucket[KL + 1] - tb.bucket[KL];
-    double2 contrib = cz(0, 0);
-    for (int it = 0; it < SE_PER_THREAD; ++it) {
-        const int sl = blockIdx.x * (SE_THREADS * SE_PER_THREAD) + it * SE_THREADS + t;
-        if (sl >= ns) break;
-        contrib = cadd(contrib, string_energy_term<KL, T, true>(tb, w, sl, ns, Bin, as, ys, wts));
+    const int blk = b - a.blk[s][k];
+    double2 v;
+    if constexpr (ONLY > 0) {
+        v = string_energy_block<ONLY, T>(tb, w, blk, a.B[s], as, ys, a.wts[s]);
+    } else {
+        switch (k) {
+        case 1: v = string_energy_block<1, T>(tb, w, blk, a.B[s], as, ys, a.wts[s]); break;
+        case 2: v = string_energy_block<2, T>(tb, w, blk, a.B[s], as, ys, a.wts[s]); break;
+        case 3: v = string_energy_block<3, T>(tb, w, blk, a.B[s], as, ys, a.wts[s]); break;
+        case 4: v = string_energy_block<4, T>(tb, w, blk, a.B[s], as, ys, a.wts[s]); break;
+        case 5: v = string_energy_block<5, T>(tb, w, blk, a.B[s], as, ys, a.wts[s]); break;
+        default: v = string_energy_block<6, T>(tb, w, blk, a.B[s], as, ys, a.wts[s]); break;
+        }
     }
-    red[t] = contrib;
+    red[t] = v;
     __syncthreads();
     for (int o = SE_THREADS / 2; o; o >>= 1) {
         if (t < o) red[t] = cadd(red[t], red[t + o]);
         __syncthreads();
     }
-    if (t == 0) part[(size_t)w * nslot + slot0 + blockIdx.x] = red[0];
+    if (t == 0) part[(size_t)w * nslot + slot0 + b] = red[0];
 }
 
 int string_energy_blocks(const SpinTables& tb, int k)
@@ -556,36 +635,45 @@ size_t string_energy_smem(const SpinTables& tb, bool fp32)
     return (fp32 ? sizeof(float2) : sizeof(double2)) * (pairs + X);
 }
 
-template <int KL>
-static void launch_se_k(const SpinTables& tb, int nw, const double2* wts,
-                        const void* B, const void* K, const void* Y, bool fp32, double2* part,
-                        int nslot, int& slot, cudaStream_t st)
+void launch_string_energy(const SpinTables& ta, const SpinTables& tb, int nw, const double2* const wts[2],
+                          const void* const B[2], const void* const K[2], const void* const Y[2], bool fp32,
+                          double2* part, int nslot, int slot0, cudaStream_t st)
 {
-    const int nb = string_energy_blocks(tb, KL);
-    if (!nb) return;
-    dim3 grid(nb, nw);
-    const size_t smem = string_energy_smem(tb, fp32);
-    if (fp32) {
-        cudaFuncSetAttribute(k_string_energy<KL, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k_string_energy<KL, float><<<grid, SE_THREADS, smem, st>>>(tb, wts, B, K, Y, part, nslot, slot); msd_note_launch();
-    } else {
-        cudaFuncSetAttribute(k_string_energy<KL, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k_string_energy<KL, double><<<grid, SE_THREADS, smem, st>>>(tb, wts, B, K, Y, part, nslot, slot); msd_note_launch();
+    SeArgs a;
+    const SpinTables* T[2] = {&ta, &tb};
+    int n = 0;
+    size_t smem = 0;
+    for (int s = 0; s < 2; ++s) {
+        a.t[s] = *T[s];
+        a.wts[s] = wts[s]; a.B[s] = B[s]; a.K[s] = K[s]; a.Y[s] = Y[s];
+        a.blk[s][0] = n;
+        for (int k = 1; k <= MSD_KMAX; ++k) { a.blk[s][k] = n; n += string_energy_blocks(*T[s], k); }
+        a.blk[s][MSD_KMAX + 1] = n;
+        const size_t b = string_energy_smem(*T[s], fp32);
+        smem = smem > b ? smem : b;
     }
-    slot += nb;
-}
-
-void launch_string_energy(const SpinTables& tb, int nw, const double2* wts,
-                          const void* B, const void* K, const void* Y, bool fp32, double2* part,
-                          int nslot, int slot0, cudaStream_t st)
-{
-    int slot = slot0;
-    launch_se_k<1>(tb, nw, wts, B, K, Y, fp32, part, nslot, slot, st);
-    launch_se_k<2>(tb, nw, wts, B, K, Y, fp32, part, nslot, slot, st);
-    launch_se_k<3>(tb, nw, wts, B, K, Y, fp32, part, nslot, slot, st);
-    launch_se_k<4>(tb, nw, wts, B, K, Y, fp32, part, nslot, slot, st);
-    launch_se_k<5>(tb, nw, wts, B, K, Y, fp32, part, nslot, slot, st);
-    launch_se_k<6>(tb, nw, wts, B, K, Y, fp32, part, nslot, slot, st);
+    if (n == 0) return;
+    auto go = [&](auto kern, int blocks) {
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        kern<<<dim3(blocks, nw), SE_THREADS, smem, st>>>(a, part, nslot, slot0);
+        msd_note_launch();
+    };
+    if ((long long)n * nw <= ONE_LAUNCH_BLOCKS * msd_sm_count()) {
+        if (fp32) go(k_string_energy<float, 0>, n); else go(k_string_energy<double, 0>, n);
+        return;
+    }
+    for (int k = 1; k <= MSD_KMAX; ++k) {
+        const int m = string_energy_blocks(ta, k) + string_energy_blocks(tb, k);
+        if (!m) continue;
+        switch (k) {
+        case 1: if (fp32) go(k_string_energy<float, 1>, m); else go(k_string_energy<double, 1>, m); break;
+        case 2: if (fp32) go(k_string_energy<float, 2>, m); else go(k_string_energy<double, 2>, m); break;
+        case 3: if (fp32) go(k_string_energy<float, 3>, m); else go(k_string_energy<double, 3>, m); break;
+        case 4: if (fp32) go(k_string_energy<float, 4>, m); else go(k_string_energy<double, 4>, m); break;
+        case 5: if (fp32) go(k_string_energy<float, 5>, m); else go(k_string_energy<double, 5>, m); break;
+        default: if (fp32) go(k_string_energy<float, 6>, m); else go(k_string_energy<double, 6>, m); break;
+        }
+    }
 }
 
 int string_energy_slots(const SpinTables& tb)
@@ -675,6 +763,7 @@ void launch_pair_cross(const SpinTables& ta, const SpinTables& tb, const PairTab
                        cudaStream_t st, bool use_runs)
 {
     int slot = slot0;
+    if (launch_pair_cross_all(ta, tb, pt, nw, ra, rb, Ba, Bb, K, fp32, part, nslot, slot0, st, use_runs)) return;
     for (int ka = 1; ka <= MSD_KMAX; ++ka) {
         launch_pc_k<1>(ta, tb, pt, ka, nw, ra, rb, Ba, Bb, K, fp32, part, nslot, slot, st, use_runs);
         launch_pc_k<2>(ta, tb, pt, ka, nw, ra, rb, Ba, Bb, K, fp32, part, nslot, slot, st, use_runs);

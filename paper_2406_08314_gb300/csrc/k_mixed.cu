@@ -136,13 +136,20 @@ void launch_fepi_f32(const SpinTables& tb, int nw, int M, int n_chol, const floa
 // sum_g C_g Lambda_g[x] as well (the one-body term of h + J, J = sum_g C_g
 // L_g, FP64). Warps split the Cholesky vectors, lanes the active entries;
 // the warp sums are added in a fixed order.
+struct GammaArgsF {
+    int X[2];
+    const double2 *v0[2], *xx[2], *Lh[2];
+    const float2 *Lact[2], *Xic[2];
+    float2* Y[2];
+};
 __global__ void __launch_bounds__(256)
-k_gamma_reduce_f32(int X, int n_chol, int spin, bool traces, const double2* __restrict__ v0a,
-                   const double2* __restrict__ v0b, const double2* __restrict__ xx,
-                   const float2* __restrict__ Lact, const float2* __restrict__ Xic,
-                   const double2* __restrict__ Lh, float2* __restrict__ Y, double2* __restrict__ scal,
+k_gamma_reduce_f32(const __grid_constant__ GammaArgsF args, int n_chol, bool traces, double2* __restrict__ scal,
                    const float2* __restrict__ v0w)
 {
+    const int spin = blockIdx.y, X = args.X[spin];
+    const double2 *v0a = args.v0[0], *v0b = args.v0[1], *xx = args.xx[spin], *Lh = args.Lh[spin];
+    const float2 *Lact = args.Lact[spin], *Xic = args.Xic[spin];
+    float2* Y = args.Y[spin];
     __shared__ float2 part[8][MSD_XMAX];
     __shared__ double2 red[2][256];
     const int w = blockIdx.x, t = threadIdx.x, warp = t >> 5, lane = t & 31;
@@ -200,11 +207,16 @@ k_gamma_reduce_f32(int X, int n_chol, int spin, bool traces, const double2* __re
     }
 }
 
-void launch_gamma_reduce_f32(int nw, int X, int n_chol, int spin, const double2* v0a, const double2* v0b,
-                             const double2* xx, const float2* Lact, const float2* Xic, const double2* Lh,
-                             float2* Y, double2* scal, cudaStream_t st, bool traces, const float2* v0w)
+void launch_gamma_reduce_f32(int nw, const int X[2], int n_chol, const double2* const v0[2], const double2* const xx[2],
+                             const float2* const Lact[2], const float2* const Xic[2], const double2* const Lh[2],
+                             float2* const Y[2], double2* scal, cudaStream_t st, bool traces, const float2* v0w)
 {
-    k_gamma_reduce_f32<<<nw, 256, 0, st>>>(X, n_chol, spin, traces, v0a, v0b, xx, Lact, Xic, Lh, Y, scal, v0w);
+    GammaArgsF a;
+    for (int s = 0; s < 2; ++s) {
+        a.X[s] = X[s]; a.v0[s] = v0[s]; a.xx[s] = xx[s]; a.Lh[s] = Lh[s]; a.Lact[s] = Lact[s]; a.Xic[s] = Xic[s];
+        a.Y[s] = Y[s];
+    }
+    k_gamma_reduce_f32<<<dim3(nw, 2), 256, 0, st>>>(a, n_chol, traces, scal, v0w);
     msd_note_launch();
 }
 

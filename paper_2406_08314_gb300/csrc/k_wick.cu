@@ -539,29 +539,36 @@ void launch_cmat(const SpinTables& ta, const SpinTables& tb, int nw, const doubl
 // minus_ref the reference part D0 D0^T (ones at (occ0_l, occ0_l)) is
 // subtracted, for the mixed path that adds its contraction in FP64.
 #define GT_COLS 16   // output columns per block
+struct GtArgs {
+    SpinTables t[2];
+    const double2 *Gr[2], *Cm[2];
+    long long off[2];
+};
 __global__ void __launch_bounds__(256)
-k_gt(SpinTables tb, int M, const double2* __restrict__ Gr, const double2* __restrict__ Cm,
-     const double2* __restrict__ Rsum, double2* __restrict__ GT, long long ld, long long off, int minus_ref)
+k_gt(const __grid_constant__ GtArgs a, int M, const double2* __restrict__ Rsum, double2* __restrict__ GT, long long ld,
+     int minus_ref)
 {
     __shared__ double2 cm[MSD_XMAX];
     __shared__ double2 y[MSD_XMAX * GT_COLS];   // [np][GT_COLS columns]
+    const int s = blockIdx.z;
+    const SpinTables& tb = a.t[s];
     const int w = blockIdx.y;
     const int c0 = blockIdx.x * GT_COLS;
     const int N = tb.N, nh = tb.nh, np = tb.np;
-    const double2* gr = Gr + (size_t)w * N * M;
-    for (int e = threadIdx.x; e < nh * np; e += blockDim.x) cm[e] = Cm[(size_t)w * nh * np + e];
+    const double2* gr = a.Gr[s] + (size_t)w * N * M;
+    for (int e = threadIdx.x; e < nh * np; e += blockDim.x) cm[e] = a.Cm[s][(size_t)w * nh * np + e];
     __syncthreads();
     const double2 R = Rsum[w];
     const double2 iR = cdiv(cz(1, 0), R);
     for (int e = threadIdx.x; e < np * GT_COLS; e += blockDim.x) {
         const int p = e / GT_COLS, c = c0 + e % GT_COLS;
-        double2 a = cz(0, 0);
+        double2 v = cz(0, 0);
         if (c < M)
-            for (int h = 0; h < nh; ++h) a = cfma(cm[p * nh + h], gr[(size_t)tb.hole_pos[h] * M + c], a);
-        y[e] = cmul(a, iR);
+            for (int h = 0; h < nh; ++h) v = cfma(cm[p * nh + h], gr[(size_t)tb.hole_pos[h] * M + c], v);
+        y[e] = cmul(v, iR);
     }
     __syncthreads();
-    double2* out = GT + (size_t)w * ld + off;
+    double2* out = GT + (size_t)w * ld + a.off[s];
     for (int e = threadIdx.x; e < (N + np) * GT_COLS; e += blockDim.x) {
         const int x = e / GT_COLS, c = c0 + e % GT_COLS;
         if (c >= M) continue;
@@ -577,11 +584,15 @@ k_gt(SpinTables tb, int M, const double2* __restrict__ Gr, const double2* __rest
     }
 }
 
-void launch_gt(const SpinTables& tb, int nw, int M, const double2* Gr, const double2* Cm,
-               const double2* R, double2* GT, long long ld, long long off, bool minus_ref, cudaStream_t st)
+// Both spins; spin s's rows go to column off[s] of a walker's row of GT.
+void launch_gt(const SpinTables& ta, const SpinTables& tb, int nw, int M, double2* const Gr[2], const double2* const Cm[2],
+               const double2* R, double2* GT, long long ld, const long long off[2], bool minus_ref, cudaStream_t st)
 {
-    dim3 grid((M + GT_COLS - 1) / GT_COLS, nw);
-    k_gt<<<grid, 256, 0, st>>>(tb, M, Gr, Cm, R, GT, ld, off, minus_ref ? 1 : 0); msd_note_launch();
+    GtArgs a;
+    a.t[0] = ta; a.t[1] = tb;
+    for (int s = 0; s < 2; ++s) { a.Gr[s] = Gr[s]; a.Cm[s] = Cm[s]; a.off[s] = off[s]; }
+    k_gt<<<dim3((M + GT_COLS - 1) / GT_COLS, nw, 2), 256, 0, st>>>(a, M, R, GT, ld, minus_ref ? 1 : 0);
+    msd_note_launch();
 }
 
 // The mixed one-body density matrix as full M x M matrices per walker and

@@ -50,8 +50,8 @@ void launch_sum_slots(int nw, const double2* part, int nslot, int slot0, int n, 
 void launch_ref_ovlp(int nw, const double2* O0a, const double2* O0b, double2* out, cudaStream_t st);
 void launch_cmat(const SpinTables& ta, const SpinTables& tb, int nw, const double2* wts_a, const double2* wts_b,
                  const void* Ba, const void* Bb, bool fp32, double2* Cm_a, double2* Cm_b, cudaStream_t st);
-void launch_gt(const SpinTables& tb, int nw, int M, const double2* Gr, const double2* Cm,
-               const double2* R, double2* GT, long long ld, long long off, bool minus_ref, cudaStream_t st);
+void launch_gt(const SpinTables& ta, const SpinTables& tb, int nw, int M, double2* const Gr[2], const double2* const Cm[2],
+               const double2* R, double2* GT, long long ld, const long long off[2], bool minus_ref, cudaStream_t st);
 void launch_rdm_scatter(const SpinTables& tb, int nw, int M, const double2* GT, long long ld, long long off, int spin,
                         double2* rdm, cudaStream_t st);
 
@@ -62,20 +62,21 @@ size_t fepi_smem(const SpinTables& tb);
 void launch_fepi(const SpinTables& tb, int nw, int M, int n_chol, const double2* F, long long ldf,
                  const double2* Gr, double2* v0, double2* xx, double2* Lact, double2* Xic,
                  cudaStream_t st);
-// hl (optional): the matrix of the Lambda_h part instead of h1.
-void launch_onebody(const SpinTables& tb, int nw, int M, const double* h1, const double2* Gr,
-                    double2* e1, double2* Lh, cudaStream_t st, const double* hl = nullptr);
-void launch_gamma_reduce(int nw, int X, int n_chol, int spin, const double2* v0a, const double2* v0b,
-                         const double2* xx, const double2* Lact, const double2* Xic,
-                         const double2* Lh, void* Y, bool fp32, double2* scal, cudaStream_t st);
+// hl: the matrix of the Lambda_h part (h1, or h1 + J).
+void launch_onebody(const SpinTables& ta, const SpinTables& tb, int nw, int M, const double* const h1[2],
+                    const double2* const Gr[2], double2* const e1[2], double2* const Lh[2], cudaStream_t st,
+                    const double* const hl[2]);
+void launch_gamma_reduce(int nw, const int X[2], int n_chol, const double2* const v0[2], const double2* const xx[2],
+                         const double2* const Lact[2], const double2* const Xic[2], const double2* const Lh[2],
+                         double2* const Y[2], double2* scal, cudaStream_t st);
 void launch_gram(int nw, int Xp, int Xq, int n_chol, const double2* P, const double2* Q, void* K,
                  bool fp32, cudaStream_t st);
 int string_energy_blocks(const SpinTables& tb, int k);
 size_t string_energy_smem(const SpinTables& tb, bool fp32);
 int string_energy_slots(const SpinTables& tb);
-void launch_string_energy(const SpinTables& tb, int nw, const double2* wts,
-                          const void* B, const void* K, const void* Y, bool fp32, double2* part,
-                          int nslot, int slot0, cudaStream_t st);
+void launch_string_energy(const SpinTables& ta, const SpinTables& tb, int nw, const double2* const wts[2],
+                          const void* const B[2], const void* const K[2], const void* const Y[2], bool fp32,
+                          double2* part, int nslot, int slot0, cudaStream_t st);
 int pair_cross_slots(const PairTables& pt, bool use_runs = false);
 // k_pair_y.cu: the opposite-spin term per beta string (mixed precision)
 bool pair_y_ok(const SpinTables& ta, const SpinTables& tb);
@@ -243,9 +244,9 @@ size_t fepi_f32_smem(const SpinTables& tb);
 void launch_fepi_f32(const SpinTables& tb, int nw, int M, int n_chol, const float* dF, long long ldf,
                      const double2* Gr, const float* F0T, const double* c0, const double* x0, double2* v0,
                      double2* xx, float2* Lact, float2* Xic, cudaStream_t st);
-void launch_gamma_reduce_f32(int nw, int X, int n_chol, int spin, const double2* v0a, const double2* v0b,
-                             const double2* xx, const float2* Lact, const float2* Xic, const double2* Lh,
-                             float2* Y, double2* scal, cudaStream_t st, bool traces,
+void launch_gamma_reduce_f32(int nw, const int X[2], int n_chol, const double2* const v0[2], const double2* const xx[2],
+                             const float2* const Lact[2], const float2* const Xic[2], const double2* const Lh[2],
+                             float2* const Y[2], double2* scal, cudaStream_t st, bool traces,
                              const float2* v0w = nullptr);
 // K[w][x][y] = sum_g P[w][g][x] Q[w][g][y] (FP32) for up to three
 // (P, Q, K) products of shapes Xp x Xq in one launch.
@@ -315,3 +316,8 @@ int launch_qr_mgs(int nw, int M, int N, double2* phi, unsigned* err, cudaStream_
 bool launch_pair_cross2(int ka, int kb, bool fp32, dim3 grid, size_t smem, const SpinTables& ta, const SpinTables& tb,
                         const PairTables& pt, int lo, int n, const void* ra, const void* rb, const void* Ba,
                         const void* Bb, const void* K, double2* part, int nslot, int slot, cudaStream_t st);
+// All level pairs (ka + kb <= 6, no runs) in one launch where that is worth it;
+// false if the caller has to launch them one by one.
+bool launch_pair_cross_all(const SpinTables& ta, const SpinTables& tb, const PairTables& pt, int nw, const void* ra,
+                           const void* rb, const void* Ba, const void* Bb, const void* K, bool fp32, double2* part,
+                           int nslot, int slot0, cudaStream_t st, bool use_runs);

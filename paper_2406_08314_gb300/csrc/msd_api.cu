@@ -1208,19 +1208,16 @@ int fb_chunk(msd_ctx* ctx, Chunk& c, FbWork& f, int w0, int nw, int cap, bool fp
     launch_sum_slots(nw, c.part, c.nslot, 0, c.nR, (double2*)f.Rs, c.O0[0], c.O0[1],
                      ov_out ? ov_out + w0 : nullptr, st);
     th.end(st);
-    long long off = 0;
     th.begin("k_cmat", st);
     launch_cmat(tables(ctx->sp[0], cap), tables(ctx->sp[1], cap), nw, c.wts[0], c.wts[1], c.B[0], c.B[1], fp32,
                 (double2*)f.Cm[0], (double2*)f.Cm[1], st);
     th.end(st);
-    for (int s = 0; s < 2; ++s) {
-        const SpinTables T = tables(ctx->sp[s], cap);
-        th.begin("k_gt", st);
-        launch_gt(T, nw, ctx->M, c.Gr[s], (double2*)f.Cm[s], (double2*)f.Rs, (double2*)f.GT, ctx->Kd, off, fp32,
-                  st);
-        th.end(st);
-        off += (long long)(T.N + T.np) * ctx->M;
-    }
+    const SpinTables T[2] = {tables(ctx->sp[0], cap), tables(ctx->sp[1], cap)};
+    const long long off[2] = {0, (long long)(T[0].N + T[0].np) * ctx->M};
+    const double2* Cm[2] = {(const double2*)f.Cm[0], (const double2*)f.Cm[1]};
+    th.begin("k_gt", st);
+    launch_gt(T[0], T[1], nw, ctx->M, c.Gr, Cm, (double2*)f.Rs, (double2*)f.GT, ctx->Kd, off, fp32, st);
+    th.end(st);
     CKLAUNCH();
     double2* out = vb_out + (size_t)w0 * ctx->n_chol;
     if (fp32) {
@@ -1469,13 +1466,15 @@ int en_rest(msd_ctx* ctx, Chunk& c, EnWork& E, int nw, int cap, bool fp32, cudaS
     const int X[2] = {T[0].nh * T[0].np, T[1].nh * T[1].np};
     const bool exact = fp32 && exact_ref_on(ctx);
     const bool traces = !exact;
-    for (int s = 0; s < 2; ++s) {
-        th.begin("k_onebody", st);
-        launch_onebody(T[s], nw, M, ctx->d_h1 + (size_t)s * M * M, c.Gr[s], (double2*)E.e1[s],
-                       (double2*)E.Lh1[s], st, exact && ctx->d_hJ ? ctx->d_hJ + (size_t)s * M * M : nullptr);
-        th.end(st);
-        CKLAUNCH();
-    }
+    const size_t MM = (size_t)M * M;
+    const double* h1[2] = {ctx->d_h1, ctx->d_h1 + MM};
+    const double* hJ[2] = {exact && ctx->d_hJ ? ctx->d_hJ : h1[0], exact && ctx->d_hJ ? ctx->d_hJ + MM : h1[1]};
+    const double2* Gr[2] = {c.Gr[0], c.Gr[1]};
+    double2 *e1[2] = {(double2*)E.e1[0], (double2*)E.e1[1]}, *Lh1[2] = {(double2*)E.Lh1[0], (double2*)E.Lh1[1]};
+    th.begin("k_onebody", st);
+    launch_onebody(T[0], T[1], nw, M, h1, Gr, e1, Lh1, st, hJ);
+    th.end(st);
+    CKLAUNCH();
     RefSpin rs[2];
     if (exact) {
         // the reference-determinant sums exactly split on the tensor cores:
@@ -1500,15 +1499,18 @@ int en_rest(msd_ctx* ctx, Chunk& c, EnWork& E, int nw, int cap, bool fp32, cudaS
         CKLAUNCH();
     }
     th.begin("k_gamma_reduce", st);
-    for (int s = 0; s < 2; ++s) {
-        if (fp32)
-            launch_gamma_reduce_f32(nw, X[s], G, s, (double2*)E.v0[0], (double2*)E.v0[1], (double2*)E.xx[s],
-                                    (float2*)E.La[s], (float2*)E.Xi[s], (double2*)E.Lh1[s], (float2*)E.Y[s],
-                                    (double2*)E.scal, st, traces, exact ? (const float2*)E.v0w : nullptr);
-        else
-            launch_gamma_reduce(nw, X[s], G, s, (double2*)E.v0[0], (double2*)E.v0[1], (double2*)E.xx[s],
-                                (double2*)E.La[s], (double2*)E.Xi[s], (double2*)E.Lh1[s], E.Y[s], false,
-                                (double2*)E.scal, st);
+    const double2* v0[2] = {(double2*)E.v0[0], (double2*)E.v0[1]};
+    const double2* xx[2] = {(double2*)E.xx[0], (double2*)E.xx[1]};
+    const double2* Lh[2] = {Lh1[0], Lh1[1]};
+    if (fp32) {
+        const float2 *La[2] = {(float2*)E.La[0], (float2*)E.La[1]}, *Xi[2] = {(float2*)E.Xi[0], (float2*)E.Xi[1]};
+        float2* Y[2] = {(float2*)E.Y[0], (float2*)E.Y[1]};
+        launch_gamma_reduce_f32(nw, X, G, v0, xx, La, Xi, Lh, Y, (double2*)E.scal, st, traces,
+                                exact ? (const float2*)E.v0w : nullptr);
+    } else {
+        const double2 *La[2] = {(double2*)E.La[0], (double2*)E.La[1]}, *Xi[2] = {(double2*)E.Xi[0], (double2*)E.Xi[1]};
+        double2* Y[2] = {(double2*)E.Y[0], (double2*)E.Y[1]};
+        launch_gamma_reduce(nw, X, G, v0, xx, La, Xi, Lh, Y, (double2*)E.scal, st);
     }
     th.end(st);
     th.begin(fp32 && tensor_gram(ctx) ? "tc_gram" : "k_gram", st);
@@ -1547,13 +1549,12 @@ int en_terms(msd_ctx* ctx, Chunk& c, EnWork& E, int w0, int nw, int cap, bool fp
     const TimerHook& th = ctx->hook;
     SpinTables T[2] = {tables(ctx->sp[0], cap), tables(ctx->sp[1], cap)};
     int slot = c.nR;
-    void* Kss[2] = {E.Kaa, E.Kbb};
+    const void *Kss[2] = {E.Kaa, E.Kbb}, *B[2] = {c.B[0], c.B[1]}, *Y[2] = {E.Y[0], E.Y[1]};
+    const double2* wts[2] = {c.wts[0], c.wts[1]};
     th.begin("k_string_energy", st);
-    for (int s = 0; s < 2; ++s) {
-        launch_string_energy(T[s], nw, c.wts[s], c.B[s], Kss[s], E.Y[s], fp32, c.part, c.nslot, slot, st);
-        slot += string_energy_slots(T[s]);
-    }
+    launch_string_energy(T[0], T[1], nw, wts, B, Kss, Y, fp32, c.part, c.nslot, slot, st);
     th.end(st);
+    slot += string_energy_slots(T[0]) + string_energy_slots(T[1]);
     CKLAUNCH();
     if (use_pair_y(ctx)) {
         th.begin("k_pair_y", st);
@@ -1741,16 +1742,18 @@ int rdm1(msd_ctx* ctx, int n_w, const double* phi_a, const double* phi_b, double
         launch_cmat(tables(ctx->sp[0], cap), tables(ctx->sp[1], cap), nw, c.wts[0], c.wts[1], c.B[0], c.B[1], fp32,
                     (double2*)f.Cm[0], (double2*)f.Cm[1], st);
         th.end(st);
-        long long off = 0;
+        const SpinTables T2[2] = {tables(ctx->sp[0], cap), tables(ctx->sp[1], cap)};
+        const long long offs[2] = {0, (long long)(T2[0].N + T2[0].np) * M};
+        const double2* Cm[2] = {(const double2*)f.Cm[0], (const double2*)f.Cm[1]};
+        th.begin("k_gt", st);
+        launch_gt(T2[0], T2[1], nw, M, c.Gr, Cm, (double2*)f.Rs, (double2*)f.GT, ctx->Kd, offs, false, st);
+        th.end(st);
         for (int s = 0; s < 2; ++s) {
-            const SpinTables T = tables(ctx->sp[s], cap);
-            th.begin("k_gt", st);
-            launch_gt(T, nw, M, c.Gr[s], (double2*)f.Cm[s], (double2*)f.Rs, (double2*)f.GT, ctx->Kd, off, false, st);
-            th.end(st);
+            const SpinTables& T = T2[s];
+            const long long off = offs[s];
             th.begin("k_rdm_scatter", st);
             launch_rdm_scatter(T, nw, M, (const double2*)f.GT, ctx->Kd, off, s, o_r.dev + (size_t)w0 * 2 * M * M, st);
             th.end(st);
-            off += (long long)(T.N + T.np) * M;
         }
         CKLAUNCH();
     }
