@@ -222,10 +222,18 @@ int oz_slices();
 // d_XT: [N Kv][G] FP64, XT[r N + l][g] = L_g[v_r][o_l]. Allocates out's arrays.
 int oz_prepare_const(int N, int Kv, int G, const double* d_XT, OzConst& out, cudaStream_t st);
 void oz_free_const(OzConst& c);
-// As: [OZ_S][pad(2 nw)][Kp] BF16 scratch, ea: [pad(2 nw)]; writes part
-// [oz_parts(NB)][pad(2 nw)] and t1 [2 nw][G].
-int oz_spin(const OzConst& K, int nw, int M, const double2* Gr, const int* virt, void* As, int* ea, double2* part,
-            double* t1, unsigned* err, cudaStream_t st);
+// One spin's walker rows: As [OZ_S][pad(2 nw)][Kp] BF16 scratch, ea [pad(2 nw)];
+// written are part [oz_parts(NB)][pad(2 nw)] and t1 [2 nw][G].
+struct OzSpin {
+    const OzConst* K;
+    const double2* Gr;
+    const int* virt;
+    void* As;
+    int* ea;
+    double2* part;
+    double* t1;
+};
+int oz_both(const OzSpin in[2], int nw, int M, unsigned* err, cudaStream_t st);
 // Also writes the walker parts t1a_g + t1b_g of V0_g as FP32 pairs v0w[w][g].
 void launch_ref_reduce(int nw, int G, const RefSpin& a, const RefSpin& b, double C2sum, double2* scal,
                        float2* v0w, cudaStream_t st);

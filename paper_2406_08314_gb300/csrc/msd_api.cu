@@ -1253,7 +1253,7 @@ int fb_chunk(msd_ctx* ctx, Chunk& c, FbWork& f, int w0, int nw, int cap, bool fp
 struct EnWork {
     void *F[2] = {nullptr, nullptr}, *F32 = nullptr, *Ah = nullptr, *Al = nullptr;
     void *v0[2], *xx[2], *La[2], *Xi[2], *Lh1[2], *e1[2], *Y[2], *Kaa, *Kbb, *Kab, *scal;
-    void *ozA = nullptr, *ozE = nullptr, *ozP[2] = {nullptr, nullptr}, *ozT[2] = {nullptr, nullptr};
+    void *ozA[2] = {nullptr, nullptr}, *ozE[2] = {nullptr, nullptr}, *ozP[2] = {nullptr, nullptr}, *ozT[2] = {nullptr, nullptr};
     void* v0w = nullptr;   // [nw][G] FP32 walker parts of V0_g (exact reference sums)
     void* GT[2] = {nullptr, nullptr};   // [nw][2X][G] Lambda rows for the tensor-core Gram
 };
@@ -1305,9 +1305,8 @@ size_t en_bytes_per_walker(msd_ctx* ctx, bool fp32)
     e += (size_t)X[0] * X[0] + (size_t)X[1] * X[1] + (size_t)X[0] * X[1];
     size_t b = e * sizeof(double2);
     if (fp32 && exact_ref_on(ctx)) {
-        int kp = 0;
-        for (int s = 0; s < 2; ++s) kp = std::max(kp, oz_k_padded(T1[s].N * (ctx->M - T1[s].N)));
-        b += (size_t)2 * oz_slices() * kp * 2 + 2 * sizeof(int);
+        for (int s = 0; s < 2; ++s)
+            b += (size_t)2 * oz_slices() * oz_k_padded(T1[s].N * (ctx->M - T1[s].N)) * 2 + 2 * sizeof(int);
         b += sizeof(float2) * (size_t)G;   // v0w
         for (int s = 0; s < 2; ++s)
             b += (size_t)2 * oz_parts_for(T1[s].N * (ctx->M - T1[s].N), G) * sizeof(double2) + 2 * sizeof(double) * G;
@@ -1372,14 +1371,14 @@ int en_alloc(msd_ctx* ctx, int cap, bool fp32, EnWork& E)
     if ((rc = arena_get(ctx, "scal", sizeof(double2) * cap * 8, &E.scal))) return rc;
     if (fp32 && exact_ref_on(ctx)) {
         const int Mpad = oz_rows_padded(2 * cap);
-        int kp = 0;
-        for (int s = 0; s < 2; ++s) kp = std::max(kp, oz_k_padded(T1[s].N * (ctx->M - T1[s].N)));
-        if ((rc = arena_get(ctx, "oz_A", (size_t)oz_slices() * Mpad * kp * 2, &E.ozA))) return rc;
-        if ((rc = arena_get(ctx, "oz_ea", sizeof(int) * Mpad, &E.ozE))) return rc;
+        static const char* na_[2] = {"oz_A_a", "oz_A_b"};
+        static const char* ne_[2] = {"oz_ea_a", "oz_ea_b"};
         static const char* np_[2] = {"oz_part_a", "oz_part_b"};
         static const char* nt_[2] = {"oz_t1_a", "oz_t1_b"};
         for (int s = 0; s < 2; ++s) {
-            const int nparts = oz_parts_for(T1[s].N * (ctx->M - T1[s].N), G);
+            const int NK = T1[s].N * (ctx->M - T1[s].N), nparts = oz_parts_for(NK, G);
+            if ((rc = arena_get(ctx, na_[s], (size_t)oz_slices() * Mpad * oz_k_padded(NK) * 2, &E.ozA[s]))) return rc;
+            if ((rc = arena_get(ctx, ne_[s], sizeof(int) * Mpad, &E.ozE[s]))) return rc;
             if ((rc = arena_get(ctx, np_[s], sizeof(double2) * nparts * Mpad, &E.ozP[s]))) return rc;
             if ((rc = arena_get(ctx, nt_[s], sizeof(double) * 2 * cap * (size_t)G, &E.ozT[s]))) return rc;
         }
@@ -1482,17 +1481,17 @@ int en_rest(msd_ctx* ctx, Chunk& c, EnWork& E, int nw, int cap, bool fp32, cudaS
         // t1_g of V0_g leave only the small part of sum_g V0_g Lambda_g to
         // the FP32 sum (the reference part C_g is in Lh1, the one-body term
         // of h + J)
+        OzSpin oz[2];
         for (int s = 0; s < 2; ++s) {
             const OzConst& K = ctx->oz[s];
-            th.begin("tc_ozaki", st);
-            if (oz_spin(K, nw, M, c.Gr[s], ctx->d_virt[s], E.ozA, (int*)E.ozE, (double2*)E.ozP[s],
-                        (double*)E.ozT[s], ctx->d_err, st))
-                return fail(ctx, MSD_ERR_CUDA, "exact reference tensor-core launch failed");
-            th.end(st);
+            oz[s] = OzSpin{&K, c.Gr[s], ctx->d_virt[s], E.ozA[s], (int*)E.ozE[s], (double2*)E.ozP[s], (double*)E.ozT[s]};
             rs[s] = RefSpin{K.N, M, K.Kv, oz_parts(K.NB), oz_rows_padded(2 * nw), c.Gr[s], ctx->d_virt[s],
                             ctx->d_JJ[s], ctx->d_KK[s], (const double*)E.ozT[s], (const double2*)E.ozP[s],
                             ctx->oz_x0sum[s]};
         }
+        th.begin("tc_ozaki", st);
+        if (oz_both(oz, nw, M, ctx->d_err, st)) return fail(ctx, MSD_ERR_CUDA, "exact reference tensor-core launch failed");
+        th.end(st);
         th.begin("k_ref_reduce", st);
         launch_ref_reduce(nw, G, rs[0], rs[1], ctx->oz_C2sum, (double2*)E.scal, (float2*)E.v0w, st);
         th.end(st);

@@ -82,6 +82,12 @@ struct OzArgs {
     const int* virt;
     double2* part;          // [n_tiles_n * 2][Mpad]
     double* t1;             // [nrow][G]
+    int tiles;              // column tiles
+};
+// Both spins of a launch (blockIdx.z).
+struct OzLaunch {
+    CUtensorMap ta[2], tb[2];
+    OzArgs s[2];
     unsigned* err;
 };
 
@@ -96,9 +102,12 @@ __device__ __forceinline__ void tmem_ld16_nowait(uint32_t taddr, uint32_t* r)
 }
 
 __global__ void __launch_bounds__(OZ_THREADS, 1)
-k_tc_ozaki(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb,
-           const __grid_constant__ OzArgs a)
+k_tc_ozaki(const __grid_constant__ OzLaunch L)
 {
+    const OzArgs& a = L.s[blockIdx.z];
+    const CUtensorMap &ta = L.ta[blockIdx.z], &tb = L.tb[blockIdx.z];
+    unsigned* const err = L.err;
+    if ((int)blockIdx.y >= a.tiles) return;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     __shared__ __align__(8) uint64_t full_bar[OZ_STAGES], empty_bar[OZ_STAGES];
@@ -113,7 +122,7 @@ k_tc_ozaki(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUten
     // V's rows are padded with zeros to whole tiles (NVp), so no tile mixes
     // V and W columns. The W tiles take the full K range and run first; the
     // V tiles follow, longest first.
-    const int nvt = a.NVp / OZ_BN, ntile = gridDim.y;
+    const int nvt = a.NVp / OZ_BN, ntile = a.tiles;
     const int tile = (int)blockIdx.y < ntile - nvt ? nvt + (int)blockIdx.y : (int)blockIdx.y - (ntile - nvt);
     const bool sym = tile < nvt;
     const int m0 = blockIdx.x * OZ_BM, n0 = tile * OZ_BN;
@@ -122,7 +131,7 @@ k_tc_ozaki(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUten
     const int first = sym ? OZ_BN / OZ_BK : OZ_KCH_KB;                   // k-blocks of chunk 0
     const int nch = nkt <= first ? 1 : 1 + (nkt - first + OZ_KCH_KB - 1) / OZ_KCH_KB;
     auto chunk_begin = [&](int ch) { return ch == 0 ? 0 : first + (ch - 1) * OZ_KCH_KB; };   // relative
-    const uint64_t wb = wait_budget(a.err);
+    const uint64_t wb = wait_budget(err);
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < OZ_STAGES; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
@@ -151,7 +160,7 @@ k_tc_ozaki(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUten
                 const int s = kb % OZ_STAGES;
                 if (!mbar_wait(&empty_bar[s], ((kb / OZ_STAGES) & 1) ^ 1, wb) || *vfail) {
                     *vfail = 1;
-                    atomicOr(a.err, MSD_DEV_ERR_TIMEOUT);
+                    atomicOr(err, MSD_DEV_ERR_TIMEOUT);
                     break;
                 }
                 uint8_t* st = smem + (size_t)s * OZ_STAGE;
@@ -211,7 +220,7 @@ k_tc_ozaki(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUten
         if (leader) {
             if (!ok) {
                 *vfail = 1;
-                atomicOr(a.err, MSD_DEV_ERR_TIMEOUT);
+                atomicOr(err, MSD_DEV_ERR_TIMEOUT);
             }
             // every product issued by this thread completes before TMEM is freed
             mma_commit(&drain_bar);
@@ -252,7 +261,7 @@ k_tc_ozaki(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUten
             if (lane == 0) mbar_arrive(&tempty);
         }
         if (!ok) {
-            if (lane == 0) { *vfail = 1; atomicOr(a.err, MSD_DEV_ERR_TIMEOUT); }
+            if (lane == 0) { *vfail = 1; atomicOr(err, MSD_DEV_ERR_TIMEOUT); }
         } else if (row < a.nrow) {
             const int w = row >> 1;
             const int er = a.ea[row] - OZ_BETA * (OZ_S + 1);
@@ -261,7 +270,7 @@ k_tc_ozaki(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUten
             for (int i = 0; i < OZ_HALF; ++i) {
                 const int n = n0 + hf * OZ_HALF + i;
                 if (n >= a.NB) break;
-                const double v = ldexp((double)acc[i], er + a.eb[n]);
+                const double v = int_to_fp64(acc[i], er + a.eb[n]);
                 if (n < a.NV) {
                     const int j = n / a.Kv, r = n - j * a.Kv;
                     const double2 u = a.Gr[((size_t)w * a.N + j) * a.M + a.virt[r]];
@@ -321,11 +330,26 @@ __device__ __forceinline__ int slice_exponent(double mx)
 
 // Slices of the walker rows: row 2w + c is part c (real, imaginary) of
 // u_w[(j, r)] = Gr[w][j][virt[r]]; rows >= nrow and columns >= N Kv are zero.
+struct OzRows {
+    int N, Kv, Kp;
+    const double2* Gr;
+    const int* virt;
+    __nv_bfloat16* As;
+    int* ea;
+    size_t slice_stride;
+};
+struct OzRowArgs { OzRows s[2]; };
 __global__ void __launch_bounds__(256)
-k_oz_slice_rows(int nrow, int N, int M, int Kv, int Kp, const double2* __restrict__ Gr, const int* __restrict__ virt,
-                __nv_bfloat16* __restrict__ As, int* __restrict__ ea, size_t slice_stride)
+k_oz_slice_rows(const __grid_constant__ OzRowArgs args, int nrow, int M)
 {
     __shared__ double red[32];
+    const OzRows& R = args.s[blockIdx.y];
+    const int N = R.N, Kv = R.Kv, Kp = R.Kp;
+    const double2* Gr = R.Gr;
+    const int* virt = R.virt;
+    __nv_bfloat16* As = R.As;
+    int* ea = R.ea;
+    const size_t slice_stride = R.slice_stride;
     const int row = blockIdx.x, NK = N * Kv;
     const int w = row >> 1, c = row & 1;
     const bool live = row < nrow;
@@ -450,9 +474,20 @@ k_ref_reduce(int nw, int G, RefSpin sa, RefSpin sb, double C2sum, double2* __res
         q = cfma(v, v, q);
         v0w[(size_t)w * G + g] = make_float2((float)v.x, (float)v.y);
     }
+    // u^T V u of both spins: the tiles' partial forms (ur.Vur, ui.Vur) and
+    // (ur.Vui, ui.Vui) of the walker's two rows
+    double2 x2[2] = {cz(0, 0), cz(0, 0)};
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+        const RefSpin& R = *S[s];
+        for (int p = t; p < R.nparts; p += blockDim.x) {
+            const double2 pr = R.part[(size_t)p * R.Mpad + 2 * w], pi = R.part[(size_t)p * R.Mpad + 2 * w + 1];
+            x2[s] = cadd(x2[s], cz(pr.x - pi.y, pi.x + pr.y));
+        }
+    }
     red[0][t] = cadd(lj[0], lj[1]);
-    red[1][t] = lk[0];
-    red[2][t] = lk[1];
+    red[1][t] = cadd(cscale(lk[0], 2.0), x2[0]);
+    red[2][t] = cadd(cscale(lk[1], 2.0), x2[1]);
     red[3][t] = q;
     __syncthreads();
     for (int o = 128; o; o >>= 1) {
@@ -461,20 +496,9 @@ k_ref_reduce(int nw, int G, RefSpin sa, RefSpin sb, double C2sum, double2* __res
         __syncthreads();
     }
     if (t == 0) {
-        double2 x2[2];
-        for (int s = 0; s < 2; ++s) {
-            const RefSpin& R = *S[s];
-            double2 v = cz(0, 0);
-            for (int p = 0; p < R.nparts; ++p) {
-                const double2 pr = R.part[(size_t)p * R.Mpad + 2 * w];       // (ur.Vur, ui.Vur)
-                const double2 pi = R.part[(size_t)p * R.Mpad + 2 * w + 1];   // (ur.Vui, ui.Vui)
-                v = cadd(v, cz(pr.x - pi.y, pi.x + pr.y));
-            }
-            x2[s] = v;
-        }
         double2* sc = scal + (size_t)w * 8;
-        sc[0] = cadd(cz(sa.x0sum, 0), cadd(cscale(red[1][0], 2.0), x2[0]));
-        sc[1] = cadd(cz(sb.x0sum, 0), cadd(cscale(red[2][0], 2.0), x2[1]));
+        sc[0] = cadd(cz(sa.x0sum, 0), red[1][0]);
+        sc[1] = cadd(cz(sb.x0sum, 0), red[2][0]);
         sc[2] = cadd(cz(C2sum, 0), cadd(cscale(red[0][0], 2.0), red[3][0]));
     }
 }
@@ -528,30 +552,31 @@ void oz_free_const(OzConst& c)
     c = OzConst{};
 }
 
-int oz_spin(const OzConst& K, int nw, int M, const double2* Gr, const int* virt, void* As, int* ea, double2* part,
-            double* t1, unsigned* err, cudaStream_t st)
+int oz_both(const OzSpin in[2], int nw, int M, unsigned* err, cudaStream_t st)
 {
     const int nrow = 2 * nw, Mpad = oz_rows_padded(nrow);
-    const size_t sa = (size_t)Mpad * K.Kp;
-    k_oz_slice_rows<<<Mpad, 256, 0, st>>>(nrow, K.N, M, K.Kv, K.Kp, Gr, virt, (__nv_bfloat16*)As, ea, sa);
-    msd_note_launch();
-    CUtensorMap ma, mb;
-    if (tc_make_map(&ma, As, K.Kp, OZ_S * Mpad, K.Kp, OZ_BM, true, 64) ||
-        tc_make_map(&mb, K.Bs, K.Kp, OZ_S * K.NBp, K.Kp, OZ_BN, true, 64))
-        return -1;
-    static bool attr = false;
-    if (!attr) {
-        if (cudaFuncSetAttribute(k_tc_ozaki, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)OZ_SMEM) !=
-            cudaSuccess)
+    OzRowArgs r;
+    OzLaunch L;
+    L.err = err;
+    int tiles = 0;
+    for (int s = 0; s < 2; ++s) {
+        const OzConst& K = *in[s].K;
+        r.s[s] = OzRows{K.N, K.Kv, K.Kp, in[s].Gr, in[s].virt, (__nv_bfloat16*)in[s].As, in[s].ea, (size_t)Mpad * K.Kp};
+        if (tc_make_map(&L.ta[s], in[s].As, K.Kp, OZ_S * Mpad, K.Kp, OZ_BM, true, 64) ||
+            tc_make_map(&L.tb[s], K.Bs, K.Kp, OZ_S * K.NBp, K.Kp, OZ_BN, true, 64))
             return -1;
-        attr = true;
+        OzArgs& a = L.s[s];
+        a.nrow = nrow; a.Mpad = Mpad; a.NB = K.NB; a.NBp = K.NBp; a.NV = K.NK; a.NVp = K.NVp; a.G = K.G; a.Kp = K.Kp;
+        a.N = K.N; a.M = M; a.Kv = K.Kv;
+        a.ea = in[s].ea; a.eb = K.eb; a.Gr = in[s].Gr; a.virt = in[s].virt; a.part = in[s].part; a.t1 = in[s].t1;
+        a.tiles = K.NBp / OZ_BN;
+        tiles = tiles > a.tiles ? tiles : a.tiles;
     }
-    OzArgs a;
-    a.nrow = nrow; a.Mpad = Mpad; a.NB = K.NB; a.NBp = K.NBp; a.NV = K.NK; a.NVp = K.NVp; a.G = K.G; a.Kp = K.Kp;
-    a.N = K.N; a.M = M; a.Kv = K.Kv;
-    a.ea = ea; a.eb = K.eb; a.Gr = Gr; a.virt = virt; a.part = part; a.t1 = t1; a.err = err;
-    dim3 grid(Mpad / OZ_BM, K.NBp / OZ_BN);
-    k_tc_ozaki<<<grid, OZ_THREADS, OZ_SMEM, st>>>(ma, mb, a);
+    k_oz_slice_rows<<<dim3(Mpad, 2), 256, 0, st>>>(r, nrow, M);
+    msd_note_launch();
+    if (cudaFuncSetAttribute(k_tc_ozaki, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)OZ_SMEM) != cudaSuccess)
+        return -1;
+    k_tc_ozaki<<<dim3(Mpad / OZ_BM, tiles, 2), OZ_THREADS, OZ_SMEM, st>>>(L);
     msd_note_launch();
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
