@@ -18,6 +18,7 @@
 
 #include "common.cuh"
 #include "det_terms.cuh"
+#include "fixed.cuh"
 #include "kernels.h"
 
 // ------------------------------------------------------------------------
@@ -136,59 +137,14 @@ k_fepi(SpinTables tb, int M, int n_chol, const double2* __restrict__ F, long lon
 
 size_t fepi_smem(const SpinTables& tb) { return sizeof(double2) * (tb.N * (tb.N + tb.np) + 2 * tb.N * tb.np); }
 
-// The same epilogue in 64-bit fixed point for N <= 32. The FP64 form is bound by
-// the FP64 unit (95 % of its rate, 6.2 ms per spin for 640 copper-oxo walkers);
-// mad.wide.s32 issues 24 times as often (44 against 1.8 per clock and SM,
-// measured). Operands are rounded to 54 fractional bits of their block's largest
-// magnitude (T per (walker, vector), G[occ0][P] per walker, Lambda per (walker,
-// vector)) and held as two signed limbs, q = h 2^26 + l, |h| <= 2^28, |l| <= 2^25;
-// a real product is h h' (weight 2^52) plus h l' + l h' (2^26), three mad.wide; l l'
-// (2^-58 of the block scales' product) is dropped. Sums of up to 64 products h h'
-// stay below 2^62, so nothing overflows for N <= 32. The result is rounded to FP64
-// once. The trace of T, which weighs most in the energy, sums 56 bits. Measured
+// The same epilogue in fixed point (fixed.cuh) for N <= 32: the FP64 form is bound
+// by the FP64 unit (95 % of its rate, 6.2 ms per spin for 640 copper-oxo walkers).
+// One scale per block of operands: T per (walker, vector), G[occ0][P] per walker,
+// Lambda per (walker, vector); sums of up to 32 complex products. The trace of T,
+// which weighs most in the energy, sums 56 bits. Measured
 // relative rms error against long double, fixed point and FP64: Lambda 5.7e-17 and
 // 2.4e-16, Xi 1.2e-16 and 3.0e-16, tr T T 3.4e-17 and 5.6e-17. 6.2 -> 2.5 ms per spin
 // (640 copper-oxo walkers), 3.1 -> 1.2 ms (64 iron-sulfur walkers).
-struct Limbs { int rh, rl, ih, il; };   // one complex value
-
-__device__ __forceinline__ Limbs to_limbs(double2 v, int e)
-{
-    Limbs o;
-    const long long r = fixed_point<54>(v.x, e), i = fixed_point<54>(v.y, e);
-    o.rl = ((int)r << 6) >> 6;                       // the low 26 bits, signed
-    o.rh = (int)((r - o.rl) >> 26);
-    o.il = ((int)i << 6) >> 6;
-    o.ih = (int)((i - o.il) >> 26);
-    return o;
-}
-
-struct LimbSum {
-    long long rr = 0, ii = 0, im = 0, crr = 0, cii = 0, cim = 0;
-    __device__ __forceinline__ void add(const Limbs& a, const Limbs& b)
-    {
-        rr += (long long)a.rh * b.rh;
-        crr += (long long)a.rh * b.rl;
-        crr += (long long)a.rl * b.rh;
-        ii += (long long)a.ih * b.ih;
-        cii += (long long)a.ih * b.il;
-        cii += (long long)a.il * b.ih;
-        im += (long long)a.rh * b.ih;
-        im += (long long)a.ih * b.rh;
-        cim += (long long)a.rh * b.il;
-        cim += (long long)a.rl * b.ih;
-        cim += (long long)a.ih * b.rl;
-        cim += (long long)a.il * b.rh;
-    }
-    // both parts in units of 2^-56 of the scales' product
-    __device__ __forceinline__ long long re() const { return (rr - ii) + ((crr - cii + (1 << 25)) >> 26); }
-    __device__ __forceinline__ long long imag() const { return im + ((cim + (1 << 25)) >> 26); }
-};
-
-__device__ __forceinline__ unsigned mag_bits(double2 v)
-{
-    return max((unsigned)__double2hiint(v.x) & 0x7fffffffu, (unsigned)__double2hiint(v.y) & 0x7fffffffu);
-}
-
 #define FEPI_INT_NMAX 32
 #define FEPI_INT_G 8      // Cholesky vectors per block: G[occ0][P] is converted once for them
 __global__ void __launch_bounds__(256)
@@ -262,10 +218,13 @@ k_fepi_int(SpinTables tb, int M, int n_chol, const double2* __restrict__ F, long
         // tr T T over the warps (each thread's sum cut at 12 bits, so that the
         // totals of both halves stay in 64 and 32 bits), tr T
         LimbSum x;
+        long long xr = 0, xi = 0;
         for (int e = t; e < N * N; e += nt) {
             const int j = e / N, l = e - j * N;
-            x.add(tl[j * NC + l], tl[l * NC + j]);
+            x.add_all(tl[j * NC + l], tl[l * NC + j], xr, xi);
         }
+        x.crr += xr >> 26;
+        x.cim += xi >> 26;
         long long q[2] = {x.re(), x.imag()};
         int lo[2];
 #pragma unroll
@@ -548,16 +507,89 @@ struct SeArgs {
     int blk[2][MSD_KMAX + 2];   // first block of each (spin, level)
 };
 
+// FP64 mode, levels 1 to 5: e_s of string_energy_value with the sums over the pair
+// table and over Y in fixed point (the FP64 unit bounds the plain form: level 4, 496
+// FP64 operations per string; here 48 and 1056 mad.wide):
+//   e_s = sum_ij b_ij Y[h_j][p_i] + sum_{i < k-1} sum_j b_ij z_ij,
+//   z_ij = sum_{m > i} sum_{l != j} (+ for l > j, - for l < j) b_ml A[h_j,h_l;p_i,p_m].
+// Scales: A, Y per walker (exponents ea, ey), b the string's largest entry.
+template <int KL>
+__device__ __forceinline__ double2 string_energy_fixed(const SpinTables& tb, int w, int sl, int ns, const void* Bin,
+                                                       const Limbs* as, int ea, const Limbs* ys, int ey)
+{
+    const int np = tb.np, nh = tb.nh, npp = np * (np - 1) / 2;
+    const uint4 rec = tb.str_hp[tb.bucket[KL] + sl];
+    const double2* B = reinterpret_cast<const double2*>(Bin) + (size_t)tb.b_off[KL] + ((size_t)w * ns + sl) * b_stride(KL);
+    Limbs b[KL * KL];
+    int eb;
+    {
+        unsigned m = 0;
+#pragma unroll
+        for (int e = 0; e < KL * KL; ++e) m = max(m, mag_bits(B[e]));
+        eb = mag_exponent(m);
+#pragma unroll
+        for (int e = 0; e < KL * KL; ++e) b[e] = to_limbs(B[e], eb);
+    }
+    LimbSum lin;
+#pragma unroll
+    for (int i = 0; i < KL; ++i)
+#pragma unroll
+        for (int j = 0; j < KL; ++j) lin.add(b[i * KL + j], ys[rec_h(rec, j) * np + rec_p(rec, i)]);
+    double2 v = limb_value(lin, eb + ey);
+#pragma unroll
+    for (int i = 0; i + 1 < KL; ++i)
+#pragma unroll
+        for (int j = 0; j < KL; ++j) {
+            LimbSum z;
+#pragma unroll
+            for (int m = i + 1; m < KL; ++m) {
+                const int pim = pair_index(rec_p(rec, i), rec_p(rec, m), np);
+#pragma unroll
+                for (int l = 0; l < KL; ++l) {
+                    if (l == j) continue;
+                    const int hp = l > j ? pair_index(rec_h(rec, j), rec_h(rec, l), nh)
+                                         : pair_index(rec_h(rec, l), rec_h(rec, j), nh);
+                    if (l > j) z.add(b[m * KL + l], as[hp * npp + pim]);
+                    else z.sub(b[m * KL + l], as[hp * npp + pim]);
+                }
+            }
+            v = cfma(B[i * KL + j], limb_value(z, eb + ea), v);
+        }
+    if (max(max(ea, ey), eb) >= FIXED_EXP_INF) v.x = v.y = __longlong_as_double(0x7ff8000000000000ll);
+    return v;
+}
+
+// The pair table and Y of a block in shared memory, FP32 / FP64, or as limbs with
+// their exponents where string_energy_fixed reads them.
+template <typename T>
+struct SeTab {
+    const cplx_t<T>*as, *ys;
+    int ea, ey;
+};
+#define SE_FIXED_MAX 5
+template <int KL, typename T>
+__device__ __forceinline__ double2 string_energy_any(const SpinTables& tb, int w, int sl, int ns, const void* B,
+                                                     const SeTab<T>& tab, const double2* wts)
+{
+    if constexpr (std::is_same<T, double>::value && KL <= SE_FIXED_MAX) {
+        const double2 e = string_energy_fixed<KL>(tb, w, sl, ns, B, reinterpret_cast<const Limbs*>(tab.as), tab.ea,
+                                                  reinterpret_cast<const Limbs*>(tab.ys), tab.ey);
+        return cmul(wts[(size_t)w * tb.n_str + tb.bucket[KL] + sl], e);   // wts holds r_s w_s
+    } else {
+        return string_energy_term<KL, T, true>(tb, w, sl, ns, B, tab.as, tab.ys, wts);
+    }
+}
+
 template <int KL, typename T>
 __device__ __forceinline__ double2 string_energy_block(const SpinTables& tb, int w, int blk, const void* B,
-                                                       const cplx_t<T>* as, const cplx_t<T>* ys, const double2* wts)
+                                                       const SeTab<T>& tab, const double2* wts)
 {
     const int ns = tb.bucket[KL + 1] - tb.bucket[KL];
     double2 contrib = cz(0, 0);
     for (int it = 0; it < SE_PER_THREAD; ++it) {
         const int sl = blk * (SE_THREADS * SE_PER_THREAD) + it * SE_THREADS + threadIdx.x;
         if (sl >= ns) break;
-        contrib = cadd(contrib, string_energy_term<KL, T, true>(tb, w, sl, ns, B, as, ys, wts));
+        contrib = cadd(contrib, string_energy_any<KL, T>(tb, w, sl, ns, B, tab, wts));
     }
     return contrib;
 }
@@ -598,19 +630,33 @@ k_string_energy(const __grid_constant__ SeArgs a, double2* __restrict__ part, in
     }
     const T2* Yw = reinterpret_cast<const T2*>(a.Y[s]) + (size_t)w * X;
     for (int e = t; e < X; e += blockDim.x) ys[e] = Yw[e];
+    SeTab<T> tab = {as, ys, 0, 0};
+    if constexpr (std::is_same<T, double>::value) {
+        if (k <= SE_FIXED_MAX) {   // each thread its own entries
+            __shared__ unsigned wm[2][SE_THREADS / 32];
+            unsigned ma = 0, my = 0;
+            for (int e = k > 1 ? t : nhp * npp; e < nhp * npp; e += blockDim.x) ma = max(ma, mag_bits(as[e]));
+            for (int e = t; e < X; e += blockDim.x) my = max(my, mag_bits(ys[e]));
+            tab.ea = mag_exponent(block_mag(ma, wm[0]));
+            tab.ey = mag_exponent(block_mag(my, wm[1]));
+            Limbs *la = reinterpret_cast<Limbs*>(as), *ly = reinterpret_cast<Limbs*>(ys);
+            for (int e = k > 1 ? t : nhp * npp; e < nhp * npp; e += blockDim.x) la[e] = to_limbs(as[e], tab.ea);
+            for (int e = t; e < X; e += blockDim.x) ly[e] = to_limbs(ys[e], tab.ey);
+        }
+    }
     __syncthreads();
     const int blk = b - a.blk[s][k];
     double2 v;
     if constexpr (ONLY > 0) {
-        v = string_energy_block<ONLY, T>(tb, w, blk, a.B[s], as, ys, a.wts[s]);
+        v = string_energy_block<ONLY, T>(tb, w, blk, a.B[s], tab, a.wts[s]);
     } else {
         switch (k) {
-        case 1: v = string_energy_block<1, T>(tb, w, blk, a.B[s], as, ys, a.wts[s]); break;
-        case 2: v = string_energy_block<2, T>(tb, w, blk, a.B[s], as, ys, a.wts[s]); break;
-        case 3: v = string_energy_block<3, T>(tb, w, blk, a.B[s], as, ys, a.wts[s]); break;
-        case 4: v = string_energy_block<4, T>(tb, w, blk, a.B[s], as, ys, a.wts[s]); break;
-        case 5: v = string_energy_block<5, T>(tb, w, blk, a.B[s], as, ys, a.wts[s]); break;
-        default: v = string_energy_block<6, T>(tb, w, blk, a.B[s], as, ys, a.wts[s]); break;
+        case 1: v = string_energy_block<1, T>(tb, w, blk, a.B[s], tab, a.wts[s]); break;
+        case 2: v = string_energy_block<2, T>(tb, w, blk, a.B[s], tab, a.wts[s]); break;
+        case 3: v = string_energy_block<3, T>(tb, w, blk, a.B[s], tab, a.wts[s]); break;
+        case 4: v = string_energy_block<4, T>(tb, w, blk, a.B[s], tab, a.wts[s]); break;
+        case 5: v = string_energy_block<5, T>(tb, w, blk, a.B[s], tab, a.wts[s]); break;
+        default: v = string_energy_block<6, T>(tb, w, blk, a.B[s], tab, a.wts[s]); break;
         }
     }
     red[t] = v;
