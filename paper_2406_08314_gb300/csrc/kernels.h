@@ -1,6 +1,8 @@
 // Host-side launchers of the libmsd kernels (internal to csrc/).
 #pragma once
 
+#include <cuda_bf16.h>
+
 #include "common.cuh"
 
 // Optional per-kernel event timing, supplied by the context.
@@ -114,8 +116,16 @@ int tc_gemm_3xtf32(const TcOperand& A, const TcOperand& B, int Mr, int Nc, int K
                    unsigned* err, cudaStream_t st, int splits = 1, long long c_split_stride = 0, int bn = 0);
 // BF16 tensor-core GEMM C[m][n] = sum_k A[m][k] B[n][k] (FP32 accumulation;
 // A, B row-major BF16 with K contiguous, K a multiple of 64).
+// epi, ep: 0 plain; 1 and 2 the network layers' epilogues (tc_gemm.cu, EPI), with C,
+// h and zin of row pitch ldc and ht [Nc][ldt].
+struct NetEpi {
+    const float* bias = nullptr;
+    const float* zin = nullptr;
+    __nv_bfloat16 *h = nullptr, *ht = nullptr;
+    int ldt = 0, Bp = 0;
+};
 int tc_gemm_bf16(const void* A, long long lda, const void* B, long long ldb, int Mr, int Nc, int K, float* C,
-                 long long ldc, unsigned* err, cudaStream_t st);
+                 long long ldc, unsigned* err, cudaStream_t st, int epi = 0, const NetEpi* ep = nullptr);
 // part_rows: rows per (block, part) in the output (0: R; larger pads each
 // part with zero rows). eye0 >= 0: columns [eye0, eye0 + 2 part_rows) hold
 // two identity blocks on the real-part rows r < R (1 at column eye0 + r and

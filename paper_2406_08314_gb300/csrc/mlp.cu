@@ -24,7 +24,6 @@ typedef __nv_bfloat16 bf16;
 
 namespace {
 
-__device__ __forceinline__ float gelu(float z) { return 0.5f * z * (1.f + erff(z * 0.70710678118654752f)); }
 __device__ __forceinline__ float gelu_d(float z)
 {
     return 0.5f * (1.f + erff(z * 0.70710678118654752f)) + z * 0.39894228040143268f * expf(-0.5f * z * z);
@@ -36,35 +35,27 @@ int grid_of(long long n)
     return (int)((n + 255) / 256 < cap ? (n + 255) / 256 : cap);
 }
 
-// x fp32 [B][n] -> row-major bf16 [B][n] and transposed bf16 [n][ldt]
-__global__ void k_in_bf16(int B, int n, const float* __restrict__ x, bf16* __restrict__ xb, bf16* __restrict__ xt,
-                          int ldt)
+// x fp32 [B][n] -> row-major bf16 [B][n] and transposed bf16 [n][ldt], whose
+// columns [B, Bp) are zero (the K padding of the weight-gradient products). A 64 x
+// 64 tile per block goes through shared memory, so that both copies are written
+// along their rows (element-wise, the transposed writes took 31 us for 512 x 6912).
+__global__ void __launch_bounds__(256) k_in_bf16(int B, int Bp, int n, const float* __restrict__ x, bf16* __restrict__ xb,
+                                                 bf16* __restrict__ xt, int ldt)
 {
-    const long long total = (long long)B * n;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
-         e += (long long)gridDim.x * blockDim.x) {
-        const int b = (int)(e / n), j = (int)(e % n);
-        const bf16 v = __float2bfloat16(x[e]);
-        xb[e] = v;
-        xt[(size_t)j * ldt + b] = v;
+    __shared__ bf16 tile[64][66];
+    const int j0 = blockIdx.x * 64, b0 = blockIdx.y * 64, c = threadIdx.x & 63, r = threadIdx.x >> 6;
+    for (int i = r; i < 64; i += 4) {
+        const int b = b0 + i, j = j0 + c;
+        bf16 v = __float2bfloat16(0.f);
+        if (b < B && j < n) {
+            v = __float2bfloat16(x[(size_t)b * n + j]);
+            xb[(size_t)b * n + j] = v;
+        }
+        tile[i][c] = v;
     }
-}
-
-// z = acc + bias (fp32, kept for the backward pass); h = GELU(z) in bf16,
-// row-major [B][n] and transposed [n][ldt]
-__global__ void k_bias_gelu(int B, int n, float* __restrict__ z, const float* __restrict__ bias,
-                            bf16* __restrict__ h, bf16* __restrict__ ht, int ldt)
-{
-    const long long total = (long long)B * n;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
-         e += (long long)gridDim.x * blockDim.x) {
-        const int b = (int)(e / n), j = (int)(e % n);
-        const float v = z[e] + bias[j];
-        z[e] = v;
-        const bf16 hv = __float2bfloat16(gelu(v));
-        h[e] = hv;
-        ht[(size_t)j * ldt + b] = hv;
-    }
+    __syncthreads();
+    for (int i = r; i < 64; i += 4)
+        if (j0 + i < n && b0 + c < Bp) xt[(size_t)(j0 + i) * ldt + b0 + c] = tile[c][i];
 }
 
 // y_b = sum_j h[b][j] w[j] + c (one warp per sample)
@@ -99,84 +90,70 @@ __global__ void k_loss(int B, const float* __restrict__ y, const float* __restri
     if (threadIdx.x == 0 && loss) loss[0] = (float)(red[0] / B);
 }
 
-// output layer backward: gw[j] = sum_b dy_b h[b][j], gc = sum_b dy_b (block j),
-// dz[b][j] = dy_b w[j] GELU'(z[b][j]) as bf16 (row-major and transposed),
-// dzf: the same in fp32 for the bias gradient of the layer below
-__global__ void k_out_back_w(int B, int n, const float* __restrict__ dy, const bf16* __restrict__ h,
-                             float* __restrict__ gw, float* __restrict__ gc)
+// output layer backward: dz[b][j] = dy_b w[j] GELU'(z[b][j]) as bf16 (row-major and
+// transposed, columns [B, Bp) zero), dzf: the same in fp32 for the bias gradient
+__global__ void k_out_back_dz(int B, int Bp, int n, const float* __restrict__ dy, const float* __restrict__ w,
+                              const float* __restrict__ z, float* __restrict__ dzf, bf16* __restrict__ dz,
+                              bf16* __restrict__ dzt, int ldt)
+{
+    __shared__ bf16 tile[32][33];
+    const int j0 = blockIdx.x * 32, b0 = blockIdx.y * 32, c = threadIdx.x & 31, r = threadIdx.x >> 5;
+    for (int i = r; i < 32; i += 8) {
+        const int b = b0 + i, j = j0 + c;
+        bf16 vb = __float2bfloat16(0.f);
+        if (b < B && j < n) {
+            const size_t e = (size_t)b * n + j;
+            const float v = dy[b] * w[j] * gelu_d(z[e]);
+            dzf[e] = v;
+            vb = __float2bfloat16(v);
+            dz[e] = vb;
+        }
+        tile[i][c] = vb;
+    }
+    __syncthreads();
+    for (int i = r; i < 32; i += 8)
+        if (j0 + i < n && b0 + c < Bp) dzt[(size_t)(j0 + i) * ldt + b0 + c] = tile[c][i];
+}
+
+// Column sums over the batch (block (j, l), fixed order): l < 3 the bias gradients
+// g[l][j] = sum_b a[l][b][j]; l = 3 the output layer's gw[j] = sum_b dy_b h[b][j], and
+// gc = sum_b dy_b from block j = 0.
+struct SumArgs {
+    const float* a[3];
+    float* g[3];
+    const float* dy;
+    const bf16* h;
+    float *gw, *gc;
+};
+__global__ void k_batch_sums(int B, int n, const __grid_constant__ SumArgs s)
 {
     __shared__ float red[256];
-    const int j = blockIdx.x;
-    float a = 0, c = 0;
-    for (int b = threadIdx.x; b < B; b += blockDim.x) {
-        a += dy[b] * __bfloat162float(h[(size_t)b * n + j]);
-        c += dy[b];
-    }
-    red[threadIdx.x] = a;
-    __syncthreads();
-    for (int o = blockDim.x / 2; o; o >>= 1) {
-        if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) gw[j] = red[0];
-    if (j == 0) {
-        __syncthreads();
-        red[threadIdx.x] = c;
+    const int j = blockIdx.x, l = blockIdx.y;
+    auto tree = [&](float v) {
+        red[threadIdx.x] = v;
         __syncthreads();
         for (int o = blockDim.x / 2; o; o >>= 1) {
             if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
             __syncthreads();
         }
-        if (threadIdx.x == 0) gc[0] = red[0];
+        return red[0];
+    };
+    float v = 0, c = 0;
+    for (int b = threadIdx.x; b < B; b += blockDim.x) {
+        if (l < 3) {
+            v += s.a[l][(size_t)b * n + j];
+        } else {
+            v += s.dy[b] * __bfloat162float(s.h[(size_t)b * n + j]);
+            c += s.dy[b];
+        }
     }
-}
-
-__global__ void k_out_back_dz(int B, int n, const float* __restrict__ dy, const float* __restrict__ w,
-                              const float* __restrict__ z, float* __restrict__ dzf, bf16* __restrict__ dz,
-                              bf16* __restrict__ dzt, int ldt)
-{
-    const long long total = (long long)B * n;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
-         e += (long long)gridDim.x * blockDim.x) {
-        const int b = (int)(e / n), j = (int)(e % n);
-        const float v = dy[b] * w[j] * gelu_d(z[e]);
-        dzf[e] = v;
-        const bf16 vb = __float2bfloat16(v);
-        dz[e] = vb;
-        dzt[(size_t)j * ldt + b] = vb;
-    }
-}
-
-// hidden backward: dz = dh * GELU'(z) with dh = (dz_above W_above) from the GEMM
-__global__ void k_gelu_back(int B, int n, const float* __restrict__ dh, const float* __restrict__ z,
-                            float* __restrict__ dzf, bf16* __restrict__ dz, bf16* __restrict__ dzt, int ldt)
-{
-    const long long total = (long long)B * n;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
-         e += (long long)gridDim.x * blockDim.x) {
-        const int b = (int)(e / n), j = (int)(e % n);
-        const float v = dh[e] * gelu_d(z[e]);
-        dzf[e] = v;
-        const bf16 vb = __float2bfloat16(v);
-        dz[e] = vb;
-        dzt[(size_t)j * ldt + b] = vb;
-    }
-}
-
-// column sums: g[j] = sum_b a[b][j] (block j, fixed order)
-__global__ void k_colsum(int B, int n, const float* __restrict__ a, float* __restrict__ g)
-{
-    __shared__ float red[256];
-    const int j = blockIdx.x;
-    float s = 0;
-    for (int b = threadIdx.x; b < B; b += blockDim.x) s += a[(size_t)b * n + j];
-    red[threadIdx.x] = s;
-    __syncthreads();
-    for (int o = blockDim.x / 2; o; o >>= 1) {
-        if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
+    v = tree(v);
+    if (threadIdx.x == 0) (l < 3 ? s.g[l] : s.gw)[j] = v;
+    if (l == 3 && j == 0) {
         __syncthreads();
+        c = tree(c);
+        if (threadIdx.x == 0) s.gc[0] = c;
     }
-    if (threadIdx.x == 0) g[j] = red[0];
 }
 
 // Adam (Kingma & Ba) on FP32 master parameters
@@ -206,8 +183,6 @@ __global__ void k_weights_bf16(int out, int in, const float* __restrict__ w, bf1
         wt[(size_t)i * out + o] = v;
     }
 }
-
-// rows x cols fp32 GEMM result -> in place add? (not needed)
 
 }  // namespace
 
@@ -280,7 +255,7 @@ struct msd_mlp {
     bf16 *xb = nullptr, *xt = nullptr;
     float* z[3] = {};
     bf16 *h[3] = {}, *ht[3] = {};
-    float *dzf[3] = {}, *dh = nullptr, *y = nullptr, *dy = nullptr, *acc = nullptr;
+    float *dzf[3] = {}, *y = nullptr, *dy = nullptr;
     bf16 *dz[3] = {}, *dzt[3] = {};
     unsigned* d_err = nullptr;
     long long step = 0;
@@ -308,7 +283,7 @@ int mfail(msd_mlp* m, int code, const char* fmt, ...)
 
 void mfree(msd_mlp* m)
 {
-    cudaFree(m->xb); cudaFree(m->xt); cudaFree(m->dh); cudaFree(m->y); cudaFree(m->dy); cudaFree(m->acc);
+    cudaFree(m->xb); cudaFree(m->xt); cudaFree(m->y); cudaFree(m->dy);
     for (int l = 0; l < 3; ++l) {
         cudaFree(m->z[l]); cudaFree(m->h[l]); cudaFree(m->ht[l]); cudaFree(m->dzf[l]); cudaFree(m->dz[l]);
         cudaFree(m->dzt[l]);
@@ -316,7 +291,7 @@ void mfree(msd_mlp* m)
         m->h[l] = m->ht[l] = m->dz[l] = m->dzt[l] = nullptr;
     }
     m->xb = m->xt = nullptr;
-    m->dh = m->y = m->dy = m->acc = nullptr;
+    m->y = m->dy = nullptr;
     m->cap = m->capt = 0;
 }
 
@@ -337,10 +312,8 @@ int ensure_batch(msd_mlp* m, int B)
         MCK(cudaMalloc(&m->dz[l], sizeof(bf16) * cap * W));
         MCK(cudaMalloc(&m->dzt[l], sizeof(bf16) * cap * W));
     }
-    MCK(cudaMalloc(&m->dh, sizeof(float) * cap * W));
     MCK(cudaMalloc(&m->y, sizeof(float) * cap));
     MCK(cudaMalloc(&m->dy, sizeof(float) * cap));
-    MCK(cudaMalloc(&m->acc, sizeof(float) * (size_t)cap * (W > m->n_in ? W : m->n_in)));
     return MSD_OK;
 }
 
@@ -360,21 +333,18 @@ int forward(msd_mlp* m, int B, const float* x, cudaStream_t st)
 {
     int rc = ensure_batch(m, B);
     if (rc) return rc;
-    const int W = m->width, ld = m->capt;
-    // transposed copies: columns beyond B stay zero (they are the K padding
-    // of the weight-gradient products)
-    MCK(cudaMemsetAsync(m->xt, 0, sizeof(bf16) * (size_t)ld * m->n_in, st));
-    for (int l = 0; l < 3; ++l) MCK(cudaMemsetAsync(m->ht[l], 0, sizeof(bf16) * (size_t)ld * W, st));
-    k_in_bf16<<<grid_of((long long)B * m->n_in), 256, 0, st>>>(B, m->n_in, x, m->xb, m->xt, ld);
+    const int W = m->width, ld = m->capt, Bp = (B + 63) / 64 * 64;
+    k_in_bf16<<<dim3((m->n_in + 63) / 64, Bp / 64), 256, 0, st>>>(B, Bp, m->n_in, x, m->xb, m->xt, ld);
     msd_note_launch();
     const bf16* in = m->xb;
     int K = m->n_in;
     for (int l = 0; l < 3; ++l) {
-        if (tc_gemm_bf16(in, K, m->wb[l], K, B, W, K, m->z[l], W, m->d_err, st))
+        NetEpi ep;
+        ep.bias = m->p + m->off_b[l];
+        ep.h = m->h[l]; ep.ht = m->ht[l];
+        ep.ldt = ld; ep.Bp = Bp;
+        if (tc_gemm_bf16(in, K, m->wb[l], K, B, W, K, m->z[l], W, m->d_err, st, 1, &ep))
             return mfail(m, MSD_ERR_CUDA, "tensor-core GEMM launch failed (forward layer %d)", l);
-        k_bias_gelu<<<grid_of((long long)B * W), 256, 0, st>>>(B, W, m->z[l], m->p + m->off_b[l], m->h[l], m->ht[l],
-                                                                ld);
-        msd_note_launch();
         in = m->h[l];
         K = W;
     }
@@ -480,32 +450,34 @@ int msd_mlp_grad(msd_mlp* m, int batch, const float* x, const float* target, flo
     MCK(cudaSetDevice(m->device));
     int rc = forward(m, batch, x, st);
     if (rc) return rc;
-    const int B = batch, W = m->width, ld = m->capt;
+    const int B = batch, W = m->width, ld = m->capt, Bp = (B + 63) / 64 * 64;
     k_loss<<<1, 1024, 0, st>>>(B, m->y, target, m->dy, loss);
     msd_note_launch();
     // output layer
-    k_out_back_w<<<W, 256, 0, st>>>(B, W, m->dy, m->h[2], m->g + m->off_w[3], m->g + m->off_b[3]);
-    msd_note_launch();
-    for (int l = 0; l < 3; ++l) MCK(cudaMemsetAsync(m->dzt[l], 0, sizeof(bf16) * (size_t)ld * W, st));
-    k_out_back_dz<<<grid_of((long long)B * W), 256, 0, st>>>(B, W, m->dy, m->p + m->off_w[3], m->z[2], m->dzf[2],
-                                                             m->dz[2], m->dzt[2], ld);
+    k_out_back_dz<<<dim3((W + 31) / 32, Bp / 32), 256, 0, st>>>(B, Bp, W, m->dy, m->p + m->off_w[3], m->z[2], m->dzf[2],
+                                                                m->dz[2], m->dzt[2], ld);
     msd_note_launch();
     for (int l = 2; l >= 0; --l) {
         const int in = l ? W : m->n_in;
         // dW_l[n][k] = sum_b dz_l[b][n] a_l[b][k]: K = batch (padded columns are zero)
         const bf16* at = l ? m->ht[l - 1] : m->xt;
-        if (tc_gemm_bf16(m->dzt[l], ld, at, ld, W, in, ld, m->g + m->off_w[l], in, m->d_err, st))
+        if (tc_gemm_bf16(m->dzt[l], ld, at, ld, W, in, Bp, m->g + m->off_w[l], in, m->d_err, st))
             return mfail(m, MSD_ERR_CUDA, "tensor-core GEMM launch failed (weight gradient %d)", l);
-        k_colsum<<<W, 256, 0, st>>>(B, W, m->dzf[l], m->g + m->off_b[l]);
-        msd_note_launch();
         if (l == 0) break;
-        // dh_{l-1}[b][k] = sum_n dz_l[b][n] W_l[n][k]
-        if (tc_gemm_bf16(m->dz[l], W, m->wt[l], W, B, W, W, m->dh, W, m->d_err, st))
+        // dz_{l-1}[b][k] = (sum_n dz_l[b][n] W_l[n][k]) GELU'(z_{l-1}[b][k])
+        NetEpi ep;
+        ep.zin = m->z[l - 1];
+        ep.h = m->dz[l - 1]; ep.ht = m->dzt[l - 1];
+        ep.ldt = ld; ep.Bp = Bp;
+        if (tc_gemm_bf16(m->dz[l], W, m->wt[l], W, B, W, W, m->dzf[l - 1], W, m->d_err, st, 2, &ep))
             return mfail(m, MSD_ERR_CUDA, "tensor-core GEMM launch failed (input gradient %d)", l);
-        k_gelu_back<<<grid_of((long long)B * W), 256, 0, st>>>(B, W, m->dh, m->z[l - 1], m->dzf[l - 1], m->dz[l - 1],
-                                                               m->dzt[l - 1], ld);
-        msd_note_launch();
     }
+    SumArgs sums;
+    for (int l = 0; l < 3; ++l) { sums.a[l] = m->dzf[l]; sums.g[l] = m->g + m->off_b[l]; }
+    sums.dy = m->dy; sums.h = m->h[2];
+    sums.gw = m->g + m->off_w[3]; sums.gc = m->g + m->off_b[3];
+    k_batch_sums<<<dim3(W, 4), 256, 0, st>>>(B, W, sums);
+    msd_note_launch();
     MCK(cudaGetLastError());
     if (grads) MCK(cudaMemcpyAsync(grads, m->g, sizeof(float) * m->n_params, cudaMemcpyDeviceToDevice, st));
     return MSD_OK;

@@ -12,6 +12,7 @@
 // wait is bounded (about 2 s of wall clock); on expiry the kernel records
 // MSD_DEV_ERR_TIMEOUT, drains what it issued and releases its TMEM.
 #include <cuda.h>
+#include <cuda_bf16.h>
 #include <cudaTypedefs.h>
 
 #include <cstdint>
@@ -26,12 +27,18 @@ using namespace tcx;
 // SPLIT: 3xTF32 (hi/lo operands, three products per K step) or a single
 // BF16 product. One k-block is 128 bytes of K per row in both cases
 // (32 FP32 or 64 BF16 elements); one MMA covers 32 bytes of K.
+__device__ __forceinline__ float net_gelu(float z) { return 0.5f * z * (1.f + erff(z * 0.70710678118654752f)); }
+__device__ __forceinline__ float net_gelu_d(float z)
+{
+    return 0.5f * (1.f + erff(z * 0.70710678118654752f)) + z * 0.39894228040143268f * expf(-0.5f * z * z);
+}
+
 template <int BN, bool SPLIT>
 struct TcCfg {
     static constexpr int BM = 128;
     static constexpr int BK = SPLIT ? 32 : 64;   // elements per k-block
     static constexpr int NOPS = SPLIT ? 2 : 1;   // hi/lo copies of each operand
-    static constexpr int STAGES = SPLIT ? (BN >= 256 ? 2 : 3) : (BN >= 256 ? 4 : 6);
+    static constexpr int STAGES = SPLIT ? (BN >= 256 ? 2 : 3) : (BN >= 256 ? 4 : BN >= 128 ? 6 : 8);
     static constexpr uint32_t A_BYTES = BM * 128;
     static constexpr uint32_t B_BYTES = BN * 128;
     static constexpr uint32_t STAGE_BYTES = NOPS * (A_BYTES + B_BYTES);
@@ -39,12 +46,19 @@ struct TcCfg {
     static constexpr size_t SMEM = (size_t)STAGES * STAGE_BYTES + 1024;
 };
 
-template <int BN, bool SPLIT>
-__global__ void __launch_bounds__(128, 1)
+// EPI: what becomes of the products v[row][n] (rows < Mr):
+//   0  C = v
+//   1  z = v + bias[n] (to C), h = GELU(z) in BF16, row-major and transposed
+//   2  v GELU'(zin[row][n]) (to C in FP32), the same in BF16, row-major and transposed
+// (the BF16 network's layers; transposed rows in [Mr, Bp) are written as zeros).
+// With an epilogue eight warps share it (halves of the columns; its erff and expf
+// on four warps took longer than the products).
+template <int BN, bool SPLIT, int EPI = 0>
+__global__ void __launch_bounds__(EPI ? 256 : 128, 1)
 k_tc_gemm(const __grid_constant__ CUtensorMap ta_hi, const __grid_constant__ CUtensorMap ta_lo,
           const __grid_constant__ CUtensorMap tb_hi, const __grid_constant__ CUtensorMap tb_lo,
           int Mr, int Nc, int K, float* __restrict__ C, long long ldc, long long c_split_stride,
-          unsigned* err)
+          unsigned* err, const __grid_constant__ NetEpi ep)
 {
     using Cfg = TcCfg<BN, SPLIT>;
     constexpr int BM = Cfg::BM, BK = Cfg::BK, STAGES = Cfg::STAGES;
@@ -146,10 +160,40 @@ k_tc_gemm(const __grid_constant__ CUtensorMap ta_hi, const __grid_constant__ CUt
     const bool ok = __all_sync(0xffffffffu, mbar_wait(&done_bar, 0, wb) ? 1 : 0);
     tc_fence_after();
     if (ok && !fail) {
-        const int row = m0 + warp * 32 + lane;
-        for (int c = 0; c < BN; c += 16) {
+        const int q = warp & 3, row = m0 + q * 32 + lane;
+        const int cb = EPI ? (warp >> 2) * (BN / 2) : 0, ce = EPI ? cb + BN / 2 : BN;
+        for (int c = cb; c < ce; c += 16) {
             float v[16];
-            tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c, v);
+            tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c, v);
+            if constexpr (EPI != 0) {
+                // n0 + c + 16 <= Nc always: the network's widths are multiples of 64
+                __align__(16) __nv_bfloat16 hv[16];
+                if (row < Mr) {
+                    const float* s = EPI == 1 ? ep.bias + n0 + c : ep.zin + (size_t)row * ldc + n0 + c;
+#pragma unroll
+                    for (int i = 0; i < 16; i += 4) {
+                        const float4 f = EPI == 1 ? make_float4(s[i], s[i + 1], s[i + 2], s[i + 3])
+                                                  : *reinterpret_cast<const float4*>(s + i);
+                        const float g[4] = {f.x, f.y, f.z, f.w};
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            float& x = v[i + k];
+                            x = EPI == 1 ? x + g[k] : x * net_gelu_d(g[k]);
+                            hv[i + k] = __float2bfloat16(EPI == 1 ? net_gelu(x) : x);
+                        }
+                    }
+                    uint4* h = reinterpret_cast<uint4*>(ep.h + (size_t)row * ldc + n0 + c);
+                    h[0] = reinterpret_cast<const uint4*>(hv)[0];
+                    h[1] = reinterpret_cast<const uint4*>(hv)[1];
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) hv[i] = __float2bfloat16(0.f);
+                }
+                if (row < ep.Bp) {   // lanes: consecutive rows
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) ep.ht[(size_t)(n0 + c + i) * ep.ldt + row] = hv[i];
+                }
+            }
             if (row < Mr) {
                 float* dst = C + (size_t)row * ldc + n0 + c;
                 if (n0 + c + 16 <= Nc && ((uintptr_t)dst & 15) == 0) {
@@ -229,10 +273,10 @@ int make_map(CUtensorMap* map, const void* base, int inner, int outer, long long
     return tc_make_map(map, base, inner, outer, ld, box_outer, bf16);
 }
 
-template <int BN, bool SPLIT>
+template <int BN, bool SPLIT, int EPI = 0>
 int launch_bn(const void* a_hi, const void* a_lo, long long lda, const void* b_hi, const void* b_lo, long long ldb,
               int Mr, int Nc, int K, float* C, long long ldc, int splits, long long c_split_stride, unsigned* err,
-              cudaStream_t st)
+              cudaStream_t st, const NetEpi& ep = NetEpi())
 {
     CUtensorMap ah, al, bh, bl;
     if (make_map(&ah, a_hi, K, Mr, lda, 128, !SPLIT) || make_map(&bh, b_hi, K, Nc, ldb, BN, !SPLIT)) return -1;
@@ -245,13 +289,13 @@ int launch_bn(const void* a_hi, const void* a_lo, long long lda, const void* b_h
     using Cfg = TcCfg<BN, SPLIT>;
     static bool attr = false;
     if (!attr) {
-        if (cudaFuncSetAttribute(k_tc_gemm<BN, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        if (cudaFuncSetAttribute(k_tc_gemm<BN, SPLIT, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)Cfg::SMEM) != cudaSuccess)
             return -1;
         attr = true;
     }
     dim3 grid((Nc + BN - 1) / BN, (Mr + 127) / 128, splits);
-    k_tc_gemm<BN, SPLIT><<<grid, 128, Cfg::SMEM, st>>>(ah, al, bh, bl, Mr, Nc, K, C, ldc, c_split_stride, err);
+    k_tc_gemm<BN, SPLIT, EPI><<<grid, EPI ? 256 : 128, Cfg::SMEM, st>>>(ah, al, bh, bl, Mr, Nc, K, C, ldc, c_split_stride, err, ep);
     msd_note_launch();
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
@@ -383,12 +427,32 @@ int tc_gemm_3xtf32(const TcOperand& A, const TcOperand& B, int Mr, int Nc, int K
     return -1;
 }
 
+namespace {
+template <int EPI>
+int gemm_bf16(const void* A, long long lda, const void* B, long long ldb, int Mr, int Nc, int K, float* C, long long ldc,
+              unsigned* err, cudaStream_t st, const NetEpi& ep)
+{
+    // the widest tile that still fills half the GPU, else the narrowest: the
+    // network's products have few tiles and a long contraction (512 x 256 x 6912:
+    // 4 tiles of 256 columns took 44 us, 16 of 64 columns 28 with the epilogue). A tile's width
+    // does not change an output's order of accumulation.
+    if (EPI && (Nc % 64 || ldc % 8)) return -1;
+    const int rt = (Mr + 127) / 128, half = msd_sm_count() / 2;
+    if (rt * ((Nc + 255) / 256) >= half && !(EPI && Nc % 256))
+        return launch_bn<256, false, EPI>(A, nullptr, lda, B, nullptr, ldb, Mr, Nc, K, C, ldc, 1, 0, err, st, ep);
+    if (rt * ((Nc + 127) / 128) >= half && !(EPI && Nc % 128))
+        return launch_bn<128, false, EPI>(A, nullptr, lda, B, nullptr, ldb, Mr, Nc, K, C, ldc, 1, 0, err, st, ep);
+    return launch_bn<64, false, EPI>(A, nullptr, lda, B, nullptr, ldb, Mr, Nc, K, C, ldc, 1, 0, err, st, ep);
+}
+}  // namespace
+
 int tc_gemm_bf16(const void* A, long long lda, const void* B, long long ldb, int Mr, int Nc, int K, float* C,
-                 long long ldc, unsigned* err, cudaStream_t st)
+                 long long ldc, unsigned* err, cudaStream_t st, int epi, const NetEpi* ep)
 {
     if (K <= 0 || K % 64 || lda % 8 || ldb % 8 || Mr <= 0 || Nc <= 0) return -1;
-    if (Nc > 128) return launch_bn<256, false>(A, nullptr, lda, B, nullptr, ldb, Mr, Nc, K, C, ldc, 1, 0, err, st);
-    return launch_bn<128, false>(A, nullptr, lda, B, nullptr, ldb, Mr, Nc, K, C, ldc, 1, 0, err, st);
+    if (epi == 1) return gemm_bf16<1>(A, lda, B, ldb, Mr, Nc, K, C, ldc, err, st, *ep);
+    if (epi == 2) return gemm_bf16<2>(A, lda, B, ldb, Mr, Nc, K, C, ldc, err, st, *ep);
+    return gemm_bf16<0>(A, lda, B, ldb, Mr, Nc, K, C, ldc, err, st, NetEpi());
 }
 
 void launch_split_complex_rows(int nb, int R, int Kg, int Kp, const double2* src, long long src_ld,
