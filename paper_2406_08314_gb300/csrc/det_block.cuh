@@ -1,0 +1,222 @@
+// The per-determinant energy terms as a block of the per-system kernels (k_energy.cu,
+// k_pair.cu) and of the persistent batched kernel (k_batch.cu) evaluates them: the
+// walker's tables in shared memory and one string's or determinant's term, in FP32
+// (mixed mode) or, in FP64 mode, with the long sums in the two-limb fixed point of
+// fixed.cuh.
+#pragma once
+
+#include <type_traits>
+
+#include "det_terms.cuh"
+#include "fixed.cuh"
+
+// The walker's K^{ab} in shared memory: FP32 entries, or in FP64 mode limbs of
+// fixed.cuh (the same 16 bytes) with their exponent.
+template <typename T>
+struct PairK { const cplx_t<T>* k; };
+template <>
+struct PairK<double> { const Limbs* k; int e; };
+
+template <typename T>
+__device__ __forceinline__ PairK<T> load_pair_k(const void* Kin, int w, int XX, unsigned char* sm)
+{
+    const cplx_t<T>* Kw = reinterpret_cast<const cplx_t<T>*>(Kin) + (size_t)w * XX;
+    cplx_t<T>* ks = reinterpret_cast<cplx_t<T>*>(sm);
+    if constexpr (std::is_same<T, float>::value) {
+        for (int e = threadIdx.x; e < XX; e += blockDim.x) ks[e] = Kw[e];
+        __syncthreads();
+        return {ks};
+    } else {
+        __shared__ unsigned wm[PC_THREADS / 32];
+        unsigned m = 0;
+        for (int e = threadIdx.x; e < XX; e += blockDim.x) {
+            const double2 v = Kw[e];
+            ks[e] = v;
+            m = max(m, mag_bits(v));
+        }
+        const int ex = mag_exponent(block_mag(m, wm));
+        Limbs* l = reinterpret_cast<Limbs*>(sm);
+        for (int e = threadIdx.x; e < XX; e += blockDim.x) l[e] = to_limbs(ks[e], ex);   // its own entries
+        __syncthreads();
+        return {l, ex};
+    }
+}
+
+// FP64 mode: c_I r_a r_b X_ab with the sum over the entries of the longer string's
+// minor in fixed point (scales: K, and the string's largest entry) and the sum over
+// the shorter one's in FP64. The FP64 unit bounds the plain double sum, 4 k_a^2
+// k_b^2 FMAs: (3, 3) determinants 360 FP64 operations, here 52 and 972 mad.wide.
+template <int KA, int KB>
+__device__ __forceinline__ double2 pair_term_fixed(const SpinTables& ta, const SpinTables& tbb, const PairTables& pt,
+                                                   int I, int w, const void* __restrict__ Ba_in,
+                                                   const void* __restrict__ Bb_in, const PairK<double>& kk,
+                                                   const double2* __restrict__ ra, const double2* __restrict__ rb)
+{
+    constexpr bool INB = KB >= KA;
+    constexpr int KI = INB ? KB : KA, KO = INB ? KA : KB;
+    const int Xb = tbb.nh * tbb.np, a = pt.a[I], b = pt.b[I];
+    const int nsa = ta.bucket[KA + 1] - ta.bucket[KA], nsb = tbb.bucket[KB + 1] - tbb.bucket[KB];
+    const double2* Ba = reinterpret_cast<const double2*>(Ba_in) + (size_t)ta.b_off[KA] +
+                        ((size_t)w * nsa + a - ta.bucket[KA]) * b_stride(KA);
+    const double2* Bb = reinterpret_cast<const double2*>(Bb_in) + (size_t)tbb.b_off[KB] +
+                        ((size_t)w * nsb + b - tbb.bucket[KB]) * b_stride(KB);
+    const double2 *Bi = INB ? Bb : Ba, *Bo = INB ? Ba : Bb;
+    const uint4 ri = INB ? tbb.str_hp[b] : ta.str_hp[a], ro = INB ? ta.str_hp[a] : tbb.str_hp[b];
+    const int npi = INB ? tbb.np : ta.np, npo = INB ? ta.np : tbb.np, si = INB ? 1 : Xb, so = INB ? Xb : 1;
+    const double2 rav = ra[(size_t)w * ta.n_str + a], rbv = rb[(size_t)w * tbb.n_str + b];
+    Limbs bi[KI * KI];
+    int xi[KI * KI], eb;
+    {
+        double2 v[KI * KI];
+        unsigned m = 0;
+#pragma unroll
+        for (int e = 0; e < KI * KI; ++e) { v[e] = Bi[e]; m = max(m, mag_bits(v[e])); }
+        eb = mag_exponent(m);
+#pragma unroll
+        for (int e = 0; e < KI * KI; ++e) {
+            bi[e] = to_limbs(v[e], eb);
+            xi[e] = (rec_h(ri, e % KI) * npi + rec_p(ri, e / KI)) * si;
+        }
+    }
+    double xr = 0, xim = 0;
+#pragma unroll
+    for (int e = 0; e < KO * KO; ++e) {
+        const double2 bo = Bo[e];
+        const Limbs* krow = kk.k + (rec_h(ro, e % KO) * npo + rec_p(ro, e / KO)) * so;
+        LimbSum s;
+#pragma unroll
+        for (int q = 0; q < KI * KI; ++q) s.add(bi[q], krow[xi[q]]);
+        const double2 z = limb_value(s, kk.e + eb);
+        xr += bo.x * z.x - bo.y * z.y;
+        xim += bo.x * z.y + bo.y * z.x;
+    }
+    if (max(kk.e, eb) >= FIXED_EXP_INF) xr = xim = __longlong_as_double(0x7ff8000000000000ll);
+    return pair_weight_times<double>(pt, I, rav, rbv, xr, xim);
+}
+
+template <int KA, int KB, typename T>
+__device__ __forceinline__ cplx_t<T> pair_term(const SpinTables& ta, const SpinTables& tbb, const PairTables& pt, int I,
+                                               int w, const void* Ba, const void* Bb, const PairK<T>& kk,
+                                               const cplx_t<T>* ra, const cplx_t<T>* rb)
+{
+    if constexpr (std::is_same<T, float>::value)
+        return pair_cross_term2<KA, KB, T>(ta, tbb, pt, I, w, Ba, Bb, kk.k, ra, rb);
+    else
+        return pair_term_fixed<KA, KB>(ta, tbb, pt, I, w, Ba, Bb, kk, ra, rb);
+}
+
+// FP64 mode, levels 1 to 5: e_s of string_energy_value with the sums over the pair
+// table and over Y in fixed point (the FP64 unit bounds the plain form: level 4, 496
+// FP64 operations per string; here 48 and 1056 mad.wide):
+//   e_s = sum_ij b_ij Y[h_j][p_i] + sum_{i < k-1} sum_j b_ij z_ij,
+//   z_ij = sum_{m > i} sum_{l != j} (+ for l > j, - for l < j) b_ml A[h_j,h_l;p_i,p_m].
+// Scales: A, Y per walker (exponents ea, ey), b the string's largest entry.
+template <int KL>
+__device__ __forceinline__ double2 string_energy_fixed(const SpinTables& tb, int w, int sl, int ns, const void* Bin,
+                                                       const Limbs* as, int ea, const Limbs* ys, int ey)
+{
+    const int np = tb.np, nh = tb.nh, npp = np * (np - 1) / 2;
+    const uint4 rec = tb.str_hp[tb.bucket[KL] + sl];
+    const double2* B = reinterpret_cast<const double2*>(Bin) + (size_t)tb.b_off[KL] + ((size_t)w * ns + sl) * b_stride(KL);
+    Limbs b[KL * KL];
+    int eb;
+    {
+        unsigned m = 0;
+#pragma unroll
+        for (int e = 0; e < KL * KL; ++e) m = max(m, mag_bits(B[e]));
+        eb = mag_exponent(m);
+#pragma unroll
+        for (int e = 0; e < KL * KL; ++e) b[e] = to_limbs(B[e], eb);
+    }
+    LimbSum lin;
+#pragma unroll
+    for (int i = 0; i < KL; ++i)
+#pragma unroll
+        for (int j = 0; j < KL; ++j) lin.add(b[i * KL + j], ys[rec_h(rec, j) * np + rec_p(rec, i)]);
+    double2 v = limb_value(lin, eb + ey);
+#pragma unroll
+    for (int i = 0; i + 1 < KL; ++i)
+#pragma unroll
+        for (int j = 0; j < KL; ++j) {
+            LimbSum z;
+#pragma unroll
+            for (int m = i + 1; m < KL; ++m) {
+                const int pim = pair_index(rec_p(rec, i), rec_p(rec, m), np);
+#pragma unroll
+                for (int l = 0; l < KL; ++l) {
+                    if (l == j) continue;
+                    const int hp = l > j ? pair_index(rec_h(rec, j), rec_h(rec, l), nh)
+                                         : pair_index(rec_h(rec, l), rec_h(rec, j), nh);
+                    if (l > j) z.add(b[m * KL + l], as[hp * npp + pim]);
+                    else z.sub(b[m * KL + l], as[hp * npp + pim]);
+                }
+            }
+            v = cfma(B[i * KL + j], limb_value(z, eb + ea), v);
+        }
+    if (max(max(ea, ey), eb) >= FIXED_EXP_INF) v.x = v.y = __longlong_as_double(0x7ff8000000000000ll);
+    return v;
+}
+
+// The pair table and Y of a block in shared memory, FP32 / FP64, or as limbs with
+// their exponents where string_energy_fixed reads them.
+template <typename T>
+struct SeTab {
+    const cplx_t<T>*as, *ys;
+    int ea, ey;
+};
+#define SE_FIXED_MAX 5
+template <int KL, typename T>
+__device__ __forceinline__ double2 string_energy_any(const SpinTables& tb, int w, int sl, int ns, const void* B,
+                                                     const SeTab<T>& tab, const double2* wts)
+{
+    if constexpr (std::is_same<T, double>::value && KL <= SE_FIXED_MAX) {
+        const double2 e = string_energy_fixed<KL>(tb, w, sl, ns, B, reinterpret_cast<const Limbs*>(tab.as), tab.ea,
+                                                  reinterpret_cast<const Limbs*>(tab.ys), tab.ey);
+        return cmul(wts[(size_t)w * tb.n_str + tb.bucket[KL] + sl], e);   // wts holds r_s w_s
+    } else {
+        return string_energy_term<KL, T, true>(tb, w, sl, ns, B, tab.as, tab.ys, wts);
+    }
+}
+
+// The walker's antisymmetrized pair table A[(h,h')][(p,p')] = K[(h,p)][(h',p')] -
+// K[(h,p')][(h',p)], h < h', p < p' (not used by level 1), and Y, in shared memory
+// for the strings of level k. The block must reach this together.
+template <typename T>
+__device__ __forceinline__ SeTab<T> load_se_table(const SpinTables& tb, const void* Kin, const void* Yin, int w, int k,
+                                                  unsigned char* sm)
+{
+    using T2 = cplx_t<T>;
+    const int X = tb.nh * tb.np, np = tb.np, nh = tb.nh, t = threadIdx.x;
+    const int nhp = nh * (nh - 1) / 2, npp = np * (np - 1) / 2, na = k > 1 ? nhp * npp : 0;
+    T2* as = reinterpret_cast<T2*>(sm);
+    T2* ys = as + nhp * npp;
+    const T2* Kw = reinterpret_cast<const T2*>(Kin) + (size_t)w * X * X;
+    for (int e = t; e < na; e += blockDim.x) {
+        int i = e / npp, c = e - i * npp, h = 0, p = 0;
+        while (i >= nh - 1 - h) { i -= nh - 1 - h; ++h; }
+        while (c >= np - 1 - p) { c -= np - 1 - p; ++p; }
+        const int h2 = h + 1 + i, p2 = p + 1 + c;
+        const T2 kc = Kw[(size_t)(h * np + p) * X + h2 * np + p2];
+        const T2 kx = Kw[(size_t)(h * np + p2) * X + h2 * np + p];
+        as[e] = T2{kc.x - kx.x, kc.y - kx.y};
+    }
+    const T2* Yw = reinterpret_cast<const T2*>(Yin) + (size_t)w * X;
+    for (int e = t; e < X; e += blockDim.x) ys[e] = Yw[e];
+    SeTab<T> tab = {as, ys, 0, 0};
+    if constexpr (std::is_same<T, double>::value) {
+        if (k <= SE_FIXED_MAX) {   // each thread its own entries
+            __shared__ unsigned wm[2][SE_THREADS / 32];
+            unsigned ma = 0, my = 0;
+            for (int e = t; e < na; e += blockDim.x) ma = max(ma, mag_bits(as[e]));
+            for (int e = t; e < X; e += blockDim.x) my = max(my, mag_bits(ys[e]));
+            tab.ea = mag_exponent(block_mag(ma, wm[0]));
+            tab.ey = mag_exponent(block_mag(my, wm[1]));
+            Limbs *la = reinterpret_cast<Limbs*>(as), *ly = reinterpret_cast<Limbs*>(ys);
+            for (int e = t; e < na; e += blockDim.x) la[e] = to_limbs(as[e], tab.ea);
+            for (int e = t; e < X; e += blockDim.x) ly[e] = to_limbs(ys[e], tab.ey);
+        }
+    }
+    __syncthreads();
+    return tab;
+}
+

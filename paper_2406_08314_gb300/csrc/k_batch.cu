@@ -7,59 +7,58 @@
 // exactly what one block of k_string_energy / k_pair_cross computes and
 // writes the same partial-sum slot, so batched and per-system results agree.
 #include "common.cuh"
-#include "det_terms.cuh"
+#include "det_block.cuh"
 #include "kernels.h"
 
-template <typename T>
-__device__ double2 batch_se(const BatchSys& S, const BatchItem& it, int t, const cplx_t<T>* ks,
-                            const cplx_t<T>* ys)
+template <int K, typename T>
+__device__ __forceinline__ double2 batch_se(const BatchSys& S, const BatchItem& it, const SeTab<T>& tab)
 {
     const SpinTables& tb = S.t[it.spin];
-    const int k = it.ka;
-    const int ns = tb.bucket[k + 1] - tb.bucket[k];
+    const int ns = tb.bucket[K + 1] - tb.bucket[K];
     double2 acc = cz(0, 0);
     for (int q = 0; q < SE_PER_THREAD; ++q) {
-        const int sl = it.blk * (SE_THREADS * SE_PER_THREAD) + q * SE_THREADS + t;
+        const int sl = it.blk * (SE_THREADS * SE_PER_THREAD) + q * SE_THREADS + threadIdx.x;
         if (sl >= ns) break;
-        double2 v;
-        switch (k) {
-        case 1: v = string_energy_term<1, T>(tb, it.w, sl, ns, S.B[it.spin], ks, ys, S.wts[it.spin]); break;
-        case 2: v = string_energy_term<2, T>(tb, it.w, sl, ns, S.B[it.spin], ks, ys, S.wts[it.spin]); break;
-        case 3: v = string_energy_term<3, T>(tb, it.w, sl, ns, S.B[it.spin], ks, ys, S.wts[it.spin]); break;
-        case 4: v = string_energy_term<4, T>(tb, it.w, sl, ns, S.B[it.spin], ks, ys, S.wts[it.spin]); break;
-        case 5: v = string_energy_term<5, T>(tb, it.w, sl, ns, S.B[it.spin], ks, ys, S.wts[it.spin]); break;
-        default: v = string_energy_term<6, T>(tb, it.w, sl, ns, S.B[it.spin], ks, ys, S.wts[it.spin]); break;
-        }
-        acc = cadd(acc, v);
+        acc = cadd(acc, string_energy_any<K, T>(tb, it.w, sl, ns, S.B[it.spin], tab, S.wts[it.spin]));
     }
     return acc;
 }
 
-template <typename T>
-__device__ double2 batch_pc(const BatchSys& S, const BatchItem& it, int t, const cplx_t<T>* ks)
+// The opposite-spin term of one block with both levels known at compile time, or
+// (levels adding up to more than 6) by the general form.
+template <int KA, int KB, typename T>
+__device__ __forceinline__ double2 batch_pc(const BatchSys& S, const BatchItem& it, const PairK<T>& ks)
 {
     using T2 = cplx_t<T>;
-    const int idx = it.ka * (MSD_KMAX + 1) + it.kb;
-    const int lo = S.pt.bucket[idx], n = S.pt.bucket[idx + 1] - lo;
+    const int idx = KA * (MSD_KMAX + 1) + KB, lo = S.pt.bucket[idx], n = S.pt.bucket[idx + 1] - lo;
     // the ratios in the working precision, as in the per-system kernels
-    const T2* ra = std::is_same<T, float>::value ? reinterpret_cast<const T2*>(S.rf[0])
-                                                 : reinterpret_cast<const T2*>(S.r[0]);
-    const T2* rb = std::is_same<T, float>::value ? reinterpret_cast<const T2*>(S.rf[1])
-                                                 : reinterpret_cast<const T2*>(S.r[1]);
+    constexpr bool F = std::is_same<T, float>::value;
+    const T2* ra = F ? reinterpret_cast<const T2*>(S.rf[0]) : reinterpret_cast<const T2*>(S.r[0]);
+    const T2* rb = F ? reinterpret_cast<const T2*>(S.rf[1]) : reinterpret_cast<const T2*>(S.r[1]);
     T2 acc = T2{0, 0};
     for (int q = 0; q < PC_PER_THREAD; ++q) {
-        const int i0 = it.blk * (PC_THREADS * PC_PER_THREAD) + q * PC_THREADS + t;
+        const int i0 = it.blk * (PC_THREADS * PC_PER_THREAD) + q * PC_THREADS + threadIdx.x;
         if (i0 >= n) break;
-        const int I = lo + i0;
-        T2 v;
-        switch (it.kb) {
-        case 1: v = pair_cross_term<1, T>(S.t[0], S.t[1], S.pt, it.ka, I, it.w, S.B[0], S.B[1], ks, ra, rb); break;
-        case 2: v = pair_cross_term<2, T>(S.t[0], S.t[1], S.pt, it.ka, I, it.w, S.B[0], S.B[1], ks, ra, rb); break;
-        case 3: v = pair_cross_term<3, T>(S.t[0], S.t[1], S.pt, it.ka, I, it.w, S.B[0], S.B[1], ks, ra, rb); break;
-        case 4: v = pair_cross_term<4, T>(S.t[0], S.t[1], S.pt, it.ka, I, it.w, S.B[0], S.B[1], ks, ra, rb); break;
-        case 5: v = pair_cross_term<5, T>(S.t[0], S.t[1], S.pt, it.ka, I, it.w, S.B[0], S.B[1], ks, ra, rb); break;
-        default: v = pair_cross_term<6, T>(S.t[0], S.t[1], S.pt, it.ka, I, it.w, S.B[0], S.B[1], ks, ra, rb); break;
-        }
+        const T2 v = pair_term<KA, KB, T>(S.t[0], S.t[1], S.pt, lo + i0, it.w, S.B[0], S.B[1], ks, ra, rb);
+        acc.x += v.x;
+        acc.y += v.y;
+    }
+    return cz((double)acc.x, (double)acc.y);
+}
+
+template <int KB, typename T>
+__device__ double2 batch_pc_any(const BatchSys& S, const BatchItem& it, const cplx_t<T>* ks)
+{
+    using T2 = cplx_t<T>;
+    const int idx = it.ka * (MSD_KMAX + 1) + KB, lo = S.pt.bucket[idx], n = S.pt.bucket[idx + 1] - lo;
+    constexpr bool F = std::is_same<T, float>::value;
+    const T2* ra = F ? reinterpret_cast<const T2*>(S.rf[0]) : reinterpret_cast<const T2*>(S.r[0]);
+    const T2* rb = F ? reinterpret_cast<const T2*>(S.rf[1]) : reinterpret_cast<const T2*>(S.r[1]);
+    T2 acc = T2{0, 0};
+    for (int q = 0; q < PC_PER_THREAD; ++q) {
+        const int i0 = it.blk * (PC_THREADS * PC_PER_THREAD) + q * PC_THREADS + threadIdx.x;
+        if (i0 >= n) break;
+        const T2 v = pair_cross_term<KB, T>(S.t[0], S.t[1], S.pt, it.ka, lo + i0, it.w, S.B[0], S.B[1], ks, ra, rb);
         acc.x += v.x;
         acc.y += v.y;
     }
@@ -67,14 +66,14 @@ __device__ double2 batch_pc(const BatchSys& S, const BatchItem& it, int t, const
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256, 2)
+// (the fixed-point sums of the FP64 mode take the registers of a whole SM)
+__global__ void __launch_bounds__(256, sizeof(T) == 8 ? 1 : 2)
 k_det_batched(const BatchSys* __restrict__ systems, const BatchItem* __restrict__ items, int n_items,
               unsigned* __restrict__ counter)
 {
     static_assert(SE_THREADS == 256 && PC_THREADS == 256, "one block shape for both item kinds");
     using T2 = cplx_t<T>;
     extern __shared__ __align__(16) unsigned char smraw[];
-    T2* ks = reinterpret_cast<T2*>(smraw);
     __shared__ BatchItem it;
     __shared__ int cur;
     __shared__ double2 red[256];
@@ -96,21 +95,46 @@ k_det_batched(const BatchSys* __restrict__ systems, const BatchItem* __restrict_
             loaded = it.sys;
             __syncthreads();
         }
-        const int X0 = S.t[0].nh * S.t[0].np, X1 = S.t[1].nh * S.t[1].np;
-        T2* ys = nullptr;
+        double2 v = cz(0, 0);
         if (it.kind == 0) {
-            const int X = it.spin ? X1 : X0;
-            const T2* K = reinterpret_cast<const T2*>(S.K[it.spin]) + (size_t)it.w * X * X;
-            const T2* Y = reinterpret_cast<const T2*>(S.Y[it.spin]) + (size_t)it.w * X;
-            ys = ks + X * X;
-            for (int e = t; e < X * X; e += blockDim.x) ks[e] = K[e];
-            for (int e = t; e < X; e += blockDim.x) ys[e] = Y[e];
+            const SeTab<T> tab = load_se_table<T>(S.t[it.spin], S.K[it.spin], S.Y[it.spin], it.w, it.ka, smraw);
+            switch (it.ka) {
+            case 1: v = batch_se<1, T>(S, it, tab); break;
+            case 2: v = batch_se<2, T>(S, it, tab); break;
+            case 3: v = batch_se<3, T>(S, it, tab); break;
+            case 4: v = batch_se<4, T>(S, it, tab); break;
+            case 5: v = batch_se<5, T>(S, it, tab); break;
+            default: v = batch_se<6, T>(S, it, tab); break;
+            }
         } else {
-            const T2* K = reinterpret_cast<const T2*>(S.K[2]) + (size_t)it.w * X0 * X1;
-            for (int e = t; e < X0 * X1; e += blockDim.x) ks[e] = K[e];
+            const int XX = S.t[0].nh * S.t[0].np * S.t[1].nh * S.t[1].np;
+            if (it.ka + it.kb <= 6) {
+                const PairK<T> ks = load_pair_k<T>(S.K[2], it.w, XX, smraw);
+                switch (it.ka * 8 + it.kb) {
+#define PAIR_CASE(A, B) case A * 8 + B: v = batch_pc<A, B, T>(S, it, ks); break;
+                PAIR_CASE(1, 1) PAIR_CASE(1, 2) PAIR_CASE(1, 3) PAIR_CASE(1, 4) PAIR_CASE(1, 5)
+                PAIR_CASE(2, 1) PAIR_CASE(2, 2) PAIR_CASE(2, 3) PAIR_CASE(2, 4)
+                PAIR_CASE(3, 1) PAIR_CASE(3, 2) PAIR_CASE(3, 3)
+                PAIR_CASE(4, 1) PAIR_CASE(4, 2)
+                PAIR_CASE(5, 1)
+#undef PAIR_CASE
+                }
+            } else {
+                const T2* K = reinterpret_cast<const T2*>(S.K[2]) + (size_t)it.w * XX;
+                T2* ks = reinterpret_cast<T2*>(smraw);
+                for (int e = t; e < XX; e += blockDim.x) ks[e] = K[e];
+                __syncthreads();
+                switch (it.kb) {
+                case 1: v = batch_pc_any<1, T>(S, it, ks); break;
+                case 2: v = batch_pc_any<2, T>(S, it, ks); break;
+                case 3: v = batch_pc_any<3, T>(S, it, ks); break;
+                case 4: v = batch_pc_any<4, T>(S, it, ks); break;
+                case 5: v = batch_pc_any<5, T>(S, it, ks); break;
+                default: v = batch_pc_any<6, T>(S, it, ks); break;
+                }
+            }
         }
-        __syncthreads();
-        red[t] = it.kind == 0 ? batch_se<T>(S, it, t, ks, ys) : batch_pc<T>(S, it, t, ks);
+        red[t] = v;
         __syncthreads();
         for (int o = 128; o; o >>= 1) {
             if (t < o) red[t] = cadd(red[t], red[t + o]);

@@ -17,8 +17,7 @@
 #include <type_traits>
 
 #include "common.cuh"
-#include "det_terms.cuh"
-#include "fixed.cuh"
+#include "det_block.cuh"
 #include "kernels.h"
 
 // ------------------------------------------------------------------------
@@ -507,79 +506,6 @@ struct SeArgs {
     int blk[2][MSD_KMAX + 2];   // first block of each (spin, level)
 };
 
-// FP64 mode, levels 1 to 5: e_s of string_energy_value with the sums over the pair
-// table and over Y in fixed point (the FP64 unit bounds the plain form: level 4, 496
-// FP64 operations per string; here 48 and 1056 mad.wide):
-//   e_s = sum_ij b_ij Y[h_j][p_i] + sum_{i < k-1} sum_j b_ij z_ij,
-//   z_ij = sum_{m > i} sum_{l != j} (+ for l > j, - for l < j) b_ml A[h_j,h_l;p_i,p_m].
-// Scales: A, Y per walker (exponents ea, ey), b the string's largest entry.
-template <int KL>
-__device__ __forceinline__ double2 string_energy_fixed(const SpinTables& tb, int w, int sl, int ns, const void* Bin,
-                                                       const Limbs* as, int ea, const Limbs* ys, int ey)
-{
-    const int np = tb.np, nh = tb.nh, npp = np * (np - 1) / 2;
-    const uint4 rec = tb.str_hp[tb.bucket[KL] + sl];
-    const double2* B = reinterpret_cast<const double2*>(Bin) + (size_t)tb.b_off[KL] + ((size_t)w * ns + sl) * b_stride(KL);
-    Limbs b[KL * KL];
-    int eb;
-    {
-        unsigned m = 0;
-#pragma unroll
-        for (int e = 0; e < KL * KL; ++e) m = max(m, mag_bits(B[e]));
-        eb = mag_exponent(m);
-#pragma unroll
-        for (int e = 0; e < KL * KL; ++e) b[e] = to_limbs(B[e], eb);
-    }
-    LimbSum lin;
-#pragma unroll
-    for (int i = 0; i < KL; ++i)
-#pragma unroll
-        for (int j = 0; j < KL; ++j) lin.add(b[i * KL + j], ys[rec_h(rec, j) * np + rec_p(rec, i)]);
-    double2 v = limb_value(lin, eb + ey);
-#pragma unroll
-    for (int i = 0; i + 1 < KL; ++i)
-#pragma unroll
-        for (int j = 0; j < KL; ++j) {
-            LimbSum z;
-#pragma unroll
-            for (int m = i + 1; m < KL; ++m) {
-                const int pim = pair_index(rec_p(rec, i), rec_p(rec, m), np);
-#pragma unroll
-                for (int l = 0; l < KL; ++l) {
-                    if (l == j) continue;
-                    const int hp = l > j ? pair_index(rec_h(rec, j), rec_h(rec, l), nh)
-                                         : pair_index(rec_h(rec, l), rec_h(rec, j), nh);
-                    if (l > j) z.add(b[m * KL + l], as[hp * npp + pim]);
-                    else z.sub(b[m * KL + l], as[hp * npp + pim]);
-                }
-            }
-            v = cfma(B[i * KL + j], limb_value(z, eb + ea), v);
-        }
-    if (max(max(ea, ey), eb) >= FIXED_EXP_INF) v.x = v.y = __longlong_as_double(0x7ff8000000000000ll);
-    return v;
-}
-
-// The pair table and Y of a block in shared memory, FP32 / FP64, or as limbs with
-// their exponents where string_energy_fixed reads them.
-template <typename T>
-struct SeTab {
-    const cplx_t<T>*as, *ys;
-    int ea, ey;
-};
-#define SE_FIXED_MAX 5
-template <int KL, typename T>
-__device__ __forceinline__ double2 string_energy_any(const SpinTables& tb, int w, int sl, int ns, const void* B,
-                                                     const SeTab<T>& tab, const double2* wts)
-{
-    if constexpr (std::is_same<T, double>::value && KL <= SE_FIXED_MAX) {
-        const double2 e = string_energy_fixed<KL>(tb, w, sl, ns, B, reinterpret_cast<const Limbs*>(tab.as), tab.ea,
-                                                  reinterpret_cast<const Limbs*>(tab.ys), tab.ey);
-        return cmul(wts[(size_t)w * tb.n_str + tb.bucket[KL] + sl], e);   // wts holds r_s w_s
-    } else {
-        return string_energy_term<KL, T, true>(tb, w, sl, ns, B, tab.as, tab.ys, wts);
-    }
-}
-
 template <int KL, typename T>
 __device__ __forceinline__ double2 string_energy_block(const SpinTables& tb, int w, int blk, const void* B,
                                                        const SeTab<T>& tab, const double2* wts)
@@ -598,7 +524,6 @@ template <typename T, int ONLY>
 __global__ void __launch_bounds__(SE_THREADS)
 k_string_energy(const __grid_constant__ SeArgs a, double2* __restrict__ part, int nslot, int slot0)
 {
-    using T2 = cplx_t<T>;
     extern __shared__ __align__(16) unsigned char smraw[];
     // this block among all (spin, level) blocks
     int b = blockIdx.x;
@@ -608,43 +533,11 @@ k_string_energy(const __grid_constant__ SeArgs a, double2* __restrict__ part, in
     }
     const int s = b >= a.blk[1][1];
     const SpinTables& tb = a.t[s];
-    const int X = tb.nh * tb.np, np = tb.np, nh = tb.nh;
-    const int nhp = nh * (nh - 1) / 2, npp = np * (np - 1) / 2;
-    T2* as = reinterpret_cast<T2*>(smraw);   // [C(nh,2)][C(np,2)] antisymmetrized pairs of K
-    T2* ys = as + nhp * npp;                 // [X]
     __shared__ double2 red[SE_THREADS];
     const int w = blockIdx.y, t = threadIdx.x;
     int k = ONLY ? ONLY : 1;
     while (!ONLY && b >= a.blk[s][k + 1]) ++k;
-    const T2* Kw = reinterpret_cast<const T2*>(a.K[s]) + (size_t)w * X * X;
-    // A[(h,h')][(p,p')] = K[(h,p)][(h',p')] - K[(h,p')][(h',p)], h < h', p < p'
-    // (not used by level 1)
-    for (int e = k > 1 ? t : nhp * npp; e < nhp * npp; e += blockDim.x) {
-        int i = e / npp, c = e - i * npp, h = 0, p = 0;
-        while (i >= nh - 1 - h) { i -= nh - 1 - h; ++h; }
-        while (c >= np - 1 - p) { c -= np - 1 - p; ++p; }
-        const int h2 = h + 1 + i, p2 = p + 1 + c;
-        const T2 kc = Kw[(size_t)(h * np + p) * X + h2 * np + p2];
-        const T2 kx = Kw[(size_t)(h * np + p2) * X + h2 * np + p];
-        as[e] = T2{kc.x - kx.x, kc.y - kx.y};
-    }
-    const T2* Yw = reinterpret_cast<const T2*>(a.Y[s]) + (size_t)w * X;
-    for (int e = t; e < X; e += blockDim.x) ys[e] = Yw[e];
-    SeTab<T> tab = {as, ys, 0, 0};
-    if constexpr (std::is_same<T, double>::value) {
-        if (k <= SE_FIXED_MAX) {   // each thread its own entries
-            __shared__ unsigned wm[2][SE_THREADS / 32];
-            unsigned ma = 0, my = 0;
-            for (int e = k > 1 ? t : nhp * npp; e < nhp * npp; e += blockDim.x) ma = max(ma, mag_bits(as[e]));
-            for (int e = t; e < X; e += blockDim.x) my = max(my, mag_bits(ys[e]));
-            tab.ea = mag_exponent(block_mag(ma, wm[0]));
-            tab.ey = mag_exponent(block_mag(my, wm[1]));
-            Limbs *la = reinterpret_cast<Limbs*>(as), *ly = reinterpret_cast<Limbs*>(ys);
-            for (int e = k > 1 ? t : nhp * npp; e < nhp * npp; e += blockDim.x) la[e] = to_limbs(as[e], tab.ea);
-            for (int e = t; e < X; e += blockDim.x) ly[e] = to_limbs(ys[e], tab.ey);
-        }
-    }
-    __syncthreads();
+    const SeTab<T> tab = load_se_table<T>(tb, a.K[s], a.Y[s], w, k, smraw);
     const int blk = b - a.blk[s][k];
     double2 v;
     if constexpr (ONLY > 0) {

@@ -8,104 +8,8 @@
 #include <type_traits>
 
 #include "common.cuh"
-#include "det_terms.cuh"
-#include "fixed.cuh"
+#include "det_block.cuh"
 #include "kernels.h"
-
-// The walker's K^{ab} in shared memory: FP32 entries, or in FP64 mode limbs of
-// fixed.cuh (the same 16 bytes) with their exponent.
-template <typename T>
-struct PairK { const cplx_t<T>* k; };
-template <>
-struct PairK<double> { const Limbs* k; int e; };
-
-template <typename T>
-__device__ __forceinline__ PairK<T> load_pair_k(const void* Kin, int w, int XX, unsigned char* sm)
-{
-    const cplx_t<T>* Kw = reinterpret_cast<const cplx_t<T>*>(Kin) + (size_t)w * XX;
-    cplx_t<T>* ks = reinterpret_cast<cplx_t<T>*>(sm);
-    if constexpr (std::is_same<T, float>::value) {
-        for (int e = threadIdx.x; e < XX; e += blockDim.x) ks[e] = Kw[e];
-        __syncthreads();
-        return {ks};
-    } else {
-        __shared__ unsigned wm[PC_THREADS / 32];
-        unsigned m = 0;
-        for (int e = threadIdx.x; e < XX; e += blockDim.x) {
-            const double2 v = Kw[e];
-            ks[e] = v;
-            m = max(m, mag_bits(v));
-        }
-        const int ex = mag_exponent(block_mag(m, wm));
-        Limbs* l = reinterpret_cast<Limbs*>(sm);
-        for (int e = threadIdx.x; e < XX; e += blockDim.x) l[e] = to_limbs(ks[e], ex);   // its own entries
-        __syncthreads();
-        return {l, ex};
-    }
-}
-
-// FP64 mode: c_I r_a r_b X_ab with the sum over the entries of the longer string's
-// minor in fixed point (scales: K, and the string's largest entry) and the sum over
-// the shorter one's in FP64. The FP64 unit bounds the plain double sum, 4 k_a^2
-// k_b^2 FMAs: (3, 3) determinants 360 FP64 operations, here 52 and 972 mad.wide.
-template <int KA, int KB>
-__device__ __forceinline__ double2 pair_term_fixed(const SpinTables& ta, const SpinTables& tbb, const PairTables& pt,
-                                                   int I, int w, const void* __restrict__ Ba_in,
-                                                   const void* __restrict__ Bb_in, const PairK<double>& kk,
-                                                   const double2* __restrict__ ra, const double2* __restrict__ rb)
-{
-    constexpr bool INB = KB >= KA;
-    constexpr int KI = INB ? KB : KA, KO = INB ? KA : KB;
-    const int Xb = tbb.nh * tbb.np, a = pt.a[I], b = pt.b[I];
-    const int nsa = ta.bucket[KA + 1] - ta.bucket[KA], nsb = tbb.bucket[KB + 1] - tbb.bucket[KB];
-    const double2* Ba = reinterpret_cast<const double2*>(Ba_in) + (size_t)ta.b_off[KA] +
-                        ((size_t)w * nsa + a - ta.bucket[KA]) * b_stride(KA);
-    const double2* Bb = reinterpret_cast<const double2*>(Bb_in) + (size_t)tbb.b_off[KB] +
-                        ((size_t)w * nsb + b - tbb.bucket[KB]) * b_stride(KB);
-    const double2 *Bi = INB ? Bb : Ba, *Bo = INB ? Ba : Bb;
-    const uint4 ri = INB ? tbb.str_hp[b] : ta.str_hp[a], ro = INB ? ta.str_hp[a] : tbb.str_hp[b];
-    const int npi = INB ? tbb.np : ta.np, npo = INB ? ta.np : tbb.np, si = INB ? 1 : Xb, so = INB ? Xb : 1;
-    const double2 rav = ra[(size_t)w * ta.n_str + a], rbv = rb[(size_t)w * tbb.n_str + b];
-    Limbs bi[KI * KI];
-    int xi[KI * KI], eb;
-    {
-        double2 v[KI * KI];
-        unsigned m = 0;
-#pragma unroll
-        for (int e = 0; e < KI * KI; ++e) { v[e] = Bi[e]; m = max(m, mag_bits(v[e])); }
-        eb = mag_exponent(m);
-#pragma unroll
-        for (int e = 0; e < KI * KI; ++e) {
-            bi[e] = to_limbs(v[e], eb);
-            xi[e] = (rec_h(ri, e % KI) * npi + rec_p(ri, e / KI)) * si;
-        }
-    }
-    double xr = 0, xim = 0;
-#pragma unroll
-    for (int e = 0; e < KO * KO; ++e) {
-        const double2 bo = Bo[e];
-        const Limbs* krow = kk.k + (rec_h(ro, e % KO) * npo + rec_p(ro, e / KO)) * so;
-        LimbSum s;
-#pragma unroll
-        for (int q = 0; q < KI * KI; ++q) s.add(bi[q], krow[xi[q]]);
-        const double2 z = limb_value(s, kk.e + eb);
-        xr += bo.x * z.x - bo.y * z.y;
-        xim += bo.x * z.y + bo.y * z.x;
-    }
-    if (max(kk.e, eb) >= FIXED_EXP_INF) xr = xim = __longlong_as_double(0x7ff8000000000000ll);
-    return pair_weight_times<double>(pt, I, rav, rbv, xr, xim);
-}
-
-template <int KA, int KB, typename T>
-__device__ __forceinline__ cplx_t<T> pair_term(const SpinTables& ta, const SpinTables& tbb, const PairTables& pt, int I,
-                                               int w, const void* Ba, const void* Bb, const PairK<T>& kk,
-                                               const cplx_t<T>* ra, const cplx_t<T>* rb)
-{
-    if constexpr (std::is_same<T, float>::value)
-        return pair_cross_term2<KA, KB, T>(ta, tbb, pt, I, w, Ba, Bb, kk.k, ra, rb);
-    else
-        return pair_term_fixed<KA, KB>(ta, tbb, pt, I, w, Ba, Bb, kk, ra, rb);
-}
 
 template <int KA, int KB, typename T>
 __global__ void __launch_bounds__(PC_THREADS)
