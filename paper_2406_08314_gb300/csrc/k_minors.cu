@@ -35,6 +35,7 @@ namespace {
 struct MinorSpin {
     int nh, np, n_str;
     int bucket[MSD_KMAX + 2];
+    int vbucket[MSD_KMAX + 2];   // strings outside the trial, by level (k_adjoint): [vbucket[k], vbucket[k + 1])
     const uint4* str_hp;
     const int8_t* str_sign;
     const int* sub;          // [n_str][MSD_KMAX] (string << 1 | negative), -1 first if one is missing
@@ -68,18 +69,18 @@ __global__ void __launch_bounds__(256) k_minor2(const __grid_constant__ MinorArg
     S.m2[e] = cfms(G(h, p2), G(h2, p), cmul(G(h, p), G(h2, p2)));
 }
 
-// Minors of the strings [bucket[k0], bucket[k1 + 1]); SUBS: through the
-// ratios of the level below where the string has them.
+// Minors of the strings of levels k0 to k1, the trial's and, for k0 = k1, those
+// outside it; subs: through the ratios of the level below where the string has them.
 __global__ void __launch_bounds__(256)
 k_minors(const __grid_constant__ MinorArgs a, int k0, int k1, bool subs, int nw)
 {
     const MinorSpin& S = a.s[blockIdx.y];
-    const int s0 = S.bucket[k0], n = S.bucket[k1 + 1] - s0;
+    const int s0 = S.bucket[k0], n = S.bucket[k1 + 1] - s0, nv = k0 == k1 ? S.vbucket[k0 + 1] - S.vbucket[k0] : 0;
     const long long e = blockIdx.x * 256ll + threadIdx.x;
-    if (e >= (long long)n * nw) return;
-    const int s = s0 + (int)(e / nw), w = (int)(e % nw);
+    if (e >= (long long)(n + nv) * nw) return;
+    const int i = (int)(e / nw), w = (int)(e % nw), s = i < n ? s0 + i : S.vbucket[k0] + i - n;
     int k = k0;
-    while (s >= S.bucket[k + 1]) ++k;
+    while (k < k1 && s >= S.bucket[k + 1]) ++k;
     double2* out = S.rT + (size_t)s * nw + w;
     if (k == 0) { *out = cz(1, 0); return; }
     const int np = S.np, nh = S.nh, npp = np * (np - 1) / 2;
@@ -154,6 +155,7 @@ struct WeightSpin {
     double2* wts;            // [nw][n_str] r_s w_s (may be NULL)
     float2* rf;              // [nw][n_str] r_s in FP32 (may be NULL)
     double2* part;           // [nw][nslot] partial sums over 32 strings (may be NULL)
+    double2* wT;             // [n_str][nw] the sums themselves (may be NULL)
 };
 struct WeightArgs { WeightSpin s[2]; };
 
@@ -193,6 +195,7 @@ __global__ void __launch_bounds__(256) k_weights(const __grid_constant__ WeightA
                 const double c = S.c[i];
                 acc = cz(fma(v.x, c, acc.x), fma(v.y, c, acc.y));
             }
+            if (S.wT) S.wT[(size_t)s * nw + w] = acc;
             r = S.self[(size_t)s * nw + w];
             rw = cmul(r, acc);
         }
@@ -349,13 +352,120 @@ MinorSpin minor_spin(const SpinTables& t, const double2* GT, double2* m2, double
 {
     MinorSpin s;
     s.nh = t.nh; s.np = t.np; s.n_str = t.n_str;
-    for (int k = 0; k < MSD_KMAX + 2; ++k) s.bucket[k] = t.bucket[k];
+    for (int k = 0; k < MSD_KMAX + 2; ++k) { s.bucket[k] = t.bucket[k]; s.vbucket[k] = 0; }
     s.str_hp = t.str_hp; s.str_sign = t.str_sign; s.sub = t.sub;
     s.GT = GT; s.m2 = m2; s.rT = rT;
     return s;
 }
 
+// --------------------------------------------------------------- adjoint
+// Cofactor matrix of the force bias and the density matrix,
+//   Cm[p][h] = sum_s w_s r_s B_s[i][j] at (p_i, h_j) = (p, h)  =  d(sum_s w_s r_s) / dG[h][p],
+// by reverse differentiation of the expansions above, without any inverse minor:
+// with every product r = ... + a b + ... of the forward pass, the adjoint of a gains b
+// times the adjoint of r. A target's users are one list of (value row, adjoint row,
+// sign), so each target is a sum over its list, lanes over the walkers:
+//   out[target] += sum +- V[a] Bv[b]   (a < 0: 1),
+// V = [G | 2 x 2 minors | ratios], Bv = [ratios' adjoints | 2 x 2 minors' adjoints],
+// both [row][nw]. Levels from the highest down, then the 2 x 2 minors, then G, whose
+// few long lists are cut in pieces and the pieces added (one list each: 1.04 ms below).
+// About 8 k FP64 FMAs per string, against 4 k^3 for its inverse minor by LU and k^2
+// scattered additions; memory bound now (16-byte rows of a warp's 32 walkers). 640
+// copper-oxo walkers, strings + cofactors: 3.05 + 1.24 -> 0.53 + 0.65 ms.
+struct AdjSpin {
+    int n0, n1;              // targets of this launch
+    const int* row;          // [target] output row of Bv, or entry of G (last stage)
+    const int* off;          // [target + 1]
+    const int2* ent;         // (a << 1 | negative, b); a = -1: (-2 | negative)
+    const double2* V;
+    double2* Bv;
+    double2* Cm;             // last stage: [nw][np][nh], entry x = h np + p to p nh + h
+    int nh, np;
+};
+struct AdjArgs { AdjSpin s[2]; };
+
+__global__ void __launch_bounds__(256) k_adjoint(const __grid_constant__ AdjArgs args, int nw)
+{
+    const AdjSpin& S = args.s[blockIdx.y];
+    const long long e = blockIdx.x * 256ll + threadIdx.x;
+    if (e >= (long long)(S.n1 - S.n0) * nw) return;
+    const int t = S.n0 + (int)(e / nw), w = (int)(e % nw);
+    double2 acc = cz(0, 0);
+    const int i1 = S.off[t + 1];
+    for (int i = S.off[t]; i < i1; i += 4) {
+        double2 a[4], b[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            if (i + q < i1) {
+                const int2 c = S.ent[i + q];
+                a[q] = c.x >= 0 ? S.V[(size_t)(c.x >> 1) * nw + w] : cz(1, 0);
+                b[q] = S.Bv[(size_t)c.y * nw + w];
+                if (c.x & 1) b[q] = cz(-b[q].x, -b[q].y);
+            } else {
+                a[q] = b[q] = cz(0, 0);
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (i + q < i1) acc = cfma(a[q], b[q], acc);
+    }
+    const int r = S.row[t];
+    if (S.Cm) {
+        const int h = r / S.np, p = r - h * S.np;
+        S.Cm[(size_t)w * S.nh * S.np + p * S.nh + h] = acc;
+    } else {
+        double2* o = S.Bv + (size_t)r * nw + w;
+        *o = cadd(*o, acc);
+    }
+}
+
 }  // namespace
+
+// Ratios of the trial's strings and of the sub-minors outside it.
+void launch_minors_ext(const GradTables g[2], const SpinTables& ta, const SpinTables& tb, int nw, double2* const V[2],
+                       cudaStream_t st)
+{
+    MinorArgs a;
+    const SpinTables* T[2] = {&ta, &tb};
+    for (int s = 0; s < 2; ++s) {
+        double2* m2 = V[s] + (size_t)T[s]->nh * T[s]->np * nw;
+        a.s[s] = minor_spin(*T[s], V[s], m2, m2 + (size_t)g[s].n2 * nw);
+        a.s[s].str_hp = g[s].str_hp; a.s[s].str_sign = g[s].str_sign; a.s[s].sub = g[s].sub;
+        for (int k = 0; k < MSD_KMAX + 2; ++k) a.s[s].vbucket[k] = g[s].vbucket[k];
+    }
+    auto blocks = [&](long long n) { return dim3((unsigned)((n * nw + 255) / 256), 2); };
+    k_minor2<<<blocks(std::max(1, std::max(g[0].n2, g[1].n2))), 256, 0, st>>>(a, nw);
+    msd_note_launch();
+    auto count = [&](int s, int k) {
+        return T[s]->bucket[k + 1] - T[s]->bucket[k] + g[s].vbucket[k + 1] - g[s].vbucket[k];
+    };
+    k_minors<<<blocks(std::max(ta.bucket[3], tb.bucket[3])), 256, 0, st>>>(a, 0, 2, false, nw);
+    msd_note_launch();
+    for (int k = 3; k <= MSD_KMAX; ++k) {
+        const int n = std::max(count(0, k), count(1, k));
+        if (n <= 0) continue;
+        k_minors<<<blocks(n), 256, 0, st>>>(a, k, k, true, nw);
+        msd_note_launch();
+    }
+}
+
+void launch_adjoint(const GradTables g[2], const SpinTables& ta, const SpinTables& tb, int nw, double2* const V[2],
+                    double2* const Bv[2], double2* const Cm[2], cudaStream_t st)
+{
+    const SpinTables* T[2] = {&ta, &tb};
+    for (int q = 0; q < GRAD_STAGES; ++q) {
+        AdjArgs a;
+        int n = 0;
+        for (int s = 0; s < 2; ++s) {
+            a.s[s] = AdjSpin{g[s].stage[q], g[s].stage[q + 1], g[s].row, g[s].off, g[s].ent, V[s], Bv[s],
+                             q == GRAD_STAGES - 1 ? Cm[s] : nullptr, T[s]->nh, T[s]->np};
+            n = std::max(n, g[s].stage[q + 1] - g[s].stage[q]);
+        }
+        if (n <= 0) continue;
+        k_adjoint<<<dim3((unsigned)(((long long)n * nw + 255) / 256), 2), 256, 0, st>>>(a, nw);
+        msd_note_launch();
+    }
+}
 
 size_t minor2_count(const SpinTables& t)
 {
@@ -411,10 +521,10 @@ int weights_blocks(const SpinTables& tb) { return (tb.n_str + WT_S - 1) / WT_S; 
 
 // wts, rf: per spin, NULL where not wanted; beta = false: the alpha sums alone.
 void launch_weights(const SpinTables& ta, const SpinTables& tb, int nw, double2* const rT[2], double2* const wts[2],
-                    float2* const rf[2], double2* part, int nslot, bool beta, cudaStream_t st)
+                    float2* const rf[2], double2* part, int nslot, bool beta, cudaStream_t st, double2* const wT[2])
 {
-    const WeightArgs a = {{{ta.n_str, ta.csr_off, ta.csr_other, ta.csr_c, rT[0], rT[1], wts[0], rf[0], part},
-                          {tb.n_str, tb.csr_off, tb.csr_other, tb.csr_c, rT[1], rT[0], wts[1], rf[1], nullptr}}};
+    const WeightArgs a = {{{ta.n_str, ta.csr_off, ta.csr_other, ta.csr_c, rT[0], rT[1], wts[0], rf[0], part, wT ? wT[0] : nullptr},
+                          {tb.n_str, tb.csr_off, tb.csr_other, tb.csr_c, rT[1], rT[0], wts[1], rf[1], nullptr, wT ? wT[1] : nullptr}}};
     const int tiles = (nw + 31) / 32, wt = (nw + tiles - 1) / tiles;   // walkers per tile, evenly
     const int nb = beta ? std::max(weights_blocks(ta), weights_blocks(tb)) : weights_blocks(ta);
     k_weights<<<dim3(nb, tiles, beta ? 2 : 1), 256, 0, st>>>(a, nw, wt, nslot);

@@ -43,7 +43,30 @@ void launch_inverse_minors(const SpinTables& ta, const SpinTables& tb, int nw, d
                            cudaStream_t st);
 int weights_blocks(const SpinTables& tb);
 void launch_weights(const SpinTables& ta, const SpinTables& tb, int nw, double2* const rT[2], double2* const wts[2],
-                    float2* const rf[2], double2* part, int nslot, bool beta, cudaStream_t st);
+                    float2* const rf[2], double2* part, int nslot, bool beta, cudaStream_t st,
+                    double2* const wT[2] = nullptr);
+// The FP64 cofactor matrix by reverse differentiation of the expansions (no inverse
+// minors): per spin the trial's strings followed by the sub-minors outside the trial
+// that their expansions need, and the targets of the reverse pass by stage (levels
+// 5, 4, 3, the 2 x 2 minors, G in n_piece pieces, their sums) with their lists.
+// V: [nh np + n2 + n_ext][nw] (G, 2 x 2 minors, ratios), its first part given;
+// Bv: [n_ext + n2 + n_piece][nw], on entry to launch_adjoint the weights of the
+// trial's strings and zeros.
+#define GRAD_STAGES 6
+struct GradTables {
+    int n_ext = 0, n2 = 0, n_piece = 0;
+    int vbucket[MSD_KMAX + 2] = {0};
+    int stage[GRAD_STAGES + 1] = {0};
+    uint4* str_hp = nullptr;     // [n_ext]
+    int8_t* str_sign = nullptr;  // [n_ext]
+    int* sub = nullptr;          // [n_ext][MSD_KMAX]
+    int *row = nullptr, *off = nullptr;
+    int2* ent = nullptr;
+};
+void launch_minors_ext(const GradTables g[2], const SpinTables& ta, const SpinTables& tb, int nw, double2* const V[2],
+                       cudaStream_t st);
+void launch_adjoint(const GradTables g[2], const SpinTables& ta, const SpinTables& tb, int nw, double2* const V[2],
+                    double2* const Bv[2], double2* const Cm[2], cudaStream_t st);
 void launch_untranspose(int n_str, int nw, const double2* rT, double2* r, cudaStream_t st);
 void launch_det_ratios(const PairTables& pt, int nw, int n_str_a, int n_str_b, const double2* ra,
                        const double2* rb, double2* out, cudaStream_t st);

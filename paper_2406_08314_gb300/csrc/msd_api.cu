@@ -188,6 +188,9 @@ struct msd_ctx {
     // spin, both spins' rows concatenated, the transposed Cholesky vectors
     // and exp(-dt h'/2)
     DgConst dg_Lh[2], dg_Lcat, dg_Lt, dg_E[2];
+    // FP64 cofactors by reverse differentiation (built on first use per trial)
+    GradTables grad[2];
+    bool grad_ready = false, grad_ok = false;
 };
 
 namespace {
@@ -195,6 +198,7 @@ namespace {
 void free_mixed(msd_ctx* ctx);
 void free_exact_ref(msd_ctx* ctx);
 void free_prop(msd_ctx* ctx);
+void free_grad(msd_ctx* ctx);
 
 int fail(msd_ctx* c, int code, const char* fmt, ...)
 {
@@ -617,6 +621,232 @@ int upload_spin(msd_ctx* ctx, SpinHost& S)
     return MSD_OK;
 }
 
+void free_grad(msd_ctx* ctx)
+{
+    for (GradTables& g : ctx->grad) {
+        cudaFree(g.str_hp); cudaFree(g.str_sign); cudaFree(g.sub); cudaFree(g.row); cudaFree(g.off); cudaFree(g.ent);
+        g = GradTables{};
+    }
+    ctx->grad_ready = ctx->grad_ok = false;
+}
+
+// A string as two words (7 bits per index, the level on top of the holes).
+struct StringKey {
+    uint64_t h = 0, p = 0;
+    bool operator==(const StringKey& o) const { return h == o.h && p == o.p; }
+    int level() const { return (int)(h >> 60); }
+    int hole(int i) const { return (int)(h >> (7 * i)) & 127; }
+    int part(int i) const { return (int)(p >> (7 * i)) & 127; }
+    // without the last hole and particle j
+    StringKey child(int j) const
+    {
+        const int k = level();
+        const uint64_t low = (1ull << (7 * j)) - 1;
+        return StringKey{(h & ((1ull << (7 * (k - 1))) - 1)) | (uint64_t)(k - 1) << 60, (p & low) | ((p >> 7) & ~low)};
+    }
+};
+static_assert(MSD_XMAX <= 127 && MSD_KMAX <= 6, "a string's indices fit 7 bits, its level 3");
+
+// String -> number (open addressing).
+struct StringMap {
+    std::vector<StringKey> key;
+    std::vector<int> val;
+    size_t used = 0;
+    explicit StringMap(size_t n) { resize(n); }
+    void resize(size_t n)
+    {
+        size_t c = 64;
+        while (c < 2 * n) c *= 2;
+        key.assign(c, StringKey{});
+        val.assign(c, -1);
+        used = 0;
+    }
+    size_t slot(const StringKey& k) const
+    {
+        size_t i = (size_t)((k.h * 0x9e3779b97f4a7c15ull ^ k.p * 0xc2b2ae3d27d4eb4full) >> 20) & (key.size() - 1);
+        while (val[i] >= 0 && !(key[i] == k)) i = (i + 1) & (key.size() - 1);
+        return i;
+    }
+    int get(const StringKey& k) const { return val[slot(k)]; }
+    void put(const StringKey& k, int v)
+    {
+        if (2 * (used + 1) > key.size()) {
+            std::vector<StringKey> ok;
+            std::vector<int> ov;
+            ok.swap(key);
+            ov.swap(val);
+            resize(ov.size());
+            for (size_t i = 0; i < ov.size(); ++i)
+                if (ov[i] >= 0) put(ok[i], ov[i]);
+        }
+        const size_t i = slot(k);
+        key[i] = k;
+        val[i] = v;
+        ++used;
+    }
+};
+
+// Tables of the FP64 cofactors' reverse pass, once per trial. A string of level k
+// >= 4 expands along its last hole over the k strings without that hole and one
+// particle; those outside the trial are appended (closed under the same expansion).
+// Trials that would need far more of them than they have strings keep the LU path.
+int prepare_grad(msd_ctx* ctx)
+{
+    if (ctx->grad_ready) return MSD_OK;
+    free_grad(ctx);
+    ctx->grad_ready = true;
+    constexpr int K = MSD_KMAX, LONG = 64;   // a G target's list is cut at LONG entries
+    std::vector<uint8_t> hp[2];
+    std::vector<int8_t> sign[2];
+    std::vector<int> sub[2], row[2], off[2];
+    std::vector<int2> ent[2];
+    for (int s = 0; s < 2; ++s) {
+        const SpinHost& S = ctx->sp[s];
+        GradTables& g = ctx->grad[s];
+        const int X = S.nh * S.np, npp = S.np * (S.np - 1) / 2;
+        const size_t limit = 4 * (size_t)S.n_str + 4096;
+        g.n2 = S.nh * (S.nh - 1) / 2 * npp;
+        std::vector<StringKey> key(S.n_str);
+        StringMap at(2 * (size_t)S.n_str);
+        for (int f = 0; f < S.n_str; ++f) {
+            const int k = S.str_k[f];
+            key[f].h = (uint64_t)k << 60;
+            for (int i = 0; i < k; ++i) {
+                key[f].h |= (uint64_t)S.str_h[(size_t)f * K + i] << (7 * i);
+                key[f].p |= (uint64_t)S.str_p[(size_t)f * K + i] << (7 * i);
+            }
+            if (k >= 3) at.put(key[f], f);
+        }
+        // strings outside the trial, by level from the highest down; their numbers
+        // follow once all are known, by level upwards
+        std::vector<StringKey> extra[K + 1];
+        size_t n_extra = 0;
+        for (int k = K; k >= 4; --k) {
+            auto expand = [&](const StringKey& q) {
+                for (int j = 0; j < k; ++j) {
+                    const StringKey c = q.child(j);
+                    if (at.get(c) < 0) { at.put(c, S.n_str); extra[k - 1].push_back(c); ++n_extra; }
+                }
+            };
+            for (int f = S.bucket[k]; f < S.bucket[k + 1]; ++f) expand(key[f]);
+            for (size_t i = 0; i < extra[k].size(); ++i) expand(extra[k][i]);
+            if (n_extra > limit) return MSD_OK;
+        }
+        for (int k = 0; k <= K; ++k) {
+            g.vbucket[k] = (int)key.size();
+            for (const StringKey& q : extra[k]) {
+                at.val[at.slot(q)] = (int)key.size();
+                key.push_back(q);
+            }
+        }
+        g.vbucket[K + 1] = g.n_ext = (int)key.size();
+        hp[s].assign((size_t)g.n_ext * 16, 0);
+        sign[s].assign(g.n_ext, 1);
+        std::copy(S.str_sign.begin(), S.str_sign.end(), sign[s].begin());
+        sub[s].assign((size_t)g.n_ext * K, -1);
+        for (int f = 0; f < g.n_ext; ++f)
+            for (int i = 0; i < key[f].level(); ++i) {
+                hp[s][(size_t)f * 16 + i] = (uint8_t)key[f].hole(i);
+                hp[s][(size_t)f * 16 + 8 + i] = (uint8_t)key[f].part(i);
+            }
+        // (target, list entry), in string order; targets: ratios, 2 x 2 minors, G
+        struct Use { int target; int2 e; };
+        std::vector<Use> uses;
+        uses.reserve((size_t)g.n_ext * 10 + (size_t)g.n2 * 4);
+        auto use = [&](int target, int a, int neg, int b) { uses.push_back(Use{target, make_int2(a * 2 + (neg & 1), b)}); };
+        auto gx = [&](int h, int p) { return h * S.np + p; };
+        const int T2 = g.n_ext, TG = g.n_ext + g.n2, V2 = X, VR = X + g.n2;
+        std::vector<char> used2(std::max(1, g.n2), 0);
+        for (int f = 0; f < g.n_ext; ++f) {
+            const StringKey& q = key[f];
+            const int k = q.level(), sf = sign[s][f] < 0;
+            auto m2 = [&](int c, int d) {
+                return pair_index(q.hole(0), q.hole(1), S.nh) * npp + pair_index(q.part(c), q.part(d), S.np);
+            };
+            if (k == 1) use(TG + gx(q.hole(0), q.part(0)), -1, sf, f);
+            if (k == 2) { use(T2 + m2(0, 1), -1, sf, f); used2[m2(0, 1)] = 1; }
+            if (k == 3)
+                for (int j = 0; j < 3; ++j) {
+                    const int m = m2(j == 0 ? 1 : 0, j == 2 ? 1 : 2), x = gx(q.hole(2), q.part(j)), neg = (j & 1) ^ sf;
+                    use(T2 + m, x, neg, f);
+                    use(TG + x, V2 + m, neg, f);
+                    used2[m] = 1;
+                }
+            if (k >= 4)
+                for (int j = 0; j < k; ++j) {
+                    const int c = at.get(q.child(j)), neg = ((k - 1 + j) & 1) ^ (sign[s][c] < 0) ^ sf;
+                    const int x = gx(q.hole(k - 1), q.part(j));
+                    sub[s][(size_t)f * K + j] = c << 1 | neg;
+                    use(c, x, neg, f);
+                    use(TG + x, VR + c, neg, f);
+                }
+        }
+        for (int h = 0; h < S.nh; ++h)
+            for (int h2 = h + 1; h2 < S.nh; ++h2)
+                for (int p = 0; p < S.np; ++p)
+                    for (int p2 = p + 1; p2 < S.np; ++p2) {
+                        const int m = pair_index(h, h2, S.nh) * npp + pair_index(p, p2, S.np), b = g.n_ext + m;
+                        if (!used2[m]) continue;   // its adjoint is zero
+                        use(TG + gx(h, p), gx(h2, p2), 0, b);
+                        use(TG + gx(h2, p2), gx(h, p), 0, b);
+                        use(TG + gx(h, p2), gx(h2, p), 1, b);
+                        use(TG + gx(h2, p), gx(h, p2), 1, b);
+                    }
+        std::vector<int> first(TG + X + 1, 0), fill;
+        for (const Use& u : uses) ++first[u.target + 1];
+        for (int i = 0; i < TG + X; ++i) first[i + 1] += first[i];
+        std::vector<int2> list(uses.size());
+        fill.assign(first.begin(), first.end() - 1);
+        for (const Use& u : uses) list[fill[u.target]++] = u.e;
+        off[s].push_back(0);
+        auto add = [&](int r, int i0, int i1) {
+            row[s].push_back(r);
+            ent[s].insert(ent[s].end(), list.begin() + i0, list.begin() + i1);
+            off[s].push_back((int)ent[s].size());
+        };
+        auto add_all = [&](int target, int r) { if (first[target] < first[target + 1]) add(r, first[target], first[target + 1]); };
+        for (int q = 0; q < 3; ++q) {   // levels 5, 4, 3
+            const int k = 5 - q;
+            g.stage[q] = (int)row[s].size();
+            for (int f = S.bucket[k]; f < S.bucket[k + 1]; ++f) add_all(f, f);
+            for (int f = g.vbucket[k]; f < g.vbucket[k + 1]; ++f) add_all(f, f);
+        }
+        g.stage[3] = (int)row[s].size();
+        for (int m = 0; m < g.n2; ++m) add_all(T2 + m, g.n_ext + m);
+        // G: the lists in pieces (few targets with long lists), then the pieces' sums
+        g.stage[4] = (int)row[s].size();
+        std::vector<int> piece(X + 1, 0);
+        for (int x = 0; x < X; ++x) {
+            for (int i = first[TG + x]; i < first[TG + x + 1]; i += LONG)
+                add(g.n_ext + g.n2 + g.n_piece++, i, std::min(i + LONG, first[TG + x + 1]));
+            piece[x + 1] = g.n_piece;
+        }
+        g.stage[5] = (int)row[s].size();
+        for (int x = 0; x < X; ++x) {
+            row[s].push_back(x);
+            for (int i = piece[x]; i < piece[x + 1]; ++i) ent[s].push_back(make_int2(-2, g.n_ext + g.n2 + i));
+            off[s].push_back((int)ent[s].size());
+        }
+        g.stage[6] = (int)row[s].size();
+        if (ent[s].empty()) ent[s].push_back(make_int2(0, 0));
+        if (row[s].empty()) row[s].push_back(0);
+    }
+    for (int s = 0; s < 2; ++s) {
+        GradTables& g = ctx->grad[s];
+        uint8_t* d_hp = nullptr;
+        int rc;
+        if ((rc = upload(ctx, &d_hp, hp[s]))) return rc;
+        g.str_hp = (uint4*)d_hp;
+        if ((rc = upload(ctx, &g.str_sign, sign[s]))) return rc;
+        if ((rc = upload(ctx, &g.sub, sub[s]))) return rc;
+        if ((rc = upload(ctx, &g.row, row[s]))) return rc;
+        if ((rc = upload(ctx, &g.off, off[s]))) return rc;
+        if ((rc = upload(ctx, &g.ent, ent[s]))) return rc;
+    }
+    ctx->grad_ok = true;
+    return MSD_OK;
+}
+
 void free_spin(SpinHost& S)
 {
     cudaFree(S.d_occ0); cudaFree(S.d_hole_pos); cudaFree(S.d_part_orb); cudaFree(S.d_str_hp);
@@ -1024,14 +1254,32 @@ struct Chunk {
     double2 *Gr[2], *O0[2], *Gact[2], *GactT[2], *m2[2], *rT[2], *r[2], *wts[2], *part;
     float2* rf[2];   // FP32 copies of r (mixed mode, with B)
     void* B[2];
+    double2 *V[2], *Bv[2];   // reverse pass of the cofactors (StringUse::Cofactors)
     int nslot, nR;
 };
 
-// What a call needs of the strings beyond rT: inverse minors and weights (and, in
-// mixed mode, FP32 ratios) with want_b; the ratios as r[w][s] for the FP64
-// per-determinant terms (want_b in FP64 mode) or for the caller (want_r).
-size_t overlap_bytes_per_walker(msd_ctx* ctx, bool want_b, int nslot, bool want_r = false)
+// What a call needs of the strings beyond their ratios.
+enum class StringUse {
+    Overlap,     // nothing
+    Minors,      // inverse minors and weights of both spins (mixed mode: FP32 ratios too)
+    Cofactors,   // the cofactor matrix alone, in FP64 (prepare_grad's tables)
+};
+
+// The use of a call that needs the cofactors, and the energy or not.
+int string_use(msd_ctx* ctx, bool energy, StringUse* use)
 {
+    *use = StringUse::Minors;
+    if (energy || ctx->prec != MSD_FP64) return MSD_OK;
+    const int rc = prepare_grad(ctx);
+    if (!rc && ctx->grad_ok) *use = StringUse::Cofactors;
+    return rc;
+}
+
+// The ratios as r[w][s] are for the FP64 per-determinant terms (Minors in FP64 mode)
+// or for the caller (want_r).
+size_t overlap_bytes_per_walker(msd_ctx* ctx, StringUse use, int nslot, bool want_r = false)
+{
+    const bool want_b = use == StringUse::Minors, cof = use == StringUse::Cofactors;
     const bool fp64_b = want_b && ctx->prec == MSD_FP64;
     size_t b = 0;
     for (int s = 0; s < 2; ++s) {
@@ -1039,6 +1287,7 @@ size_t overlap_bytes_per_walker(msd_ctx* ctx, bool want_b, int nslot, bool want_
         b += (size_t)S.N * ctx->M + 1 + 2 * (size_t)S.nh * S.np + (size_t)S.n_str;
         b += ref_dg_bytes(ctx->M, S.N) / sizeof(double2) + 1;
         if (!fp64_b) b += minor2_count(tables(S, 1));
+        if (cof) b += 2 * (size_t)ctx->grad[s].n_ext + ctx->grad[s].n2 + ctx->grad[s].n_piece - S.n_str;
         if (fp64_b || want_r) b += S.n_str;
         if (want_b) b += S.n_str + S.b_per_walker + (S.n_str + 1) / 2;
     }
@@ -1046,13 +1295,14 @@ size_t overlap_bytes_per_walker(msd_ctx* ctx, bool want_b, int nslot, bool want_
     return b * sizeof(double2);
 }
 
-int chunk_alloc(msd_ctx* ctx, int cap, bool want_b, int nslot, Chunk& c, bool want_r = false)
+int chunk_alloc(msd_ctx* ctx, int cap, StringUse use, int nslot, Chunk& c, bool want_r = false)
 {
     int rc;
+    const bool want_b = use == StringUse::Minors, cof = use == StringUse::Cofactors;
     const bool fp64_b = want_b && ctx->prec == MSD_FP64;
-    static const char* names[2][10] = {
-        {"Gr_a", "O0_a", "Gact_a", "GactT_a", "m2_a", "rT_a", "r_a", "wts_a", "B_a", "rf_a"},
-        {"Gr_b", "O0_b", "Gact_b", "GactT_b", "m2_b", "rT_b", "r_b", "wts_b", "B_b", "rf_b"}};
+    static const char* names[2][12] = {
+        {"Gr_a", "O0_a", "Gact_a", "GactT_a", "m2_a", "rT_a", "r_a", "wts_a", "B_a", "rf_a", "V_a", "Bv_a"},
+        {"Gr_b", "O0_b", "Gact_b", "GactT_b", "m2_b", "rT_b", "r_b", "wts_b", "B_b", "rf_b", "V_b", "Bv_b"}};
     for (int s = 0; s < 2; ++s) {
         const SpinHost& S = ctx->sp[s];
         const size_t X = std::max(1, S.nh * S.np), w16 = sizeof(double2) * (size_t)cap;
@@ -1063,9 +1313,13 @@ int chunk_alloc(msd_ctx* ctx, int cap, bool want_b, int nslot, Chunk& c, bool wa
         if ((rc = get(0, w16 * S.N * ctx->M, true, (void**)&c.Gr[s]))) return rc;
         if ((rc = get(1, w16, true, (void**)&c.O0[s]))) return rc;
         if ((rc = get(2, w16 * X, true, (void**)&c.Gact[s]))) return rc;
-        if ((rc = get(3, w16 * X, true, (void**)&c.GactT[s]))) return rc;
-        if ((rc = get(4, w16 * minor2_count(tables(S, 1)), !fp64_b, (void**)&c.m2[s]))) return rc;
-        if ((rc = get(5, w16 * S.n_str, true, (void**)&c.rT[s]))) return rc;
+        if ((rc = get(3, w16 * X, !cof, (void**)&c.GactT[s]))) return rc;
+        if ((rc = get(4, w16 * minor2_count(tables(S, 1)), !fp64_b && !cof, (void**)&c.m2[s]))) return rc;
+        if ((rc = get(5, w16 * S.n_str, !cof, (void**)&c.rT[s]))) return rc;
+        const GradTables& g = ctx->grad[s];
+        if ((rc = get(10, w16 * (X + (size_t)g.n2 + g.n_ext), cof, (void**)&c.V[s]))) return rc;
+        if ((rc = get(11, w16 * ((size_t)g.n_ext + g.n2 + g.n_piece), cof, (void**)&c.Bv[s]))) return rc;
+        if (cof) c.GactT[s] = c.V[s];   // the head of V
         if ((rc = get(6, w16 * S.n_str, fp64_b || want_r, (void**)&c.r[s]))) return rc;
         if ((rc = get(7, w16 * S.n_str, want_b, (void**)&c.wts[s]))) return rc;
         if ((rc = get(8, sizeof(double2) * std::max<long long>(1, cap * S.b_per_walker), want_b, &c.B[s]))) return rc;
@@ -1117,11 +1371,31 @@ int run_refs(msd_ctx* ctx, const Staged& in, int w0, int nw, int cap, Chunk& c, 
 }
 
 // String minors, ratios and weights of a chunk whose reference inverse is done.
-// Without want_b only the alpha weights' partial sums are formed.
-int run_strings_weights(msd_ctx* ctx, int nw, int cap, Chunk& c, bool want_b, bool fp32_b, cudaStream_t st)
+// For the overlap alone only the alpha weights' partial sums are formed.
+int run_strings_weights(msd_ctx* ctx, int nw, int cap, Chunk& c, StringUse use, bool fp32_b, cudaStream_t st)
 {
     const TimerHook& th = ctx->hook;
+    const bool want_b = use == StringUse::Minors;
     SpinTables T[2] = {tables(ctx->sp[0], cap), tables(ctx->sp[1], cap)};
+    if (use == StringUse::Cofactors) {
+        double2 *rT[2], *none[2] = {nullptr, nullptr};
+        float2* no_f[2] = {nullptr, nullptr};
+        for (int s = 0; s < 2; ++s) {
+            const GradTables& g = ctx->grad[s];
+            rT[s] = c.V[s] + ((size_t)T[s].nh * T[s].np + g.n2) * nw;
+            // adjoints: the weights in the trial's strings, zero elsewhere
+            CK(cudaMemsetAsync(c.Bv[s] + (size_t)T[s].n_str * nw, 0,
+                               sizeof(double2) * (size_t)nw * (g.n_ext - T[s].n_str + g.n2 + g.n_piece), st));
+        }
+        th.begin("k_strings", st);
+        launch_minors_ext(ctx->grad, T[0], T[1], nw, c.V, st);
+        th.end(st);
+        th.begin("k_weights", st);
+        launch_weights(T[0], T[1], nw, rT, none, no_f, c.part, c.nslot, true, st, c.Bv);
+        th.end(st);
+        CKLAUNCH();
+        return MSD_OK;
+    }
     if (want_b && !fp32_b) {
         for (int s = 0; s < 2; ++s) launch_strings(T[s], nw, c.Gact[s], c.r[s], c.rT[s], c.B[s], st, th);
     } else {
@@ -1141,10 +1415,22 @@ int run_strings_weights(msd_ctx* ctx, int nw, int cap, Chunk& c, bool want_b, bo
 
 // Reference inverse, string minors and weights for walkers [w0, w0 + nw).
 int run_overlap_part(msd_ctx* ctx, const Staged& in, int w0, int nw, int cap, Chunk& c,
-                     bool want_b, bool fp32_b, cudaStream_t st)
+                     StringUse use, bool fp32_b, cudaStream_t st)
 {
     int rc = run_refs(ctx, in, w0, nw, cap, c, st);
-    return rc ? rc : run_strings_weights(ctx, nw, cap, c, want_b, fp32_b, st);
+    return rc ? rc : run_strings_weights(ctx, nw, cap, c, use, fp32_b, st);
+}
+
+// The cofactor matrices of both spins.
+int run_cofactors(msd_ctx* ctx, int nw, int cap, Chunk& c, StringUse use, bool fp32, double2* const Cm[2], cudaStream_t st)
+{
+    const SpinTables T[2] = {tables(ctx->sp[0], cap), tables(ctx->sp[1], cap)};
+    ctx->hook.begin("k_cmat", st);
+    if (use == StringUse::Cofactors) launch_adjoint(ctx->grad, T[0], T[1], nw, c.V, c.Bv, Cm, st);
+    else launch_cmat(T[0], T[1], nw, c.wts[0], c.wts[1], c.B[0], c.B[1], fp32, Cm[0], Cm[1], st);
+    ctx->hook.end(st);
+    CKLAUNCH();
+    return MSD_OK;
 }
 
 int begin_call(msd_ctx* ctx, int n_w, const double* pa, const double* pb, cudaStream_t st)
@@ -1199,7 +1485,7 @@ int fb_alloc(msd_ctx* ctx, int cap, bool fp32, FbWork& f)
     return MSD_OK;
 }
 
-int fb_chunk(msd_ctx* ctx, Chunk& c, FbWork& f, int w0, int nw, int cap, bool fp32, double2* vb_out,
+int fb_chunk(msd_ctx* ctx, Chunk& c, FbWork& f, int w0, int nw, int cap, StringUse use, bool fp32, double2* vb_out,
              double2* ov_out, cudaStream_t st)
 {
     const TimerHook& th = ctx->hook;
@@ -1208,10 +1494,8 @@ int fb_chunk(msd_ctx* ctx, Chunk& c, FbWork& f, int w0, int nw, int cap, bool fp
     launch_sum_slots(nw, c.part, c.nslot, 0, c.nR, (double2*)f.Rs, c.O0[0], c.O0[1],
                      ov_out ? ov_out + w0 : nullptr, st);
     th.end(st);
-    th.begin("k_cmat", st);
-    launch_cmat(tables(ctx->sp[0], cap), tables(ctx->sp[1], cap), nw, c.wts[0], c.wts[1], c.B[0], c.B[1], fp32,
-                (double2*)f.Cm[0], (double2*)f.Cm[1], st);
-    th.end(st);
+    double2* const cm[2] = {(double2*)f.Cm[0], (double2*)f.Cm[1]};
+    if ((rc = run_cofactors(ctx, nw, cap, c, use, fp32, cm, st))) return rc;
     const SpinTables T[2] = {tables(ctx->sp[0], cap), tables(ctx->sp[1], cap)};
     const long long off[2] = {0, (long long)(T[0].N + T[0].np) * ctx->M};
     const double2* Cm[2] = {(const double2*)f.Cm[0], (const double2*)f.Cm[1]};
@@ -1621,12 +1905,14 @@ int evaluate_impl(msd_ctx* ctx, int n_w, const double* phi_a, const double* phi_
     const bool want_v = vbias != nullptr, want_e = e_loc != nullptr;
     const int nR = weights_blocks(tables(ctx->sp[0], 1));
     const int nslot = nR + (want_e ? energy_slots(ctx) : 0);
-    size_t per = overlap_bytes_per_walker(ctx, true, nslot);
+    StringUse use = want_v || want_e ? StringUse::Minors : StringUse::Overlap;
+    if (want_v && !want_e && (rc = string_use(ctx, false, &use))) return rc;
+    size_t per = overlap_bytes_per_walker(ctx, use, nslot);
     if (want_v) per += fb_bytes_per_walker(ctx, fp32);
     if (want_e) per += en_bytes_per_walker(ctx, fp32);
     const int cap = chunk_for(ctx, per, n_w);
     Chunk c;
-    if ((rc = chunk_alloc(ctx, cap, true, nslot, c))) return rc;
+    if ((rc = chunk_alloc(ctx, cap, use, nslot, c))) return rc;
     FbWork f;
     EnWork E;
     if (want_v && (rc = fb_alloc(ctx, cap, fp32, f))) return rc;
@@ -1671,13 +1957,13 @@ int evaluate_impl(msd_ctx* ctx, int n_w, const double* phi_a, const double* phi_
             join.ev = ctx->ev_join;
             if ((rc = en_rest(ctx, c, E, nw, cap, fp32, ctx->side_st))) return rc;
             CK(cudaEventRecord(ctx->ev_rest, ctx->side_st));
-            if ((rc = run_strings_weights(ctx, nw, cap, c, true, fp32, st))) return rc;
+            if ((rc = run_strings_weights(ctx, nw, cap, c, use, fp32, st))) return rc;
             // the force bias (cofactors, G_T, contraction) follows the weights
             // on the second stream, beside the per-determinant terms here
             if (want_v) {
                 CK(cudaEventRecord(ctx->ev_w, st));
                 CK(cudaStreamWaitEvent(ctx->side_st, ctx->ev_w, 0));
-                if ((rc = fb_chunk(ctx, c, f, w0, nw, cap, fp32, o_v.dev, nullptr, ctx->side_st))) return rc;
+                if ((rc = fb_chunk(ctx, c, f, w0, nw, cap, use, fp32, o_v.dev, nullptr, ctx->side_st))) return rc;
             }
             CK(cudaStreamWaitEvent(st, ctx->ev_rest, 0));
             if ((rc = en_terms(ctx, c, E, w0, nw, cap, fp32, o_e.dev, o_ov.dev, st))) return rc;
@@ -1685,8 +1971,8 @@ int evaluate_impl(msd_ctx* ctx, int n_w, const double* phi_a, const double* phi_
             CKLAUNCH();
             continue;
         }
-        if ((rc = run_overlap_part(ctx, in, w0, nw, cap, c, true, fp32, st))) return rc;
-        if (want_v && (rc = fb_chunk(ctx, c, f, w0, nw, cap, fp32, o_v.dev, want_e ? nullptr : o_ov.dev, st)))
+        if ((rc = run_overlap_part(ctx, in, w0, nw, cap, c, use, fp32, st))) return rc;
+        if (want_v && (rc = fb_chunk(ctx, c, f, w0, nw, cap, use, fp32, o_v.dev, want_e ? nullptr : o_ov.dev, st)))
             return rc;
         if (want_e && (rc = en_chunk(ctx, c, E, w0, nw, cap, fp32, o_e.dev, o_ov.dev, st, defer != nullptr)))
             return rc;
@@ -1725,22 +2011,22 @@ int rdm1(msd_ctx* ctx, int n_w, const double* phi_a, const double* phi_b, double
     if ((rc = stage_output(ctx, "out_rdm", rdm, (size_t)n_w * 2 * M * M, o_r))) return rc;
     CK(cudaMemsetAsync(o_r.dev, 0, o_r.bytes, st));
     const int nR = weights_blocks(tables(ctx->sp[0], 1));
-    const int cap = chunk_for(ctx, overlap_bytes_per_walker(ctx, true, nR) + fb_bytes_per_walker(ctx, false), n_w);
+    StringUse use;
+    if ((rc = string_use(ctx, false, &use))) return rc;
+    const int cap = chunk_for(ctx, overlap_bytes_per_walker(ctx, use, nR) + fb_bytes_per_walker(ctx, false), n_w);
     Chunk c;
     FbWork f;
-    if ((rc = chunk_alloc(ctx, cap, true, nR, c))) return rc;
+    if ((rc = chunk_alloc(ctx, cap, use, nR, c))) return rc;
     if ((rc = fb_alloc(ctx, cap, false, f))) return rc;
     const TimerHook& th = ctx->hook;
     for (int w0 = 0; w0 < n_w; w0 += cap) {
         const int nw = std::min(cap, n_w - w0);
-        if ((rc = run_overlap_part(ctx, in, w0, nw, cap, c, true, fp32, st))) return rc;
+        if ((rc = run_overlap_part(ctx, in, w0, nw, cap, c, use, fp32, st))) return rc;
         th.begin("k_sum_slots", st);
         launch_sum_slots(nw, c.part, c.nslot, 0, c.nR, (double2*)f.Rs, c.O0[0], c.O0[1], nullptr, st);
         th.end(st);
-        th.begin("k_cmat", st);
-        launch_cmat(tables(ctx->sp[0], cap), tables(ctx->sp[1], cap), nw, c.wts[0], c.wts[1], c.B[0], c.B[1], fp32,
-                    (double2*)f.Cm[0], (double2*)f.Cm[1], st);
-        th.end(st);
+        double2* const cm[2] = {(double2*)f.Cm[0], (double2*)f.Cm[1]};
+        if ((rc = run_cofactors(ctx, nw, cap, c, use, fp32, cm, st))) return rc;
         const SpinTables T2[2] = {tables(ctx->sp[0], cap), tables(ctx->sp[1], cap)};
         const long long offs[2] = {0, (long long)(T2[0].N + T2[0].np) * M};
         const double2* Cm[2] = {(const double2*)f.Cm[0], (const double2*)f.Cm[1]};
@@ -1794,15 +2080,15 @@ int det_energies(msd_ctx* ctx, int n_w, const double* phi_a, const double* phi_b
     if ((rc = arena_get(ctx, "det_rec", sizeof(DetRec) * n_pairs, &d_rec))) return rc;
     CK(cudaMemcpyAsync(d_rec, recs.data(), sizeof(DetRec) * n_pairs, cudaMemcpyHostToDevice, st));
     const int nR = weights_blocks(tables(ctx->sp[0], 1));
-    const size_t per = overlap_bytes_per_walker(ctx, true, nR) + en_bytes_per_walker(ctx, fp32);
+    const size_t per = overlap_bytes_per_walker(ctx, StringUse::Minors, nR) + en_bytes_per_walker(ctx, fp32);
     const int cap = chunk_for(ctx, per, n_w);
     Chunk c;
     EnWork E;
-    if ((rc = chunk_alloc(ctx, cap, true, nR, c))) return rc;
+    if ((rc = chunk_alloc(ctx, cap, StringUse::Minors, nR, c))) return rc;
     if ((rc = en_alloc(ctx, cap, fp32, E))) return rc;
     for (int w0 = 0; w0 < n_w; w0 += cap) {
         const int nw = std::min(cap, n_w - w0);
-        if ((rc = run_overlap_part(ctx, in, w0, nw, cap, c, true, fp32, st))) return rc;
+        if ((rc = run_overlap_part(ctx, in, w0, nw, cap, c, StringUse::Minors, fp32, st))) return rc;
         if ((rc = en_chunk(ctx, c, E, w0, nw, cap, fp32, nullptr, nullptr, st, true))) return rc;
         launch_det_energy(n_pairs, (const DetRec*)d_rec, w0, nw, tables(ctx->sp[0], cap), tables(ctx->sp[1], cap),
                           c.B[0], c.B[1], E.Kaa, E.Kbb, E.Kab, E.Y[0], E.Y[1], (const double2*)E.scal,
@@ -2080,6 +2366,7 @@ void msd_destroy(msd_ctx* ctx)
     cudaFree(ctx->pairs.d_det_index); cudaFree(ctx->pairs.d_cf);
     free_mixed(ctx);
     free_prop(ctx);
+    free_grad(ctx);
     cudaFree(ctx->d_h1); cudaFree(ctx->d_Lcat); cudaFree(ctx->d_err);
     cudaFreeHost(ctx->h_err);
     for (auto& p : ctx->pending) { ctx->ev_pool.push_back(p.a); ctx->ev_pool.push_back(p.b); }
@@ -2121,6 +2408,7 @@ int msd_set_trial(msd_ctx* ctx, int n_det, const double* coeff, const int32_t* o
     if (n_det <= 0 || !coeff || !occ_a || !occ_b) return fail(ctx, MSD_ERR_ARG, "empty trial");
     CK(cudaSetDevice(ctx->device));
     ctx->have_trial = false;
+    free_grad(ctx);
     std::vector<int> sid[2];
     const int32_t* occ[2] = {occ_a, occ_b};
     for (int s = 0; s < 2; ++s) {
@@ -2300,12 +2588,12 @@ int msd_overlap(msd_ctx* ctx, int n_w, const double* phi_a, const double* phi_b,
     if ((rc = stage_output(ctx, "out_ovlp", ovlp, n_w, o_ov))) return rc;
     if ((rc = stage_output(ctx, "out_rsum", ratio_sum, n_w, o_rs))) return rc;
     const int nR = weights_blocks(tables(ctx->sp[0], 1));
-    const int cap = chunk_for(ctx, overlap_bytes_per_walker(ctx, false, nR), n_w);
+    const int cap = chunk_for(ctx, overlap_bytes_per_walker(ctx, StringUse::Overlap, nR), n_w);
     Chunk c;
-    if ((rc = chunk_alloc(ctx, cap, false, nR, c))) return rc;
+    if ((rc = chunk_alloc(ctx, cap, StringUse::Overlap, nR, c))) return rc;
     for (int w0 = 0; w0 < n_w; w0 += cap) {
         const int nw = std::min(cap, n_w - w0);
-        if ((rc = run_overlap_part(ctx, in, w0, nw, cap, c, false, false, st))) return rc;
+        if ((rc = run_overlap_part(ctx, in, w0, nw, cap, c, StringUse::Overlap, false, st))) return rc;
         ctx->hook.begin("k_sum_slots", st);
         launch_sum_slots(nw, c.part, c.nslot, 0, c.nR, o_rs.dev ? o_rs.dev + w0 : nullptr, c.O0[0],
                          c.O0[1], o_ov.dev ? o_ov.dev + w0 : nullptr, st);
@@ -2329,12 +2617,12 @@ int msd_det_ratios(msd_ctx* ctx, int n_w, const double* phi_a, const double* phi
     if ((rc = stage_output(ctx, "out_ratios", ratios, (size_t)n_w * ctx->pairs.n_det, o_r))) return rc;
     if ((rc = stage_output(ctx, "out_refovlp", ref_ovlp, n_w, o_o))) return rc;
     const int nR = weights_blocks(tables(ctx->sp[0], 1));
-    const int cap = chunk_for(ctx, overlap_bytes_per_walker(ctx, false, nR, true), n_w);
+    const int cap = chunk_for(ctx, overlap_bytes_per_walker(ctx, StringUse::Overlap, nR, true), n_w);
     Chunk c;
-    if ((rc = chunk_alloc(ctx, cap, false, nR, c, true))) return rc;
+    if ((rc = chunk_alloc(ctx, cap, StringUse::Overlap, nR, c, true))) return rc;
     for (int w0 = 0; w0 < n_w; w0 += cap) {
         const int nw = std::min(cap, n_w - w0);
-        if ((rc = run_overlap_part(ctx, in, w0, nw, cap, c, false, false, st))) return rc;
+        if ((rc = run_overlap_part(ctx, in, w0, nw, cap, c, StringUse::Overlap, false, st))) return rc;
         ctx->hook.begin("k_det_ratios", st);
         for (int s = 0; s < 2; ++s) launch_untranspose(ctx->sp[s].n_str, nw, c.rT[s], c.r[s], st);
         launch_det_ratios(pair_tables(ctx->pairs), nw, ctx->sp[0].n_str, ctx->sp[1].n_str, c.r[0],
@@ -2397,9 +2685,9 @@ int msd_features(msd_ctx* ctx, int n_w, const double* phi_a, const double* phi_b
     Staged in;
     if ((rc = stage_inputs(ctx, n_w, phi_a, phi_b, st, in))) return rc;
     const int nR = weights_blocks(tables(ctx->sp[0], 1));
-    const int cap = chunk_for(ctx, overlap_bytes_per_walker(ctx, false, nR), n_w);
+    const int cap = chunk_for(ctx, overlap_bytes_per_walker(ctx, StringUse::Overlap, nR), n_w);
     Chunk c;
-    if ((rc = chunk_alloc(ctx, cap, false, nR, c))) return rc;
+    if ((rc = chunk_alloc(ctx, cap, StringUse::Overlap, nR, c))) return rc;
     const int M = ctx->M;
     for (int w0 = 0; w0 < n_w; w0 += cap) {
         const int nw = std::min(cap, n_w - w0);
@@ -2427,9 +2715,9 @@ int msd_features_rows(msd_ctx* ctx, int n_w, const double* phi_a, const double* 
     Staged in;
     if ((rc = stage_inputs(ctx, n_w, phi_a, phi_b, st, in))) return rc;
     const int nR = weights_blocks(tables(ctx->sp[0], 1));
-    const int cap = chunk_for(ctx, overlap_bytes_per_walker(ctx, false, nR), n_w);
+    const int cap = chunk_for(ctx, overlap_bytes_per_walker(ctx, StringUse::Overlap, nR), n_w);
     Chunk c;
-    if ((rc = chunk_alloc(ctx, cap, false, nR, c))) return rc;
+    if ((rc = chunk_alloc(ctx, cap, StringUse::Overlap, nR, c))) return rc;
     const int M = ctx->M;
     if (ld > need) CK(cudaMemsetAsync(feat, 0, sizeof(float) * (size_t)n_w * ld, st));
     for (int w0 = 0; w0 < n_w; w0 += cap) {
