@@ -348,6 +348,95 @@ __global__ void __launch_bounds__(128) k_inverse_minors(const __grid_constant__ 
     }
 }
 
+// ------------------------------------------------------ FP64 inverse minors
+// B = A^-1 of every string as its cofactors over its determinant. The cofactors are
+// the (k - 1)-minors that the ratios' expansions leave (and the sub-minors that the
+// trial does not hold, appended to its strings): 4 FP64 FMAs per entry and one
+// reciprocal per string, against 8 k^3 / 3 and k reciprocals of an LU with its column
+// solves, which the FP64 unit bounds. The relative error of an entry is that of two
+// division-free minors. Bound by memory now: k^2 gathered rows of the walkers in, k^2
+// entries out per string and walker. A warp takes 32 (string, walker) pairs, walkers
+// fastest, and writes their entries through shared memory, up to 16 (256 bytes) of a
+// pair at a time. 640 copper-oxo walkers, ratios and inverses 3.06 -> 1.28 ms.
+struct InvRatioSpin {
+    int bucket[MSD_KMAX + 2];
+    const int* row;
+    long long row_off[MSD_KMAX + 2];
+    const double2* V;        // [row][nw]
+    const double2* r;        // [string][nw], within V
+    double2* B;
+    long long b_off[MSD_KMAX + 2];
+    int blk[MSD_KMAX + 2];   // first block of each level
+};
+struct InvRatioArgs { InvRatioSpin s[2]; };
+
+#define IR_E 16   // entries per pass
+template <int K>
+__device__ __forceinline__ void inverse_ratios(const InvRatioSpin& S, int nw, double2 (*tile)[IR_E + 1])
+{
+    constexpr int KK = K * K, KST = b_stride(K);
+    const int ns = S.bucket[K + 1] - S.bucket[K], lane = threadIdx.x & 31;
+    const long long items = (long long)ns * nw;
+    const long long e0 = ((long long)blockIdx.x - S.blk[K]) * 128 + (threadIdx.x & ~31), e = e0 + lane;
+    if (e0 >= items) return;
+    const bool on = e < items;
+    // 32-bit division where the count allows it
+    const int sl = !on ? 0 : items < 0x7fffffff ? (int)((unsigned)e / (unsigned)nw) : (int)(e / nw);
+    const int w = on ? (int)(e - (long long)sl * nw) : 0;
+    const double2 r = S.r[(size_t)(S.bucket[K] + sl) * nw + w];
+    // 1 / r at a scale where |r|^2 neither underflows nor overflows; 0 for r = 0
+    const double m = fmax(fabs(r.x), fabs(r.y));
+    const int ex = min(1000, max(-1000, ((__double2hiint(m) >> 20) & 2047) - 1023));
+    const double sc = __hiloint2double((1023 - ex) << 20, 0);
+    const double2 q = cscale(r, sc);
+    const double d = r.x == 0 && r.y == 0 ? 0.0 : 1.0 / fma(q.x, q.x, q.y * q.y);
+    const double2 inv = cz(q.x * d * sc, -q.y * d * sc);
+    const int* row = S.row + S.row_off[K] + (size_t)sl * KK;
+    const double2* V = S.V + w;
+    const long long base = ((long long)w * ns + sl) * KST;
+    double2* B = S.B + S.b_off[K];
+#pragma unroll 1
+    for (int p = 0; p < KST; p += IR_E) {
+        const int n = KST < IR_E ? KST : min(IR_E, KST - p);
+#pragma unroll 4
+        for (int i = 0; i < n; ++i) {
+            double2 v = cz(0, 0);
+            if (p + i < KK) {
+                const int c = row[p + i];
+                if (K == 1) v = inv;
+                else v = cmul(V[(size_t)(c >> 1) * nw], inv);
+                if (c & 1) v = cz(-v.x, -v.y);
+            }
+            tile[lane][i] = v;
+        }
+        __syncwarp();
+        for (int i = 0; i < n; ++i) {
+            const int f = i * 32 + lane, it = f / n;   // pair, entry
+            const long long b = __shfl_sync(0xffffffffu, base, it);
+            if (e0 + it < items) B[b + p + f - it * n] = tile[it][f - it * n];
+        }
+        __syncwarp();
+    }
+}
+
+__global__ void __launch_bounds__(128) k_inverse_ratios(const __grid_constant__ InvRatioArgs a, int nw)
+{
+    const InvRatioSpin& S = a.s[blockIdx.y];
+    __shared__ double2 tile[4][32][IR_E + 1];
+    if ((int)blockIdx.x >= S.blk[MSD_KMAX + 1]) return;
+    int k = 1;
+    while ((int)blockIdx.x >= S.blk[k + 1]) ++k;
+    double2 (*t)[IR_E + 1] = tile[threadIdx.x >> 5];
+    switch (k) {
+    case 1: inverse_ratios<1>(S, nw, t); break;
+    case 2: inverse_ratios<2>(S, nw, t); break;
+    case 3: inverse_ratios<3>(S, nw, t); break;
+    case 4: inverse_ratios<4>(S, nw, t); break;
+    case 5: inverse_ratios<5>(S, nw, t); break;
+    default: inverse_ratios<6>(S, nw, t); break;
+    }
+}
+
 MinorSpin minor_spin(const SpinTables& t, const double2* GT, double2* m2, double2* rT)
 {
     MinorSpin s;
@@ -514,6 +603,29 @@ void launch_inverse_minors(const SpinTables& ta, const SpinTables& tb, int nw, d
     }
     if (nb <= 0) return;
     k_inverse_minors<<<dim3(nb, nw, 2), 128, 0, st>>>(args);
+    msd_note_launch();
+}
+
+void launch_inverse_ratios(const GradTables g[2], const SpinTables& ta, const SpinTables& tb, int nw,
+                           double2* const V[2], void* const B[2], cudaStream_t st)
+{
+    InvRatioArgs args;
+    const SpinTables* t[2] = {&ta, &tb};
+    int nb = 0;
+    for (int i = 0; i < 2; ++i) {
+        InvRatioSpin& s = args.s[i];
+        s.row = g[i].row; s.V = V[i]; s.B = (double2*)B[i];
+        s.r = V[i] + ((size_t)t[i]->nh * t[i]->np + g[i].n2) * nw;
+        s.blk[0] = s.blk[1] = 0;
+        for (int k = 0; k < MSD_KMAX + 2; ++k) {
+            s.bucket[k] = t[i]->bucket[k]; s.b_off[k] = t[i]->b_off[k]; s.row_off[k] = t[i]->cmx_off[k];
+        }
+        for (int k = 1; k <= MSD_KMAX; ++k)
+            s.blk[k + 1] = s.blk[k] + (int)(((long long)(s.bucket[k + 1] - s.bucket[k]) * nw + 127) / 128);
+        nb = std::max(nb, s.blk[MSD_KMAX + 1]);
+    }
+    if (nb <= 0) return;
+    k_inverse_ratios<<<dim3(nb, 2), 128, 0, st>>>(args, nw);
     msd_note_launch();
 }
 

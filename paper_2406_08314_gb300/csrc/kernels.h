@@ -60,11 +60,14 @@ struct GradTables {
     uint4* str_hp = nullptr;     // [n_ext]
     int8_t* str_sign = nullptr;  // [n_ext]
     int* sub = nullptr;          // [n_ext][MSD_KMAX]
-    int *row = nullptr, *off = nullptr;
+    int *row = nullptr, *off = nullptr;   // launch_inverse_ratios: row alone, at SpinTables::cmx_off
     int2* ent = nullptr;
 };
 void launch_minors_ext(const GradTables g[2], const SpinTables& ta, const SpinTables& tb, int nw, double2* const V[2],
                        cudaStream_t st);
+// FP64 inverse minors from V as launch_minors_ext left it.
+void launch_inverse_ratios(const GradTables g[2], const SpinTables& ta, const SpinTables& tb, int nw,
+                           double2* const V[2], void* const B[2], cudaStream_t st);
 void launch_adjoint(const GradTables g[2], const SpinTables& ta, const SpinTables& tb, int nw, double2* const V[2],
                     double2* const Bv[2], double2* const Cm[2], cudaStream_t st);
 void launch_untranspose(int n_str, int nw, const double2* rT, double2* r, cudaStream_t st);

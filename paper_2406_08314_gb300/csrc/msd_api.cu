@@ -191,6 +191,9 @@ struct msd_ctx {
     // FP64 cofactors by reverse differentiation (built on first use per trial)
     GradTables grad[2];
     bool grad_ready = false, grad_ok = false;
+    // FP64 inverse minors from the ratios (built on first use per trial)
+    GradTables inv[2];
+    bool inv_ready = false, inv_ok = false;
 };
 
 namespace {
@@ -623,11 +626,11 @@ int upload_spin(msd_ctx* ctx, SpinHost& S)
 
 void free_grad(msd_ctx* ctx)
 {
-    for (GradTables& g : ctx->grad) {
-        cudaFree(g.str_hp); cudaFree(g.str_sign); cudaFree(g.sub); cudaFree(g.row); cudaFree(g.off); cudaFree(g.ent);
-        g = GradTables{};
+    for (GradTables* g : {&ctx->grad[0], &ctx->grad[1], &ctx->inv[0], &ctx->inv[1]}) {
+        cudaFree(g->str_hp); cudaFree(g->str_sign); cudaFree(g->sub); cudaFree(g->row); cudaFree(g->off); cudaFree(g->ent);
+        *g = GradTables{};
     }
-    ctx->grad_ready = ctx->grad_ok = false;
+    ctx->grad_ready = ctx->grad_ok = ctx->inv_ready = ctx->inv_ok = false;
 }
 
 // A string as two words (7 bits per index, the level on top of the holes).
@@ -637,12 +640,11 @@ struct StringKey {
     int level() const { return (int)(h >> 60); }
     int hole(int i) const { return (int)(h >> (7 * i)) & 127; }
     int part(int i) const { return (int)(p >> (7 * i)) & 127; }
-    // without the last hole and particle j
-    StringKey child(int j) const
+    // without hole i and particle j
+    StringKey child(int i, int j) const
     {
-        const int k = level();
-        const uint64_t low = (1ull << (7 * j)) - 1;
-        return StringKey{(h & ((1ull << (7 * (k - 1))) - 1)) | (uint64_t)(k - 1) << 60, (p & low) | ((p >> 7) & ~low)};
+        const uint64_t li = (1ull << (7 * i)) - 1, lj = (1ull << (7 * j)) - 1, hh = h & ~(15ull << 60);
+        return StringKey{(hh & li) | ((hh >> 7) & ~li) | (uint64_t)(level() - 1) << 60, (p & lj) | ((p >> 7) & ~lj)};
     }
 };
 static_assert(MSD_XMAX <= 127 && MSD_KMAX <= 6, "a string's indices fit 7 bits, its level 3");
@@ -686,28 +688,24 @@ struct StringMap {
     }
 };
 
-// Tables of the FP64 cofactors' reverse pass, once per trial. A string of level k
-// >= 4 expands along its last hole over the k strings without that hole and one
-// particle; those outside the trial are appended (closed under the same expansion).
-// Trials that would need far more of them than they have strings keep the LU path.
-int prepare_grad(msd_ctx* ctx)
-{
-    if (ctx->grad_ready) return MSD_OK;
-    free_grad(ctx);
-    ctx->grad_ready = true;
-    constexpr int K = MSD_KMAX, LONG = 64;   // a G target's list is cut at LONG entries
-    std::vector<uint8_t> hp[2];
-    std::vector<int8_t> sign[2];
-    std::vector<int> sub[2], row[2], off[2];
-    std::vector<int2> ent[2];
-    for (int s = 0; s < 2; ++s) {
-        const SpinHost& S = ctx->sp[s];
-        GradTables& g = ctx->grad[s];
-        const int X = S.nh * S.np, npp = S.np * (S.np - 1) / 2;
+// One spin's strings, the trial's followed by those outside it that are needed, by
+// level upwards. A string of level k >= 4 is evaluated over the k strings without its
+// last hole and one particle; with `all`, the k^2 sub-minors (one hole and one
+// particle less) of the trial's strings are needed too.
+struct Closure {
+    std::vector<StringKey> key;
+    StringMap at{64};            // level >= 3: number
+    std::vector<uint8_t> hp;     // records (SpinTables::str_hp)
+    std::vector<int8_t> sign;
+    std::vector<int> sub;        // [string][MSD_KMAX] (string << 1 | negative)
+    // false: far more of them than the trial has strings
+    bool build(const SpinHost& S, bool all, GradTables& g)
+    {
+        constexpr int K = MSD_KMAX;
         const size_t limit = 4 * (size_t)S.n_str + 4096;
-        g.n2 = S.nh * (S.nh - 1) / 2 * npp;
-        std::vector<StringKey> key(S.n_str);
-        StringMap at(2 * (size_t)S.n_str);
+        g.n2 = S.nh * (S.nh - 1) / 2 * (S.np * (S.np - 1) / 2);
+        key.assign(S.n_str, StringKey{});
+        at.resize(2 * (size_t)S.n_str);
         for (int f = 0; f < S.n_str; ++f) {
             const int k = S.str_k[f];
             key[f].h = (uint64_t)k << 60;
@@ -717,20 +715,20 @@ int prepare_grad(msd_ctx* ctx)
             }
             if (k >= 3) at.put(key[f], f);
         }
-        // strings outside the trial, by level from the highest down; their numbers
-        // follow once all are known, by level upwards
+        // from the highest level down; their numbers follow once all are known
         std::vector<StringKey> extra[K + 1];
         size_t n_extra = 0;
         for (int k = K; k >= 4; --k) {
-            auto expand = [&](const StringKey& q) {
-                for (int j = 0; j < k; ++j) {
-                    const StringKey c = q.child(j);
-                    if (at.get(c) < 0) { at.put(c, S.n_str); extra[k - 1].push_back(c); ++n_extra; }
-                }
+            auto expand = [&](const StringKey& q, int i0) {
+                for (int i = i0; i < k; ++i)
+                    for (int j = 0; j < k; ++j) {
+                        const StringKey c = q.child(i, j);
+                        if (at.get(c) < 0) { at.put(c, S.n_str); extra[k - 1].push_back(c); ++n_extra; }
+                    }
             };
-            for (int f = S.bucket[k]; f < S.bucket[k + 1]; ++f) expand(key[f]);
-            for (size_t i = 0; i < extra[k].size(); ++i) expand(extra[k][i]);
-            if (n_extra > limit) return MSD_OK;
+            for (int f = S.bucket[k]; f < S.bucket[k + 1]; ++f) expand(key[f], all ? 0 : k - 1);
+            for (size_t i = 0; i < extra[k].size(); ++i) expand(extra[k][i], k - 1);
+            if (n_extra > limit) return false;
         }
         for (int k = 0; k <= K; ++k) {
             g.vbucket[k] = (int)key.size();
@@ -740,15 +738,98 @@ int prepare_grad(msd_ctx* ctx)
             }
         }
         g.vbucket[K + 1] = g.n_ext = (int)key.size();
-        hp[s].assign((size_t)g.n_ext * 16, 0);
-        sign[s].assign(g.n_ext, 1);
-        std::copy(S.str_sign.begin(), S.str_sign.end(), sign[s].begin());
-        sub[s].assign((size_t)g.n_ext * K, -1);
-        for (int f = 0; f < g.n_ext; ++f)
-            for (int i = 0; i < key[f].level(); ++i) {
-                hp[s][(size_t)f * 16 + i] = (uint8_t)key[f].hole(i);
-                hp[s][(size_t)f * 16 + 8 + i] = (uint8_t)key[f].part(i);
+        hp.assign((size_t)g.n_ext * 16, 0);
+        sign.assign(g.n_ext, 1);
+        std::copy(S.str_sign.begin(), S.str_sign.end(), sign.begin());
+        sub.assign((size_t)g.n_ext * K, -1);
+        for (int f = 0; f < g.n_ext; ++f) {
+            const int k = key[f].level();
+            for (int i = 0; i < k; ++i) {
+                hp[(size_t)f * 16 + i] = (uint8_t)key[f].hole(i);
+                hp[(size_t)f * 16 + 8 + i] = (uint8_t)key[f].part(i);
             }
+            for (int j = 0; k >= 4 && j < k; ++j) {
+                const int c = at.get(key[f].child(k - 1, j));
+                sub[(size_t)f * K + j] = c << 1 | (((k - 1 + j) & 1) ^ (sign[c] < 0) ^ (sign[f] < 0));
+            }
+        }
+        return true;
+    }
+    int upload_to(msd_ctx* ctx, GradTables& g)
+    {
+        int rc;
+        uint8_t* d_hp = nullptr;
+        if ((rc = upload(ctx, &d_hp, hp))) return rc;
+        g.str_hp = (uint4*)d_hp;
+        if ((rc = upload(ctx, &g.str_sign, sign))) return rc;
+        return upload(ctx, &g.sub, sub);
+    }
+};
+
+// Row of the 2 x 2 minor of the string's holes a < b and particles c < d.
+int minor2_row(const StringKey& q, int a, int b, int c, int d, int nh, int np)
+{
+    return pair_index(q.hole(a), q.hole(b), nh) * (np * (np - 1) / 2) + pair_index(q.part(c), q.part(d), np);
+}
+
+// Tables of the FP64 inverse minors, once per trial: for entry (i, j) of a string's
+// k x k inverse the row of V = [G | 2 x 2 minors | ratios] that holds its cofactor
+// (the minor without hole j and particle i), twice, plus 1 where its sign is negative.
+// Trials with far more sub-minors than strings keep the LU path.
+int prepare_inverse(msd_ctx* ctx)
+{
+    if (ctx->inv_ready) return MSD_OK;
+    ctx->inv_ready = true;
+    Closure C[2];
+    std::vector<int> row[2];
+    for (int s = 0; s < 2; ++s) {
+        const SpinHost& S = ctx->sp[s];
+        GradTables& g = ctx->inv[s];
+        if (!C[s].build(S, true, g)) return MSD_OK;
+        const int X = S.nh * S.np;
+        for (int f = S.bucket[1]; f < S.n_str; ++f) {
+            const StringKey& q = C[s].key[f];
+            const int k = q.level();
+            for (int i = 0; i < k; ++i)
+                for (int j = 0; j < k; ++j) {
+                    int r = 0, neg = (i + j) & 1;   // k = 1: no row, the cofactor is 1
+                    if (k == 2) r = q.hole(1 - j) * S.np + q.part(1 - i);
+                    if (k == 3) r = X + minor2_row(q, j == 0, j == 2 ? 1 : 2, i == 0, i == 2 ? 1 : 2, S.nh, S.np);
+                    if (k >= 4) {
+                        const int c = C[s].at.get(q.child(j, i));
+                        neg ^= C[s].sign[c] < 0;
+                        r = X + g.n2 + c;
+                    }
+                    row[s].push_back(r << 1 | (neg ^ (C[s].sign[f] < 0)));
+                }
+        }
+        if (row[s].empty()) row[s].push_back(0);
+    }
+    for (int s = 0; s < 2; ++s) {
+        int rc;
+        if ((rc = C[s].upload_to(ctx, ctx->inv[s]))) return rc;
+        if ((rc = upload(ctx, &ctx->inv[s].row, row[s]))) return rc;
+    }
+    ctx->inv_ok = true;
+    return MSD_OK;
+}
+
+// Tables of the FP64 cofactors' reverse pass, once per trial. Trials that would need
+// far more strings than they have keep the LU path.
+int prepare_grad(msd_ctx* ctx)
+{
+    if (ctx->grad_ready) return MSD_OK;
+    ctx->grad_ready = true;
+    constexpr int LONG = 64;   // a G target's list is cut at LONG entries
+    Closure C[2];
+    std::vector<int> row[2], off[2];
+    std::vector<int2> ent[2];
+    for (int s = 0; s < 2; ++s) {
+        const SpinHost& S = ctx->sp[s];
+        GradTables& g = ctx->grad[s];
+        if (!C[s].build(S, false, g)) return MSD_OK;
+        const int X = S.nh * S.np, npp = S.np * (S.np - 1) / 2;
+        const std::vector<StringKey>& key = C[s].key;
         // (target, list entry), in string order; targets: ratios, 2 x 2 minors, G
         struct Use { int target; int2 e; };
         std::vector<Use> uses;
@@ -759,10 +840,8 @@ int prepare_grad(msd_ctx* ctx)
         std::vector<char> used2(std::max(1, g.n2), 0);
         for (int f = 0; f < g.n_ext; ++f) {
             const StringKey& q = key[f];
-            const int k = q.level(), sf = sign[s][f] < 0;
-            auto m2 = [&](int c, int d) {
-                return pair_index(q.hole(0), q.hole(1), S.nh) * npp + pair_index(q.part(c), q.part(d), S.np);
-            };
+            const int k = q.level(), sf = C[s].sign[f] < 0;
+            auto m2 = [&](int c, int d) { return minor2_row(q, 0, 1, c, d, S.nh, S.np); };
             if (k == 1) use(TG + gx(q.hole(0), q.part(0)), -1, sf, f);
             if (k == 2) { use(T2 + m2(0, 1), -1, sf, f); used2[m2(0, 1)] = 1; }
             if (k == 3)
@@ -774,9 +853,8 @@ int prepare_grad(msd_ctx* ctx)
                 }
             if (k >= 4)
                 for (int j = 0; j < k; ++j) {
-                    const int c = at.get(q.child(j)), neg = ((k - 1 + j) & 1) ^ (sign[s][c] < 0) ^ sf;
+                    const int c = C[s].sub[(size_t)f * MSD_KMAX + j] >> 1, neg = C[s].sub[(size_t)f * MSD_KMAX + j] & 1;
                     const int x = gx(q.hole(k - 1), q.part(j));
-                    sub[s][(size_t)f * K + j] = c << 1 | neg;
                     use(c, x, neg, f);
                     use(TG + x, VR + c, neg, f);
                 }
@@ -833,12 +911,8 @@ int prepare_grad(msd_ctx* ctx)
     }
     for (int s = 0; s < 2; ++s) {
         GradTables& g = ctx->grad[s];
-        uint8_t* d_hp = nullptr;
         int rc;
-        if ((rc = upload(ctx, &d_hp, hp[s]))) return rc;
-        g.str_hp = (uint4*)d_hp;
-        if ((rc = upload(ctx, &g.str_sign, sign[s]))) return rc;
-        if ((rc = upload(ctx, &g.sub, sub[s]))) return rc;
+        if ((rc = C[s].upload_to(ctx, g))) return rc;
         if ((rc = upload(ctx, &g.row, row[s]))) return rc;
         if ((rc = upload(ctx, &g.off, off[s]))) return rc;
         if ((rc = upload(ctx, &g.ent, ent[s]))) return rc;
@@ -1254,7 +1328,7 @@ struct Chunk {
     double2 *Gr[2], *O0[2], *Gact[2], *GactT[2], *m2[2], *rT[2], *r[2], *wts[2], *part;
     float2* rf[2];   // FP32 copies of r (mixed mode, with B)
     void* B[2];
-    double2 *V[2], *Bv[2];   // reverse pass of the cofactors (StringUse::Cofactors)
+    double2 *V[2], *Bv[2];   // expansions (launch_minors_ext) and their reverse pass
     int nslot, nR;
 };
 
@@ -1265,11 +1339,18 @@ enum class StringUse {
     Cofactors,   // the cofactor matrix alone, in FP64 (prepare_grad's tables)
 };
 
-// The use of a call that needs the cofactors, and the energy or not.
+// FP64 inverse minors of a call: from the ratios' tables where the trial has them.
+bool ratio_inverse(const msd_ctx* ctx, StringUse use)
+{
+    return use == StringUse::Minors && ctx->prec == MSD_FP64 && ctx->inv_ok;
+}
+
+// The use of a call that needs the cofactors or inverse minors (energy).
 int string_use(msd_ctx* ctx, bool energy, StringUse* use)
 {
     *use = StringUse::Minors;
-    if (energy || ctx->prec != MSD_FP64) return MSD_OK;
+    if (ctx->prec != MSD_FP64) return MSD_OK;
+    if (energy) return prepare_inverse(ctx);
     const int rc = prepare_grad(ctx);
     if (!rc && ctx->grad_ok) *use = StringUse::Cofactors;
     return rc;
@@ -1280,13 +1361,14 @@ int string_use(msd_ctx* ctx, bool energy, StringUse* use)
 size_t overlap_bytes_per_walker(msd_ctx* ctx, StringUse use, int nslot, bool want_r = false)
 {
     const bool want_b = use == StringUse::Minors, cof = use == StringUse::Cofactors;
-    const bool fp64_b = want_b && ctx->prec == MSD_FP64;
+    const bool fp64_b = want_b && ctx->prec == MSD_FP64, inv = ratio_inverse(ctx, use);
     size_t b = 0;
     for (int s = 0; s < 2; ++s) {
         const SpinHost& S = ctx->sp[s];
         b += (size_t)S.N * ctx->M + 1 + 2 * (size_t)S.nh * S.np + (size_t)S.n_str;
         b += ref_dg_bytes(ctx->M, S.N) / sizeof(double2) + 1;
         if (!fp64_b) b += minor2_count(tables(S, 1));
+        if (inv) b += ctx->inv[s].n2 + ctx->inv[s].n_ext - S.n_str;
         if (cof) b += 2 * (size_t)ctx->grad[s].n_ext + ctx->grad[s].n2 + ctx->grad[s].n_piece - S.n_str;
         if (fp64_b || want_r) b += S.n_str;
         if (want_b) b += S.n_str + S.b_per_walker + (S.n_str + 1) / 2;
@@ -1299,7 +1381,7 @@ int chunk_alloc(msd_ctx* ctx, int cap, StringUse use, int nslot, Chunk& c, bool 
 {
     int rc;
     const bool want_b = use == StringUse::Minors, cof = use == StringUse::Cofactors;
-    const bool fp64_b = want_b && ctx->prec == MSD_FP64;
+    const bool fp64_b = want_b && ctx->prec == MSD_FP64, inv = ratio_inverse(ctx, use);
     static const char* names[2][12] = {
         {"Gr_a", "O0_a", "Gact_a", "GactT_a", "m2_a", "rT_a", "r_a", "wts_a", "B_a", "rf_a", "V_a", "Bv_a"},
         {"Gr_b", "O0_b", "Gact_b", "GactT_b", "m2_b", "rT_b", "r_b", "wts_b", "B_b", "rf_b", "V_b", "Bv_b"}};
@@ -1313,13 +1395,13 @@ int chunk_alloc(msd_ctx* ctx, int cap, StringUse use, int nslot, Chunk& c, bool 
         if ((rc = get(0, w16 * S.N * ctx->M, true, (void**)&c.Gr[s]))) return rc;
         if ((rc = get(1, w16, true, (void**)&c.O0[s]))) return rc;
         if ((rc = get(2, w16 * X, true, (void**)&c.Gact[s]))) return rc;
-        if ((rc = get(3, w16 * X, !cof, (void**)&c.GactT[s]))) return rc;
+        if ((rc = get(3, w16 * X, !cof && !inv, (void**)&c.GactT[s]))) return rc;
         if ((rc = get(4, w16 * minor2_count(tables(S, 1)), !fp64_b && !cof, (void**)&c.m2[s]))) return rc;
-        if ((rc = get(5, w16 * S.n_str, !cof, (void**)&c.rT[s]))) return rc;
-        const GradTables& g = ctx->grad[s];
-        if ((rc = get(10, w16 * (X + (size_t)g.n2 + g.n_ext), cof, (void**)&c.V[s]))) return rc;
+        if ((rc = get(5, w16 * S.n_str, !cof && !inv, (void**)&c.rT[s]))) return rc;
+        const GradTables& g = inv ? ctx->inv[s] : ctx->grad[s];
+        if ((rc = get(10, w16 * (X + (size_t)g.n2 + g.n_ext), cof || inv, (void**)&c.V[s]))) return rc;
         if ((rc = get(11, w16 * ((size_t)g.n_ext + g.n2 + g.n_piece), cof, (void**)&c.Bv[s]))) return rc;
-        if (cof) c.GactT[s] = c.V[s];   // the head of V
+        if (cof || inv) c.GactT[s] = c.V[s];   // the head of V
         if ((rc = get(6, w16 * S.n_str, fp64_b || want_r, (void**)&c.r[s]))) return rc;
         if ((rc = get(7, w16 * S.n_str, want_b, (void**)&c.wts[s]))) return rc;
         if ((rc = get(8, sizeof(double2) * std::max<long long>(1, cap * S.b_per_walker), want_b, &c.B[s]))) return rc;
@@ -1396,7 +1478,14 @@ int run_strings_weights(msd_ctx* ctx, int nw, int cap, Chunk& c, StringUse use, 
         CKLAUNCH();
         return MSD_OK;
     }
-    if (want_b && !fp32_b) {
+    if (ratio_inverse(ctx, use)) {
+        for (int s = 0; s < 2; ++s) c.rT[s] = c.V[s] + ((size_t)T[s].nh * T[s].np + ctx->inv[s].n2) * nw;
+        th.begin("k_strings", st);
+        launch_minors_ext(ctx->inv, T[0], T[1], nw, c.V, st);
+        launch_inverse_ratios(ctx->inv, T[0], T[1], nw, c.V, c.B, st);
+        for (int s = 0; s < 2; ++s) launch_untranspose(T[s].n_str, nw, c.rT[s], c.r[s], st);
+        th.end(st);
+    } else if (want_b && !fp32_b) {
         for (int s = 0; s < 2; ++s) launch_strings(T[s], nw, c.Gact[s], c.r[s], c.rT[s], c.B[s], st, th);
     } else {
         th.begin("k_strings", st);
@@ -1905,8 +1994,8 @@ int evaluate_impl(msd_ctx* ctx, int n_w, const double* phi_a, const double* phi_
     const bool want_v = vbias != nullptr, want_e = e_loc != nullptr;
     const int nR = weights_blocks(tables(ctx->sp[0], 1));
     const int nslot = nR + (want_e ? energy_slots(ctx) : 0);
-    StringUse use = want_v || want_e ? StringUse::Minors : StringUse::Overlap;
-    if (want_v && !want_e && (rc = string_use(ctx, false, &use))) return rc;
+    StringUse use = StringUse::Overlap;
+    if ((want_v || want_e) && (rc = string_use(ctx, want_e, &use))) return rc;
     size_t per = overlap_bytes_per_walker(ctx, use, nslot);
     if (want_v) per += fb_bytes_per_walker(ctx, fp32);
     if (want_e) per += en_bytes_per_walker(ctx, fp32);
@@ -2080,15 +2169,17 @@ int det_energies(msd_ctx* ctx, int n_w, const double* phi_a, const double* phi_b
     if ((rc = arena_get(ctx, "det_rec", sizeof(DetRec) * n_pairs, &d_rec))) return rc;
     CK(cudaMemcpyAsync(d_rec, recs.data(), sizeof(DetRec) * n_pairs, cudaMemcpyHostToDevice, st));
     const int nR = weights_blocks(tables(ctx->sp[0], 1));
-    const size_t per = overlap_bytes_per_walker(ctx, StringUse::Minors, nR) + en_bytes_per_walker(ctx, fp32);
+    StringUse use;
+    if ((rc = string_use(ctx, true, &use))) return rc;
+    const size_t per = overlap_bytes_per_walker(ctx, use, nR) + en_bytes_per_walker(ctx, fp32);
     const int cap = chunk_for(ctx, per, n_w);
     Chunk c;
     EnWork E;
-    if ((rc = chunk_alloc(ctx, cap, StringUse::Minors, nR, c))) return rc;
+    if ((rc = chunk_alloc(ctx, cap, use, nR, c))) return rc;
     if ((rc = en_alloc(ctx, cap, fp32, E))) return rc;
     for (int w0 = 0; w0 < n_w; w0 += cap) {
         const int nw = std::min(cap, n_w - w0);
-        if ((rc = run_overlap_part(ctx, in, w0, nw, cap, c, StringUse::Minors, fp32, st))) return rc;
+        if ((rc = run_overlap_part(ctx, in, w0, nw, cap, c, use, fp32, st))) return rc;
         if ((rc = en_chunk(ctx, c, E, w0, nw, cap, fp32, nullptr, nullptr, st, true))) return rc;
         launch_det_energy(n_pairs, (const DetRec*)d_rec, w0, nw, tables(ctx->sp[0], cap), tables(ctx->sp[1], cap),
                           c.B[0], c.B[1], E.Kaa, E.Kbb, E.Kab, E.Y[0], E.Y[1], (const double2*)E.scal,
