@@ -79,7 +79,7 @@ __device__ __forceinline__ double2 pair_term_fixed(const SpinTables& ta, const S
         }
     }
     double xr = 0, xim = 0;
-#pragma unroll
+#pragma unroll 1
     for (int e = 0; e < KO * KO; ++e) {
         const double2 bo = Bo[e];
         const Limbs* krow = kk.k + (rec_h(ro, e % KO) * npo + rec_p(ro, e / KO)) * so;
@@ -105,7 +105,7 @@ __device__ __forceinline__ cplx_t<T> pair_term(const SpinTables& ta, const SpinT
         return pair_term_fixed<KA, KB>(ta, tbb, pt, I, w, Ba, Bb, kk, ra, rb);
 }
 
-// FP64 mode, levels 1 to 5: e_s of string_energy_value with the sums over the pair
+// FP64 mode, levels 1 and 2 (string_energy_lanes: 3 to 6): e_s of string_energy_value with the sums over the pair
 // table and over Y in fixed point (the FP64 unit bounds the plain form: level 4, 496
 // FP64 operations per string; here 48 and 1056 mad.wide):
 //   e_s = sum_ij b_ij Y[h_j][p_i] + sum_{i < k-1} sum_j b_ij z_ij,
@@ -157,25 +157,119 @@ __device__ __forceinline__ double2 string_energy_fixed(const SpinTables& tb, int
     return v;
 }
 
-// The pair table and Y of a block in shared memory, FP32 / FP64, or as limbs with
-// their exponents where string_energy_fixed reads them.
+// The pair table and Y of a block in shared memory, in FP64 mode as limbs with their
+// exponents and with room for the strings' minors (string_energy_lanes).
 template <typename T>
 struct SeTab {
     const cplx_t<T>*as, *ys;
     int ea, ey;
+    Limbs* bs;
 };
-#define SE_FIXED_MAX 5
-template <int KL, typename T>
-__device__ __forceinline__ double2 string_energy_any(const SpinTables& tb, int w, int sl, int ns, const void* B,
-                                                     const SeTab<T>& tab, const double2* wts)
+#define SE_LANES_MIN 3   // levels that string_energy_lanes takes
+static_assert(MSD_KMAX <= 8, "a group of 8 lanes holds a string's columns");
+__host__ __device__ __forceinline__ constexpr int se_group(int k) { return k <= 4 ? 4 : 8; }
+__host__ __device__ __forceinline__ constexpr int se_pitch(int k) { return (k * k) | 1; }
+// limbs of a block's strings, the most of any level (se_group 4: level 4, 8: level 6)
+#define SE_LIMBS (SE_THREADS / 8 * se_pitch(MSD_KMAX) > SE_THREADS / 4 * se_pitch(4) \
+                      ? SE_THREADS / 8 * se_pitch(MSD_KMAX) : SE_THREADS / 4 * se_pitch(4))
+
+// FP64 mode, levels 3 to 6: this block's strings (SE_THREADS SE_PER_THREAD from blk) in
+// the sums of string_energy_fixed, a group of 4 or 8 lanes to a string, lane j taking
+// the columns j: b_ij Y[h_j][p_i] and b_ij z_ij for all i. The string's limbs are made
+// once, by the group's lanes, in shared memory. A thread per string holds them in
+// registers (254 at level 4: 8 warps per SM, every instruction waiting for the last)
+// and leaves the SM idle where strings are few (one level-6 string in 640 walkers: 0.66
+// ms). 640 copper-oxo walkers, levels 3 to 6: 2.94 -> 1.31 ms.
+template <int KL>
+__device__ __forceinline__ double2 string_energy_lanes(const SpinTables& tb, int w, int blk, int ns, const void* Bin,
+                                                       const SeTab<double>& tab, const double2* wts)
 {
-    if constexpr (std::is_same<T, double>::value && KL <= SE_FIXED_MAX) {
-        const double2 e = string_energy_fixed<KL>(tb, w, sl, ns, B, reinterpret_cast<const Limbs*>(tab.as), tab.ea,
-                                                  reinterpret_cast<const Limbs*>(tab.ys), tab.ey);
-        return cmul(wts[(size_t)w * tb.n_str + tb.bucket[KL] + sl], e);   // wts holds r_s w_s
-    } else {
-        return string_energy_term<KL, T, true>(tb, w, sl, ns, B, tab.as, tab.ys, wts);
+    constexpr int KK = KL * KL, G = se_group(KL), SPW = 32 / G, PITCH = se_pitch(KL), EPL = (KK + G - 1) / G;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane / G, j = lane % G;
+    const int np = tb.np, nh = tb.nh, npp = np * (np - 1) / 2;
+    const Limbs *as = reinterpret_cast<const Limbs*>(tab.as), *ys = reinterpret_cast<const Limbs*>(tab.ys);
+    Limbs* bs = tab.bs + (warp * SPW + g) * PITCH;
+    double2 sum = cz(0, 0);
+    for (int it = 0; it < SE_PER_THREAD * G; ++it) {
+        const int s0 = blk * (SE_THREADS * SE_PER_THREAD) + (it * (SE_THREADS / 32) + warp) * SPW, sl = s0 + g;
+        if (s0 >= ns) break;   // the warp's
+        const bool on = sl < ns;
+        const int sc = on ? sl : ns - 1;
+        const double2* B = reinterpret_cast<const double2*>(Bin) + (size_t)tb.b_off[KL] + ((size_t)w * ns + sc) * b_stride(KL);
+        const uint4 rec = tb.str_hp[tb.bucket[KL] + sc];
+        double2 bv[EPL];
+        unsigned mag = 0;
+#pragma unroll
+        for (int q = 0; q < EPL; ++q) {
+            bv[q] = j + q * G < KK ? B[j + q * G] : cz(0, 0);
+            mag = max(mag, mag_bits(bv[q]));
+        }
+#pragma unroll
+        for (int o = 1; o < G; o <<= 1) mag = max(mag, __shfl_xor_sync(0xffffffffu, mag, o));
+        const int eb = mag_exponent(mag);
+        __syncwarp();   // the previous strings' limbs consumed
+#pragma unroll
+        for (int q = 0; q < EPL; ++q)
+            if (j + q * G < KK) bs[j + q * G] = to_limbs(bv[q], eb);
+        __syncwarp();
+        if (on && j < KL) {
+            int hp[KL - 1], lc[KL - 1];   // pair rows of (h_j, h_l) and columns l, j + 1 on, in a circle
+            const int hj = rec_h(rec, j);
+#pragma unroll
+            for (int d = 1; d < KL; ++d) {
+                const int l = j + d < KL ? j + d : j + d - KL, hl = rec_h(rec, l);
+                lc[d - 1] = l;
+                hp[d - 1] = (l > j ? pair_index(hj, hl, nh) : pair_index(hl, hj, nh)) * npp;
+            }
+            LimbSum lin;
+#pragma unroll
+            for (int i = 0; i < KL; ++i) lin.add(bs[i * KL + j], ys[hj * np + rec_p(rec, i)]);
+            double2 v = limb_value(lin, eb + tab.ey);
+#pragma unroll 1
+            for (int i = 0; i + 1 < KL; ++i) {
+                LimbSum z;
+                const int pi = rec_p(rec, i);
+#pragma unroll 1
+                for (int m = i + 1; m < KL; ++m) {
+                    const int pim = pair_index(pi, rec_p(rec, m), np);
+#pragma unroll
+                    for (int d = 0; d < KL - 1; ++d) {
+                        const Limbs x = bs[m * KL + lc[d]], y = as[hp[d] + pim];
+                        if (lc[d] > j) z.add(x, y);
+                        else z.sub(x, y);
+                    }
+                }
+                v = cfma(B[i * KL + j], limb_value(z, eb + tab.ea), v);
+            }
+            if (max(max(tab.ea, tab.ey), eb) >= FIXED_EXP_INF) v.x = v.y = __longlong_as_double(0x7ff8000000000000ll);
+            sum = cfma(wts[(size_t)w * tb.n_str + tb.bucket[KL] + sl], v, sum);   // wts holds r_s w_s
+        }
     }
+    return sum;
+}
+
+// The same-spin term of one block's strings of one level, this thread's part.
+template <int KL, typename T>
+__device__ __forceinline__ double2 string_energy_block(const SpinTables& tb, int w, int blk, const void* B,
+                                                       const SeTab<T>& tab, const double2* wts)
+{
+    const int ns = tb.bucket[KL + 1] - tb.bucket[KL];
+    double2 sum = cz(0, 0);
+    if constexpr (std::is_same<T, double>::value && KL >= SE_LANES_MIN) {
+        sum = string_energy_lanes<KL>(tb, w, blk, ns, B, tab, wts);
+    } else {
+        for (int it = 0; it < SE_PER_THREAD; ++it) {
+            const int sl = blk * (SE_THREADS * SE_PER_THREAD) + it * SE_THREADS + threadIdx.x;
+            if (sl >= ns) break;
+            if constexpr (std::is_same<T, double>::value)
+                sum = cadd(sum, cmul(wts[(size_t)w * tb.n_str + tb.bucket[KL] + sl],
+                                     string_energy_fixed<KL>(tb, w, sl, ns, B, reinterpret_cast<const Limbs*>(tab.as), tab.ea,
+                                                             reinterpret_cast<const Limbs*>(tab.ys), tab.ey)));
+            else
+                sum = cadd(sum, string_energy_term<KL, T, true>(tb, w, sl, ns, B, tab.as, tab.ys, wts));
+        }
+    }
+    return sum;
 }
 
 // The walker's antisymmetrized pair table A[(h,h')][(p,p')] = K[(h,p)][(h',p')] -
@@ -202,19 +296,18 @@ __device__ __forceinline__ SeTab<T> load_se_table(const SpinTables& tb, const vo
     }
     const T2* Yw = reinterpret_cast<const T2*>(Yin) + (size_t)w * X;
     for (int e = t; e < X; e += blockDim.x) ys[e] = Yw[e];
-    SeTab<T> tab = {as, ys, 0, 0};
+    SeTab<T> tab = {as, ys, 0, 0, reinterpret_cast<Limbs*>(ys + X)};
     if constexpr (std::is_same<T, double>::value) {
-        if (k <= SE_FIXED_MAX) {   // each thread its own entries
-            __shared__ unsigned wm[2][SE_THREADS / 32];
-            unsigned ma = 0, my = 0;
-            for (int e = t; e < na; e += blockDim.x) ma = max(ma, mag_bits(as[e]));
-            for (int e = t; e < X; e += blockDim.x) my = max(my, mag_bits(ys[e]));
-            tab.ea = mag_exponent(block_mag(ma, wm[0]));
-            tab.ey = mag_exponent(block_mag(my, wm[1]));
-            Limbs *la = reinterpret_cast<Limbs*>(as), *ly = reinterpret_cast<Limbs*>(ys);
-            for (int e = t; e < na; e += blockDim.x) la[e] = to_limbs(as[e], tab.ea);
-            for (int e = t; e < X; e += blockDim.x) ly[e] = to_limbs(ys[e], tab.ey);
-        }
+        // each thread its own entries
+        __shared__ unsigned wm[2][SE_THREADS / 32];
+        unsigned ma = 0, my = 0;
+        for (int e = t; e < na; e += blockDim.x) ma = max(ma, mag_bits(as[e]));
+        for (int e = t; e < X; e += blockDim.x) my = max(my, mag_bits(ys[e]));
+        tab.ea = mag_exponent(block_mag(ma, wm[0]));
+        tab.ey = mag_exponent(block_mag(my, wm[1]));
+        Limbs *la = reinterpret_cast<Limbs*>(as), *ly = reinterpret_cast<Limbs*>(ys);
+        for (int e = t; e < na; e += blockDim.x) la[e] = to_limbs(as[e], tab.ea);
+        for (int e = t; e < X; e += blockDim.x) ly[e] = to_limbs(ys[e], tab.ey);
     }
     __syncthreads();
     return tab;

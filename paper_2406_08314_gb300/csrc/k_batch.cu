@@ -10,20 +10,6 @@
 #include "det_block.cuh"
 #include "kernels.h"
 
-template <int K, typename T>
-__device__ __forceinline__ double2 batch_se(const BatchSys& S, const BatchItem& it, const SeTab<T>& tab)
-{
-    const SpinTables& tb = S.t[it.spin];
-    const int ns = tb.bucket[K + 1] - tb.bucket[K];
-    double2 acc = cz(0, 0);
-    for (int q = 0; q < SE_PER_THREAD; ++q) {
-        const int sl = it.blk * (SE_THREADS * SE_PER_THREAD) + q * SE_THREADS + threadIdx.x;
-        if (sl >= ns) break;
-        acc = cadd(acc, string_energy_any<K, T>(tb, it.w, sl, ns, S.B[it.spin], tab, S.wts[it.spin]));
-    }
-    return acc;
-}
-
 // The opposite-spin term of one block with both levels known at compile time, or
 // (levels adding up to more than 6) by the general form.
 template <int KA, int KB, typename T>
@@ -98,13 +84,16 @@ k_det_batched(const BatchSys* __restrict__ systems, const BatchItem* __restrict_
         double2 v = cz(0, 0);
         if (it.kind == 0) {
             const SeTab<T> tab = load_se_table<T>(S.t[it.spin], S.K[it.spin], S.Y[it.spin], it.w, it.ka, smraw);
+            const int s = it.spin;
             switch (it.ka) {
-            case 1: v = batch_se<1, T>(S, it, tab); break;
-            case 2: v = batch_se<2, T>(S, it, tab); break;
-            case 3: v = batch_se<3, T>(S, it, tab); break;
-            case 4: v = batch_se<4, T>(S, it, tab); break;
-            case 5: v = batch_se<5, T>(S, it, tab); break;
-            default: v = batch_se<6, T>(S, it, tab); break;
+#define BATCH_SE(K) string_energy_block<K, T>(S.t[s], it.w, it.blk, S.B[s], tab, S.wts[s])
+            case 1: v = BATCH_SE(1); break;
+            case 2: v = BATCH_SE(2); break;
+            case 3: v = BATCH_SE(3); break;
+            case 4: v = BATCH_SE(4); break;
+            case 5: v = BATCH_SE(5); break;
+            default: v = BATCH_SE(6); break;
+#undef BATCH_SE
             }
         } else {
             const int XX = S.t[0].nh * S.t[0].np * S.t[1].nh * S.t[1].np;

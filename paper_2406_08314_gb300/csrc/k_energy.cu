@@ -506,20 +506,6 @@ struct SeArgs {
     int blk[2][MSD_KMAX + 2];   // first block of each (spin, level)
 };
 
-template <int KL, typename T>
-__device__ __forceinline__ double2 string_energy_block(const SpinTables& tb, int w, int blk, const void* B,
-                                                       const SeTab<T>& tab, const double2* wts)
-{
-    const int ns = tb.bucket[KL + 1] - tb.bucket[KL];
-    double2 contrib = cz(0, 0);
-    for (int it = 0; it < SE_PER_THREAD; ++it) {
-        const int sl = blk * (SE_THREADS * SE_PER_THREAD) + it * SE_THREADS + threadIdx.x;
-        if (sl >= ns) break;
-        contrib = cadd(contrib, string_energy_any<KL, T>(tb, w, sl, ns, B, tab, wts));
-    }
-    return contrib;
-}
-
 template <typename T, int ONLY>
 __global__ void __launch_bounds__(SE_THREADS)
 k_string_energy(const __grid_constant__ SeArgs a, double2* __restrict__ part, int nslot, int slot0)
@@ -571,7 +557,7 @@ size_t string_energy_smem(const SpinTables& tb, bool fp32)
 {
     const int X = tb.nh * tb.np;
     const size_t pairs = (size_t)(tb.nh * (tb.nh - 1) / 2) * (tb.np * (tb.np - 1) / 2);
-    return (fp32 ? sizeof(float2) : sizeof(double2)) * (pairs + X);
+    return fp32 ? sizeof(float2) * (pairs + X) : sizeof(double2) * (pairs + X) + sizeof(Limbs) * SE_LIMBS;
 }
 
 void launch_string_energy(const SpinTables& ta, const SpinTables& tb, int nw, const double2* const wts[2],

@@ -12,7 +12,7 @@
 #include "kernels.h"
 
 template <int KA, int KB, typename T>
-__global__ void __launch_bounds__(PC_THREADS)
+__global__ void __launch_bounds__(PC_THREADS, std::is_same<T, double>::value ? 2 : 1)
 k_pair_cross2(SpinTables ta, SpinTables tbb, PairTables pt, int lo, int n, const void* __restrict__ ra_in,
               const void* __restrict__ rb_in, const void* __restrict__ Ba_in, const void* __restrict__ Bb_in,
               const void* __restrict__ Kin, double2* __restrict__ part, int nslot, int slot0)
