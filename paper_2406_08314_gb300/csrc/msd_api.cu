@@ -3219,7 +3219,8 @@ int batch_run(msd_batch* b, const int* n_w, const double* const* pa, const doubl
             S.part = d[i].c.part;
             S.nslot = d[i].c.nslot;
             const size_t X0 = (size_t)S.t[0].nh * S.t[0].np, X1 = (size_t)S.t[1].nh * S.t[1].np;
-            smem = std::max(smem, std::max(std::max(X0 * X0 + X0, X1 * X1 + X1), X0 * X1));
+            for (int s = 0; s < 2; ++s) smem = std::max(smem, string_energy_smem(S.t[s], b->fp32));
+            smem = std::max(smem, X0 * X1 * (b->fp32 ? sizeof(float2) : sizeof(double2)));
             system_items(ctx, i, n_w[i], items, cost);
         }
         if (b->order == 1) {          // largest work first
@@ -3233,7 +3234,7 @@ int batch_run(msd_batch* b, const int* n_w, const double* const* pa, const doubl
             std::stable_sort(items.begin(), items.end(),
                              [](const BatchItem& x, const BatchItem& y) { return x.w < y.w; });
         }
-        b->smem = smem * (b->fp32 ? sizeof(float2) : sizeof(double2));
+        b->smem = smem;
         if (b->sys_cap < (size_t)n) {
             cudaFree(b->d_sys);
             BCK(cudaMalloc(&b->d_sys, sizeof(BatchSys) * n));
