@@ -10,28 +10,8 @@
 #include "det_block.cuh"
 #include "kernels.h"
 
-// The opposite-spin term of one block with both levels known at compile time, or
-// (levels adding up to more than 6) by the general form.
-template <int KA, int KB, typename T>
-__device__ __forceinline__ double2 batch_pc(const BatchSys& S, const BatchItem& it, const PairK<T>& ks)
-{
-    using T2 = cplx_t<T>;
-    const int idx = KA * (MSD_KMAX + 1) + KB, lo = S.pt.bucket[idx], n = S.pt.bucket[idx + 1] - lo;
-    // the ratios in the working precision, as in the per-system kernels
-    constexpr bool F = std::is_same<T, float>::value;
-    const T2* ra = F ? reinterpret_cast<const T2*>(S.rf[0]) : reinterpret_cast<const T2*>(S.r[0]);
-    const T2* rb = F ? reinterpret_cast<const T2*>(S.rf[1]) : reinterpret_cast<const T2*>(S.r[1]);
-    T2 acc = T2{0, 0};
-    for (int q = 0; q < PC_PER_THREAD; ++q) {
-        const int i0 = it.blk * (PC_THREADS * PC_PER_THREAD) + q * PC_THREADS + threadIdx.x;
-        if (i0 >= n) break;
-        const T2 v = pair_term<KA, KB, T>(S.t[0], S.t[1], S.pt, lo + i0, it.w, S.B[0], S.B[1], ks, ra, rb);
-        acc.x += v.x;
-        acc.y += v.y;
-    }
-    return cz((double)acc.x, (double)acc.y);
-}
-
+// The opposite-spin term of one block whose levels add up to more than 6, in the
+// general form.
 template <int KB, typename T>
 __device__ double2 batch_pc_any(const BatchSys& S, const BatchItem& it, const cplx_t<T>* ks)
 {
@@ -99,8 +79,15 @@ k_det_batched(const BatchSys* __restrict__ systems, const BatchItem* __restrict_
             const int XX = S.t[0].nh * S.t[0].np * S.t[1].nh * S.t[1].np;
             if (it.ka + it.kb <= 6) {
                 const PairK<T> ks = load_pair_k<T>(S.K[2], it.w, XX, smraw);
+                // the ratios in the working precision, as in the per-system kernels
+                constexpr bool F = std::is_same<T, float>::value;
+                const void *ra = F ? (const void*)S.rf[0] : S.r[0], *rb = F ? (const void*)S.rf[1] : S.r[1];
+                const int i = it.ka * (MSD_KMAX + 1) + it.kb, lo = S.pt.bucket[i], n = S.pt.bucket[i + 1] - lo;
                 switch (it.ka * 8 + it.kb) {
-#define PAIR_CASE(A, B) case A * 8 + B: v = batch_pc<A, B, T>(S, it, ks); break;
+#define PAIR_CASE(KA, KB)                                                                                         \
+    case KA * 8 + KB:                                                                                             \
+        v = pair_block<KA, KB, T, false>(S.t[0], S.t[1], S.pt, lo, n, it.blk, it.w, S.B[0], S.B[1], ks, ra, rb, nullptr); \
+        break;
                 PAIR_CASE(1, 1) PAIR_CASE(1, 2) PAIR_CASE(1, 3) PAIR_CASE(1, 4) PAIR_CASE(1, 5)
                 PAIR_CASE(2, 1) PAIR_CASE(2, 2) PAIR_CASE(2, 3) PAIR_CASE(2, 4)
                 PAIR_CASE(3, 1) PAIR_CASE(3, 2) PAIR_CASE(3, 3)

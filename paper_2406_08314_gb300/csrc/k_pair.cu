@@ -1,62 +1,79 @@
 // Opposite-spin cross term (fill_os) per determinant with both excitation
-// levels (ka, kb) known at compile time, for ka + kb <= 8: the indices and
-// both inverse minors sit in registers and the ka^2 kb^2 gathers from the
-// shared Gram matrix K^{ab} are fully unrolled, so a determinant's global
-// loads are all issued before its first gather. Same value, partial-sum
-// slots and block shape as k_pair_cross in k_energy.cu, which serves the
-// other level pairs.
+// levels (ka, kb) known at compile time, for ka + kb <= 8. Mixed mode: a thread
+// per determinant, the indices and both inverse minors in registers, the ka^2 kb^2
+// gathers from the shared Gram matrix K^{ab} fully unrolled, so a determinant's
+// global loads are all issued before its first gather. FP64 mode: groups of lanes
+// (pair_lanes). Same partial-sum slots as k_pair_cross in k_energy.cu, which
+// serves the other level pairs.
+#include <algorithm>
 #include <type_traits>
 
 #include "common.cuh"
 #include "det_block.cuh"
 #include "kernels.h"
 
+// Mixed mode: PC_THREADS threads, one per determinant; FP64 mode: groups of lanes,
+// any number of warps.
 template <int KA, int KB, typename T>
-__global__ void __launch_bounds__(PC_THREADS, std::is_same<T, double>::value ? 2 : 1)
-k_pair_cross2(SpinTables ta, SpinTables tbb, PairTables pt, int lo, int n, const void* __restrict__ ra_in,
-              const void* __restrict__ rb_in, const void* __restrict__ Ba_in, const void* __restrict__ Bb_in,
+__global__ void __launch_bounds__(std::is_same<T, double>::value ? 1024 : PC_THREADS)
+k_pair_cross2(SpinTables ta, SpinTables tbb, PairTables pt, int lo, int n, const void* __restrict__ ra,
+              const void* __restrict__ rb, const void* __restrict__ Ba, const void* __restrict__ Bb,
               const void* __restrict__ Kin, double2* __restrict__ part, int nslot, int slot0)
 {
-    using T2 = cplx_t<T>;
+    constexpr bool LANES = std::is_same<T, double>::value;
     extern __shared__ __align__(16) unsigned char smraw[];
-    const int Xa = ta.nh * ta.np, Xb = tbb.nh * tbb.np;
-    __shared__ double2 red[PC_THREADS];
+    const int XX = ta.nh * ta.np * tbb.nh * tbb.np;
+    __shared__ double2 red[LANES ? 32 : PC_THREADS];
     const int w = blockIdx.y, t = threadIdx.x;
-    const PairK<T> ks = load_pair_k<T>(Kin, w, Xa * Xb, smraw);   // [Xa][Xb]
-    const T2* ra = reinterpret_cast<const T2*>(ra_in);
-    const T2* rb = reinterpret_cast<const T2*>(rb_in);
-    T2 contrib = T2{0, 0};   // this thread's determinants, in the working precision
-    for (int it = 0; it < PC_PER_THREAD; ++it) {
-        const int i0 = blockIdx.x * (PC_THREADS * PC_PER_THREAD) + it * PC_THREADS + t;
-        if (i0 >= n) break;
-        const T2 v = pair_term<KA, KB, T>(ta, tbb, pt, lo + i0, w, Ba_in, Bb_in, ks, ra, rb);
-        contrib.x += v.x;
-        contrib.y += v.y;
-    }
-    red[t] = cz((double)contrib.x, (double)contrib.y);
-    __syncthreads();
-    for (int o = PC_THREADS / 2; o; o >>= 1) {
-        if (t < o) red[t] = cadd(red[t], red[t + o]);
+    const PairK<T> ks = load_pair_k<T>(Kin, w, XX, smraw);   // [Xa][Xb]
+    double2 v = pair_block<KA, KB, T, LANES>(ta, tbb, pt, lo, n, blockIdx.x, w, Ba, Bb, ks, ra, rb,
+                                             reinterpret_cast<Limbs*>(smraw) + XX);
+    if constexpr (LANES) {
+#pragma unroll
+        for (int o = 16; o; o >>= 1) {
+            v.x += __shfl_down_sync(0xffffffffu, v.x, o);
+            v.y += __shfl_down_sync(0xffffffffu, v.y, o);
+        }
+        if ((t & 31) == 0) red[t >> 5] = v;
         __syncthreads();
+        for (int q = 1; t == 0 && q < (int)(blockDim.x >> 5); ++q) v = cadd(v, red[q]);
+    } else {
+        red[t] = v;
+        __syncthreads();
+        for (int o = PC_THREADS / 2; o; o >>= 1) {
+            if (t < o) red[t] = cadd(red[t], red[t + o]);
+            __syncthreads();
+        }
+        v = red[0];
     }
-    if (t == 0) part[(size_t)w * nslot + slot0 + blockIdx.x] = red[0];
+    if (t == 0) part[(size_t)w * nslot + slot0 + blockIdx.x] = v;
 }
+
+// Shared memory of a block in the lanes form, beside its static part.
+static size_t lanes_smem(size_t k_bytes, int limbs) { return k_bytes + sizeof(Limbs) * limbs; }
+static bool lanes_fit(size_t dyn, int blocks) { return (dyn + 5 * 1024) * blocks <= 227 * 1024; }
 
 template <int KA, int KB>
 static bool go(bool fp32, dim3 grid, size_t smem, const SpinTables& ta, const SpinTables& tb, const PairTables& pt,
                int lo, int n, const void* ra, const void* rb, const void* Ba, const void* Bb, const void* K,
                double2* part, int nslot, int slot, cudaStream_t st)
 {
+    auto run = [&](auto kern, int threads, size_t sm) {
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        kern<<<grid, threads, sm, st>>>(ta, tb, pt, lo, n, ra, rb, Ba, Bb, K, part, nslot, slot);
+        msd_note_launch();
+    };
     if (fp32) {
-        cudaFuncSetAttribute(k_pair_cross2<KA, KB, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k_pair_cross2<KA, KB, float><<<grid, PC_THREADS, smem, st>>>(ta, tb, pt, lo, n, ra, rb, Ba, Bb, K, part,
-                                                                     nslot, slot);
-    } else {
-        cudaFuncSetAttribute(k_pair_cross2<KA, KB, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k_pair_cross2<KA, KB, double><<<grid, PC_THREADS, smem, st>>>(ta, tb, pt, lo, n, ra, rb, Ba, Bb, K, part,
-                                                                      nslot, slot);
+        run(k_pair_cross2<KA, KB, float>, PC_THREADS, smem);
+        return true;
     }
-    msd_note_launch();
+    // 32 warps per SM where they fit: two blocks of 512 threads, one loading its Gram
+    // matrix while the other computes, else one of 1024 (75 x 75 active pairs); fewer
+    // only beside the largest Gram matrices (112 x 112: 196 KB)
+    auto bytes = [&](int threads) { return lanes_smem(smem, pair_limbs(KA, KB, threads)); };
+    int threads = lanes_fit(bytes(512), 2) ? 512 : 1024;
+    while (threads > 64 && !lanes_fit(bytes(threads), 1)) threads /= 2;
+    run(k_pair_cross2<KA, KB, double>, threads, bytes(threads));
     return true;
 }
 
@@ -107,28 +124,10 @@ struct PairAll {
     int blk[MSD_KMAX * MSD_KMAX + 1];   // first block of pair (ka - 1) KMAX + kb - 1
 };
 
-template <int KA, int KB, typename T>
-__device__ __forceinline__ cplx_t<T> pair_block(const PairAll& a, int w, int blk, const PairK<T>& ks)
-{
-    using T2 = cplx_t<T>;
-    const int idx = KA * (MSD_KMAX + 1) + KB, lo = a.pt.bucket[idx], n = a.pt.bucket[idx + 1] - lo;
-    T2 contrib = T2{0, 0};
-    for (int it = 0; it < PC_PER_THREAD; ++it) {
-        const int i0 = blk * (PC_THREADS * PC_PER_THREAD) + it * PC_THREADS + threadIdx.x;
-        if (i0 >= n) break;
-        const T2 v = pair_term<KA, KB, T>(a.t[0], a.t[1], a.pt, lo + i0, w, a.B[0], a.B[1], ks,
-                                          reinterpret_cast<const T2*>(a.r[0]), reinterpret_cast<const T2*>(a.r[1]));
-        contrib.x += v.x;
-        contrib.y += v.y;
-    }
-    return contrib;
-}
-
 template <typename T>
 __global__ void __launch_bounds__(PC_THREADS)
 k_pair_all(const __grid_constant__ PairAll a, double2* __restrict__ part, int nslot, int slot0)
 {
-    using T2 = cplx_t<T>;
     extern __shared__ __align__(16) unsigned char smraw[];
     const int XX = a.t[0].nh * a.t[0].np * a.t[1].nh * a.t[1].np;
     __shared__ double2 red[PC_THREADS];
@@ -137,9 +136,16 @@ k_pair_all(const __grid_constant__ PairAll a, double2* __restrict__ part, int ns
     int q = 0;
     while ((int)blockIdx.x >= a.blk[q + 1]) ++q;
     const int blk = (int)blockIdx.x - a.blk[q];
-    T2 v = T2{0, 0};
+    double2 v = cz(0, 0);
+    Limbs* bs = reinterpret_cast<Limbs*>(smraw) + XX;
     switch ((q / MSD_KMAX + 1) * 8 + q % MSD_KMAX + 1) {
-#define PAIR_CASE(A, B) case A * 8 + B: v = pair_block<A, B, T>(a, w, blk, ks); break;
+#define PAIR_CASE(KA, KB)                                                                                      \
+    case KA * 8 + KB: {                                                                                        \
+        const int i = KA * (MSD_KMAX + 1) + KB, lo = a.pt.bucket[i];                                           \
+        v = pair_block<KA, KB, T, true>(a.t[0], a.t[1], a.pt, lo, a.pt.bucket[i + 1] - lo, blk, w, a.B[0],     \
+                                        a.B[1], ks, a.r[0], a.r[1], bs);                                       \
+        break;                                                                                                 \
+    }
     PAIR_CASE(1, 1) PAIR_CASE(1, 2) PAIR_CASE(1, 3) PAIR_CASE(1, 4) PAIR_CASE(1, 5)
     PAIR_CASE(2, 1) PAIR_CASE(2, 2) PAIR_CASE(2, 3) PAIR_CASE(2, 4)
     PAIR_CASE(3, 1) PAIR_CASE(3, 2) PAIR_CASE(3, 3)
@@ -147,7 +153,7 @@ k_pair_all(const __grid_constant__ PairAll a, double2* __restrict__ part, int ns
     PAIR_CASE(5, 1)
 #undef PAIR_CASE
     }
-    red[t] = cz((double)v.x, (double)v.y);
+    red[t] = v;
     __syncthreads();
     for (int o = PC_THREADS / 2; o; o >>= 1) {
         if (t < o) red[t] = cadd(red[t], red[t + o]);
@@ -161,7 +167,7 @@ bool launch_pair_cross_all(const SpinTables& ta, const SpinTables& tb, const Pai
                            int nslot, int slot0, cudaStream_t st, bool use_runs)
 {
     PairAll a;
-    int n = 0, used = 0;
+    int n = 0, used = 0, limbs = 0;
     for (int ka = 1; ka <= MSD_KMAX; ++ka)
         for (int kb = 1; kb <= MSD_KMAX; ++kb) {
             const int idx = ka * (MSD_KMAX + 1) + kb, c = pt.bucket[idx + 1] - pt.bucket[idx];
@@ -169,13 +175,16 @@ bool launch_pair_cross_all(const SpinTables& ta, const SpinTables& tb, const Pai
             if (c <= 0) continue;
             if (ka + kb > 6 || (use_runs && pt.run_side[idx])) return false;
             n += (c + PC_THREADS * PC_PER_THREAD - 1) / (PC_THREADS * PC_PER_THREAD);
+            limbs = std::max(limbs, pair_limbs(ka, kb, PC_THREADS));
             ++used;
         }
     a.blk[MSD_KMAX * MSD_KMAX] = n;
     if (used < 2 || (long long)n * nw > ONE_LAUNCH_BLOCKS * msd_sm_count()) return false;
     a.t[0] = ta; a.t[1] = tb; a.pt = pt;
     a.r[0] = ra; a.r[1] = rb; a.B[0] = Ba; a.B[1] = Bb; a.K = K;
-    const size_t smem = (fp32 ? sizeof(float2) : sizeof(double2)) * (size_t)(ta.nh * ta.np) * (tb.nh * tb.np);
+    const size_t smem = (fp32 ? sizeof(float2) : sizeof(double2)) * (size_t)(ta.nh * ta.np) * (tb.nh * tb.np) +
+                        (fp32 ? 0 : sizeof(Limbs) * limbs);
+    if (!fp32 && !lanes_fit(smem, 1)) return false;
     if (fp32) {
         cudaFuncSetAttribute(k_pair_all<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         k_pair_all<float><<<dim3(n, nw), PC_THREADS, smem, st>>>(a, part, nslot, slot0);
