@@ -256,9 +256,11 @@ def algorithmic_work(s, n_w):
     w = {}
     # reference inverse: LU + inverse + Theta product + active block, both spins
     w["k_ref"] = sum(8 * (4 / 3 * sp["N"] ** 3 + M * sp["N"] ** 2 + sp["X"] * sp["N"]) for sp in spins) * n_w
-    # string minors: the FP64 part, LU with partial pivoting (k^3/3 complex
-    # MACs); the inverse from the factors runs in the working precision
-    w["k_strings"] = sum(float(np.sum(sp["lv"] * 8 * k ** 3 / 3)) for sp in spins) * n_w
+    # string minors: the FP64 part, expansions over all 2 x 2 minors of the
+    # active block (two complex products each) and, from level 3 on, k complex
+    # products per string; the inverse minors beside them are not counted
+    w["k_strings"] = sum(16.0 * sp["nh"] * (sp["nh"] - 1) * sp["np"] * (sp["np"] - 1) / 4
+                         + float(np.sum(sp["lv"][3:] * 8 * k[3:len(sp["lv"])])) for sp in spins) * n_w
     w["k_gemm_F"] = sum(4.0 * sp["N"] * M * G * sp["NC"] for sp in spins) * n_w
     w["k_fepi"] = sum(8.0 * (sp["N"] ** 2 + sp["N"] ** 2 * sp["np"] + sp["nh"] * sp["N"] * sp["np"]) * G
                       for sp in spins) * n_w
@@ -304,6 +306,10 @@ def algorithmic_work(s, n_w):
     return w, spins
 
 
+# FP64 mode: products by the exact-integer split on the tensor cores, and sums in
+# integer fixed point
+FP64_SPLIT = {"k_gemm_F", "k_gemm_vbias", "k_gemm_V", "k_gram", "k_apply_rows"}
+FP64_FIXED = {"k_fepi", "k_string_energy", "k_pair_cross", "k_pair_run"}
 FP64_KERNELS = {"k_ref", "k_strings", "k_weights", "k_gt", "k_onebody", "k_final", "k_sum_slots"}
 
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per launch of a
@@ -344,6 +350,11 @@ def kernel_peak(name, precision, peaks):
     if name.startswith("tc_"):
         return ("tensor", peaks["tf32_gflops"] / 3,
                 "measured TF32 GEMM / 3 products of the 3xTF32 split")
+    if precision == "fp64" and name in FP64_SPLIT:
+        return ("tensor", peaks["bf16_tflops"] * 1e3 / 36,
+                "measured bf16 burst / 36 BF16 slice products of the exact split")
+    if precision == "fp64" and name in FP64_FIXED:
+        return ("alu", peaks["fp64_gflops"], "measured FP64 GEMM (the sums run on the integer units: can exceed 1)")
     if precision == "fp64" or name in FP64_KERNELS:
         return ("alu", peaks["fp64_gflops"], "measured FP64 GEMM")
     return ("alu", peaks["fp32_gflops"], "measured FP32 GEMM (TF32 off)")
@@ -960,22 +971,22 @@ def run_prop(args, rank, world, local):
     work = {"k_gemm_V": 4.0 * M * M * G * n_w,
             "k_apply_rows": sum(2 * 4.0 * M * M * n + 6 * 8.0 * M * M * n for n in (s.n_alpha, s.n_beta)) * n_w}
     peaks, _ = load_peaks(dev)
-    fp64_peak = peaks["fp64_gflops"]
     kernels = {}
     for name, (n_launch, ms) in kstats.items():
         entry = {"launches": n_launch, "ms_per_step": ms / args.steps,
                  "share": ms / max(1e-9, sum(v[1] for v in kstats.values()))}
         if name in work and ms > 0:
             entry["gflops"] = work[name] * args.steps / (ms / 1e3) / 1e9
-            entry["frac"] = entry["gflops"] / fp64_peak
+            entry["frac"] = entry["gflops"] / kernel_peak(name, "fp64", peaks)[1]
         kernels[name] = entry
     dom = max(kstats.items(), key=lambda kv: kv[1][1])[0] if kstats else None
     roofline = None
     if dom is not None:
         d = kernels[dom]
-        roofline = {"kernel": dom, "bound": "alu", "achieved": d.get("gflops"), "peak": fp64_peak,
+        b, pk, src = kernel_peak(dom, "fp64", peaks)
+        roofline = {"kernel": dom, "bound": b, "achieved": d.get("gflops"), "peak": pk,
                     "unit": "GFLOP/s", "frac": d.get("frac"), "traffic": ncu_traffic(dom, "propagate"),
-                    "peak_source": "measured FP64 GEMM (" + peaks["alu_how"] + ")"}
+                    "peak_source": src}
     cpu = None
     if rank == 0 and world == 1 and not args.no_cpu_baseline:
         from oracle import prop_oracle

@@ -46,6 +46,8 @@ __device__ __forceinline__ PairK<T> load_pair_k(const void* Kin, int w, int XX, 
 // minor in fixed point (scales: K, and the string's largest entry) and the sum over
 // the shorter one's in FP64. The FP64 unit bounds the plain double sum, 4 k_a^2
 // k_b^2 FMAs: (3, 3) determinants 360 FP64 operations, here 52 and 972 mad.wide.
+// A thread per determinant, for the batched kernel (its items share a block shape);
+// the per-system kernels use pair_lanes.
 template <int KA, int KB>
 __device__ __forceinline__ double2 pair_term_fixed(const SpinTables& ta, const SpinTables& tbb, const PairTables& pt,
                                                    int I, int w, const void* __restrict__ Ba_in,
@@ -208,8 +210,8 @@ __device__ __forceinline__ double2 pair_lanes(const SpinTables& ta, const SpinTa
 }
 
 // One block's part of the opposite-spin term of levels (KA, KB), this thread's share:
-// in FP64 mode by groups of lanes where bs has room for their limbs (LANES), else a
-// thread per determinant.
+// in FP64 mode by groups of lanes (LANES, bs with room for their limbs), else a thread
+// per determinant.
 template <int KA, int KB, typename T, bool LANES>
 __device__ __forceinline__ double2 pair_block(const SpinTables& ta, const SpinTables& tbb, const PairTables& pt, int lo,
                                               int n, int blk, int w, const void* Ba, const void* Bb, const PairK<T>& kk,

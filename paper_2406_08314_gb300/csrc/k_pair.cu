@@ -114,9 +114,9 @@ bool launch_pair_cross2(int ka, int kb, bool fp32, dim3 grid, size_t smem, const
 
 // All level pairs in one launch, for calls whose blocks are few: a launch per
 // pair was most of this term's time there (7 us each, up to 15 of them). Block b
-// writes slot slot0 + b, the slots and values of the separate launches, which
-// stay where the blocks fill the GPU: one kernel for every pair takes the
-// registers of the largest.
+// writes slot slot0 + b, the slots of the separate launches (and in mixed mode their
+// values; in FP64 mode the same terms in the order of fewer lanes), which stay where
+// the blocks fill the GPU: one kernel for every pair takes the registers of the largest.
 struct PairAll {
     SpinTables t[2];
     PairTables pt;

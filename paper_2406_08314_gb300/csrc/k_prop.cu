@@ -1,6 +1,6 @@
 // One phaseless AFQMC propagation step (Sec. II A, Eq. 7-12), FP64:
 //   c_g     = i sqrt(dt) (x_g - xbar_g) = i sqrt(dt) x_g - dt vbias_g,  xbar = -i sqrt(dt) vbias
-//   V       = sum_g c_g L_g                                (a GEMM over g, k_gemm_zd)
+//   V       = sum_g c_g L_g                                (a GEMM over g)
 //   phi'    = E T_n(V) E phi,  E = exp(-dt h'/2),  T_n(V) = sum_{k<=n} V^k / k!
 //   I       = S exp(x.xbar - xbar.xbar/2),  S = O_T(phi') / O_T(phi)
 //   w'      = w |I| max(0, cos arg S)

@@ -214,7 +214,8 @@ int launch_refs(const RefSpinIn* in, int n_spin, int nw, int M, unsigned* err, c
 
 // ------------------------------------------------------------------------
 // Excitation strings of level K for one spin with their FP64 inverse minors
-// (the FP64 path; ratios alone and the mixed path's FP32 inverses: k_minors.cu):
+// by an LU of its own, for FP64 energies and force bias of trials whose sub-minors are
+// far more than their strings (all else: k_minors.cu):
 // A[i][j] = G[h_i][p_j] (a K x K minor of G). LU with partial pivoting in
 // FP64 gives r = sign * det A, the overlap ratio <D_s|phi>/<D_0|phi> of the
 // string's spin sector, and B = A^-1 from its factors, K*K entries

@@ -30,7 +30,8 @@ struct RefSpinIn {
 bool ref_dg_use(int M, int N);
 size_t ref_dg_bytes(int M, int N);   // that scratch per walker (0 if unused)
 int launch_refs(const RefSpinIn* in, int n_spin, int nw, int M, unsigned* err, cudaStream_t st);
-// FP64 ratios r[w][s] and rT[s][w] and FP64 inverse minors by pivoted LU.
+// FP64 ratios r[w][s] and rT[s][w] and FP64 inverse minors by pivoted LU (trials whose
+// sub-minors are too many for launch_inverse_ratios).
 void launch_strings(const SpinTables& tb, int nw, const double2* Gact, double2* r, double2* rT, void* B, cudaStream_t st,
                     const TimerHook& th);
 // k_minors.cu: FP64 ratios rT[s][w] of both spins by expansions over shared
