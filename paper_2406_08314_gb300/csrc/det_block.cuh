@@ -114,7 +114,7 @@ __device__ __forceinline__ cplx_t<T> pair_term(const SpinTables& ta, const SpinT
 // entries); where the shorter has one entry they are used as they are made. A thread
 // per determinant holds them and their table offsets in registers (226 at (2, 4), 164
 // at (3, 3)): 8 warps per SM, each instruction waiting for the last. 640 copper-oxo
-// walkers 3.31 -> 2.12 ms, 64 iron-sulfur ones 3.37 -> 2.24.
+// walkers 3.31 -> 2.05 ms, 64 iron-sulfur ones 3.37 -> 2.24.
 __host__ __device__ __forceinline__ constexpr int pair_group(int ka, int kb)
 {
     const int ko = ka < kb ? ka : kb;
@@ -170,7 +170,7 @@ __device__ __forceinline__ double2 pair_lanes(const SpinTables& ta, const SpinTa
         int hx[KI];
 #pragma unroll
         for (int l = 0; l < KI; ++l) hx[l] = rec_h(ri, l) * npi * si;
-        double xr = 0, xim = 0;
+        double2 x = cz(0, 0);
         if constexpr (G > 1) {
             __syncwarp();   // the previous determinants' limbs consumed
             if (g < DPW)
@@ -198,12 +198,12 @@ __device__ __forceinline__ double2 pair_lanes(const SpinTables& ta, const SpinTa
                 }
             }
             const double2 z = limb_value(s, kk.e + eb), bo = Bo[e];
-            xr += bo.x * z.x - bo.y * z.y;
-            xim += bo.x * z.y + bo.y * z.x;
+            x = cfma(bo, z, x);
         }
         if (on) {
-            if (max(kk.e, eb) >= FIXED_EXP_INF) xr = xim = __longlong_as_double(0x7ff8000000000000ll);
-            sum = cadd(sum, pair_weight_times<double>(pt, I, rav, rbv, xr, xim));
+            if (max(kk.e, eb) >= FIXED_EXP_INF) x.x = x.y = __longlong_as_double(0x7ff8000000000000ll);
+            // fused explicitly: the same rounding in every kernel that holds this
+            sum = cfma(cfma(rav, rbv, cz(0, 0)), cscale(x, pt.c[I]), sum);
         }
     }
     return sum;
@@ -392,9 +392,9 @@ __device__ __forceinline__ double2 string_energy_block(const SpinTables& tb, int
             const int sl = blk * (SE_THREADS * SE_PER_THREAD) + it * SE_THREADS + threadIdx.x;
             if (sl >= ns) break;
             if constexpr (std::is_same<T, double>::value)
-                sum = cadd(sum, cmul(wts[(size_t)w * tb.n_str + tb.bucket[KL] + sl],
-                                     string_energy_fixed<KL>(tb, w, sl, ns, B, reinterpret_cast<const Limbs*>(tab.as), tab.ea,
-                                                             reinterpret_cast<const Limbs*>(tab.ys), tab.ey)));
+                sum = cfma(wts[(size_t)w * tb.n_str + tb.bucket[KL] + sl],
+                           string_energy_fixed<KL>(tb, w, sl, ns, B, reinterpret_cast<const Limbs*>(tab.as), tab.ea,
+                                                   reinterpret_cast<const Limbs*>(tab.ys), tab.ey), sum);
             else
                 sum = cadd(sum, string_energy_term<KL, T, true>(tb, w, sl, ns, B, tab.as, tab.ys, wts));
         }

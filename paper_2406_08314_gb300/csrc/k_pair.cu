@@ -12,6 +12,33 @@
 #include "det_block.cuh"
 #include "kernels.h"
 
+// The block's total, on thread 0: in FP64 mode the lanes of a warp, then the warps in
+// order (red: 32), else a tree (red: PC_THREADS).
+template <typename T>
+__device__ __forceinline__ double2 block_total(double2 v, double2* red)
+{
+    const int t = threadIdx.x;
+    if constexpr (std::is_same<T, double>::value) {
+#pragma unroll
+        for (int o = 16; o; o >>= 1) {
+            v.x += __shfl_down_sync(0xffffffffu, v.x, o);
+            v.y += __shfl_down_sync(0xffffffffu, v.y, o);
+        }
+        if ((t & 31) == 0) red[t >> 5] = v;
+        __syncthreads();
+        for (int q = 1; t == 0 && q < (int)(blockDim.x >> 5); ++q) v = cadd(v, red[q]);
+        return v;
+    } else {
+        red[t] = v;
+        __syncthreads();
+        for (int o = PC_THREADS / 2; o; o >>= 1) {
+            if (t < o) red[t] = cadd(red[t], red[t + o]);
+            __syncthreads();
+        }
+        return red[0];
+    }
+}
+
 // Mixed mode: PC_THREADS threads, one per determinant; FP64 mode: groups of lanes,
 // any number of warps.
 template <int KA, int KB, typename T>
@@ -28,30 +55,14 @@ k_pair_cross2(SpinTables ta, SpinTables tbb, PairTables pt, int lo, int n, const
     const PairK<T> ks = load_pair_k<T>(Kin, w, XX, smraw);   // [Xa][Xb]
     double2 v = pair_block<KA, KB, T, LANES>(ta, tbb, pt, lo, n, blockIdx.x, w, Ba, Bb, ks, ra, rb,
                                              reinterpret_cast<Limbs*>(smraw) + XX);
-    if constexpr (LANES) {
-#pragma unroll
-        for (int o = 16; o; o >>= 1) {
-            v.x += __shfl_down_sync(0xffffffffu, v.x, o);
-            v.y += __shfl_down_sync(0xffffffffu, v.y, o);
-        }
-        if ((t & 31) == 0) red[t >> 5] = v;
-        __syncthreads();
-        for (int q = 1; t == 0 && q < (int)(blockDim.x >> 5); ++q) v = cadd(v, red[q]);
-    } else {
-        red[t] = v;
-        __syncthreads();
-        for (int o = PC_THREADS / 2; o; o >>= 1) {
-            if (t < o) red[t] = cadd(red[t], red[t + o]);
-            __syncthreads();
-        }
-        v = red[0];
-    }
+    v = block_total<T>(v, red);
     if (t == 0) part[(size_t)w * nslot + slot0 + blockIdx.x] = v;
 }
 
 // Shared memory of a block in the lanes form, beside its static part.
 static size_t lanes_smem(size_t k_bytes, int limbs) { return k_bytes + sizeof(Limbs) * limbs; }
 static bool lanes_fit(size_t dyn, int blocks) { return (dyn + 5 * 1024) * blocks <= 227 * 1024; }
+#define PL_THREADS 512   // two blocks per SM
 
 template <int KA, int KB>
 static bool go(bool fp32, dim3 grid, size_t smem, const SpinTables& ta, const SpinTables& tb, const PairTables& pt,
@@ -71,7 +82,7 @@ static bool go(bool fp32, dim3 grid, size_t smem, const SpinTables& ta, const Sp
     // matrix while the other computes, else one of 1024 (75 x 75 active pairs); fewer
     // only beside the largest Gram matrices (112 x 112: 196 KB)
     auto bytes = [&](int threads) { return lanes_smem(smem, pair_limbs(KA, KB, threads)); };
-    int threads = lanes_fit(bytes(512), 2) ? 512 : 1024;
+    int threads = lanes_fit(bytes(PL_THREADS), 2) ? PL_THREADS : 1024;
     while (threads > 64 && !lanes_fit(bytes(threads), 1)) threads /= 2;
     run(k_pair_cross2<KA, KB, double>, threads, bytes(threads));
     return true;
@@ -114,9 +125,10 @@ bool launch_pair_cross2(int ka, int kb, bool fp32, dim3 grid, size_t smem, const
 
 // All level pairs in one launch, for calls whose blocks are few: a launch per
 // pair was most of this term's time there (7 us each, up to 15 of them). Block b
-// writes slot slot0 + b, the slots of the separate launches (and in mixed mode their
-// values; in FP64 mode the same terms in the order of fewer lanes), which stay where
-// the blocks fill the GPU: one kernel for every pair takes the registers of the largest.
+// writes slot slot0 + b, the slots and values of the separate launches, which stay
+// where the blocks fill the GPU: one kernel for every pair takes the registers of the
+// largest. (FP64: where those take PL_THREADS too, so that a walker's value does not
+// depend on how many there are.)
 struct PairAll {
     SpinTables t[2];
     PairTables pt;
@@ -125,12 +137,12 @@ struct PairAll {
 };
 
 template <typename T>
-__global__ void __launch_bounds__(PC_THREADS)
+__global__ void __launch_bounds__(std::is_same<T, double>::value ? PL_THREADS : PC_THREADS)
 k_pair_all(const __grid_constant__ PairAll a, double2* __restrict__ part, int nslot, int slot0)
 {
     extern __shared__ __align__(16) unsigned char smraw[];
     const int XX = a.t[0].nh * a.t[0].np * a.t[1].nh * a.t[1].np;
-    __shared__ double2 red[PC_THREADS];
+    __shared__ double2 red[std::is_same<T, double>::value ? 32 : PC_THREADS];
     const int w = blockIdx.y, t = threadIdx.x;
     const PairK<T> ks = load_pair_k<T>(a.K, w, XX, smraw);   // [Xa][Xb]
     int q = 0;
@@ -153,13 +165,8 @@ k_pair_all(const __grid_constant__ PairAll a, double2* __restrict__ part, int ns
     PAIR_CASE(5, 1)
 #undef PAIR_CASE
     }
-    red[t] = v;
-    __syncthreads();
-    for (int o = PC_THREADS / 2; o; o >>= 1) {
-        if (t < o) red[t] = cadd(red[t], red[t + o]);
-        __syncthreads();
-    }
-    if (t == 0) part[(size_t)w * nslot + slot0 + blockIdx.x] = red[0];
+    v = block_total<T>(v, red);
+    if (t == 0) part[(size_t)w * nslot + slot0 + blockIdx.x] = v;
 }
 
 bool launch_pair_cross_all(const SpinTables& ta, const SpinTables& tb, const PairTables& pt, int nw, const void* ra,
@@ -175,7 +182,7 @@ bool launch_pair_cross_all(const SpinTables& ta, const SpinTables& tb, const Pai
             if (c <= 0) continue;
             if (ka + kb > 6 || (use_runs && pt.run_side[idx])) return false;
             n += (c + PC_THREADS * PC_PER_THREAD - 1) / (PC_THREADS * PC_PER_THREAD);
-            limbs = std::max(limbs, pair_limbs(ka, kb, PC_THREADS));
+            limbs = std::max(limbs, pair_limbs(ka, kb, PL_THREADS));
             ++used;
         }
     a.blk[MSD_KMAX * MSD_KMAX] = n;
@@ -184,13 +191,13 @@ bool launch_pair_cross_all(const SpinTables& ta, const SpinTables& tb, const Pai
     a.r[0] = ra; a.r[1] = rb; a.B[0] = Ba; a.B[1] = Bb; a.K = K;
     const size_t smem = (fp32 ? sizeof(float2) : sizeof(double2)) * (size_t)(ta.nh * ta.np) * (tb.nh * tb.np) +
                         (fp32 ? 0 : sizeof(Limbs) * limbs);
-    if (!fp32 && !lanes_fit(smem, 1)) return false;
+    if (!fp32 && !lanes_fit(smem, 2)) return false;   // the separate launches take another block size
     if (fp32) {
         cudaFuncSetAttribute(k_pair_all<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         k_pair_all<float><<<dim3(n, nw), PC_THREADS, smem, st>>>(a, part, nslot, slot0);
     } else {
         cudaFuncSetAttribute(k_pair_all<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k_pair_all<double><<<dim3(n, nw), PC_THREADS, smem, st>>>(a, part, nslot, slot0);
+        k_pair_all<double><<<dim3(n, nw), PL_THREADS, smem, st>>>(a, part, nslot, slot0);
     }
     msd_note_launch();
     return true;

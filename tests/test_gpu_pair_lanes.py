@@ -49,3 +49,22 @@ def test_energy(n_o, n_act, pairs, n_w):
     assert np.all(np.abs(e - ref["e_loc"]) <= 1e-10 * scale)   # the parity tests' bound
     assert np.abs(one[0] - e[0]) <= 1e-12 * scale[0]
     ctx.close()
+
+
+def test_one_launch_and_separate_launches_agree():
+    """Few walkers take every level pair in one launch, many a launch per pair: the
+    same value for the same walker."""
+    import torch
+
+    from paper_2406_08314_gb300 import msd, synth
+    n_o, n_act, n_w = 5, 10, 200
+    s = synth.make_system(11, n_act + 2, n_o, n_o, 0, n_act, 6, 12, 0.7, 10)
+    s = _trial(s, n_o, n_act, [(1, 1, 25), (1, 2, 30), (2, 2, 400), (3, 3, 500), (2, 4, 50), (4, 2, 31), (1, 5, 3)], 5)
+    w = synth.make_walkers(np.random.default_rng(4), n_act + 2, n_o, n_o, n_w, noise=0.4)
+    da, db = torch.from_numpy(w.phi_a).cuda(), torch.from_numpy(w.phi_b).cuda()
+    for precision in ("fp64", "mixed"):
+        ctx = msd.Context(s, precision)
+        e = ctx.local_energy(da, db)
+        few = ctx.local_energy(da[:3].contiguous(), db[:3].contiguous())
+        assert torch.equal(e[:3], few), precision
+        ctx.close()
