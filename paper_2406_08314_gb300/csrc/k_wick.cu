@@ -20,7 +20,11 @@
 // one thread per column with a serial chain: 35 us for a 5 x 5 block, and two
 // thirds of the inversion's FP64 operations on one warp). The product with phi,
 // (M - N) N^2 complex FMAs and most of the FP64 work at larger N, runs on the
-// tensor cores from ref_dg_use on (S^-1 then goes out to Sinv), else here.
+// tensor cores from ref_dg_use on (S^-1 then goes out to Sinv), else here. Its operands
+// are rounded to 56 bits of a row's largest value over the walker's columns, and G does
+// not depend on the columns' scales: so column k of phi enters as phi_k 2^-e_k, |phi_k|
+// < 2^e_k, and row k of S^-1 as 2^e_k of it (exact; without it columns 1e8 apart left 9
+// digits of G). Reading phi once more for the e_k: k_ref 1.15 -> 1.15 ms as below.
 // Measured, both spins: N = 5, 16 walkers 70 -> 21 us; iron-sulfur (N = 30, M = 160)
 // 640 walkers 1.95 -> 1.15 ms, 64 walkers 0.81 -> 0.24 ms; copper-oxo (N = 16, M =
 // 108) 640 walkers 0.73 -> 0.46 ms.
@@ -31,6 +35,7 @@ struct RefIn {
     double2 *Gr, *O0;
     double2 *Gact, *GactT;  // [nw][nh np], [nh np][nw] (either may be NULL)
     double2* Sinv;          // [nw][N][N], or NULL: form Gr and the active block here
+    double* cs;             // [nw][N] with Sinv: the columns' scales
 };
 struct RefArgs { RefIn s[2]; };
 
@@ -52,6 +57,7 @@ k_ref(const __grid_constant__ RefArgs args, int M, unsigned* err)
     __shared__ double2 prow[MSD_NMAX], pcol[MSD_NMAX], pinv;
     __shared__ int piv[MSD_NMAX], col[MSD_NMAX];
     __shared__ double cn[MSD_NMAX];
+    __shared__ int ce[MSD_NMAX];     // with Sinv: largest magnitude (high word), then exponent of phi's columns
     __shared__ int singular;
     const RefIn& R = args.s[blockIdx.y];
     const int w = blockIdx.x, nw = gridDim.x, N = R.N;
@@ -60,8 +66,18 @@ k_ref(const __grid_constant__ RefArgs args, int M, unsigned* err)
 
     for (int e = t; e < N * N; e += nt) S[e] = ph[(size_t)R.occ0[e / N] * N + e % N];
     if (t == 0) singular = 0;
+    if (R.Sinv)
+        for (int j = t; j < N; j += nt) ce[j] = 0;
     __syncthreads();
+    if (R.Sinv) {
+        for (int e = t; e < M * N; e += nt) atomicMax(&ce[e % N], mag_key(ph[e]));
+        __syncthreads();
+    }
     for (int j = t; j < N; j += nt) {
+        if (R.Sinv) {
+            ce[j] = min(1000, max(-1000, (ce[j] >> 20) - 1022));
+            R.cs[(size_t)w * N + j] = ldexp(1.0, -ce[j]);
+        }
         double a = 0;
         for (int i = 0; i < N; ++i) a += S[i * N + j].x * S[i * N + j].x + S[i * N + j].y * S[i * N + j].y;
         cn[j] = sqrt(a);
@@ -124,7 +140,8 @@ k_ref(const __grid_constant__ RefArgs args, int M, unsigned* err)
     double2* gr = R.Gr + (size_t)w * N * M;
     if (R.Sinv) {
         double2* out = R.Sinv + (size_t)w * N * N;
-        for (int e = t; e < N * N; e += nt) out[e] = singular ? cz(0, 0) : S[e - e % N + col[e % N]];
+        for (int e = t; e < N * N; e += nt)   // row k: of S^-1, so of the walker's column k
+            out[e] = singular ? cz(0, 0) : cscale(S[e - e % N + col[e % N]], ldexp(1.0, ce[e / N]));
         return;
     }
     for (int e = t; e < M * N; e += nt) {
@@ -169,7 +186,8 @@ __global__ void __launch_bounds__(256) k_gact(const __grid_constant__ RefArgs ar
 bool ref_dg_use(int M, int N) { return (long long)(M - N) * N * N >= 16384; }
 size_t ref_dg_bytes(int M, int N)
 {
-    return ref_dg_use(M, N) ? sizeof(double2) * (size_t)N * N + dg_row_bytes(2 * N) * (M + 2 * (size_t)N) : 0;
+    return ref_dg_use(M, N) ? sizeof(double2) * (size_t)N * N + sizeof(double) * N + dg_row_bytes(2 * N) * (M + 2 * (size_t)N)
+                            : 0;
 }
 
 int launch_refs(const RefSpinIn* in, int n_spin, int nw, int M, unsigned* err, cudaStream_t st)
@@ -180,7 +198,7 @@ int launch_refs(const RefSpinIn* in, int n_spin, int nw, int M, unsigned* err, c
     for (int s = 0; s < n_spin; ++s) {
         const SpinTables& T = *in[s].T;
         a.s[s] = RefIn{in[s].phi, T.N, T.nh, T.np, T.occ0, T.pos0, T.hole_pos, T.part_orb, in[s].Gr, in[s].O0, in[s].Gact,
-                       in[s].GactT, in[s].Sinv};
+                       in[s].GactT, in[s].Sinv, in[s].cs};
         Nmax = Nmax > T.N ? Nmax : T.N;
         X = X > T.nh * T.np ? X : T.nh * T.np;
         dg = dg || in[s].Sinv;
@@ -195,7 +213,7 @@ int launch_refs(const RefSpinIn* in, int n_spin, int nw, int M, unsigned* err, c
     for (int s = 0; s < n_spin; ++s) {
         if (!in[s].Sinv) continue;
         const int N = in[s].T->N;
-        dg_slice_real((long long)nw * M, 2 * N, (const double*)in[s].phi, 2 * N, in[s].sa, in[s].ea, st);
+        dg_slice_real((long long)nw * M, 2 * N, (const double*)in[s].phi, 2 * N, in[s].sa, in[s].ea, st, in[s].cs, M);
         dg_slice_columns(1, N, N, nw, in[s].Sinv, N, (long long)N * N, 0, N, nullptr, nullptr, in[s].sb, in[s].eb, st);
         DgOut o;
         o.Mr = M; o.Nc = N; o.batch = nw;

@@ -16,14 +16,15 @@ struct TimerHook {
 
 // k_wick.cu
 // Reference inverse of one spin: inputs, outputs and, where ref_dg_use, the
-// scratch of the tensor-core product (Sinv [nw][N][N]; sa, ea: M rows, sb, eb: 2 N
-// rows of dg_row_bytes(2 N) per walker; all NULL otherwise). GactT: the active
-// block with the walkers contiguous, [nh np][nw].
+// scratch of the tensor-core product (Sinv [nw][N][N]; cs [nw][N], the columns' scales;
+// sa, ea: M rows, sb, eb: 2 N rows of dg_row_bytes(2 N) per walker; all NULL
+// otherwise). GactT: the active block with the walkers contiguous, [nh np][nw].
 struct RefSpinIn {
     const SpinTables* T = nullptr;
     const double2* phi = nullptr;
     double2 *Gr = nullptr, *O0 = nullptr, *Gact = nullptr, *GactT = nullptr;
     double2* Sinv = nullptr;
+    double* cs = nullptr;
     void *sa = nullptr, *sb = nullptr;
     int *ea = nullptr, *eb = nullptr;
 };
@@ -202,7 +203,10 @@ struct DgOut {
 int dg_k_padded(int K);
 size_t dg_row_bytes(int K);              // slices and exponent of one real row
 int dg_splits(int Mr, int K);
-void dg_slice_real(long long R, int K, const double* src, long long ld, void* S, int* ex, cudaStream_t st);
+// scale (optional): row r's elements 2 k and 2 k + 1 times scale[r / rows][k], a power
+// of two (K / 2 of them).
+void dg_slice_real(long long R, int K, const double* src, long long ld, void* S, int* ex, cudaStream_t st,
+                   const double* scale = nullptr, int rows = 1);
 void dg_slice_complex(long long R, int K, const double2* src, long long ld, void* S, int* ex, cudaStream_t st);
 // Columns of src[z][k][c] (k < K, c < nc) as the operand rows z rows + row0 + c:
 // mode 0 a left operand (Sa, length 2 K) and the matching complex right operand

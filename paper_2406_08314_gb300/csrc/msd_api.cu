@@ -1423,8 +1423,8 @@ int run_refs(msd_ctx* ctx, const Staged& in, int w0, int nw, int cap, Chunk& c, 
     const TimerHook& th = ctx->hook;
     const SpinTables T[2] = {tables(ctx->sp[0], cap), tables(ctx->sp[1], cap)};
     RefSpinIn r[2];
-    static const char* names[2][5] = {{"ref_inv_a", "ref_sa_a", "ref_ea_a", "ref_sb_a", "ref_eb_a"},
-                                      {"ref_inv_b", "ref_sa_b", "ref_ea_b", "ref_sb_b", "ref_eb_b"}};
+    static const char* names[2][6] = {{"ref_inv_a", "ref_sa_a", "ref_ea_a", "ref_sb_a", "ref_eb_a", "ref_cs_a"},
+                                      {"ref_inv_b", "ref_sa_b", "ref_ea_b", "ref_sb_b", "ref_eb_b", "ref_cs_b"}};
     for (int s = 0; s < 2; ++s) {
         const int N = ctx->n[s];
         r[s].T = &T[s];
@@ -1439,6 +1439,7 @@ int run_refs(msd_ctx* ctx, const Staged& in, int w0, int nw, int cap, Chunk& c, 
         if ((rc = arena_get(ctx, names[s][2], sizeof(int) * cap * (size_t)M, (void**)&r[s].ea))) return rc;
         if ((rc = arena_get(ctx, names[s][3], rb * cap * 2 * (size_t)N, &r[s].sb))) return rc;
         if ((rc = arena_get(ctx, names[s][4], sizeof(int) * cap * 2 * (size_t)N, (void**)&r[s].eb))) return rc;
+        if ((rc = arena_get(ctx, names[s][5], sizeof(double) * cap * (size_t)N, (void**)&r[s].cs))) return rc;
     }
     th.begin("k_ref", st);
     int g = launch_refs(r, in.b_ready ? 1 : 2, nw, M, ctx->d_err, st);

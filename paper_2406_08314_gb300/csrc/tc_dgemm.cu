@@ -390,16 +390,19 @@ __device__ __forceinline__ unsigned dg_mag(double x) { return (unsigned)__double
 
 // Rows of a row-major matrix: src[r ld + k], real, or the two parts of a complex
 // row as rows 2r, 2r + 1. LR lanes per row, each 8 consecutive elements of the
-// row at a time (one 16-byte store per digit).
-template <bool CPLX, int LR>
+// row at a time (one 16-byte store per digit). SCALED: elements 2 k, 2 k + 1 of a real
+// row times scale[r / rows][k].
+template <bool CPLX, int LR, bool SCALED>
 __global__ void __launch_bounds__(256)
 k_dg_rows(long long R, int K, int Kp, const double* __restrict__ src, long long ld, __nv_bfloat16* __restrict__ S,
-          int* __restrict__ ex, size_t stride)
+          int* __restrict__ ex, size_t stride, const double* __restrict__ scale, int rows)
 {
     const long long r = ((long long)blockIdx.x * 256 + threadIdx.x) / LR;
     const int lane = threadIdx.x % LR;
     const bool live = r < R;
     const double* p = src + (CPLX ? 2 : 1) * (live ? r : 0) * ld;
+    const double* sc = SCALED ? scale + (live ? r / rows : 0) * (K / 2) : nullptr;
+    auto at = [&](int k) { return SCALED ? p[k] * sc[k >> 1] : p[k]; };
     unsigned t0 = 0, t1 = 0;
     if (live) {
         if (CPLX) {
@@ -410,7 +413,7 @@ k_dg_rows(long long R, int K, int Kp, const double* __restrict__ src, long long 
                 t1 = max(t1, dg_mag(v.y));
             }
         } else {
-            for (int k = lane; k < K; k += LR) t0 = max(t0, dg_mag(p[k]));
+            for (int k = lane; k < K; k += LR) t0 = max(t0, dg_mag(at(k)));
         }
     }
 #pragma unroll
@@ -435,7 +438,7 @@ k_dg_rows(long long R, int K, int Kp, const double* __restrict__ src, long long 
                 q0[j] = fixed56(v.x, e0);
                 q1[j] = fixed56(v.y, e1);
             } else {
-                q0[j] = fixed56(k < K ? p[k] : 0.0, e0);
+                q0[j] = fixed56(k < K ? at(k) : 0.0, e0);
             }
         }
         dg_store8(q0, o0 + k0, stride);
@@ -443,18 +446,19 @@ k_dg_rows(long long R, int K, int Kp, const double* __restrict__ src, long long 
     }
 }
 
-template <bool CPLX>
-void launch_dg_rows(long long R, int K, const double* src, long long ld, void* S, int* ex, size_t stride, cudaStream_t st)
+template <bool CPLX, bool SCALED = false>
+void launch_dg_rows(long long R, int K, const double* src, long long ld, void* S, int* ex, size_t stride, cudaStream_t st,
+                    const double* scale = nullptr, int rows = 1)
 {
     const int Kp = dg_k_padded(K);
     // lanes per row: as many as have a group of 8 elements to write
     const int lr = Kp > 128 ? 32 : Kp > 64 ? 16 : Kp > 32 ? 8 : 4;
     const unsigned grid = (unsigned)((R * lr + 255) / 256);
     __nv_bfloat16* s = (__nv_bfloat16*)S;
-    if (lr == 32) k_dg_rows<CPLX, 32><<<grid, 256, 0, st>>>(R, K, Kp, src, ld, s, ex, stride);
-    else if (lr == 16) k_dg_rows<CPLX, 16><<<grid, 256, 0, st>>>(R, K, Kp, src, ld, s, ex, stride);
-    else if (lr == 8) k_dg_rows<CPLX, 8><<<grid, 256, 0, st>>>(R, K, Kp, src, ld, s, ex, stride);
-    else k_dg_rows<CPLX, 4><<<grid, 256, 0, st>>>(R, K, Kp, src, ld, s, ex, stride);
+    if (lr == 32) k_dg_rows<CPLX, 32, SCALED><<<grid, 256, 0, st>>>(R, K, Kp, src, ld, s, ex, stride, scale, rows);
+    else if (lr == 16) k_dg_rows<CPLX, 16, SCALED><<<grid, 256, 0, st>>>(R, K, Kp, src, ld, s, ex, stride, scale, rows);
+    else if (lr == 8) k_dg_rows<CPLX, 8, SCALED><<<grid, 256, 0, st>>>(R, K, Kp, src, ld, s, ex, stride, scale, rows);
+    else k_dg_rows<CPLX, 4, SCALED><<<grid, 256, 0, st>>>(R, K, Kp, src, ld, s, ex, stride, scale, rows);
     msd_note_launch();
 }
 
@@ -564,9 +568,12 @@ __global__ void k_dg_sum(int R, int Cc, int splits, const double2* __restrict__ 
 int dg_k_padded(int K) { return (K + DG_BK - 1) / DG_BK * DG_BK; }
 size_t dg_row_bytes(int K) { return (size_t)DG_S * dg_k_padded(K) * sizeof(__nv_bfloat16) + sizeof(int); }
 
-void dg_slice_real(long long R, int K, const double* src, long long ld, void* S, int* ex, cudaStream_t st)
+void dg_slice_real(long long R, int K, const double* src, long long ld, void* S, int* ex, cudaStream_t st,
+                   const double* scale, int rows)
 {
-    launch_dg_rows<false>(R, K, src, ld, S, ex, (size_t)R * dg_k_padded(K), st);
+    const size_t stride = (size_t)R * dg_k_padded(K);
+    if (scale) launch_dg_rows<false, true>(R, K, src, ld, S, ex, stride, st, scale, rows);
+    else launch_dg_rows<false>(R, K, src, ld, S, ex, stride, st);
 }
 
 void dg_slice_complex(long long R, int K, const double2* src, long long ld, void* S, int* ex, cudaStream_t st)
