@@ -235,54 +235,32 @@ __device__ __forceinline__ double2 pair_block(const SpinTables& ta, const SpinTa
     }
 }
 
-// FP64 mode, levels 1 and 2 (string_energy_lanes: 3 to 6): e_s of string_energy_value with the sums over the pair
-// table and over Y in fixed point (the FP64 unit bounds the plain form: level 4, 496
-// FP64 operations per string; here 48 and 1056 mad.wide):
-//   e_s = sum_ij b_ij Y[h_j][p_i] + sum_{i < k-1} sum_j b_ij z_ij,
-//   z_ij = sum_{m > i} sum_{l != j} (+ for l > j, - for l < j) b_ml A[h_j,h_l;p_i,p_m].
-// Scales: A, Y per walker (exponents ea, ey), b the string's largest entry.
+// FP64 mode, levels 1 and 2 (string_energy_lanes: 3 to 6): e_s of string_energy_value
+// with the sum over Y in fixed point (scales: Y per walker, exponent ey, and the string's
+// largest entry) and, level 2, its one pair of entries in FP64.
 template <int KL>
 __device__ __forceinline__ double2 string_energy_fixed(const SpinTables& tb, int w, int sl, int ns, const void* Bin,
                                                        const Limbs* as, int ea, const Limbs* ys, int ey)
 {
+    static_assert(KL <= 2, "one pair of holes and particles at most");
     const int np = tb.np, nh = tb.nh, npp = np * (np - 1) / 2;
     const uint4 rec = tb.str_hp[tb.bucket[KL] + sl];
     const double2* B = reinterpret_cast<const double2*>(Bin) + (size_t)tb.b_off[KL] + ((size_t)w * ns + sl) * b_stride(KL);
-    Limbs b[KL * KL];
-    int eb;
-    {
-        unsigned m = 0;
+    double2 b[KL * KL];
+    unsigned m = 0;
 #pragma unroll
-        for (int e = 0; e < KL * KL; ++e) m = max(m, mag_bits(B[e]));
-        eb = mag_exponent(m);
-#pragma unroll
-        for (int e = 0; e < KL * KL; ++e) b[e] = to_limbs(B[e], eb);
-    }
+    for (int e = 0; e < KL * KL; ++e) { b[e] = B[e]; m = max(m, mag_bits(b[e])); }
+    const int eb = mag_exponent(m);
     LimbSum lin;
 #pragma unroll
     for (int i = 0; i < KL; ++i)
 #pragma unroll
-        for (int j = 0; j < KL; ++j) lin.add(b[i * KL + j], ys[rec_h(rec, j) * np + rec_p(rec, i)]);
+        for (int j = 0; j < KL; ++j) lin.add(to_limbs(b[i * KL + j], eb), ys[rec_h(rec, j) * np + rec_p(rec, i)]);
     double2 v = limb_value(lin, eb + ey);
-#pragma unroll
-    for (int i = 0; i + 1 < KL; ++i)
-#pragma unroll
-        for (int j = 0; j < KL; ++j) {
-            LimbSum z;
-#pragma unroll
-            for (int m = i + 1; m < KL; ++m) {
-                const int pim = pair_index(rec_p(rec, i), rec_p(rec, m), np);
-#pragma unroll
-                for (int l = 0; l < KL; ++l) {
-                    if (l == j) continue;
-                    const int hp = l > j ? pair_index(rec_h(rec, j), rec_h(rec, l), nh)
-                                         : pair_index(rec_h(rec, l), rec_h(rec, j), nh);
-                    if (l > j) z.add(b[m * KL + l], as[hp * npp + pim]);
-                    else z.sub(b[m * KL + l], as[hp * npp + pim]);
-                }
-            }
-            v = cfma(B[i * KL + j], limb_value(z, eb + ea), v);
-        }
+    if constexpr (KL == 2) {
+        const int x = pair_index(rec_h(rec, 0), rec_h(rec, 1), nh) * npp + pair_index(rec_p(rec, 0), rec_p(rec, 1), np);
+        v = cfma(cfms(b[1], b[2], cfma(b[0], b[3], cz(0, 0))), limbs_fp64(as[x], ea), v);   // fused explicitly, as pair_lanes
+    }
     if (max(max(ea, ey), eb) >= FIXED_EXP_INF) v.x = v.y = __longlong_as_double(0x7ff8000000000000ll);
     return v;
 }
@@ -303,13 +281,27 @@ __host__ __device__ __forceinline__ constexpr int se_pitch(int k) { return (k * 
 #define SE_LIMBS (SE_THREADS / 8 * se_pitch(MSD_KMAX) > SE_THREADS / 4 * se_pitch(4) \
                       ? SE_THREADS / 8 * se_pitch(MSD_KMAX) : SE_THREADS / 4 * se_pitch(4))
 
-// FP64 mode, levels 3 to 6: this block's strings (SE_THREADS SE_PER_THREAD from blk) in
-// the sums of string_energy_fixed, a group of 4 or 8 lanes to a string, lane j taking
-// the columns j: b_ij Y[h_j][p_i] and b_ij z_ij for all i. The string's limbs are made
-// once, by the group's lanes, in shared memory. A thread per string holds them in
-// registers (254 at level 4: 8 warps per SM, every instruction waiting for the last)
-// and leaves the SM idle where strings are few (one level-6 string in 640 walkers: 0.66
-// ms). 640 copper-oxo walkers, levels 3 to 6: 2.94 -> 1.31 ms.
+// FP64 mode, levels 3 to 6: this block's strings (SE_THREADS SE_PER_THREAD from blk),
+// e_s of string_energy_value with its long sums in fixed point (the FP64 unit bounds the
+// plain form: level 4, 496 FP64 operations per string; here 48 and 1056 mad.wide):
+//   e_s = sum_ij b_ij Y[h_j][p_i] + sum_{i < k-1} sum_j b_ij z_ij,
+//   z_ij = sum_{m > i} sum_{l != j} (+ for l > j, - for l < j) b_ml A[h_j,h_l;p_i,p_m].
+// Scales: A, Y per walker (exponents ea, ey), b the string's largest entry. A group of 4
+// or 8 lanes takes a string, lane j the columns j: b_ij Y[h_j][p_i] and b_ij z_ij for all
+// i. The string's limbs are made once, by the group's lanes, in shared memory. A thread
+// per string holds them in registers (254 at level 4: 8 warps per SM, every instruction
+// waiting for the last) and leaves the SM idle where strings are few (one level-6 string
+// in 640 walkers: 0.66 ms). 640 copper-oxo walkers, levels 3 to 6: 2.94 -> 1.31 ms.
+//
+// The b_ml of z_ij carry 54 bits of the string's largest entry b_ab, and the term is of
+// the size of the largest product b_ij b_ml, i != m, j != l: of
+//   b_ab max_{m != a, l != b} b_ml   or   max_{m != a} b_mb max_{l != b} b_al,
+// far below b_ab^2 where a column or row of b is large by itself (a hole or particle that
+// the walker mixes with a small amplitude x: 1 / x). A string whose b_ab^2 is above 2^3
+// times that takes z_ij in FP64. Error relative to the term, random minors: FP64 5e-16 to
+// 2e-15 (levels 3 to 6), here 2e-16 to 7e-16, of which 0.1 % and less take FP64; at x =
+// 1e-8 without the rule 1e-9.
+#define SE_SPREAD 3   // bits
 template <int KL>
 __device__ __forceinline__ double2 string_energy_lanes(const SpinTables& tb, int w, int blk, int ns, const void* Bin,
                                                        const SeTab<double>& tab, const double2* wts)
@@ -337,6 +329,30 @@ __device__ __forceinline__ double2 string_energy_lanes(const SpinTables& tb, int
 #pragma unroll
         for (int o = 1; o < G; o <<= 1) mag = max(mag, __shfl_xor_sync(0xffffffffu, mag, o));
         const int eb = mag_exponent(mag);
+        // the keys' high bits are log2 to 0.09: a bit is 2^16
+        int at = KK, rest = 0, col = 0, row = 0;
+#pragma unroll
+        for (int q = 0; q < EPL; ++q)
+            if (j + q * G < KK && mag_bits(bv[q]) == mag) at = min(at, j + q * G);
+#pragma unroll
+        for (int o = 1; o < G; o <<= 1) at = min(at, __shfl_xor_sync(0xffffffffu, at, o));
+#pragma unroll
+        for (int q = 0; q < EPL; ++q) {
+            const int e = j + q * G, key = (int)(mag_bits(bv[q]) >> 4);
+            if (e >= KK) continue;
+            const bool r = e / KL == at / KL, c = e % KL == at % KL;
+            if (!r && !c) rest = max(rest, key);
+            if (!r && c) col = max(col, key);
+            if (r && !c) row = max(row, key);
+        }
+#pragma unroll
+        for (int o = 1; o < G; o <<= 1) {
+            rest = max(rest, __shfl_xor_sync(0xffffffffu, rest, o));
+            col = max(col, __shfl_xor_sync(0xffffffffu, col, o));
+            row = max(row, __shfl_xor_sync(0xffffffffu, row, o));
+        }
+        const int top = (int)(mag >> 4);
+        const bool wide = 2 * top - max(top + rest, col + row) > (SE_SPREAD << 16);
         __syncwarp();   // the previous strings' limbs consumed
 #pragma unroll
         for (int q = 0; q < EPL; ++q)
@@ -355,8 +371,24 @@ __device__ __forceinline__ double2 string_energy_lanes(const SpinTables& tb, int
 #pragma unroll
             for (int i = 0; i < KL; ++i) lin.add(bs[i * KL + j], ys[hj * np + rec_p(rec, i)]);
             double2 v = limb_value(lin, eb + tab.ey);
+            if (wide) {
 #pragma unroll 1
-            for (int i = 0; i + 1 < KL; ++i) {
+                for (int i = 0; i + 1 < KL; ++i) {
+                    double2 z = cz(0, 0);
+#pragma unroll 1
+                    for (int m = i + 1; m < KL; ++m) {
+                        const int pim = pair_index(rec_p(rec, i), rec_p(rec, m), np);
+#pragma unroll
+                        for (int d = 0; d < KL - 1; ++d) {
+                            const double2 x = B[m * KL + lc[d]], y = limbs_fp64(as[hp[d] + pim], tab.ea);
+                            z = lc[d] > j ? cfma(x, y, z) : cfms(x, y, z);
+                        }
+                    }
+                    v = cfma(B[i * KL + j], z, v);
+                }
+            }
+#pragma unroll 1
+            for (int i = 0; i + 1 < KL && !wide; ++i) {
                 LimbSum z;
                 const int pi = rec_p(rec, i);
 #pragma unroll 1

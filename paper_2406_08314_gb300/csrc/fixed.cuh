@@ -27,6 +27,13 @@ __device__ __forceinline__ Limbs to_limbs(double2 v, int e)
     return o;
 }
 
+// The value of limbs with exponent e, as FP64.
+__device__ __forceinline__ double2 limbs_fp64(const Limbs& x, int e)
+{
+    return make_double2(int_to_fp64((long long)x.rh * (1 << 26) + x.rl, e - 54),
+                        int_to_fp64((long long)x.ih * (1 << 26) + x.il, e - 54));
+}
+
 struct LimbSum {
     long long rr = 0, ii = 0, im = 0, crr = 0, cii = 0, cim = 0;
     __device__ __forceinline__ void add(const Limbs& a, const Limbs& b)
