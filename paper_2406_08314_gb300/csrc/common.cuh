@@ -125,6 +125,36 @@ __device__ __forceinline__ int rec_p(const uint4& r, int i) { return (int)(((i <
 
 
 #ifdef __CUDACC__
+// 1 / m for m > 0: y <- y + y (1 - m y) (Newton-Raphson for f(y) = 1/y - m),
+// two steps from the FP32 reciprocal (~2^-22 relative) reach FP64 rounding
+// (2^-44, then below 2^-53 before rounding). Outside the FP32 normal range
+// the quotient is taken directly.
+__device__ __forceinline__ double recip_nr(double m)
+{
+    if (!(m > 1e-36 && m < 1e36)) return 1.0 / m;
+    float yf;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(yf) : "f"((float)m));
+    double y = (double)yf;
+    double e = fma(-m, y, 1.0);
+    y = fma(y, e, y);
+    e = fma(-m, y, 1.0);
+    return fma(y, e, y);
+}
+
+__device__ __forceinline__ double2 crecip(double2 z)
+{
+    const double m2 = fma(z.x, z.x, z.y * z.y);
+    if (!(m2 > 1e-280 && m2 < 1e280)) return cdiv(cz(1, 0), z);
+    const double i = recip_nr(m2);
+    return cz(z.x * i, -z.y * i);
+}
+
+// monotone in max(|Re v|, |Im v|) up to the low 32 bits of each mantissa
+__device__ __forceinline__ int mag_key(double2 v)
+{
+    return max(__double2hiint(v.x) & 0x7fffffff, __double2hiint(v.y) & 0x7fffffff);
+}
+
 // x 2^-e (|x| < 2^e) as an integer of BITS fractional bits, the magnitude rounded
 // to nearest (integer operations only: FP64 ones issue at a sixty-fourth of
 // their rate).

@@ -10,9 +10,19 @@
 // and 6 along the last row over the level below (5, 6) where the trial holds all
 // the k strings that takes, else over the 2 x 2 minors (35, 105). GB300 issues
 // two FP64 FMAs per clock and SM, so the operation count is the time.
-// Division-free expansions of these sizes have no growth: against exact rational
-// arithmetic their relative error is 1.5e-16 to 2.9e-16 (levels 3 to 6, random
-// blocks), the pivoted LU's 5e-16 to 8e-16.
+//
+// Cancellation. An expansion is off by a few ulps of its largest product, a pivoted LU
+// by those times the minor's own conditioning. The two are alike for blocks whose
+// products do not cancel (random ones, levels 3 to 6: 1.1e-16 to 2.2e-16 relative,
+// median, the LU 1.4e-16 to 3.1e-16; graded rows and columns: the expansions half the
+// LU's), but the active block of a walker that overlaps the reference little is a large
+// part of low rank plus one of order one, and there the expansions lose g^(k-1) where
+// the LU loses g. So every minor carries log2 of its largest product, the maximum over
+// all permutations (max-plus arithmetic on the operands' high words, 16 fractional
+// bits: no FP64 operation), and a minor 2^3 below that is evaluated once more by an LU
+// of its own (k_minor_lu). Random blocks: 0.1 to 0.4 % of the minors, error then at or
+// below the LU's; with blocks of rank 1 or 2 times 3 to 1e4 added the error stays
+// within 1.2 of it (limits of 2^4: 1.5, 2^6: 3).
 //
 // Layout. Arrays of a string (or an active entry) hold its walkers contiguously,
 // rT[s][nw]: a warp's lanes are walkers of the same string, so index lists are
@@ -42,9 +52,19 @@ struct MinorSpin {
     const double2* GT;       // [nh np][nw]
     double2* m2;             // [C(nh,2) C(np,2)][nw]
     double2* rT;             // [n_str][nw]
+    int* t2;                 // as m2: log2 of the larger product (log_mag)
+    int* tr;                 // from string bucket[3] on, as rT: log2 of the largest product; odd: evaluate by LU
 };
 // Both spins of a launch (indexed by the block, in constant memory).
 struct MinorArgs { MinorSpin s[2]; };
+
+// log2 max(|Re v|, |Im v|) to 0.09, 16 fractional bits; far below any sum of six for 0.
+__device__ __forceinline__ int log_mag(double2 v)
+{
+    const int k = mag_key(v) >> 4;
+    return k ? k - (1023 << 16) : -(2400 << 16);
+}
+#define MINOR_BITS 3   // a minor this far below its largest product takes the LU
 
 __device__ __forceinline__ void pair_of(int e, int n, int& a, int& b)
 {
@@ -66,12 +86,14 @@ __global__ void __launch_bounds__(256) k_minor2(const __grid_constant__ MinorArg
     pair_of(pr % npp, S.np, p, p2);
     const double2* g = S.GT + w;
     auto G = [&](int a, int b) { return g[(size_t)(a * S.np + b) * nw]; };
-    S.m2[e] = cfms(G(h, p2), G(h2, p), cmul(G(h, p), G(h2, p2)));
+    const double2 g0 = G(h, p), g1 = G(h, p2), g2 = G(h2, p), g3 = G(h2, p2);
+    S.m2[e] = cfms(g1, g2, cmul(g0, g3));
+    S.t2[e] = max(log_mag(g0) + log_mag(g3), log_mag(g1) + log_mag(g2));
 }
 
 // Minors of the strings of levels k0 to k1, the trial's and, for k0 = k1, those
 // outside it; subs: through the ratios of the level below where the string has them.
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 4)
 k_minors(const __grid_constant__ MinorArgs a, int k0, int k1, bool subs, int nw)
 {
     const MinorSpin& S = a.s[blockIdx.y];
@@ -87,61 +109,174 @@ k_minors(const __grid_constant__ MinorArgs a, int k0, int k1, bool subs, int nw)
     const uint4 rec = S.str_hp[s];
     const double2* g = S.GT + w;
     const double2* m2 = S.m2 + w;
+    const int* t2 = S.t2 + w;
+    int* tr = S.tr + w;
     const double sg = S.str_sign[s];
     auto G = [&](int i, int j) { return g[(size_t)(rec_h(rec, i) * np + rec_p(rec, j)) * nw]; };
-    // 2 x 2 minor of rows a < b, columns c < d of the string's block
-    auto M2 = [&](int a, int b, int c, int d) {
+    // 2 x 2 minor of rows a < b, columns c < d of the string's block, and its row
+    auto R2 = [&](int a, int b, int c, int d) {
         const int hp = pair_index(rec_h(rec, a), rec_h(rec, b), nh), pp = pair_index(rec_p(rec, c), rec_p(rec, d), np);
-        return m2[(size_t)(hp * npp + pp) * nw];
+        return (size_t)(hp * npp + pp) * nw;
     };
-    // 4 x 4 minor of rows a < b < c < d, columns q0 < q1 < q2 < q3
-    auto M4 = [&](int a, int b, int c, int d, int q0, int q1, int q2, int q3) {
-        double2 v = cmul(M2(a, b, q0, q1), M2(c, d, q2, q3));
-        v = cfms(M2(a, b, q0, q2), M2(c, d, q1, q3), v);
-        v = cfma(M2(a, b, q0, q3), M2(c, d, q1, q2), v);
-        v = cfma(M2(a, b, q1, q2), M2(c, d, q0, q3), v);
-        v = cfms(M2(a, b, q1, q3), M2(c, d, q0, q2), v);
-        return cfma(M2(a, b, q2, q3), M2(c, d, q0, q1), v);
-    };
+    auto M2 = [&](int a, int b, int c, int d) { return m2[R2(a, b, c, d)]; };
     if (k == 1) { *out = cscale(G(0, 0), sg); return; }
     if (k == 2) { *out = cscale(M2(0, 1, 0, 1), sg); return; }
-    if (k == 3) {
-        double2 v = cmul(G(2, 0), M2(0, 1, 1, 2));
-        v = cfms(G(2, 1), M2(0, 1, 0, 2), v);
-        *out = cscale(cfma(G(2, 2), M2(0, 1, 0, 1), v), sg);
-        return;
-    }
+    // 4 x 4 minor of rows a < b < c < d, columns q0 < q1 < q2 < q3, log2 of its largest
+    // product to l
+    auto M4 = [&](int a, int b, int c, int d, int q0, int q1, int q2, int q3, int& l) {
+        const size_t r01 = R2(a, b, q0, q1), r02 = R2(a, b, q0, q2), r03 = R2(a, b, q0, q3), r12 = R2(a, b, q1, q2),
+                     r13 = R2(a, b, q1, q3), r23 = R2(a, b, q2, q3);
+        const size_t s01 = R2(c, d, q0, q1), s02 = R2(c, d, q0, q2), s03 = R2(c, d, q0, q3), s12 = R2(c, d, q1, q2),
+                     s13 = R2(c, d, q1, q3), s23 = R2(c, d, q2, q3);
+        double2 v = cmul(m2[r01], m2[s23]);
+        v = cfms(m2[r02], m2[s13], v);
+        v = cfma(m2[r03], m2[s12], v);
+        v = cfma(m2[r12], m2[s03], v);
+        v = cfms(m2[r13], m2[s02], v);
+        v = cfma(m2[r23], m2[s01], v);
+        l = max(max(max(t2[r01] + t2[s23], t2[r02] + t2[s13]), max(t2[r03] + t2[s12], t2[r12] + t2[s03])),
+                max(t2[r13] + t2[s02], t2[r23] + t2[s01]));
+        return v;
+    };
     const int* sub = S.sub + (size_t)s * MSD_KMAX;
-    if (subs && sub[0] >= 0) {
-        double2 v = cz(0, 0);
+    double2 v = cz(0, 0);
+    int top = -(1 << 30);   // log2 of the largest product
+    if (k == 3) {
+        const size_t r0 = R2(0, 1, 1, 2), r1 = R2(0, 1, 0, 2), r2 = R2(0, 1, 0, 1);
+        const double2 g0 = G(2, 0), g1 = G(2, 1), g2 = G(2, 2);
+        v = cmul(g0, m2[r0]);
+        v = cfms(g1, m2[r1], v);
+        v = cscale(cfma(g2, m2[r2], v), sg);
+        top = max(max(log_mag(g0) + t2[r0], log_mag(g1) + t2[r1]), log_mag(g2) + t2[r2]);
+    } else if (subs && sub[0] >= 0) {
         for (int j = 0; j < k; ++j) {
             const int q = sub[j];
             double2 gj = G(k - 1, j);
+            top = max(top, log_mag(gj) + tr[(size_t)((q >> 1) - S.bucket[3]) * nw]);
             if (q & 1) gj = cz(-gj.x, -gj.y);
             v = cfma(gj, S.rT[(size_t)(q >> 1) * nw + w], v);
         }
-        *out = v;
-        return;
-    }
-    double2 v = cz(0, 0);
-    if (k == 4) {
-        v = M4(0, 1, 2, 3, 0, 1, 2, 3);
+    } else if (k == 4) {
+        v = cscale(M4(0, 1, 2, 3, 0, 1, 2, 3, top), sg);
     } else if (k == 5) {
         for (int j = 0; j < 5; ++j) {
             const int a = j > 0 ? 0 : 1, b = j > 1 ? 1 : 2, c = j > 2 ? 2 : 3, d = j > 3 ? 3 : 4;
-            const double2 m = M4(0, 1, 2, 3, a, b, c, d), gj = G(4, j);
+            int l;
+            const double2 m = M4(0, 1, 2, 3, a, b, c, d, l), gj = G(4, j);
             v = (j & 1) ? cfms(gj, m, v) : cfma(gj, m, v);
+            top = max(top, log_mag(gj) + l);
         }
+        v = cscale(v, sg);
     } else {
         // rows 4, 5 over all column pairs; sign (-1)^(4 + 5 + c + d)
         for (int c = 0; c < 5; ++c)
             for (int d = c + 1; d < 6; ++d) {
                 auto q = [&](int j) { j += j >= c; return j + (j >= d); };   // the other columns
-                const double2 x = M4(0, 1, 2, 3, q(0), q(1), q(2), q(3)), y = M2(4, 5, c, d);
+                int l;
+                const double2 x = M4(0, 1, 2, 3, q(0), q(1), q(2), q(3), l), y = M2(4, 5, c, d);
                 v = ((c + d) & 1) ? cfma(y, x, v) : cfms(y, x, v);
+                top = max(top, l + t2[R2(4, 5, c, d)]);
             }
+        v = cscale(v, sg);
     }
-    *out = cscale(v, sg);
+    *out = v;
+    const bool lu = top - ((mag_key(v) >> 4) - (1023 << 16)) > (MINOR_BITS << 16);
+    tr[(size_t)(s - S.bucket[3]) * nw] = (top & ~1) | (lu ? 1 : 0);
+}
+
+// sign * det A of one string by an LU with partial pivoting (by the larger of |Re|, |Im|).
+template <int K>
+__device__ __forceinline__ double2 lu_minor(const uint4 rec, int np, const double2* __restrict__ g, int nw, double sign)
+{
+    double2 a[K][K];
+#pragma unroll
+    for (int i = 0; i < K; ++i)
+#pragma unroll
+        for (int j = 0; j < K; ++j) a[i][j] = g[(size_t)(rec_h(rec, i) * np + rec_p(rec, j)) * nw];
+    double2 det = cz(sign, 0);
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        int p = k, best = mag_key(a[k][k]);
+#pragma unroll
+        for (int i = k + 1; i < K; ++i) {
+            const int v = mag_key(a[i][k]);
+            if (v > best) { best = v; p = i; }
+        }
+#pragma unroll
+        for (int i = k + 1; i < K; ++i)
+            if (i == p) {
+#pragma unroll
+                for (int j = k; j < K; ++j) { const double2 t = a[k][j]; a[k][j] = a[i][j]; a[i][j] = t; }
+                det = cz(-det.x, -det.y);
+            }
+        const double2 v = a[k][k];
+        det = cmul(det, v);
+        const double2 inv = v.x == 0.0 && v.y == 0.0 ? cz(0, 0) : crecip(v);
+#pragma unroll
+        for (int i = k + 1; i < K; ++i) {
+            const double2 f = cmul(a[i][k], inv);
+#pragma unroll
+            for (int j = k + 1; j < K; ++j) a[i][j] = cfms(f, a[k][j], a[i][j]);
+        }
+    }
+    return det;
+}
+
+// The minors that k_minors marked, by LU: a block looks through LU_PAIRS (string, walker)
+// pairs from string s0 on and then its threads take those marked (few: one in a warp
+// would occupy all of it). No marks (tr NULL): all of them. The marks are 4 bytes a pair:
+// 64 MB, 20 us, at 640 iron-sulfur walkers.
+#define LU_PAIRS 2048
+#define LU_THREADS 128
+__global__ void __launch_bounds__(LU_THREADS) k_minor_lu(const __grid_constant__ MinorArgs a, int level0, int nw)
+{
+    const MinorSpin& S = a.s[blockIdx.y];
+    __shared__ unsigned short list[LU_PAIRS];
+    __shared__ int count;
+    const int s0 = S.bucket[level0], t = threadIdx.x;
+    const int n_all = S.vbucket[MSD_KMAX + 1] > S.n_str ? S.vbucket[MSD_KMAX + 1] : S.n_str;
+    const long long pairs = (long long)(n_all - s0) * nw, e0 = blockIdx.x * (long long)LU_PAIRS;
+    if (e0 >= pairs) return;
+    const int n = (int)(pairs - e0 < LU_PAIRS ? pairs - e0 : LU_PAIRS);
+    if (t == 0) count = S.tr ? 0 : n;
+    __syncthreads();
+    if (S.tr) {
+        for (int i = t * 4; i < n; i += LU_THREADS * 4) {
+            int m[4] = {0, 0, 0, 0};
+            if (i + 4 <= n) {
+                const int4 v = *reinterpret_cast<const int4*>(S.tr + e0 + i);
+                m[0] = v.x; m[1] = v.y; m[2] = v.z; m[3] = v.w;
+            } else {
+                for (int q = 0; i + q < n; ++q) m[q] = S.tr[e0 + i + q];
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (m[q] & 1) list[atomicAdd(&count, 1)] = (unsigned short)(i + q);
+        }
+        __syncthreads();
+    }
+    const int total = count;
+    for (int i = t; i < total; i += LU_THREADS) {
+        const long long e = e0 + (S.tr ? list[i] : i);
+        const int s = s0 + (int)(e / nw), w = (int)(e % nw);
+        int k = 0;
+        if (s < S.n_str) while (s >= S.bucket[k + 1]) ++k;
+        else while (s >= S.vbucket[k + 1]) ++k;
+        const uint4 rec = S.str_hp[s];
+        const double2* g = S.GT + w;
+        const double sg = S.str_sign[s];
+        double2 r = cz(1, 0);
+        switch (k) {
+        case 0: break;
+        case 1: r = lu_minor<1>(rec, S.np, g, nw, sg); break;
+        case 2: r = lu_minor<2>(rec, S.np, g, nw, sg); break;
+        case 3: r = lu_minor<3>(rec, S.np, g, nw, sg); break;
+        case 4: r = lu_minor<4>(rec, S.np, g, nw, sg); break;
+        case 5: r = lu_minor<5>(rec, S.np, g, nw, sg); break;
+        default: r = lu_minor<6>(rec, S.np, g, nw, sg); break;
+        }
+        S.rT[(size_t)s * nw + w] = r;
+    }
 }
 
 // ----------------------------------------------------------------- weights
@@ -437,14 +572,25 @@ __global__ void __launch_bounds__(128) k_inverse_ratios(const __grid_constant__ 
     }
 }
 
-MinorSpin minor_spin(const SpinTables& t, const double2* GT, double2* m2, double2* rT)
+MinorSpin minor_spin(const SpinTables& t, const double2* GT, double2* m2, double2* rT, int* t2, int* tr)
 {
     MinorSpin s;
     s.nh = t.nh; s.np = t.np; s.n_str = t.n_str;
     for (int k = 0; k < MSD_KMAX + 2; ++k) { s.bucket[k] = t.bucket[k]; s.vbucket[k] = 0; }
     s.str_hp = t.str_hp; s.str_sign = t.str_sign; s.sub = t.sub;
-    s.GT = GT; s.m2 = m2; s.rT = rT;
+    s.GT = GT; s.m2 = m2; s.rT = rT; s.t2 = t2; s.tr = tr;
     return s;
+}
+
+// The marked minors of both spins from level 3 on (all of every level without marks).
+void launch_lu(const MinorArgs& a, int nw, cudaStream_t st)
+{
+    const int level0 = a.s[0].tr ? 3 : 0;
+    long long n = 0;
+    for (const MinorSpin& s : a.s) n = std::max(n, (long long)std::max(s.n_str, s.vbucket[MSD_KMAX + 1]) - s.bucket[level0]);
+    if (n <= 0) return;
+    k_minor_lu<<<dim3((unsigned)((n * nw + LU_PAIRS - 1) / LU_PAIRS), 2), LU_THREADS, 0, st>>>(a, level0, nw);
+    msd_note_launch();
 }
 
 // --------------------------------------------------------------- adjoint
@@ -512,13 +658,13 @@ __global__ void __launch_bounds__(256) k_adjoint(const __grid_constant__ AdjArgs
 
 // Ratios of the trial's strings and of the sub-minors outside it.
 void launch_minors_ext(const GradTables g[2], const SpinTables& ta, const SpinTables& tb, int nw, double2* const V[2],
-                       cudaStream_t st)
+                       int* const t2[2], int* const tr[2], cudaStream_t st)
 {
     MinorArgs a;
     const SpinTables* T[2] = {&ta, &tb};
     for (int s = 0; s < 2; ++s) {
         double2* m2 = V[s] + (size_t)T[s]->nh * T[s]->np * nw;
-        a.s[s] = minor_spin(*T[s], V[s], m2, m2 + (size_t)g[s].n2 * nw);
+        a.s[s] = minor_spin(*T[s], V[s], m2, m2 + (size_t)g[s].n2 * nw, t2[s], tr[s]);
         a.s[s].str_hp = g[s].str_hp; a.s[s].str_sign = g[s].str_sign; a.s[s].sub = g[s].sub;
         for (int k = 0; k < MSD_KMAX + 2; ++k) a.s[s].vbucket[k] = g[s].vbucket[k];
     }
@@ -536,6 +682,7 @@ void launch_minors_ext(const GradTables g[2], const SpinTables& ta, const SpinTa
         k_minors<<<blocks(n), 256, 0, st>>>(a, k, k, true, nw);
         msd_note_launch();
     }
+    launch_lu(a, nw, st);
 }
 
 void launch_adjoint(const GradTables g[2], const SpinTables& ta, const SpinTables& tb, int nw, double2* const V[2],
@@ -561,10 +708,13 @@ size_t minor2_count(const SpinTables& t)
     return std::max<size_t>(1, (size_t)(t.nh * (t.nh - 1) / 2) * (t.np * (t.np - 1) / 2));
 }
 
+size_t minor_marks(const SpinTables& t) { return std::max(1, t.n_str - t.bucket[3]); }
+
 void launch_minors(const SpinTables& ta, const SpinTables& tb, int nw, double2* const GT[2], double2* const m2[2],
-                   double2* const rT[2], cudaStream_t st)
+                   int* const t2[2], int* const tr[2], double2* const rT[2], cudaStream_t st)
 {
-    const MinorArgs a = {{minor_spin(ta, GT[0], m2[0], rT[0]), minor_spin(tb, GT[1], m2[1], rT[1])}};
+    const MinorArgs a = {{minor_spin(ta, GT[0], m2[0], rT[0], t2[0], tr[0]), minor_spin(tb, GT[1], m2[1], rT[1], t2[1], tr[1])}};
+    if (!m2[0]) { launch_lu(a, nw, st); return; }
     auto blocks = [&](long long n) { return dim3((unsigned)((n * nw + 255) / 256), 2); };
     k_minor2<<<blocks(std::max(minor2_count(ta), minor2_count(tb))), 256, 0, st>>>(a, nw);
     msd_note_launch();
@@ -582,6 +732,7 @@ void launch_minors(const SpinTables& ta, const SpinTables& tb, int nw, double2* 
         k_minors<<<blocks(count(k, k)), 256, 0, st>>>(a, k, k, true, nw);
         msd_note_launch();
     }
+    launch_lu(a, nw, st);
 }
 
 void launch_inverse_minors(const SpinTables& ta, const SpinTables& tb, int nw, double2* const Gact[2], void* const B[2],

@@ -39,17 +39,6 @@ struct RefIn {
 };
 struct RefArgs { RefIn s[2]; };
 
-__device__ __forceinline__ double recip_nr(double m);
-__device__ __forceinline__ int mag_key(double2 v);
-
-__device__ __forceinline__ double2 crecip(double2 z)
-{
-    const double m2 = fma(z.x, z.x, z.y * z.y);
-    if (!(m2 > 1e-280 && m2 < 1e280)) return cdiv(cz(1, 0), z);
-    const double i = recip_nr(m2);
-    return cz(z.x * i, -z.y * i);
-}
-
 __global__ void __launch_bounds__(256)
 k_ref(const __grid_constant__ RefArgs args, int M, unsigned* err)
 {
@@ -247,28 +236,6 @@ int launch_refs(const RefSpinIn* in, int n_spin, int nw, int M, unsigned* err, c
 // larger high word of |Re|, |Im|: partial pivoting by the max-norm), the row
 // swaps count parity in an integer, and the pivot reciprocals are
 // Newton-Raphson iterations from an FP32 seed.
-
-// 1 / m for m > 0: y <- y + y (1 - m y) (Newton-Raphson for f(y) = 1/y - m),
-// two steps from the FP32 reciprocal (~2^-22 relative) reach FP64 rounding
-// (2^-44, then below 2^-53 before rounding). Outside the FP32 normal range
-// the quotient is taken directly.
-__device__ __forceinline__ double recip_nr(double m)
-{
-    if (!(m > 1e-36 && m < 1e36)) return 1.0 / m;
-    float yf;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(yf) : "f"((float)m));
-    double y = (double)yf;
-    double e = fma(-m, y, 1.0);
-    y = fma(y, e, y);
-    e = fma(-m, y, 1.0);
-    return fma(y, e, y);
-}
-
-// monotone in max(|Re v|, |Im v|) up to the low 32 bits of each mantissa
-__device__ __forceinline__ int mag_key(double2 v)
-{
-    return max(__double2hiint(v.x) & 0x7fffffff, __double2hiint(v.y) & 0x7fffffff);
-}
 
 template <int K>
 __global__ void __launch_bounds__(128)

@@ -36,11 +36,13 @@ int launch_refs(const RefSpinIn* in, int n_spin, int nw, int M, unsigned* err, c
 void launch_strings(const SpinTables& tb, int nw, const double2* Gact, double2* r, double2* rT, void* B, cudaStream_t st,
                     const TimerHook& th);
 // k_minors.cu: FP64 ratios rT[s][w] of both spins by expansions over shared
-// minors (m2: scratch, minor2_count entries per walker), FP32 inverse minors,
-// and the CI weights.
+// minors, those that cancel by LU (m2, t2: scratch, minor2_count entries per walker;
+// tr: minor_marks entries; all NULL: every ratio by LU), FP32 inverse minors, and the CI
+// weights.
 size_t minor2_count(const SpinTables& t);
+size_t minor_marks(const SpinTables& t);
 void launch_minors(const SpinTables& ta, const SpinTables& tb, int nw, double2* const GT[2], double2* const m2[2],
-                   double2* const rT[2], cudaStream_t st);
+                   int* const t2[2], int* const tr[2], double2* const rT[2], cudaStream_t st);
 void launch_inverse_minors(const SpinTables& ta, const SpinTables& tb, int nw, double2* const Gact[2], void* const B[2],
                            cudaStream_t st);
 int weights_blocks(const SpinTables& tb);
@@ -65,8 +67,9 @@ struct GradTables {
     int *row = nullptr, *off = nullptr;   // launch_inverse_ratios: row alone, at SpinTables::cmx_off
     int2* ent = nullptr;
 };
+// t2 [n2][nw], tr [n_ext - bucket[3]][nw]: scratch.
 void launch_minors_ext(const GradTables g[2], const SpinTables& ta, const SpinTables& tb, int nw, double2* const V[2],
-                       cudaStream_t st);
+                       int* const t2[2], int* const tr[2], cudaStream_t st);
 // FP64 inverse minors from V as launch_minors_ext left it.
 void launch_inverse_ratios(const GradTables g[2], const SpinTables& ta, const SpinTables& tb, int nw,
                            double2* const V[2], void* const B[2], cudaStream_t st);

@@ -1329,6 +1329,7 @@ struct Chunk {
     float2* rf[2];   // FP32 copies of r (mixed mode, with B)
     void* B[2];
     double2 *V[2], *Bv[2];   // expansions (launch_minors_ext) and their reverse pass
+    int *t2[2], *tr[2];      // the minors' largest products (launch_minors)
     int nslot, nR;
 };
 
@@ -1356,6 +1357,14 @@ int string_use(msd_ctx* ctx, bool energy, StringUse* use)
     return rc;
 }
 
+// Rows of the minors' marks of spin s (launch_minors, launch_minors_ext).
+size_t mark_rows(const msd_ctx* ctx, int s, StringUse use)
+{
+    const SpinHost& S = ctx->sp[s];
+    const int n = use == StringUse::Cofactors ? ctx->grad[s].n_ext : ratio_inverse(ctx, use) ? ctx->inv[s].n_ext : S.n_str;
+    return std::max(1, n - S.bucket[3]);
+}
+
 // The ratios as r[w][s] are for the FP64 per-determinant terms (Minors in FP64 mode)
 // or for the caller (want_r).
 size_t overlap_bytes_per_walker(msd_ctx* ctx, StringUse use, int nslot, bool want_r = false)
@@ -1368,6 +1377,7 @@ size_t overlap_bytes_per_walker(msd_ctx* ctx, StringUse use, int nslot, bool wan
         b += (size_t)S.N * ctx->M + 1 + 2 * (size_t)S.nh * S.np + (size_t)S.n_str;
         b += ref_dg_bytes(ctx->M, S.N) / sizeof(double2) + 1;
         if (!fp64_b) b += minor2_count(tables(S, 1));
+        if (!fp64_b || inv) b += (minor2_count(tables(S, 1)) + mark_rows(ctx, s, use)) / 4 + 2;
         if (inv) b += ctx->inv[s].n2 + ctx->inv[s].n_ext - S.n_str;
         if (cof) b += 2 * (size_t)ctx->grad[s].n_ext + ctx->grad[s].n2 + ctx->grad[s].n_piece - S.n_str;
         if (fp64_b || want_r) b += S.n_str;
@@ -1382,9 +1392,9 @@ int chunk_alloc(msd_ctx* ctx, int cap, StringUse use, int nslot, Chunk& c, bool 
     int rc;
     const bool want_b = use == StringUse::Minors, cof = use == StringUse::Cofactors;
     const bool fp64_b = want_b && ctx->prec == MSD_FP64, inv = ratio_inverse(ctx, use);
-    static const char* names[2][12] = {
-        {"Gr_a", "O0_a", "Gact_a", "GactT_a", "m2_a", "rT_a", "r_a", "wts_a", "B_a", "rf_a", "V_a", "Bv_a"},
-        {"Gr_b", "O0_b", "Gact_b", "GactT_b", "m2_b", "rT_b", "r_b", "wts_b", "B_b", "rf_b", "V_b", "Bv_b"}};
+    static const char* names[2][14] = {
+        {"Gr_a", "O0_a", "Gact_a", "GactT_a", "m2_a", "rT_a", "r_a", "wts_a", "B_a", "rf_a", "V_a", "Bv_a", "t2_a", "tr_a"},
+        {"Gr_b", "O0_b", "Gact_b", "GactT_b", "m2_b", "rT_b", "r_b", "wts_b", "B_b", "rf_b", "V_b", "Bv_b", "t2_b", "tr_b"}};
     for (int s = 0; s < 2; ++s) {
         const SpinHost& S = ctx->sp[s];
         const size_t X = std::max(1, S.nh * S.np), w16 = sizeof(double2) * (size_t)cap;
@@ -1402,6 +1412,9 @@ int chunk_alloc(msd_ctx* ctx, int cap, StringUse use, int nslot, Chunk& c, bool 
         if ((rc = get(10, w16 * (X + (size_t)g.n2 + g.n_ext), cof || inv, (void**)&c.V[s]))) return rc;
         if ((rc = get(11, w16 * ((size_t)g.n_ext + g.n2 + g.n_piece), cof, (void**)&c.Bv[s]))) return rc;
         if (cof || inv) c.GactT[s] = c.V[s];   // the head of V
+        const bool marks = !fp64_b || inv;
+        if ((rc = get(12, sizeof(int) * cap * minor2_count(tables(S, 1)), marks, (void**)&c.t2[s]))) return rc;
+        if ((rc = get(13, sizeof(int) * cap * mark_rows(ctx, s, use), marks, (void**)&c.tr[s]))) return rc;
         if ((rc = get(6, w16 * S.n_str, fp64_b || want_r, (void**)&c.r[s]))) return rc;
         if ((rc = get(7, w16 * S.n_str, want_b, (void**)&c.wts[s]))) return rc;
         if ((rc = get(8, sizeof(double2) * std::max<long long>(1, cap * S.b_per_walker), want_b, &c.B[s]))) return rc;
@@ -1471,7 +1484,7 @@ int run_strings_weights(msd_ctx* ctx, int nw, int cap, Chunk& c, StringUse use, 
                                sizeof(double2) * (size_t)nw * (g.n_ext - T[s].n_str + g.n2 + g.n_piece), st));
         }
         th.begin("k_strings", st);
-        launch_minors_ext(ctx->grad, T[0], T[1], nw, c.V, st);
+        launch_minors_ext(ctx->grad, T[0], T[1], nw, c.V, c.t2, c.tr, st);
         th.end(st);
         th.begin("k_weights", st);
         launch_weights(T[0], T[1], nw, rT, none, no_f, c.part, c.nslot, true, st, c.Bv);
@@ -1482,7 +1495,7 @@ int run_strings_weights(msd_ctx* ctx, int nw, int cap, Chunk& c, StringUse use, 
     if (ratio_inverse(ctx, use)) {
         for (int s = 0; s < 2; ++s) c.rT[s] = c.V[s] + ((size_t)T[s].nh * T[s].np + ctx->inv[s].n2) * nw;
         th.begin("k_strings", st);
-        launch_minors_ext(ctx->inv, T[0], T[1], nw, c.V, st);
+        launch_minors_ext(ctx->inv, T[0], T[1], nw, c.V, c.t2, c.tr, st);
         launch_inverse_ratios(ctx->inv, T[0], T[1], nw, c.V, c.B, st);
         for (int s = 0; s < 2; ++s) launch_untranspose(T[s].n_str, nw, c.rT[s], c.r[s], st);
         th.end(st);
@@ -1490,7 +1503,7 @@ int run_strings_weights(msd_ctx* ctx, int nw, int cap, Chunk& c, StringUse use, 
         for (int s = 0; s < 2; ++s) launch_strings(T[s], nw, c.Gact[s], c.r[s], c.rT[s], c.B[s], st, th);
     } else {
         th.begin("k_strings", st);
-        launch_minors(T[0], T[1], nw, c.GactT, c.m2, c.rT, st);
+        launch_minors(T[0], T[1], nw, c.GactT, c.m2, c.t2, c.tr, c.rT, st);
         if (want_b) launch_inverse_minors(T[0], T[1], nw, c.Gact, c.B, st);
         th.end(st);
     }
@@ -3018,14 +3031,17 @@ extern "C" int msd_overlap_noalloc(msd_ctx* ctx, int n_w, const double* phi_a, c
     const int M = ctx->M;
     SpinTables T1[2] = {tables(ctx->sp[0], 1), tables(ctx->sp[1], 1)};
     const int nR = weights_blocks(T1[0]);
-    // scratch per walker: Gr, O0, active block, 2 x 2 minors and ratios of both
-    // spins, partial sums
-    size_t per = 0;
-    for (int s = 0; s < 2; ++s)
-        per += sizeof(double2) * ((size_t)T1[s].N * M + 1 + std::max(1, T1[s].nh * T1[s].np) + minor2_count(T1[s]) +
-                                  T1[s].n_str);
-    per += sizeof(double2) * (size_t)nR;
+    // scratch per walker: Gr, O0, active block and ratios of both spins, partial sums,
+    // and the 2 x 2 minors with the marks of the expansions (without them, where a
+    // walker's do not fit, every ratio by LU)
+    size_t per = sizeof(double2) * (size_t)nR, shared = 0;
+    for (int s = 0; s < 2; ++s) {
+        per += sizeof(double2) * ((size_t)T1[s].N * M + 1 + std::max(1, T1[s].nh * T1[s].np) + T1[s].n_str);
+        shared += (sizeof(double2) + sizeof(int)) * minor2_count(T1[s]) + sizeof(int) * minor_marks(T1[s]);
+    }
     const size_t slack = 16 * 256;   // alignment of the carved arrays
+    const bool expand = per + shared + slack <= (size_t)MSD_STATIC_SCRATCH_BYTES;
+    if (expand) per += shared;
     if (per + slack > (size_t)MSD_STATIC_SCRATCH_BYTES)
         return fail(ctx, MSD_ERR_SHAPE,
                     "one walker needs %zu bytes of scratch; the static scratch holds %zu bytes", per + slack,
@@ -3036,13 +3052,18 @@ extern "C" int msd_overlap_noalloc(msd_ctx* ctx, int n_w, const double* phi_a, c
     unsigned char* base = (unsigned char*)scratch;
     size_t off = 0;
     auto take = [&](size_t bytes) { void* p = base + off; off += align256(bytes); return p; };
-    double2 *Gr[2], *O0[2], *GactT[2], *m2[2], *r[2], *no_wts[2] = {nullptr, nullptr};
+    double2 *Gr[2], *O0[2], *GactT[2], *m2[2] = {nullptr, nullptr}, *r[2], *no_wts[2] = {nullptr, nullptr};
+    int *t2[2] = {nullptr, nullptr}, *tr[2] = {nullptr, nullptr};
     float2* no_rf[2] = {nullptr, nullptr};
     for (int s = 0; s < 2; ++s) {
         Gr[s] = (double2*)take(sizeof(double2) * cap * T1[s].N * (size_t)M);
         O0[s] = (double2*)take(sizeof(double2) * cap);
         GactT[s] = (double2*)take(sizeof(double2) * cap * (size_t)std::max(1, T1[s].nh * T1[s].np));
-        m2[s] = (double2*)take(sizeof(double2) * cap * minor2_count(T1[s]));
+        if (expand) {
+            m2[s] = (double2*)take(sizeof(double2) * cap * minor2_count(T1[s]));
+            t2[s] = (int*)take(sizeof(int) * cap * minor2_count(T1[s]));
+            tr[s] = (int*)take(sizeof(int) * cap * minor_marks(T1[s]));
+        }
         r[s] = (double2*)take(sizeof(double2) * cap * (size_t)T1[s].n_str);
     }
     double2* part = (double2*)take(sizeof(double2) * cap * (size_t)nR);
@@ -3061,7 +3082,7 @@ extern "C" int msd_overlap_noalloc(msd_ctx* ctx, int n_w, const double* phi_a, c
             in[s].Gr = Gr[s]; in[s].O0 = O0[s]; in[s].GactT = GactT[s];
         }
         launch_refs(in, 2, nw, M, ctx->d_err, st);
-        launch_minors(T[0], T[1], nw, GactT, m2, r, st);
+        launch_minors(T[0], T[1], nw, GactT, m2, t2, tr, r, st);
         launch_weights(T[0], T[1], nw, r, no_wts, no_rf, part, nR, false, st);
         launch_sum_slots(nw, part, nR, 0, nR, ratio_sum ? (double2*)ratio_sum + w0 : nullptr, O0[0], O0[1],
                          ovlp ? (double2*)ovlp + w0 : nullptr, st);
