@@ -45,7 +45,7 @@ namespace {
 struct MinorSpin {
     int nh, np, n_str;
     int bucket[MSD_KMAX + 2];
-    int vbucket[MSD_KMAX + 2];   // strings outside the trial, by level (k_adjoint): [vbucket[k], vbucket[k + 1])
+    int vbucket[MSD_KMAX + 2];   // strings outside the trial, by level: [vbucket[k], vbucket[k + 1])
     const uint4* str_hp;
     const int8_t* str_sign;
     const int* sub;          // [n_str][MSD_KMAX] (string << 1 | negative), -1 first if one is missing
@@ -291,6 +291,7 @@ struct WeightSpin {
     float2* rf;              // [nw][n_str] r_s in FP32 (may be NULL)
     double2* part;           // [nw][nslot] partial sums over 32 strings (may be NULL)
     double2* wT;             // [n_str][nw] the sums themselves (may be NULL)
+    const int* big;          // [nw] with wT: walkers whose sums go to wT for vanishing ratios only
 };
 struct WeightArgs { WeightSpin s[2]; };
 
@@ -330,8 +331,8 @@ __global__ void __launch_bounds__(256) k_weights(const __grid_constant__ WeightA
                 const double c = S.c[i];
                 acc = cz(fma(v.x, c, acc.x), fma(v.y, c, acc.y));
             }
-            if (S.wT) S.wT[(size_t)s * nw + w] = acc;
             r = S.self[(size_t)s * nw + w];
+            if (S.wT) S.wT[(size_t)s * nw + w] = S.big[w] && (r.x != 0 || r.y != 0) ? cz(0, 0) : acc;
             rw = cmul(r, acc);
         }
         tw[sl][wl] = rw;
@@ -593,38 +594,35 @@ void launch_lu(const MinorArgs& a, int nw, cudaStream_t st)
     msd_note_launch();
 }
 
-// --------------------------------------------------------------- adjoint
-// Cofactor matrix of the force bias and the density matrix,
-//   Cm[p][h] = sum_s w_s r_s B_s[i][j] at (p_i, h_j) = (p, h)  =  d(sum_s w_s r_s) / dG[h][p],
-// by reverse differentiation of the expansions above, without any inverse minor:
-// with every product r = ... + a b + ... of the forward pass, the adjoint of a gains b
-// times the adjoint of r. A target's users are one list of (value row, adjoint row,
-// sign), so each target is a sum over its list, lanes over the walkers:
-//   out[target] += sum +- V[a] Bv[b]   (a < 0: 1),
-// V = [G | 2 x 2 minors | ratios], Bv = [ratios' adjoints | 2 x 2 minors' adjoints],
-// both [row][nw]. Levels from the highest down, then the 2 x 2 minors, then G, whose
-// few long lists are cut in pieces and the pieces added (one list each: 1.04 ms below).
-// About 8 k FP64 FMAs per string, against 4 k^3 for its inverse minor by LU and k^2
-// scattered additions; memory bound now (16-byte rows of a warp's 32 walkers). 640
-// copper-oxo walkers, strings + cofactors: 3.05 + 1.24 -> 0.53 + 0.65 ms.
-struct AdjSpin {
-    int n0, n1;              // targets of this launch
-    const int* row;          // [target] output row of Bv, or entry of G (last stage)
+// ------------------------------------------------------------- cofactors
+// Cofactor matrix of the FP64 force bias and density matrix,
+//   Cm[p][h] = sum_s w_s r_s B_s[i][j] at (p_i, h_j) = (p, h),
+// from the cofactors r_s B_s themselves, which are rows of V: no inverse minor, and right
+// where a ratio vanishes and its cofactors do not. An entry's list holds (row of V, string,
+// sign); the lists are cut in pieces of 64 (few entries with long lists), then the
+// pieces are added. 4 FP64 FMAs and two 16-byte rows of a warp's 32 walkers per entry.
+// Walkers with a large active block (k_large in k_wick.cu) take theirs from the LU's
+// inverse minors, the vanishing ratios excepted. 640 copper-oxo walkers 0.76 ms. (Reverse
+// differentiation of the expansions takes half the operations, 0.65 ms; but it sums the
+// cofactors' own expansions again, with their cancellation.)
+struct CofSpin {
+    int t0, t1;              // targets of this launch
+    const int* row;          // [target] row of Bv, or entry of G (the sums)
     const int* off;          // [target + 1]
-    const int2* ent;         // (a << 1 | negative, b); a = -1: (-2 | negative)
+    const int2* ent;         // (a << 1 | negative, b): +-V[a] Bv[b]; a = -1: +-Bv[b]
     const double2* V;
     double2* Bv;
-    double2* Cm;             // last stage: [nw][np][nh], entry x = h np + p to p nh + h
+    double2* Cm;             // the sums: [nw][np][nh], entry x = h np + p to p nh + h
     int nh, np;
 };
-struct AdjArgs { AdjSpin s[2]; };
+struct CofArgs { CofSpin s[2]; };
 
-__global__ void __launch_bounds__(256) k_adjoint(const __grid_constant__ AdjArgs args, int nw)
+__global__ void __launch_bounds__(256) k_cofactors(const __grid_constant__ CofArgs args, int nw)
 {
-    const AdjSpin& S = args.s[blockIdx.y];
+    const CofSpin& S = args.s[blockIdx.y];
     const long long e = blockIdx.x * 256ll + threadIdx.x;
-    if (e >= (long long)(S.n1 - S.n0) * nw) return;
-    const int t = S.n0 + (int)(e / nw), w = (int)(e % nw);
+    if (e >= (long long)(S.t1 - S.t0) * nw) return;
+    const int t = S.t0 + (int)(e / nw), w = (int)(e % nw);
     double2 acc = cz(0, 0);
     const int i1 = S.off[t + 1];
     for (int i = S.off[t]; i < i1; i += 4) {
@@ -649,15 +647,14 @@ __global__ void __launch_bounds__(256) k_adjoint(const __grid_constant__ AdjArgs
         const int h = r / S.np, p = r - h * S.np;
         S.Cm[(size_t)w * S.nh * S.np + p * S.nh + h] = acc;
     } else {
-        double2* o = S.Bv + (size_t)r * nw + w;
-        *o = cadd(*o, acc);
+        S.Bv[(size_t)r * nw + w] = acc;
     }
 }
 
 }  // namespace
 
 // Ratios of the trial's strings and of the sub-minors outside it.
-void launch_minors_ext(const GradTables g[2], const SpinTables& ta, const SpinTables& tb, int nw, double2* const V[2],
+void launch_minors_ext(const ExtTables g[2], const SpinTables& ta, const SpinTables& tb, int nw, double2* const V[2],
                        int* const t2[2], int* const tr[2], cudaStream_t st)
 {
     MinorArgs a;
@@ -685,20 +682,21 @@ void launch_minors_ext(const GradTables g[2], const SpinTables& ta, const SpinTa
     launch_lu(a, nw, st);
 }
 
-void launch_adjoint(const GradTables g[2], const SpinTables& ta, const SpinTables& tb, int nw, double2* const V[2],
-                    double2* const Bv[2], double2* const Cm[2], cudaStream_t st)
+void launch_cofactors(const ExtTables g[2], const SpinTables& ta, const SpinTables& tb, int nw, double2* const V[2],
+                      double2* const Bv[2], double2* const Cm[2], cudaStream_t st)
 {
     const SpinTables* T[2] = {&ta, &tb};
-    for (int q = 0; q < GRAD_STAGES; ++q) {
-        AdjArgs a;
+    for (int sums = 0; sums < 2; ++sums) {
+        CofArgs a;
         int n = 0;
         for (int s = 0; s < 2; ++s) {
-            a.s[s] = AdjSpin{g[s].stage[q], g[s].stage[q + 1], g[s].row, g[s].off, g[s].ent, V[s], Bv[s],
-                             q == GRAD_STAGES - 1 ? Cm[s] : nullptr, T[s]->nh, T[s]->np};
-            n = std::max(n, g[s].stage[q + 1] - g[s].stage[q]);
+            const int t0 = sums ? g[s].n_piece : 0, t1 = g[s].n_piece + (sums ? T[s]->nh * T[s]->np : 0);
+            a.s[s] = CofSpin{t0, t1, g[s].cof_row, g[s].cof_off, g[s].cof_ent, V[s], Bv[s], sums ? Cm[s] : nullptr, T[s]->nh,
+                             T[s]->np};
+            n = std::max(n, t1 - t0);
         }
         if (n <= 0) continue;
-        k_adjoint<<<dim3((unsigned)(((long long)n * nw + 255) / 256), 2), 256, 0, st>>>(a, nw);
+        k_cofactors<<<dim3((unsigned)(((long long)n * nw + 255) / 256), 2), 256, 0, st>>>(a, nw);
         msd_note_launch();
     }
 }
@@ -757,7 +755,7 @@ void launch_inverse_minors(const SpinTables& ta, const SpinTables& tb, int nw, d
     msd_note_launch();
 }
 
-void launch_inverse_ratios(const GradTables g[2], const SpinTables& ta, const SpinTables& tb, int nw,
+void launch_inverse_ratios(const ExtTables g[2], const SpinTables& ta, const SpinTables& tb, int nw,
                            double2* const V[2], void* const B[2], cudaStream_t st)
 {
     InvRatioArgs args;
@@ -784,10 +782,13 @@ int weights_blocks(const SpinTables& tb) { return (tb.n_str + WT_S - 1) / WT_S; 
 
 // wts, rf: per spin, NULL where not wanted; beta = false: the alpha sums alone.
 void launch_weights(const SpinTables& ta, const SpinTables& tb, int nw, double2* const rT[2], double2* const wts[2],
-                    float2* const rf[2], double2* part, int nslot, bool beta, cudaStream_t st, double2* const wT[2])
+                    float2* const rf[2], double2* part, int nslot, bool beta, cudaStream_t st, double2* const wT[2],
+                    int* const big[2])
 {
-    const WeightArgs a = {{{ta.n_str, ta.csr_off, ta.csr_other, ta.csr_c, rT[0], rT[1], wts[0], rf[0], part, wT ? wT[0] : nullptr},
-                          {tb.n_str, tb.csr_off, tb.csr_other, tb.csr_c, rT[1], rT[0], wts[1], rf[1], nullptr, wT ? wT[1] : nullptr}}};
+    const WeightArgs a = {{{ta.n_str, ta.csr_off, ta.csr_other, ta.csr_c, rT[0], rT[1], wts[0], rf[0], part,
+                           wT ? wT[0] : nullptr, wT ? big[0] : nullptr},
+                          {tb.n_str, tb.csr_off, tb.csr_other, tb.csr_c, rT[1], rT[0], wts[1], rf[1], nullptr,
+                           wT ? wT[1] : nullptr, wT ? big[1] : nullptr}}};
     const int tiles = (nw + 31) / 32, wt = (nw + tiles - 1) / tiles;   // walkers per tile, evenly
     const int nb = beta ? std::max(weights_blocks(ta), weights_blocks(tb)) : weights_blocks(ta);
     k_weights<<<dim3(nb, tiles, beta ? 2 : 1), 256, 0, st>>>(a, nw, wt, nslot);

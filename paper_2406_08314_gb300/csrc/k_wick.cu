@@ -237,20 +237,12 @@ int launch_refs(const RefSpinIn* in, int n_spin, int nw, int M, unsigned* err, c
 // swaps count parity in an integer, and the pivot reciprocals are
 // Newton-Raphson iterations from an FP32 seed.
 
+// String s = bucket[K] + sl of walker w, its active block in shared memory (g).
 template <int K>
-__global__ void __launch_bounds__(128)
-k_strings(SpinTables tb, int nw, const double2* __restrict__ Gact, double2* __restrict__ r, double2* __restrict__ rT,
-          double2* __restrict__ Bout)
+__device__ __forceinline__ void string_lu(const SpinTables& tb, int nw, int w, int sl, const double2* g, double2* r,
+                                          double2* rT, double2* Bout)
 {
-    __shared__ double2 g[MSD_XMAX];
-    const int w = blockIdx.y;
-    const int X = tb.nh * tb.np;
-    for (int e = threadIdx.x; e < X; e += blockDim.x) g[e] = Gact[(size_t)w * X + e];
-    __syncthreads();
-    const int ns = tb.bucket[K + 1] - tb.bucket[K];
-    const int sl = blockIdx.x * blockDim.x + threadIdx.x;
-    if (sl >= ns) return;
-    const int s = tb.bucket[K] + sl;
+    const int ns = tb.bucket[K + 1] - tb.bucket[K], s = tb.bucket[K] + sl;
     const uint4 rec = tb.str_hp[s];
     double2 a[K][K];
 #pragma unroll
@@ -299,7 +291,7 @@ k_strings(SpinTables tb, int nw, const double2* __restrict__ Gact, double2* __re
     }
     if (odd) det = cz(-det.x, -det.y);
     if (sing) det = cz(0, 0);
-    r[(size_t)w * tb.n_str + s] = det;
+    if (r) r[(size_t)w * tb.n_str + s] = det;
     rT[(size_t)s * nw + w] = det;
     // B = A^-1 from P A = L U: column c solves L U x = P e_c
     double2* B = Bout + (size_t)tb.b_off[K] + ((size_t)w * ns + sl) * b_stride(K);
@@ -322,6 +314,20 @@ k_strings(SpinTables tb, int nw, const double2* __restrict__ Gact, double2* __re
 #pragma unroll
         for (int i = 0; i < K; ++i) B[i * K + c] = x[i];
     }
+}
+
+template <int K>
+__global__ void __launch_bounds__(128)
+k_strings(SpinTables tb, int nw, const double2* __restrict__ Gact, double2* __restrict__ r, double2* __restrict__ rT,
+          double2* __restrict__ Bout)
+{
+    __shared__ double2 g[MSD_XMAX];
+    const int w = blockIdx.y;
+    const int X = tb.nh * tb.np;
+    for (int e = threadIdx.x; e < X; e += blockDim.x) g[e] = Gact[(size_t)w * X + e];
+    __syncthreads();
+    const int sl = blockIdx.x * blockDim.x + threadIdx.x;
+    if (sl < tb.bucket[K + 1] - tb.bucket[K]) string_lu<K>(tb, nw, w, sl, g, r, rT, Bout);
 }
 
 template <int K>
@@ -358,6 +364,105 @@ void launch_strings(const SpinTables& tb, int nw, const double2* Gact, double2* 
     launch_strings_k<5>(tb, nw, Gact, r, rT, B, st);
     launch_strings_k<6>(tb, nw, Gact, r, rT, B, st);
     th.end(st);
+}
+
+// Walkers whose active block has an entry above 1 in magnitude (the larger of |Re|, |Im|):
+// big[w]. GT [nh np][nw], both spins. A block takes 32 walkers.
+struct LargeArgs {
+    const double2* GT[2];
+    int X[2];
+    int* big[2];
+};
+__global__ void __launch_bounds__(256) k_large(const __grid_constant__ LargeArgs a, int nw)
+{
+    __shared__ int red[8][32];
+    const int s = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, w = blockIdx.x * 32 + lane;
+    int m = 0;
+    if (w < nw)
+        for (int x = warp; x < a.X[s]; x += 8) m = max(m, mag_key(a.GT[s][(size_t)x * nw + w]));
+    red[warp][lane] = m;
+    __syncthreads();
+    if (warp || w >= nw) return;
+    for (int q = 1; q < 8; ++q) m = max(m, red[q][lane]);
+    a.big[s][w] = m >= 0x3ff00000;
+}
+
+// Ratios and inverse minors of the walkers marked by k_large, by LU, over what the
+// expansions left (k_minors.cu). A minor's LU is the exact one of a nearby block, so G - G
+// B G keeps its cancellation; inverse entries as ratios of separately rounded minors do
+// not, and lose the square of the block's magnitude (rank-1 part of 30: density matrix
+// 4e-13 against 3e-14, of 1e4: 4e-8 against 8e-12; entries up to 1: alike). A block takes
+// 128 strings of a level; the blocks of a column share the marked walkers. None marked: 3 us.
+struct StringsLargeArgs {
+    SpinTables t[2];
+    const double2* Gact[2];
+    const int* big[2];
+    double2 *r[2], *rT[2], *B[2];
+    int blk[2][MSD_KMAX + 2];   // first block of each level
+};
+__global__ void __launch_bounds__(128) k_strings_large(const __grid_constant__ StringsLargeArgs a, int nw)
+{
+    const int spin = blockIdx.z, t = threadIdx.x;
+    const SpinTables& tb = a.t[spin];
+    if ((int)blockIdx.x >= a.blk[spin][MSD_KMAX + 1]) return;
+    __shared__ double2 g[MSD_XMAX];
+    __shared__ unsigned marks[32];
+    int k = 1;
+    while ((int)blockIdx.x >= a.blk[spin][k + 1]) ++k;
+    const int X = tb.nh * tb.np, sl = ((int)blockIdx.x - a.blk[spin][k]) * 128 + t;
+    const bool on = sl < tb.bucket[k + 1] - tb.bucket[k];
+    unsigned turn = 0;
+    for (int w0 = 0; w0 < nw; w0 += 1024) {
+        __syncthreads();
+        for (int q = t >> 5; q < 32; q += 4) {
+            const int w = w0 + q * 32 + (t & 31);
+            const unsigned m = __ballot_sync(0xffffffffu, w < nw && a.big[spin][w]);
+            if ((t & 31) == 0) marks[q] = m;
+        }
+        __syncthreads();
+        for (int q = 0; q < 32; ++q)
+            for (unsigned m = marks[q]; m; m &= m - 1) {
+                if (turn++ % gridDim.y != blockIdx.y) continue;
+                const int w = w0 + q * 32 + __ffs(m) - 1;
+                __syncthreads();
+                for (int e = t; e < X; e += 128) g[e] = a.Gact[spin][(size_t)w * X + e];
+                __syncthreads();
+                if (!on) continue;
+                switch (k) {
+                case 1: string_lu<1>(tb, nw, w, sl, g, a.r[spin], a.rT[spin], a.B[spin]); break;
+                case 2: string_lu<2>(tb, nw, w, sl, g, a.r[spin], a.rT[spin], a.B[spin]); break;
+                case 3: string_lu<3>(tb, nw, w, sl, g, a.r[spin], a.rT[spin], a.B[spin]); break;
+                case 4: string_lu<4>(tb, nw, w, sl, g, a.r[spin], a.rT[spin], a.B[spin]); break;
+                case 5: string_lu<5>(tb, nw, w, sl, g, a.r[spin], a.rT[spin], a.B[spin]); break;
+                default: string_lu<6>(tb, nw, w, sl, g, a.r[spin], a.rT[spin], a.B[spin]); break;
+                }
+            }
+    }
+}
+
+// r may be NULL (both).
+void launch_strings_large(const SpinTables& ta, const SpinTables& tb, int nw, double2* const GT[2], double2* const Gact[2],
+                          int* const big[2], double2* const r[2], double2* const rT[2], void* const B[2], cudaStream_t st)
+{
+    LargeArgs l;
+    StringsLargeArgs a;
+    const SpinTables* T[2] = {&ta, &tb};
+    int nb = 0;
+    for (int s = 0; s < 2; ++s) {
+        l.GT[s] = GT[s]; l.X[s] = T[s]->nh * T[s]->np; l.big[s] = big[s];
+        a.t[s] = *T[s]; a.Gact[s] = Gact[s]; a.big[s] = big[s];
+        a.r[s] = r[s]; a.rT[s] = rT[s]; a.B[s] = (double2*)B[s];
+        a.blk[s][0] = a.blk[s][1] = 0;
+        for (int k = 1; k <= MSD_KMAX; ++k) a.blk[s][k + 1] = a.blk[s][k] + (T[s]->bucket[k + 1] - T[s]->bucket[k] + 127) / 128;
+        nb = nb > a.blk[s][MSD_KMAX + 1] ? nb : a.blk[s][MSD_KMAX + 1];
+    }
+    k_large<<<dim3((nw + 31) / 32, 2), 256, 0, st>>>(l, nw);
+    msd_note_launch();
+    if (nb <= 0) return;
+    // columns enough to fill the GPU when many walkers are marked
+    const int cols = nb >= 512 ? 4 : nb >= 128 ? 16 : 64;
+    k_strings_large<<<dim3(nb, nw < cols ? nw : cols, 2), 128, 0, st>>>(a, nw);
+    msd_note_launch();
 }
 
 // ------------------------------------------------------------------------
@@ -457,7 +562,7 @@ __device__ __forceinline__ void cmat_level(T* __restrict__ a, int g, int ng, int
 
 template <typename T>
 __device__ __forceinline__ void cmat_walker(const SpinTables& tb, int w, const double2* __restrict__ wts,
-                                            const void* __restrict__ Bin, double2* __restrict__ Cm, T* accp)
+                                            const void* __restrict__ Bin, double2* __restrict__ Cm, T* accp, bool add)
 {
     T (*acc)[2 * MSD_XMAX] = reinterpret_cast<T (*)[2 * MSD_XMAX]>(accp);
     const int X = tb.nh * tb.np;
@@ -484,33 +589,38 @@ __device__ __forceinline__ void cmat_walker(const SpinTables& tb, int w, const d
     for (int x = threadIdx.x; x < X; x += blockDim.x) {
         double re = 0, im = 0;
         for (int q = 0; q < CMAT_COPIES; ++q) { re += (double)acc[q][2 * x]; im += (double)acc[q][2 * x + 1]; }
-        Cm[(size_t)w * X + x] = cz(re, im);
+        double2* o = Cm + (size_t)w * X + x;
+        *o = add ? cadd(*o, cz(re, im)) : cz(re, im);
     }
 }
 
 // Both spins in one grid (blockIdx.y = spin), so the two spins' blocks fill
-// the machine together.
+// the machine together. big (may be NULL): only the walkers marked there, added to Cm.
 template <typename T>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 5 : 3)
 k_cmat(SpinTables ta, SpinTables tb, const double2* __restrict__ wts_a, const double2* __restrict__ wts_b,
        const void* __restrict__ Ba, const void* __restrict__ Bb, double2* __restrict__ Cm_a,
-       double2* __restrict__ Cm_b)
+       double2* __restrict__ Cm_b, const int* __restrict__ big_a, const int* __restrict__ big_b)
 {
     __shared__ T acc[CMAT_COPIES][2 * MSD_XMAX];
+    const int* big = blockIdx.y == 0 ? big_a : big_b;
+    if (big && !big[blockIdx.x]) return;
     if (blockIdx.y == 0) {
-        if (ta.nh * ta.np > 0) cmat_walker<T>(ta, blockIdx.x, wts_a, Ba, Cm_a, &acc[0][0]);
+        if (ta.nh * ta.np > 0) cmat_walker<T>(ta, blockIdx.x, wts_a, Ba, Cm_a, &acc[0][0], big != nullptr);
     } else {
-        if (tb.nh * tb.np > 0) cmat_walker<T>(tb, blockIdx.x, wts_b, Bb, Cm_b, &acc[0][0]);
+        if (tb.nh * tb.np > 0) cmat_walker<T>(tb, blockIdx.x, wts_b, Bb, Cm_b, &acc[0][0], big != nullptr);
     }
 }
 
 void launch_cmat(const SpinTables& ta, const SpinTables& tb, int nw, const double2* wts_a, const double2* wts_b,
-                 const void* Ba, const void* Bb, bool fp32, double2* Cm_a, double2* Cm_b, cudaStream_t st)
+                 const void* Ba, const void* Bb, bool fp32, double2* Cm_a, double2* Cm_b, cudaStream_t st,
+                 int* const big[2])
 {
+    const int *ga = big ? big[0] : nullptr, *gb = big ? big[1] : nullptr;
     if (ta.nh * ta.np <= 0 && tb.nh * tb.np <= 0) return;
     const dim3 grid(nw, 2);
-    if (fp32) k_cmat<float><<<grid, 256, 0, st>>>(ta, tb, wts_a, wts_b, Ba, Bb, Cm_a, Cm_b);
-    else k_cmat<double><<<grid, 256, 0, st>>>(ta, tb, wts_a, wts_b, Ba, Bb, Cm_a, Cm_b);
+    if (fp32) k_cmat<float><<<grid, 256, 0, st>>>(ta, tb, wts_a, wts_b, Ba, Bb, Cm_a, Cm_b, ga, gb);
+    else k_cmat<double><<<grid, 256, 0, st>>>(ta, tb, wts_a, wts_b, Ba, Bb, Cm_a, Cm_b, ga, gb);
     msd_note_launch();
 }
 

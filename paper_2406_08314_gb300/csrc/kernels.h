@@ -35,6 +35,10 @@ int launch_refs(const RefSpinIn* in, int n_spin, int nw, int M, unsigned* err, c
 // sub-minors are too many for launch_inverse_ratios).
 void launch_strings(const SpinTables& tb, int nw, const double2* Gact, double2* r, double2* rT, void* B, cudaStream_t st,
                     const TimerHook& th);
+// Marks the walkers with large active blocks (big [nw]) and replaces their ratios and FP64
+// inverse minors by those of the LU.
+void launch_strings_large(const SpinTables& ta, const SpinTables& tb, int nw, double2* const GT[2], double2* const Gact[2],
+                          int* const big[2], double2* const r[2], double2* const rT[2], void* const B[2], cudaStream_t st);
 // k_minors.cu: FP64 ratios rT[s][w] of both spins by expansions over shared
 // minors, those that cancel by LU (m2, t2: scratch, minor2_count entries per walker;
 // tr: minor_marks entries; all NULL: every ratio by LU), FP32 inverse minors, and the CI
@@ -48,33 +52,31 @@ void launch_inverse_minors(const SpinTables& ta, const SpinTables& tb, int nw, d
 int weights_blocks(const SpinTables& tb);
 void launch_weights(const SpinTables& ta, const SpinTables& tb, int nw, double2* const rT[2], double2* const wts[2],
                     float2* const rf[2], double2* part, int nslot, bool beta, cudaStream_t st,
-                    double2* const wT[2] = nullptr);
-// The FP64 cofactor matrix by reverse differentiation of the expansions (no inverse
-// minors): per spin the trial's strings followed by the sub-minors outside the trial
-// that their expansions need, and the targets of the reverse pass by stage (levels
-// 5, 4, 3, the 2 x 2 minors, G in n_piece pieces, their sums) with their lists.
-// V: [nh np + n2 + n_ext][nw] (G, 2 x 2 minors, ratios), its first part given;
-// Bv: [n_ext + n2 + n_piece][nw], on entry to launch_adjoint the weights of the
-// trial's strings and zeros.
-#define GRAD_STAGES 6
-struct GradTables {
+                    double2* const wT[2] = nullptr, int* const big[2] = nullptr);
+// FP64 inverse minors and the FP64 cofactor matrix from the minors: per spin the trial's
+// strings followed by the sub-minors outside the trial. V: [nh np + n2 + n_ext][nw] (G, 2
+// x 2 minors, ratios), its first part given. Bv: [n_str + n_piece][nw], on entry to
+// launch_cofactors the weights of the trial's strings (of a walker with a large active
+// block those of its vanishing ratios only: the others go by their inverse minors).
+struct ExtTables {
     int n_ext = 0, n2 = 0, n_piece = 0;
     int vbucket[MSD_KMAX + 2] = {0};
-    int stage[GRAD_STAGES + 1] = {0};
     uint4* str_hp = nullptr;     // [n_ext]
     int8_t* str_sign = nullptr;  // [n_ext]
     int* sub = nullptr;          // [n_ext][MSD_KMAX]
-    int *row = nullptr, *off = nullptr;   // launch_inverse_ratios: row alone, at SpinTables::cmx_off
-    int2* ent = nullptr;
+    int* row = nullptr;          // rows of V of the inverse minors' entries, at SpinTables::cmx_off
+    // lists of the cofactor matrix: n_piece pieces, then the nh np sums of pieces
+    int *cof_row = nullptr, *cof_off = nullptr;
+    int2* cof_ent = nullptr;
 };
 // t2 [n2][nw], tr [n_ext - bucket[3]][nw]: scratch.
-void launch_minors_ext(const GradTables g[2], const SpinTables& ta, const SpinTables& tb, int nw, double2* const V[2],
+void launch_minors_ext(const ExtTables g[2], const SpinTables& ta, const SpinTables& tb, int nw, double2* const V[2],
                        int* const t2[2], int* const tr[2], cudaStream_t st);
 // FP64 inverse minors from V as launch_minors_ext left it.
-void launch_inverse_ratios(const GradTables g[2], const SpinTables& ta, const SpinTables& tb, int nw,
+void launch_inverse_ratios(const ExtTables g[2], const SpinTables& ta, const SpinTables& tb, int nw,
                            double2* const V[2], void* const B[2], cudaStream_t st);
-void launch_adjoint(const GradTables g[2], const SpinTables& ta, const SpinTables& tb, int nw, double2* const V[2],
-                    double2* const Bv[2], double2* const Cm[2], cudaStream_t st);
+void launch_cofactors(const ExtTables g[2], const SpinTables& ta, const SpinTables& tb, int nw, double2* const V[2],
+                      double2* const Bv[2], double2* const Cm[2], cudaStream_t st);
 void launch_untranspose(int n_str, int nw, const double2* rT, double2* r, cudaStream_t st);
 void launch_det_ratios(const PairTables& pt, int nw, int n_str_a, int n_str_b, const double2* ra,
                        const double2* rb, double2* out, cudaStream_t st);
@@ -82,7 +84,8 @@ void launch_sum_slots(int nw, const double2* part, int nslot, int slot0, int n, 
                       const double2* O0a, const double2* O0b, double2* ovlp, cudaStream_t st);
 void launch_ref_ovlp(int nw, const double2* O0a, const double2* O0b, double2* out, cudaStream_t st);
 void launch_cmat(const SpinTables& ta, const SpinTables& tb, int nw, const double2* wts_a, const double2* wts_b,
-                 const void* Ba, const void* Bb, bool fp32, double2* Cm_a, double2* Cm_b, cudaStream_t st);
+                 const void* Ba, const void* Bb, bool fp32, double2* Cm_a, double2* Cm_b, cudaStream_t st,
+                 int* const big[2] = nullptr);
 void launch_gt(const SpinTables& ta, const SpinTables& tb, int nw, int M, double2* const Gr[2], const double2* const Cm[2],
                const double2* R, double2* GT, long long ld, const long long off[2], bool minus_ref, cudaStream_t st);
 void launch_rdm_scatter(const SpinTables& tb, int nw, int M, const double2* GT, long long ld, long long off, int spin,

@@ -188,12 +188,10 @@ struct msd_ctx {
     // spin, both spins' rows concatenated, the transposed Cholesky vectors
     // and exp(-dt h'/2)
     DgConst dg_Lh[2], dg_Lcat, dg_Lt, dg_E[2];
-    // FP64 cofactors by reverse differentiation (built on first use per trial)
-    GradTables grad[2];
-    bool grad_ready = false, grad_ok = false;
-    // FP64 inverse minors from the ratios (built on first use per trial)
-    GradTables inv[2];
-    bool inv_ready = false, inv_ok = false;
+    // FP64 inverse minors and cofactors from the minors themselves (built on first
+    // use per trial)
+    ExtTables ext[2];
+    bool ext_ready = false, ext_ok = false;
 };
 
 namespace {
@@ -201,7 +199,7 @@ namespace {
 void free_mixed(msd_ctx* ctx);
 void free_exact_ref(msd_ctx* ctx);
 void free_prop(msd_ctx* ctx);
-void free_grad(msd_ctx* ctx);
+void free_ext(msd_ctx* ctx);
 
 int fail(msd_ctx* c, int code, const char* fmt, ...)
 {
@@ -624,13 +622,14 @@ int upload_spin(msd_ctx* ctx, SpinHost& S)
     return MSD_OK;
 }
 
-void free_grad(msd_ctx* ctx)
+void free_ext(msd_ctx* ctx)
 {
-    for (GradTables* g : {&ctx->grad[0], &ctx->grad[1], &ctx->inv[0], &ctx->inv[1]}) {
-        cudaFree(g->str_hp); cudaFree(g->str_sign); cudaFree(g->sub); cudaFree(g->row); cudaFree(g->off); cudaFree(g->ent);
-        *g = GradTables{};
+    for (ExtTables& g : ctx->ext) {
+        cudaFree(g.str_hp); cudaFree(g.str_sign); cudaFree(g.sub); cudaFree(g.row);
+        cudaFree(g.cof_row); cudaFree(g.cof_off); cudaFree(g.cof_ent);
+        g = ExtTables{};
     }
-    ctx->grad_ready = ctx->grad_ok = ctx->inv_ready = ctx->inv_ok = false;
+    ctx->ext_ready = ctx->ext_ok = false;
 }
 
 // A string as two words (7 bits per index, the level on top of the holes).
@@ -689,9 +688,9 @@ struct StringMap {
 };
 
 // One spin's strings, the trial's followed by those outside it that are needed, by
-// level upwards. A string of level k >= 4 is evaluated over the k strings without its
-// last hole and one particle; with `all`, the k^2 sub-minors (one hole and one
-// particle less) of the trial's strings are needed too.
+// level upwards: the k^2 sub-minors (one hole and one particle less) of the trial's
+// strings of level k >= 4, and, as a string is evaluated over the k strings without its
+// last hole and one particle, those of the strings added.
 struct Closure {
     std::vector<StringKey> key;
     StringMap at{64};            // level >= 3: number
@@ -699,7 +698,7 @@ struct Closure {
     std::vector<int8_t> sign;
     std::vector<int> sub;        // [string][MSD_KMAX] (string << 1 | negative)
     // false: far more of them than the trial has strings
-    bool build(const SpinHost& S, bool all, GradTables& g)
+    bool build(const SpinHost& S, ExtTables& g)
     {
         constexpr int K = MSD_KMAX;
         const size_t limit = 4 * (size_t)S.n_str + 4096;
@@ -726,8 +725,8 @@ struct Closure {
                         if (at.get(c) < 0) { at.put(c, S.n_str); extra[k - 1].push_back(c); ++n_extra; }
                     }
             };
-            for (int f = S.bucket[k]; f < S.bucket[k + 1]; ++f) expand(key[f], all ? 0 : k - 1);
-            for (size_t i = 0; i < extra[k].size(); ++i) expand(extra[k][i], k - 1);
+            for (int f = S.bucket[k]; f < S.bucket[k + 1] && n_extra <= limit; ++f) expand(key[f], 0);
+            for (size_t i = 0; i < extra[k].size() && n_extra <= limit; ++i) expand(extra[k][i], k - 1);
             if (n_extra > limit) return false;
         }
         for (int k = 0; k <= K; ++k) {
@@ -755,7 +754,7 @@ struct Closure {
         }
         return true;
     }
-    int upload_to(msd_ctx* ctx, GradTables& g)
+    int upload_to(msd_ctx* ctx, ExtTables& g)
     {
         int rc;
         uint8_t* d_hp = nullptr;
@@ -772,21 +771,29 @@ int minor2_row(const StringKey& q, int a, int b, int c, int d, int nh, int np)
     return pair_index(q.hole(a), q.hole(b), nh) * (np * (np - 1) / 2) + pair_index(q.part(c), q.part(d), np);
 }
 
-// Tables of the FP64 inverse minors, once per trial: for entry (i, j) of a string's
-// k x k inverse the row of V = [G | 2 x 2 minors | ratios] that holds its cofactor
-// (the minor without hole j and particle i), twice, plus 1 where its sign is negative.
+// Tables of the FP64 inverse minors and of the cofactor matrix, once per trial. For
+// entry (i, j) of a string's k x k inverse, the row of V = [G | 2 x 2 minors | ratios] that
+// holds its cofactor (the minor without hole j and particle i), twice, plus 1 where its
+// sign is negative; and the same entries by (hole, particle), in pieces of at most LONG.
 // Trials with far more sub-minors than strings keep the LU path.
-int prepare_inverse(msd_ctx* ctx)
+int prepare_ext(msd_ctx* ctx)
 {
-    if (ctx->inv_ready) return MSD_OK;
-    ctx->inv_ready = true;
+    if (ctx->ext_ready) return MSD_OK;
+    ctx->ext_ready = true;
+    constexpr int LONG = 64;
     Closure C[2];
-    std::vector<int> row[2];
+    std::vector<int> row[2], crow[2], coff[2];
+    std::vector<int2> cent[2];
     for (int s = 0; s < 2; ++s) {
         const SpinHost& S = ctx->sp[s];
-        GradTables& g = ctx->inv[s];
-        if (!C[s].build(S, true, g)) return MSD_OK;
+        ExtTables& g = ctx->ext[s];
+        if (!C[s].build(S, g)) return MSD_OK;
         const int X = S.nh * S.np;
+        struct Use { int x; int2 e; };
+        std::vector<Use> uses;
+        std::vector<int> first(X + 1, 0);
+        row[s].reserve((size_t)S.b_per_walker);
+        uses.reserve((size_t)S.b_per_walker);
         for (int f = S.bucket[1]; f < S.n_str; ++f) {
             const StringKey& q = C[s].key[f];
             const int k = q.level();
@@ -800,124 +807,46 @@ int prepare_inverse(msd_ctx* ctx)
                         neg ^= C[s].sign[c] < 0;
                         r = X + g.n2 + c;
                     }
-                    row[s].push_back(r << 1 | (neg ^ (C[s].sign[f] < 0)));
+                    neg ^= C[s].sign[f] < 0;
+                    row[s].push_back(r << 1 | neg);
+                    const int x = q.hole(j) * S.np + q.part(i);
+                    uses.push_back(Use{x, make_int2((k == 1 ? -2 : r * 2) | neg, f)});
+                    ++first[x + 1];
                 }
         }
-        if (row[s].empty()) row[s].push_back(0);
-    }
-    for (int s = 0; s < 2; ++s) {
-        int rc;
-        if ((rc = C[s].upload_to(ctx, ctx->inv[s]))) return rc;
-        if ((rc = upload(ctx, &ctx->inv[s].row, row[s]))) return rc;
-    }
-    ctx->inv_ok = true;
-    return MSD_OK;
-}
-
-// Tables of the FP64 cofactors' reverse pass, once per trial. Trials that would need
-// far more strings than they have keep the LU path.
-int prepare_grad(msd_ctx* ctx)
-{
-    if (ctx->grad_ready) return MSD_OK;
-    ctx->grad_ready = true;
-    constexpr int LONG = 64;   // a G target's list is cut at LONG entries
-    Closure C[2];
-    std::vector<int> row[2], off[2];
-    std::vector<int2> ent[2];
-    for (int s = 0; s < 2; ++s) {
-        const SpinHost& S = ctx->sp[s];
-        GradTables& g = ctx->grad[s];
-        if (!C[s].build(S, false, g)) return MSD_OK;
-        const int X = S.nh * S.np, npp = S.np * (S.np - 1) / 2;
-        const std::vector<StringKey>& key = C[s].key;
-        // (target, list entry), in string order; targets: ratios, 2 x 2 minors, G
-        struct Use { int target; int2 e; };
-        std::vector<Use> uses;
-        uses.reserve((size_t)g.n_ext * 10 + (size_t)g.n2 * 4);
-        auto use = [&](int target, int a, int neg, int b) { uses.push_back(Use{target, make_int2(a * 2 + (neg & 1), b)}); };
-        auto gx = [&](int h, int p) { return h * S.np + p; };
-        const int T2 = g.n_ext, TG = g.n_ext + g.n2, V2 = X, VR = X + g.n2;
-        std::vector<char> used2(std::max(1, g.n2), 0);
-        for (int f = 0; f < g.n_ext; ++f) {
-            const StringKey& q = key[f];
-            const int k = q.level(), sf = C[s].sign[f] < 0;
-            auto m2 = [&](int c, int d) { return minor2_row(q, 0, 1, c, d, S.nh, S.np); };
-            if (k == 1) use(TG + gx(q.hole(0), q.part(0)), -1, sf, f);
-            if (k == 2) { use(T2 + m2(0, 1), -1, sf, f); used2[m2(0, 1)] = 1; }
-            if (k == 3)
-                for (int j = 0; j < 3; ++j) {
-                    const int m = m2(j == 0 ? 1 : 0, j == 2 ? 1 : 2), x = gx(q.hole(2), q.part(j)), neg = (j & 1) ^ sf;
-                    use(T2 + m, x, neg, f);
-                    use(TG + x, V2 + m, neg, f);
-                    used2[m] = 1;
-                }
-            if (k >= 4)
-                for (int j = 0; j < k; ++j) {
-                    const int c = C[s].sub[(size_t)f * MSD_KMAX + j] >> 1, neg = C[s].sub[(size_t)f * MSD_KMAX + j] & 1;
-                    const int x = gx(q.hole(k - 1), q.part(j));
-                    use(c, x, neg, f);
-                    use(TG + x, VR + c, neg, f);
-                }
-        }
-        for (int h = 0; h < S.nh; ++h)
-            for (int h2 = h + 1; h2 < S.nh; ++h2)
-                for (int p = 0; p < S.np; ++p)
-                    for (int p2 = p + 1; p2 < S.np; ++p2) {
-                        const int m = pair_index(h, h2, S.nh) * npp + pair_index(p, p2, S.np), b = g.n_ext + m;
-                        if (!used2[m]) continue;   // its adjoint is zero
-                        use(TG + gx(h, p), gx(h2, p2), 0, b);
-                        use(TG + gx(h2, p2), gx(h, p), 0, b);
-                        use(TG + gx(h, p2), gx(h2, p), 1, b);
-                        use(TG + gx(h2, p), gx(h, p2), 1, b);
-                    }
-        std::vector<int> first(TG + X + 1, 0), fill;
-        for (const Use& u : uses) ++first[u.target + 1];
-        for (int i = 0; i < TG + X; ++i) first[i + 1] += first[i];
+        for (int x = 0; x < X; ++x) first[x + 1] += first[x];
         std::vector<int2> list(uses.size());
-        fill.assign(first.begin(), first.end() - 1);
-        for (const Use& u : uses) list[fill[u.target]++] = u.e;
-        off[s].push_back(0);
-        auto add = [&](int r, int i0, int i1) {
-            row[s].push_back(r);
-            ent[s].insert(ent[s].end(), list.begin() + i0, list.begin() + i1);
-            off[s].push_back((int)ent[s].size());
-        };
-        auto add_all = [&](int target, int r) { if (first[target] < first[target + 1]) add(r, first[target], first[target + 1]); };
-        for (int q = 0; q < 3; ++q) {   // levels 5, 4, 3
-            const int k = 5 - q;
-            g.stage[q] = (int)row[s].size();
-            for (int f = S.bucket[k]; f < S.bucket[k + 1]; ++f) add_all(f, f);
-            for (int f = g.vbucket[k]; f < g.vbucket[k + 1]; ++f) add_all(f, f);
-        }
-        g.stage[3] = (int)row[s].size();
-        for (int m = 0; m < g.n2; ++m) add_all(T2 + m, g.n_ext + m);
-        // G: the lists in pieces (few targets with long lists), then the pieces' sums
-        g.stage[4] = (int)row[s].size();
+        std::vector<int> fill(first.begin(), first.end() - 1);
+        for (const Use& u : uses) list[fill[u.x]++] = u.e;
+        coff[s].push_back(0);
         std::vector<int> piece(X + 1, 0);
         for (int x = 0; x < X; ++x) {
-            for (int i = first[TG + x]; i < first[TG + x + 1]; i += LONG)
-                add(g.n_ext + g.n2 + g.n_piece++, i, std::min(i + LONG, first[TG + x + 1]));
+            for (int i = first[x]; i < first[x + 1]; i += LONG) {
+                crow[s].push_back(S.n_str + g.n_piece++);
+                coff[s].push_back(std::min(i + LONG, first[x + 1]));
+            }
             piece[x + 1] = g.n_piece;
         }
-        g.stage[5] = (int)row[s].size();
-        for (int x = 0; x < X; ++x) {
-            row[s].push_back(x);
-            for (int i = piece[x]; i < piece[x + 1]; ++i) ent[s].push_back(make_int2(-2, g.n_ext + g.n2 + i));
-            off[s].push_back((int)ent[s].size());
+        cent[s] = std::move(list);
+        for (int x = 0; x < X; ++x) {   // the pieces' sums
+            crow[s].push_back(x);
+            for (int i = piece[x]; i < piece[x + 1]; ++i) cent[s].push_back(make_int2(-2, S.n_str + i));
+            coff[s].push_back((int)cent[s].size());
         }
-        g.stage[6] = (int)row[s].size();
-        if (ent[s].empty()) ent[s].push_back(make_int2(0, 0));
-        if (row[s].empty()) row[s].push_back(0);
+        for (auto* v : {&row[s], &crow[s]})
+            if (v->empty()) v->push_back(0);
+        if (cent[s].empty()) cent[s].push_back(make_int2(0, 0));
     }
     for (int s = 0; s < 2; ++s) {
-        GradTables& g = ctx->grad[s];
+        ExtTables& g = ctx->ext[s];
         int rc;
         if ((rc = C[s].upload_to(ctx, g))) return rc;
         if ((rc = upload(ctx, &g.row, row[s]))) return rc;
-        if ((rc = upload(ctx, &g.off, off[s]))) return rc;
-        if ((rc = upload(ctx, &g.ent, ent[s]))) return rc;
+        if ((rc = upload(ctx, &g.cof_row, crow[s]))) return rc;
+        if ((rc = upload(ctx, &g.cof_off, coff[s]))) return rc;
+        if ((rc = upload(ctx, &g.cof_ent, cent[s]))) return rc;
     }
-    ctx->grad_ok = true;
+    ctx->ext_ok = true;
     return MSD_OK;
 }
 
@@ -1328,8 +1257,9 @@ struct Chunk {
     double2 *Gr[2], *O0[2], *Gact[2], *GactT[2], *m2[2], *rT[2], *r[2], *wts[2], *part;
     float2* rf[2];   // FP32 copies of r (mixed mode, with B)
     void* B[2];
-    double2 *V[2], *Bv[2];   // expansions (launch_minors_ext) and their reverse pass
+    double2 *V[2], *Bv[2];   // expansions (launch_minors_ext); weights and pieces (launch_cofactors)
     int *t2[2], *tr[2];      // the minors' largest products (launch_minors)
+    int* big[2];             // walkers with large active blocks (launch_strings_large)
     int nslot, nR;
 };
 
@@ -1337,13 +1267,13 @@ struct Chunk {
 enum class StringUse {
     Overlap,     // nothing
     Minors,      // inverse minors and weights of both spins (mixed mode: FP32 ratios too)
-    Cofactors,   // the cofactor matrix alone, in FP64 (prepare_grad's tables)
+    Cofactors,   // the cofactor matrix alone, in FP64 from the minors (prepare_ext's tables)
 };
 
-// FP64 inverse minors of a call: from the ratios' tables where the trial has them.
-bool ratio_inverse(const msd_ctx* ctx, StringUse use)
+// The call's minors are those of prepare_ext's tables (V).
+bool use_ext(const msd_ctx* ctx, StringUse use)
 {
-    return use == StringUse::Minors && ctx->prec == MSD_FP64 && ctx->inv_ok;
+    return use == StringUse::Cofactors || (use == StringUse::Minors && ctx->prec == MSD_FP64 && ctx->ext_ok);
 }
 
 // The use of a call that needs the cofactors or inverse minors (energy).
@@ -1351,9 +1281,8 @@ int string_use(msd_ctx* ctx, bool energy, StringUse* use)
 {
     *use = StringUse::Minors;
     if (ctx->prec != MSD_FP64) return MSD_OK;
-    if (energy) return prepare_inverse(ctx);
-    const int rc = prepare_grad(ctx);
-    if (!rc && ctx->grad_ok) *use = StringUse::Cofactors;
+    const int rc = prepare_ext(ctx);
+    if (!rc && ctx->ext_ok && !energy) *use = StringUse::Cofactors;
     return rc;
 }
 
@@ -1361,40 +1290,41 @@ int string_use(msd_ctx* ctx, bool energy, StringUse* use)
 size_t mark_rows(const msd_ctx* ctx, int s, StringUse use)
 {
     const SpinHost& S = ctx->sp[s];
-    const int n = use == StringUse::Cofactors ? ctx->grad[s].n_ext : ratio_inverse(ctx, use) ? ctx->inv[s].n_ext : S.n_str;
-    return std::max(1, n - S.bucket[3]);
+    return std::max(1, (use_ext(ctx, use) ? ctx->ext[s].n_ext : S.n_str) - S.bucket[3]);
 }
 
-// The ratios as r[w][s] are for the FP64 per-determinant terms (Minors in FP64 mode)
-// or for the caller (want_r).
-size_t overlap_bytes_per_walker(msd_ctx* ctx, StringUse use, int nslot, bool want_r = false)
+// want_r: the ratios as r[w][s] are for the caller (the FP64 per-determinant terms read
+// them in any case). cof: the cofactor matrix is needed.
+size_t overlap_bytes_per_walker(msd_ctx* ctx, StringUse use, int nslot, bool want_r = false, bool cof = false)
 {
-    const bool want_b = use == StringUse::Minors, cof = use == StringUse::Cofactors;
-    const bool fp64_b = want_b && ctx->prec == MSD_FP64, inv = ratio_inverse(ctx, use);
+    const bool want_b = use == StringUse::Minors, ext = use_ext(ctx, use);
+    const bool fp64_b = want_b && ctx->prec == MSD_FP64;
     size_t b = 0;
     for (int s = 0; s < 2; ++s) {
         const SpinHost& S = ctx->sp[s];
         b += (size_t)S.N * ctx->M + 1 + 2 * (size_t)S.nh * S.np + (size_t)S.n_str;
         b += ref_dg_bytes(ctx->M, S.N) / sizeof(double2) + 1;
-        if (!fp64_b) b += minor2_count(tables(S, 1));
-        if (!fp64_b || inv) b += (minor2_count(tables(S, 1)) + mark_rows(ctx, s, use)) / 4 + 2;
-        if (inv) b += ctx->inv[s].n2 + ctx->inv[s].n_ext - S.n_str;
-        if (cof) b += 2 * (size_t)ctx->grad[s].n_ext + ctx->grad[s].n2 + ctx->grad[s].n_piece - S.n_str;
+        if (ext) b += ctx->ext[s].n2 + ctx->ext[s].n_ext - S.n_str;
+        else if (!fp64_b) b += minor2_count(tables(S, 1));
+        if (ext || !fp64_b) b += (minor2_count(tables(S, 1)) + mark_rows(ctx, s, use)) / 4 + 2;
+        if (ext && cof) b += S.n_str + ctx->ext[s].n_piece;
         if (fp64_b || want_r) b += S.n_str;
-        if (want_b) b += S.n_str + S.b_per_walker + (S.n_str + 1) / 2;
+        if (want_b || cof) b += S.n_str + S.b_per_walker;
+        if (want_b && !fp64_b) b += (S.n_str + 1) / 2;
+        if (ext) b += 1;
     }
     b += nslot;
     return b * sizeof(double2);
 }
 
-int chunk_alloc(msd_ctx* ctx, int cap, StringUse use, int nslot, Chunk& c, bool want_r = false)
+int chunk_alloc(msd_ctx* ctx, int cap, StringUse use, int nslot, Chunk& c, bool want_r = false, bool cof = false)
 {
     int rc;
-    const bool want_b = use == StringUse::Minors, cof = use == StringUse::Cofactors;
-    const bool fp64_b = want_b && ctx->prec == MSD_FP64, inv = ratio_inverse(ctx, use);
-    static const char* names[2][14] = {
-        {"Gr_a", "O0_a", "Gact_a", "GactT_a", "m2_a", "rT_a", "r_a", "wts_a", "B_a", "rf_a", "V_a", "Bv_a", "t2_a", "tr_a"},
-        {"Gr_b", "O0_b", "Gact_b", "GactT_b", "m2_b", "rT_b", "r_b", "wts_b", "B_b", "rf_b", "V_b", "Bv_b", "t2_b", "tr_b"}};
+    const bool want_b = use == StringUse::Minors, ext = use_ext(ctx, use);
+    const bool fp64_b = want_b && ctx->prec == MSD_FP64;
+    static const char* names[2][15] = {
+        {"Gr_a", "O0_a", "Gact_a", "GactT_a", "m2_a", "rT_a", "r_a", "wts_a", "B_a", "rf_a", "V_a", "Bv_a", "t2_a", "tr_a", "big_a"},
+        {"Gr_b", "O0_b", "Gact_b", "GactT_b", "m2_b", "rT_b", "r_b", "wts_b", "B_b", "rf_b", "V_b", "Bv_b", "t2_b", "tr_b", "big_b"}};
     for (int s = 0; s < 2; ++s) {
         const SpinHost& S = ctx->sp[s];
         const size_t X = std::max(1, S.nh * S.np), w16 = sizeof(double2) * (size_t)cap;
@@ -1405,20 +1335,21 @@ int chunk_alloc(msd_ctx* ctx, int cap, StringUse use, int nslot, Chunk& c, bool 
         if ((rc = get(0, w16 * S.N * ctx->M, true, (void**)&c.Gr[s]))) return rc;
         if ((rc = get(1, w16, true, (void**)&c.O0[s]))) return rc;
         if ((rc = get(2, w16 * X, true, (void**)&c.Gact[s]))) return rc;
-        if ((rc = get(3, w16 * X, !cof && !inv, (void**)&c.GactT[s]))) return rc;
-        if ((rc = get(4, w16 * minor2_count(tables(S, 1)), !fp64_b && !cof, (void**)&c.m2[s]))) return rc;
-        if ((rc = get(5, w16 * S.n_str, !cof && !inv, (void**)&c.rT[s]))) return rc;
-        const GradTables& g = inv ? ctx->inv[s] : ctx->grad[s];
-        if ((rc = get(10, w16 * (X + (size_t)g.n2 + g.n_ext), cof || inv, (void**)&c.V[s]))) return rc;
-        if ((rc = get(11, w16 * ((size_t)g.n_ext + g.n2 + g.n_piece), cof, (void**)&c.Bv[s]))) return rc;
-        if (cof || inv) c.GactT[s] = c.V[s];   // the head of V
-        const bool marks = !fp64_b || inv;
+        if ((rc = get(3, w16 * X, !ext, (void**)&c.GactT[s]))) return rc;
+        if ((rc = get(4, w16 * minor2_count(tables(S, 1)), !ext && !fp64_b, (void**)&c.m2[s]))) return rc;
+        if ((rc = get(5, w16 * S.n_str, !ext, (void**)&c.rT[s]))) return rc;
+        const ExtTables& g = ctx->ext[s];
+        if ((rc = get(10, w16 * (X + (size_t)g.n2 + g.n_ext), ext, (void**)&c.V[s]))) return rc;
+        if ((rc = get(11, w16 * ((size_t)S.n_str + g.n_piece), ext && cof, (void**)&c.Bv[s]))) return rc;
+        if (ext) c.GactT[s] = c.V[s];   // the head of V
+        const bool marks = ext || !fp64_b;
         if ((rc = get(12, sizeof(int) * cap * minor2_count(tables(S, 1)), marks, (void**)&c.t2[s]))) return rc;
         if ((rc = get(13, sizeof(int) * cap * mark_rows(ctx, s, use), marks, (void**)&c.tr[s]))) return rc;
         if ((rc = get(6, w16 * S.n_str, fp64_b || want_r, (void**)&c.r[s]))) return rc;
-        if ((rc = get(7, w16 * S.n_str, want_b, (void**)&c.wts[s]))) return rc;
-        if ((rc = get(8, sizeof(double2) * std::max<long long>(1, cap * S.b_per_walker), want_b, &c.B[s]))) return rc;
-        if ((rc = get(9, sizeof(float2) * cap * (size_t)S.n_str, want_b, (void**)&c.rf[s]))) return rc;
+        if ((rc = get(7, w16 * S.n_str, want_b || cof, (void**)&c.wts[s]))) return rc;
+        if ((rc = get(8, sizeof(double2) * std::max<long long>(1, cap * S.b_per_walker), want_b || cof, &c.B[s]))) return rc;
+        if ((rc = get(9, sizeof(float2) * cap * (size_t)S.n_str, want_b && !fp64_b, (void**)&c.rf[s]))) return rc;
+        if ((rc = get(14, sizeof(int) * cap, ext, (void**)&c.big[s]))) return rc;
     }
     void* p;
     if ((rc = arena_get(ctx, "part", sizeof(double2) * cap * std::max(1, nslot), &p))) return rc;
@@ -1473,31 +1404,16 @@ int run_strings_weights(msd_ctx* ctx, int nw, int cap, Chunk& c, StringUse use, 
     const TimerHook& th = ctx->hook;
     const bool want_b = use == StringUse::Minors;
     SpinTables T[2] = {tables(ctx->sp[0], cap), tables(ctx->sp[1], cap)};
-    if (use == StringUse::Cofactors) {
-        double2 *rT[2], *none[2] = {nullptr, nullptr};
-        float2* no_f[2] = {nullptr, nullptr};
-        for (int s = 0; s < 2; ++s) {
-            const GradTables& g = ctx->grad[s];
-            rT[s] = c.V[s] + ((size_t)T[s].nh * T[s].np + g.n2) * nw;
-            // adjoints: the weights in the trial's strings, zero elsewhere
-            CK(cudaMemsetAsync(c.Bv[s] + (size_t)T[s].n_str * nw, 0,
-                               sizeof(double2) * (size_t)nw * (g.n_ext - T[s].n_str + g.n2 + g.n_piece), st));
+    if (use_ext(ctx, use)) {
+        // the ratios are V's last rows
+        for (int s = 0; s < 2; ++s) c.rT[s] = c.V[s] + ((size_t)T[s].nh * T[s].np + ctx->ext[s].n2) * nw;
+        th.begin("k_strings", st);
+        launch_minors_ext(ctx->ext, T[0], T[1], nw, c.V, c.t2, c.tr, st);
+        if (want_b) {
+            launch_inverse_ratios(ctx->ext, T[0], T[1], nw, c.V, c.B, st);
+            for (int s = 0; s < 2; ++s) launch_untranspose(T[s].n_str, nw, c.rT[s], c.r[s], st);
         }
-        th.begin("k_strings", st);
-        launch_minors_ext(ctx->grad, T[0], T[1], nw, c.V, c.t2, c.tr, st);
-        th.end(st);
-        th.begin("k_weights", st);
-        launch_weights(T[0], T[1], nw, rT, none, no_f, c.part, c.nslot, true, st, c.Bv);
-        th.end(st);
-        CKLAUNCH();
-        return MSD_OK;
-    }
-    if (ratio_inverse(ctx, use)) {
-        for (int s = 0; s < 2; ++s) c.rT[s] = c.V[s] + ((size_t)T[s].nh * T[s].np + ctx->inv[s].n2) * nw;
-        th.begin("k_strings", st);
-        launch_minors_ext(ctx->inv, T[0], T[1], nw, c.V, c.t2, c.tr, st);
-        launch_inverse_ratios(ctx->inv, T[0], T[1], nw, c.V, c.B, st);
-        for (int s = 0; s < 2; ++s) launch_untranspose(T[s].n_str, nw, c.rT[s], c.r[s], st);
+        launch_strings_large(T[0], T[1], nw, c.GactT, c.Gact, c.big, c.r, c.rT, c.B, st);
         th.end(st);
     } else if (want_b && !fp32_b) {
         for (int s = 0; s < 2; ++s) launch_strings(T[s], nw, c.Gact[s], c.r[s], c.rT[s], c.B[s], st, th);
@@ -1510,7 +1426,9 @@ int run_strings_weights(msd_ctx* ctx, int nw, int cap, Chunk& c, StringUse use, 
     CKLAUNCH();
     float2* no_rf[2] = {nullptr, nullptr};
     th.begin("k_weights", st);
-    launch_weights(T[0], T[1], nw, c.rT, c.wts, want_b && fp32_b ? c.rf : no_rf, c.part, c.nslot, want_b, st);
+    const bool cof = use_ext(ctx, use) && c.Bv[0];
+    launch_weights(T[0], T[1], nw, c.rT, c.wts, want_b && fp32_b ? c.rf : no_rf, c.part, c.nslot, want_b || cof, st,
+                   cof ? c.Bv : nullptr, c.big);
     th.end(st);
     CKLAUNCH();
     return MSD_OK;
@@ -1529,8 +1447,9 @@ int run_cofactors(msd_ctx* ctx, int nw, int cap, Chunk& c, StringUse use, bool f
 {
     const SpinTables T[2] = {tables(ctx->sp[0], cap), tables(ctx->sp[1], cap)};
     ctx->hook.begin("k_cmat", st);
-    if (use == StringUse::Cofactors) launch_adjoint(ctx->grad, T[0], T[1], nw, c.V, c.Bv, Cm, st);
-    else launch_cmat(T[0], T[1], nw, c.wts[0], c.wts[1], c.B[0], c.B[1], fp32, Cm[0], Cm[1], st);
+    const bool ext = use_ext(ctx, use);
+    if (ext) launch_cofactors(ctx->ext, T[0], T[1], nw, c.V, c.Bv, Cm, st);
+    launch_cmat(T[0], T[1], nw, c.wts[0], c.wts[1], c.B[0], c.B[1], fp32, Cm[0], Cm[1], st, ext ? c.big : nullptr);
     ctx->hook.end(st);
     CKLAUNCH();
     return MSD_OK;
@@ -2010,12 +1929,12 @@ int evaluate_impl(msd_ctx* ctx, int n_w, const double* phi_a, const double* phi_
     const int nslot = nR + (want_e ? energy_slots(ctx) : 0);
     StringUse use = StringUse::Overlap;
     if ((want_v || want_e) && (rc = string_use(ctx, want_e, &use))) return rc;
-    size_t per = overlap_bytes_per_walker(ctx, use, nslot);
+    size_t per = overlap_bytes_per_walker(ctx, use, nslot, false, want_v);
     if (want_v) per += fb_bytes_per_walker(ctx, fp32);
     if (want_e) per += en_bytes_per_walker(ctx, fp32);
     const int cap = chunk_for(ctx, per, n_w);
     Chunk c;
-    if ((rc = chunk_alloc(ctx, cap, use, nslot, c))) return rc;
+    if ((rc = chunk_alloc(ctx, cap, use, nslot, c, false, want_v))) return rc;
     FbWork f;
     EnWork E;
     if (want_v && (rc = fb_alloc(ctx, cap, fp32, f))) return rc;
@@ -2116,10 +2035,10 @@ int rdm1(msd_ctx* ctx, int n_w, const double* phi_a, const double* phi_b, double
     const int nR = weights_blocks(tables(ctx->sp[0], 1));
     StringUse use;
     if ((rc = string_use(ctx, false, &use))) return rc;
-    const int cap = chunk_for(ctx, overlap_bytes_per_walker(ctx, use, nR) + fb_bytes_per_walker(ctx, false), n_w);
+    const int cap = chunk_for(ctx, overlap_bytes_per_walker(ctx, use, nR, false, true) + fb_bytes_per_walker(ctx, false), n_w);
     Chunk c;
     FbWork f;
-    if ((rc = chunk_alloc(ctx, cap, use, nR, c))) return rc;
+    if ((rc = chunk_alloc(ctx, cap, use, nR, c, false, true))) return rc;
     if ((rc = fb_alloc(ctx, cap, false, f))) return rc;
     const TimerHook& th = ctx->hook;
     for (int w0 = 0; w0 < n_w; w0 += cap) {
@@ -2471,7 +2390,7 @@ void msd_destroy(msd_ctx* ctx)
     cudaFree(ctx->pairs.d_det_index); cudaFree(ctx->pairs.d_cf);
     free_mixed(ctx);
     free_prop(ctx);
-    free_grad(ctx);
+    free_ext(ctx);
     cudaFree(ctx->d_h1); cudaFree(ctx->d_Lcat); cudaFree(ctx->d_err);
     cudaFreeHost(ctx->h_err);
     for (auto& p : ctx->pending) { ctx->ev_pool.push_back(p.a); ctx->ev_pool.push_back(p.b); }
@@ -2513,7 +2432,7 @@ int msd_set_trial(msd_ctx* ctx, int n_det, const double* coeff, const int32_t* o
     if (n_det <= 0 || !coeff || !occ_a || !occ_b) return fail(ctx, MSD_ERR_ARG, "empty trial");
     CK(cudaSetDevice(ctx->device));
     ctx->have_trial = false;
-    free_grad(ctx);
+    free_ext(ctx);
     std::vector<int> sid[2];
     const int32_t* occ[2] = {occ_a, occ_b};
     for (int s = 0; s < 2; ++s) {

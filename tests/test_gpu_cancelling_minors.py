@@ -1,6 +1,7 @@
 """Walkers that overlap the reference little: the Green's function's active block is a
 large part of low rank plus one of order one, and the minors from level 3 on are sums
-that cancel. Ratios and overlaps against 60-digit arithmetic, within what a pivoted LU of every minor may be off."""
+that cancel. Ratios, overlaps, density matrix, force bias and energy against 60-digit
+arithmetic, within what a pivoted LU of every minor may be off."""
 import numpy as np
 import pytest
 
@@ -79,3 +80,32 @@ def test_ratios(rank, size, complete):
         ctx.overlap_noalloc(*dev, o)
         assert np.all(np.abs(o.cpu().numpy() - total) <= tt), prec
         ctx.close()
+
+
+@pytest.mark.parametrize("rank,size", CASES)
+def test_observables(rank, size):
+    import torch
+
+    from paper_2406_08314_gb300 import msd
+    s, w = _system(2, False), _walkers(rank, size, 1, 9)
+    ref = exact_msd.msd(s, *w)
+    # a determinant's relative error as of the LU bounds of its two strings (their
+    # inverses are off by no more), its Green's function and energy weighted with it;
+    # FP64 sums of terms as large as the reference's and the determinants' own
+    (ra, ba), (rb, bb) = _ratios(s, w)
+    rel = 4 * (ba / np.abs(ra) + bb / np.abs(rb)) + 1e-14
+    f = np.abs(s.coeff * ref["det_ovlp"]) / np.abs(ref["ovlp"])[:, None]
+    g = np.abs(ref["det_g"]).max(axis=(2, 3, 4))
+    tol_g = np.sum(f * rel * (g + g[:, :1]), 1)
+    lam = np.abs(s.L).sum(axis=(1, 2)).max()
+    big = np.abs(ref["det_e"]) + np.abs(ref["det_e"][:, :1]) + lam ** 2 * (g + g[:, :1]) ** 2
+    tol_e = np.sum(f * rel * big, 1)
+    dev = [torch.from_numpy(x).cuda() for x in w]
+    ctx = msd.Context(s, "fp64")
+    rdm = ctx.rdm1(*dev).cpu().numpy()
+    assert np.all(np.abs(rdm - ref["G_T"]).max((1, 2, 3)) <= tol_g)
+    _, v, e = (t.cpu().numpy() for t in ctx.evaluate(*dev))
+    for x in (v, ctx.force_bias(*dev).cpu().numpy()):
+        assert np.all(np.abs(x - ref["vbias"]).max(1) <= tol_g * lam)
+    assert np.all(np.abs(e - ref["e_loc"]) <= tol_e)
+    ctx.close()
