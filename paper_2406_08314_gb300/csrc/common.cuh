@@ -155,9 +155,10 @@ __device__ __forceinline__ int mag_key(double2 v)
     return max(__double2hiint(v.x) & 0x7fffffff, __double2hiint(v.y) & 0x7fffffff);
 }
 
-// x 2^-e (|x| < 2^e) as an integer of BITS fractional bits, the magnitude rounded
-// to nearest (integer operations only: FP64 ones issue at a sixty-fourth of
-// their rate).
+// x 2^-e (|x| < 2^e) as an integer of BITS fractional bits, rounded to nearest, ties to
+// even (integer operations only: FP64 ones issue at a sixty-fourth of their rate). Ties are
+// common: a value some bits below the scale drops that many bits, so halves upwards
+// would bias every magnitude by up to 2^-53 of it.
 template <int BITS>
 __device__ __forceinline__ long long fixed_point(double x, int e)
 {
@@ -167,7 +168,7 @@ __device__ __forceinline__ long long fixed_point(double x, int e)
     if (f) m |= 1ll << 52;
     const int sh = (f ? f : 1) - 1075 + BITS - e;   // <= BITS - 53
     if (sh >= 0) m <<= min(sh, BITS - 53);
-    else m = sh > -56 ? (m + (1ll << (-sh - 1))) >> -sh : 0;
+    else m = sh > -56 ? (m + (1ll << (-sh - 1)) - 1 + ((m >> -sh) & 1)) >> -sh : 0;
     return b < 0 ? -m : m;
 }
 __device__ __forceinline__ long long fixed56(double x, int e) { return fixed_point<56>(x, e); }
@@ -180,7 +181,7 @@ static __device__ __noinline__ double int_to_fp64_slow(long long hi, long long l
     return ldexp(fma((double)hi, 268435456.0, (double)lo), s);
 }
 
-// v 2^s rounded to FP64 by integer operations (a conversion from 64 bits and a
+// v 2^s rounded to FP64 (to nearest, ties to even) by integer operations (a conversion from 64 bits and a
 // scaling are two operations of the FP64 unit, 2 per clock and SM).
 __device__ __forceinline__ double int_to_fp64(long long v, int s)
 {
@@ -190,7 +191,8 @@ __device__ __forceinline__ double int_to_fp64(long long v, int s)
     u <<= lz;
     // the mantissa's leading bit adds one to the exponent field, a carry out of
     // the rounding another one
-    const unsigned long long m = (u >> 11) + ((u >> 10) & 1);
+    unsigned long long m = u >> 11;
+    m += (((unsigned)u & 2047u) + 1023u + ((unsigned)m & 1u)) >> 11;
     return __longlong_as_double((long long)((((unsigned long long)(ex - 1)) << 52) + m) | (v & (long long)(1ull << 63)));
 }
 
