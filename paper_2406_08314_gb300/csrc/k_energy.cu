@@ -363,7 +363,8 @@ void launch_onebody(const SpinTables& ta, const SpinTables& tb, int nw, int M, c
 //   Y[x] = Lh[x] + sum_g V0_g Lact_g[x] - sum_g Xic_g[x],  V0_g = v0a_g + v0b_g
 //   scal[w][0 + s] = sum_g xx_g (exchange of G),  scal[w][2] = sum_g V0_g^2
 // One block per (walker, spin): warp k takes the vectors g = k mod 8, lanes over
-// the entries x (contiguous rows); the warps' sums are added in order. (A serial
+// the entries x (contiguous rows); the warps' sums are added in pairs (added in a row,
+// most round at the size of the total: energies 1.75e-16 rms off). (A serial
 // sum over g per entry left 64 walkers with 64 x 75 chains of 1600 dependent FP64
 // operations: 1.05 ms for both iron-sulfur spins.)
 struct GammaArgs {
@@ -395,8 +396,10 @@ k_gamma_reduce(const __grid_constant__ GammaArgs a, int n_chol, double2* __restr
 #pragma unroll
     for (int q = 0; q < (MSD_XMAX + 31) / 32; ++q)
         if (q * 32 + lane < X) part[warp][q * 32 + lane] = acc[q];
+    // consecutive vectors go to different warps: they come in descending order as a
+    // rule, and partial sums of one size round at the size of the total once only
     double2 s0 = cz(0, 0), s1 = cz(0, 0);
-    for (int g = t; g < n_chol; g += blockDim.x) {
+    for (int g = lane * 8 + warp; g < n_chol; g += 256) {
         s0 = cadd(s0, a.xx[spin][base + g]);
         const double2 V0 = cadd(va[g], vb[g]);
         s1 = cfma(V0, V0, s1);
@@ -408,13 +411,12 @@ k_gamma_reduce(const __grid_constant__ GammaArgs a, int n_chol, double2* __restr
     if (lane == 0) { red[0][warp] = s0; red[1][warp] = s1; }
     __syncthreads();
     for (int x = t; x < X; x += blockDim.x) {
-        double2 y = a.Lh[spin][(size_t)w * X + x];
-        for (int q = 0; q < 8; ++q) y = cadd(y, part[q][x]);
-        a.Y[spin][(size_t)w * X + x] = y;
+        auto y = [&](int q) { return cadd(part[q][x], part[q + 1][x]); };
+        a.Y[spin][(size_t)w * X + x] = cadd(a.Lh[spin][(size_t)w * X + x], cadd(cadd(y(0), y(2)), cadd(y(4), y(6))));
     }
     if (t < 2) {
-        double2 s = red[t][0];
-        for (int q = 1; q < 8; ++q) s = cadd(s, red[t][q]);
+        auto r = [&](int q) { return cadd(red[t][q], red[t][q + 1]); };
+        const double2 s = cadd(cadd(r(0), r(2)), cadd(r(4), r(6)));
         if (t == 0) scal[(size_t)w * 8 + spin] = s;
         else if (spin == 0) scal[(size_t)w * 8 + 2] = s;
     }

@@ -1,4 +1,5 @@
-"""FP64 energies of D_0 with Cholesky vectors on which a way of rounding shows: E = 1/2 sum_g (2 sum_j L_jj)^2 - sum_g sum_jl L_jl^2 over the occupied
+"""FP64 energies of D_0 with Cholesky vectors on which an order of summation or a way of
+rounding shows: E = 1/2 sum_g (2 sum_j L_jj)^2 - sum_g sum_jl L_jl^2 over the occupied
 block, in exact rational arithmetic."""
 from fractions import Fraction
 
@@ -26,6 +27,16 @@ def _energy(L, n):
         want += 2 * sum(q[j][j] for j in range(n)) ** 2 - sum(x * x for r in q for x in r)
     assert e.imag == 0.0
     return e.real, want
+
+
+def test_sum_over_vectors():
+    # one vector of 1 and seven of 2^-27, 32 vectors apart: sum of squares 1 + 7 2^-54
+    L = np.zeros((256, 4, 4))
+    L[::32, 0, 0] = 2.0 ** -27
+    L[0, 0, 0] = 1.0
+    e, want = _energy(L, 1)
+    # eight partial sums added in pairs: three roundings of half an ulp
+    assert abs(Fraction(e) - want) <= Fraction(3, 2) * Fraction(1, 2 ** 52), float(Fraction(e) - want)
 
 
 def test_ties_round_to_even():
