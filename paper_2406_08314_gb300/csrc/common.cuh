@@ -166,8 +166,8 @@ __device__ __forceinline__ long long fixed_point(double x, int e)
     const int f = (int)((b >> 52) & 0x7ff);
     long long m = b & 0xfffffffffffffll;
     if (f) m |= 1ll << 52;
-    const int sh = (f ? f : 1) - 1075 + BITS - e;   // <= BITS - 53
-    if (sh >= 0) m <<= min(sh, BITS - 53);
+    const int sh = (f ? f : 1) - 1075 + BITS - e;   // below 63 (e >= -1073), m 2^sh below 2^BITS
+    if (sh >= 0) m <<= sh;
     else m = sh > -56 ? (m + (1ll << (-sh - 1)) - 1 + ((m >> -sh) & 1)) >> -sh : 0;
     return b < 0 ? -m : m;
 }

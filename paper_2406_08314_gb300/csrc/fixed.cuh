@@ -70,9 +70,9 @@ __device__ __forceinline__ unsigned mag_bits(double2 v)
     return max((unsigned)__double2hiint(v.x) & 0x7fffffffu, (unsigned)__double2hiint(v.y) & 0x7fffffffu);
 }
 
-// Exponent e of a largest magnitude in mag_bits form: every |x| < 2^e (1025 marks an
-// infinity or a NaN).
-__device__ __forceinline__ int mag_exponent(unsigned m) { return (int)(m >> 20) - 1022; }
+// Exponent e of a largest magnitude in mag_bits form: every |x| < 2^e (-1021 for
+// subnormal ones; 1025 marks an infinity or a NaN).
+__device__ __forceinline__ int mag_exponent(unsigned m) { return max((int)(m >> 20), 1) - 1022; }
 #define FIXED_EXP_INF 1025
 
 // The sum of `s` with operand exponents adding up to e, as FP64.

@@ -166,7 +166,7 @@ k_fepi_int(SpinTables tb, int M, int n_chol, const double2* __restrict__ F, long
     auto exponent = [&](int i) {      // of the largest magnitude the warps left in wmax[i]
         unsigned m = 0;
         for (int k = 0; k < nwarp; ++k) m = max(m, wmax[i][k]);
-        return (int)(m >> 20) - 1022;   // every |x| < 2^e (1025: an infinity or a NaN)
+        return mag_exponent(m);
     };
     const double2* gr = Gr + (size_t)w * N * M;
     unsigned m = 0;

@@ -341,11 +341,11 @@ k_tc_dgemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUten
 
 // ---------------------------------------------------------------- slicing
 // Exponent e of a row with largest magnitude bits `top` (the sign-free high
-// word of an FP64 value): every |x| < 2^e.
+// word of an FP64 value): every |x| < 2^e, -1021 for subnormal rows.
 __device__ __forceinline__ int dg_exponent(unsigned top)
 {
     const int f = (int)(top >> 20);
-    return f == 0x7ff ? DG_NAN : f - 1022;
+    return f == 0x7ff ? DG_NAN : max(f, 1) - 1022;
 }
 
 // The eight digits of eight fixed-point values as BF16: u[i] packs digit i (most
