@@ -208,6 +208,7 @@ int launch_refs(const RefSpinIn* in, int n_spin, int nw, int M, unsigned* err, c
         o.Mr = M; o.Nc = N; o.batch = nw;
         o.C = in[s].Gr; o.c_batch = (long long)N * M; o.c_n = M; o.c_m = 1;
         o.eye = in[s].T->pos0;
+        o.live = in[s].O0;   // 0 for a singular walker: zero rows, as k_ref writes them
         if (dg_gemm({in[s].sa, in[s].ea, nw * M, M}, {in[s].sb, in[s].eb, 2 * N * nw, 2 * N}, o, 2 * N, err, st)) return -1;
     }
     if (X > 0 && (in[0].Gact || in[0].GactT)) {

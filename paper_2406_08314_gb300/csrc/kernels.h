@@ -194,7 +194,8 @@ struct DgOperand {
 // part at z c_batch, for dg_sum_splits. gx >= 0: the rows of A and B stack gx
 // alpha and gy beta entries, and the (alpha, alpha), (beta, beta) and (alpha,
 // beta) blocks go to K[0], K[2], K[1] ([batch][rows][columns] each) instead of C.
-// eye [Mr]: rows m with eye[m] >= 0 are written as unit vectors (1 at n = eye[m]).
+// eye [Mr]: rows m with eye[m] >= 0 are written as unit vectors (1 at n = eye[m]); live
+// [batch]: entries z with live[z] = 0 are written as zeros.
 struct DgOut {
     int Mr = 0, Nc = 0, batch = 1, splits = 1;
     double2* C = nullptr;
@@ -205,6 +206,7 @@ struct DgOut {
     int gx = -1, gy = 0;
     double2* K[3] = {nullptr, nullptr, nullptr};
     const int* eye = nullptr;
+    const double2* live = nullptr;
 };
 int dg_k_padded(int K);
 size_t dg_row_bytes(int K);              // slices and exponent of one real row

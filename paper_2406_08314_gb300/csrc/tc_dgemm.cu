@@ -84,6 +84,7 @@ struct DgArgs {
     int gx, gy;
     double2* K[3];
     const int* eye;          // [Mr] or NULL: rows with eye[m] >= 0 are unit vectors
+    const double2* live;     // [batch] with eye: entries z with live[z] = 0 are zero
     unsigned* err;
 };
 
@@ -302,6 +303,7 @@ k_tc_dgemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUten
                 const int ea = a.ea[bz * a.a_batch + m];
                 const int* ebp = a.eb + (size_t)bz * a.b_batch;
                 const int unit_n = a.eye ? a.eye[m] : -1;
+                const bool dead = a.eye && a.live[tl.z].x == 0.0 && a.live[tl.z].y == 0.0;
                 const long long o0 = (long long)tl.z * a.c_batch + (long long)m * a.c_m;
 #pragma unroll
                 for (int i = 0; i < DG_HALF; i += 2) {
@@ -311,6 +313,7 @@ k_tc_dgemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUten
                                                  dg_value(hi[i + 1], lo[i + 1], ea + ebp[n2 + 1]));
                         if (a.mul != 1.0) v = make_double2(v.x * a.mul, v.y * a.mul);
                         if (unit_n >= 0) v = make_double2(n == unit_n ? 1.0 : 0.0, 0.0);
+                        if (dead) v = make_double2(0.0, 0.0);
                         if (a.gx >= 0) {
                             const int X = a.gx, Y = a.gy;
                             if (n >= X) {
@@ -626,7 +629,7 @@ int dg_gemm(const DgOperand& A, const DgOperand& B, const DgOut& o, int K, unsig
     a.ea = A.e; a.eb = B.e;
     a.C = o.C; a.c_batch = o.c_batch; a.c_n = o.c_n; a.c_m = o.c_m;
     a.acc = o.acc; a.acc_in = o.acc_in; a.mul = o.mul; a.err = err;
-    a.gx = o.gx; a.gy = o.gy; a.eye = o.eye;
+    a.gx = o.gx; a.gy = o.gy; a.eye = o.eye; a.live = o.live;
     for (int i = 0; i < 3; ++i) a.K[i] = o.K[i];
     const long long tiles = (long long)a.mt * a.nt * a.batch * a.splits;
     if (tiles <= 0) return 0;
