@@ -313,10 +313,26 @@ void free_dg(DgConst& c)
 // of the persistent kernel outweigh the products. The rule does not look at the
 // number of walkers, so a walker's result does not depend on the chunk it is in.
 bool dg_use(long long rows, long long K) { return K >= 24 && rows * K >= 65536 && rows < (1ll << 27); }
-size_t dg_bytes(long long rows, int K, int complex_rows)
-{
-    return dg_use(rows, K) ? 2 * dg_row_bytes(K) * (size_t)complex_rows : 0;
-}
+// Scratch per walker of a call's products: each of these buffers is shared by them and
+// as large as its largest use (gemm_zd, dg_gram, apply_tc).
+struct DgScratch {
+    size_t s = 0, sa = 0, part = 0;   // dg_s and dg_e; dg_sa and dg_ea; dg_part
+    // complex_rows rows against [rows][K]
+    void gemm(long long rows, int K, int complex_rows)
+    {
+        if (!dg_use(rows, K)) return;
+        const int splits = dg_splits((int)rows, K);
+        s = std::max(s, 2 * dg_row_bytes(K) * complex_rows);
+        if (splits > 1) part = std::max(part, sizeof(double2) * splits * (size_t)rows * complex_rows);
+    }
+    // left and right operand rows of length K
+    void pair(int K, size_t left, size_t right)
+    {
+        s = std::max(s, dg_row_bytes(K) * right);
+        sa = std::max(sa, dg_row_bytes(K) * left);
+    }
+    size_t bytes() const { return s + sa + part; }
+};
 
 // Slices of a constant real [rows][K] operand on first use; false where their
 // memory cannot be had (the FP64 kernels run then).
@@ -367,10 +383,6 @@ int gemm_zd(msd_ctx* ctx, int Mr, int Nc, int K, const double2* A, long long lda
 // The FP64 Gram matrices of a walker, (Xa + Xb)^2 products of length n_chol, run
 // on the tensor cores from this size on (as dg_use: by shape only).
 bool dg_gram_use(int Xa, int Xb, int G) { return (long long)(Xa + Xb) * (Xa + Xb) * G >= 262144; }
-size_t dg_gram_bytes(int Xa, int Xb, int G)
-{
-    return dg_gram_use(Xa, Xb, G) ? 3 * (size_t)(Xa + Xb) * dg_row_bytes(2 * G) : 0;
-}
 
 // K_aa, K_bb, K_ab of nw walkers from the Lambda rows [w][g][x] of both spins.
 int dg_gram(msd_ctx* ctx, int nw, int Xa, int Xb, const double2* La, const double2* Lb, double2* Kaa, double2* Kbb,
@@ -1483,8 +1495,11 @@ size_t fb_bytes_per_walker(msd_ctx* ctx, bool fp32)
         b += sizeof(double2) * (size_t)t.nh * t.np;
     }
     if (fp32) b += sizeof(float) * 2 * 2 * ctx->Kdp + sizeof(float) * 16 * 2 * ctx->n_chol;
-    else if (dg_use(ctx->n_chol, ctx->Kd))
-        b += dg_bytes(ctx->n_chol, (int)ctx->Kd, 1) + sizeof(double2) * dg_splits(ctx->n_chol, (int)ctx->Kd) * ctx->n_chol;
+    if (!fp32) {
+        DgScratch d;
+        d.gemm(ctx->n_chol, (int)ctx->Kd, 1);
+        b += d.bytes();
+    }
     return b;
 }
 
@@ -1627,13 +1642,14 @@ size_t en_bytes_per_walker(msd_ctx* ctx, bool fp32)
         }
         b += f + a;
     } else {
-        size_t d = 0;
+        DgScratch d;
         for (int s = 0; s < 2; ++s) {
             const int NC = T1[s].N + T1[s].np;
             b += sizeof(double2) * T1[s].N * (size_t)G * NC;
-            d = std::max(d, dg_bytes((long long)G * NC, ctx->M, T1[s].N));
+            d.gemm((long long)G * NC, ctx->M, T1[s].N);
         }
-        b += std::max(d, dg_gram_bytes(X[0], X[1], G));
+        if (dg_gram_use(X[0], X[1], G)) d.pair(2 * G, X[0] + X[1], 2 * (size_t)(X[0] + X[1]));
+        b += d.bytes();
     }
     return b;
 }
@@ -2285,8 +2301,10 @@ int propagate(msd_ctx* ctx, int n_w, double* phi_a, double* phi_b, double* weigh
     bool tc = dg_apply_use(M);
     for (int s = 0; s < 2 && tc; ++s) tc = dg_ready(ctx->dg_E[s], M, M, ctx->d_E[s], M, st);
     const int Nt = ctx->n[0] + ctx->n[1], Nw = tc ? Nt : Nm;   // columns of the work arrays
-    const size_t per = sizeof(double2) * ((size_t)M * M + 3 * (size_t)M * Nw) +
-                       std::max(dg_bytes((long long)M * M, G, 1), tc ? dg_row_bytes(2 * M) * (M + 2 * (size_t)Nt) : 0);
+    DgScratch d;
+    d.gemm((long long)M * M, G, 1);
+    if (tc) d.pair(2 * M, M, 2 * (size_t)Nt);
+    const size_t per = sizeof(double2) * ((size_t)M * M + 3 * (size_t)M * Nw) + d.bytes();
     const int cap = (int)std::max<size_t>(1, std::min<size_t>((size_t)n_w, ctx->ws_limit / 2 / per));
     void *V, *t0, *t1, *ac;
     if ((rc = arena_get(ctx, "pr_V", sizeof(double2) * (size_t)cap * M * M, &V))) return rc;
