@@ -354,29 +354,34 @@ bool dg_ready(DgConst& c, long long rows, int K, const double* src, long long ld
 }
 
 // C[m][n] = sum_k A[m][k] B[n][k] in FP64: A Mr complex rows (walkers), B the
-// constant real operand [Nc][K] whose slices `cB` keeps.
+// constant real operand [Nc][K] whose slices `cB` keeps. step: rows that the scratch is for.
 int gemm_zd(msd_ctx* ctx, int Mr, int Nc, int K, const double2* A, long long lda, const double* B, long long ldb,
-            DgConst& cB, double2* C, long long ldc, cudaStream_t st)
+            DgConst& cB, double2* C, long long ldc, int step, cudaStream_t st)
 {
     if (!dg_use(Nc, K) || !dg_ready(cB, Nc, K, B, ldb, st)) {
         launch_gemm_zd(Mr, Nc, K, A, lda, B, ldb, C, ldc, st);
         return MSD_OK;
     }
-    int rc;
-    void *s, *e, *part = C;
     const int splits = dg_splits(Nc, K);
-    if ((rc = arena_get(ctx, "dg_s", dg_row_bytes(K) * 2 * (size_t)Mr, &s))) return rc;
-    if ((rc = arena_get(ctx, "dg_e", sizeof(int) * 2 * (size_t)Mr, &e))) return rc;
-    if (splits > 1 && (rc = arena_get(ctx, "dg_part", sizeof(double2) * splits * (size_t)Mr * Nc, &part))) return rc;
-    dg_slice_complex(Mr, K, A, lda, s, (int*)e, st);
-    DgOut o;
-    o.Mr = Nc; o.Nc = Mr; o.splits = splits;
-    o.C = (double2*)part;
-    o.c_n = splits > 1 ? Nc : ldc;
-    o.c_batch = (long long)Mr * Nc;
-    if (dg_gemm({cB.s, cB.e, Nc, 0}, {s, (int*)e, 2 * Mr, 0}, o, K, ctx->d_err, st))
-        return fail(ctx, MSD_ERR_CUDA, "FP64 tensor-core contraction launch failed");
-    if (splits > 1) dg_sum_splits(Mr, Nc, splits, (const double2*)part, C, ldc, st);
+    step = std::min(step, Mr);
+    int rc;
+    void *s, *e, *part = nullptr;
+    if ((rc = arena_get(ctx, "dg_s", dg_row_bytes(K) * 2 * (size_t)step, &s))) return rc;
+    if ((rc = arena_get(ctx, "dg_e", sizeof(int) * 2 * (size_t)step, &e))) return rc;
+    if (splits > 1 && (rc = arena_get(ctx, "dg_part", sizeof(double2) * splits * (size_t)step * Nc, &part))) return rc;
+    for (int m0 = 0; m0 < Mr; m0 += step) {
+        const int m = std::min(step, Mr - m0);
+        double2* out = C + m0 * ldc;
+        dg_slice_complex(m, K, A + m0 * lda, lda, s, (int*)e, st);
+        DgOut o;
+        o.Mr = Nc; o.Nc = m; o.splits = splits;
+        o.C = splits > 1 ? (double2*)part : out;
+        o.c_n = splits > 1 ? Nc : ldc;
+        o.c_batch = (long long)m * Nc;
+        if (dg_gemm({cB.s, cB.e, Nc, 0}, {s, (int*)e, 2 * m, 0}, o, K, ctx->d_err, st))
+            return fail(ctx, MSD_ERR_CUDA, "FP64 tensor-core contraction launch failed");
+        if (splits > 1) dg_sum_splits(m, Nc, splits, (const double2*)part, out, ldc, st);
+    }
     return MSD_OK;
 }
 
@@ -384,26 +389,31 @@ int gemm_zd(msd_ctx* ctx, int Mr, int Nc, int K, const double2* A, long long lda
 // on the tensor cores from this size on (as dg_use: by shape only).
 bool dg_gram_use(int Xa, int Xb, int G) { return (long long)(Xa + Xb) * (Xa + Xb) * G >= 262144; }
 
-// K_aa, K_bb, K_ab of nw walkers from the Lambda rows [w][g][x] of both spins.
+// K_aa, K_bb, K_ab of nw walkers from the Lambda rows [w][g][x] of both spins, step
+// walkers at a time.
 int dg_gram(msd_ctx* ctx, int nw, int Xa, int Xb, const double2* La, const double2* Lb, double2* Kaa, double2* Kbb,
-            double2* Kab, cudaStream_t st)
+            double2* Kab, int step, cudaStream_t st)
 {
     const int G = ctx->n_chol, X = Xa + Xb;
-    const long long rows = (long long)nw * X;
+    step = std::min(step, nw);
     int rc;
     void *sa, *ea, *sb, *eb;
-    if ((rc = arena_get(ctx, "dg_s", dg_row_bytes(2 * G) * 2 * rows, &sb))) return rc;
-    if ((rc = arena_get(ctx, "dg_e", sizeof(int) * 2 * rows, &eb))) return rc;
-    if ((rc = arena_get(ctx, "dg_sa", dg_row_bytes(2 * G) * rows, &sa))) return rc;
-    if ((rc = arena_get(ctx, "dg_ea", sizeof(int) * rows, &ea))) return rc;
-    dg_slice_columns(0, G, Xa, nw, La, Xa, (long long)G * Xa, 0, X, sa, (int*)ea, sb, (int*)eb, st);
-    dg_slice_columns(0, G, Xb, nw, Lb, Xb, (long long)G * Xb, Xa, X, sa, (int*)ea, sb, (int*)eb, st);
-    DgOut o;
-    o.Mr = o.Nc = X; o.batch = nw;
-    o.gx = Xa; o.gy = Xb;
-    o.K[0] = Kaa; o.K[1] = Kab; o.K[2] = Kbb;
-    if (dg_gemm({sa, (int*)ea, (int)rows, X}, {sb, (int*)eb, (int)(2 * rows), 2 * X}, o, 2 * G, ctx->d_err, st))
-        return fail(ctx, MSD_ERR_CUDA, "FP64 tensor-core Gram launch failed");
+    if ((rc = arena_get(ctx, "dg_s", dg_row_bytes(2 * G) * 2 * (size_t)step * X, &sb))) return rc;
+    if ((rc = arena_get(ctx, "dg_e", sizeof(int) * 2 * (size_t)step * X, &eb))) return rc;
+    if ((rc = arena_get(ctx, "dg_sa", dg_row_bytes(2 * G) * (size_t)step * X, &sa))) return rc;
+    if ((rc = arena_get(ctx, "dg_ea", sizeof(int) * (size_t)step * X, &ea))) return rc;
+    for (int w0 = 0; w0 < nw; w0 += step) {
+        const int n = std::min(step, nw - w0);
+        const size_t w = w0;
+        dg_slice_columns(0, G, Xa, n, La + w * G * Xa, Xa, (long long)G * Xa, 0, X, sa, (int*)ea, sb, (int*)eb, st);
+        dg_slice_columns(0, G, Xb, n, Lb + w * G * Xb, Xb, (long long)G * Xb, Xa, X, sa, (int*)ea, sb, (int*)eb, st);
+        DgOut o;
+        o.Mr = o.Nc = X; o.batch = n;
+        o.gx = Xa; o.gy = Xb;
+        o.K[0] = Kaa + w * Xa * Xa; o.K[1] = Kab + w * Xa * Xb; o.K[2] = Kbb + w * Xb * Xb;
+        if (dg_gemm({sa, (int*)ea, n * X, X}, {sb, (int*)eb, 2 * n * X, 2 * X}, o, 2 * G, ctx->d_err, st))
+            return fail(ctx, MSD_ERR_CUDA, "FP64 tensor-core Gram launch failed");
+    }
     return MSD_OK;
 }
 
@@ -414,7 +424,8 @@ bool is_device_ptr(const void* p)
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
-SpinTables tables(const SpinHost& s, int cap)
+// cap: walkers of the chunk; w0: the walker that walker 0 of the call is in it.
+SpinTables tables(const SpinHost& s, int cap, int w0 = 0)
 {
     SpinTables t;
     t.N = s.N; t.nh = s.nh; t.np = s.np; t.n_str = s.n_str;
@@ -428,7 +439,7 @@ SpinTables tables(const SpinHost& s, int cap)
     t.csr_cf = s.d_csr_cf;
     long long off = 0, xo = 0;
     for (int k = 0; k <= MSD_KMAX; ++k) {
-        t.b_off[k] = off;
+        t.b_off[k] = off + (long long)w0 * b_stride(k) * (s.bucket[k + 1] - s.bucket[k]);
         t.cmx_off[k] = xo;
         off += (long long)cap * b_stride(k) * (s.bucket[k + 1] - s.bucket[k]);
         xo += (long long)k * k * (s.bucket[k + 1] - s.bucket[k]);
@@ -1166,9 +1177,18 @@ int check_ready(msd_ctx* ctx)
     return MSD_OK;
 }
 
+// Workspace per walker: what a chunk of walkers keeps, and scratch that its stages use
+// up as they go (a chunk can take them in several pieces of walkers).
+struct Bytes {
+    size_t keep = 0, scratch = 0;
+    size_t all() const { return keep + scratch; }
+    Bytes& operator+=(const Bytes& o) { keep += o.keep; scratch += o.scratch; return *this; }
+};
+
 // Walkers per chunk for a given per-walker footprint.
-int chunk_for(msd_ctx* ctx, size_t per_walker, int n_w)
+int chunk_for(msd_ctx* ctx, const Bytes& per, int n_w)
 {
+    const size_t per_walker = per.all();
     size_t c = per_walker ? ctx->ws_limit / per_walker : (size_t)n_w;
     if (c < 1) c = 1;
     if (c > (size_t)n_w) c = n_w;
@@ -1266,6 +1286,7 @@ int finish(msd_ctx* ctx, cudaStream_t st, std::initializer_list<Out*> outs, bool
 
 // Per-chunk workspace for the overlap part.
 struct Chunk {
+    int cap, piece, w0 = 0;   // walkers; walkers that the scratch is for; first walker (at)
     double2 *Gr[2], *O0[2], *Gact[2], *GactT[2], *m2[2], *rT[2], *r[2], *wts[2], *part;
     float2* rf[2];   // FP32 copies of r (mixed mode, with B)
     void* B[2];
@@ -1273,6 +1294,24 @@ struct Chunk {
     int *t2[2], *tr[2];      // the minors' largest products (launch_minors)
     int* big[2];             // walkers with large active blocks (launch_strings_large)
     int nslot, nR;
+    // the same from walker p0 on (scratch arrays from their start)
+    Chunk at(const msd_ctx* ctx, int p0) const
+    {
+        Chunk c = *this;
+        c.w0 = w0 + p0;
+        const size_t p = p0;
+        for (int s = 0; s < 2; ++s) {
+            const SpinHost& S = ctx->sp[s];
+            c.Gr[s] += p * S.N * ctx->M;
+            c.O0[s] += p;
+            c.Gact[s] += p * S.nh * S.np;
+            if (r[s]) c.r[s] += p * S.n_str;
+            if (wts[s]) c.wts[s] += p * S.n_str;
+            if (rf[s]) c.rf[s] += p * S.n_str;
+        }
+        c.part += p * nslot;
+        return c;
+    }
 };
 
 // What a call needs of the strings beyond their ratios.
@@ -1307,39 +1346,42 @@ size_t mark_rows(const msd_ctx* ctx, int s, StringUse use)
 
 // want_r: the ratios as r[w][s] are for the caller (the FP64 per-determinant terms read
 // them in any case). cof: the cofactor matrix is needed.
-size_t overlap_bytes_per_walker(msd_ctx* ctx, StringUse use, int nslot, bool want_r = false, bool cof = false)
+Bytes overlap_bytes_per_walker(msd_ctx* ctx, StringUse use, int nslot, bool want_r = false, bool cof = false)
 {
     const bool want_b = use == StringUse::Minors, ext = use_ext(ctx, use);
     const bool fp64_b = want_b && ctx->prec == MSD_FP64;
-    size_t b = 0;
-    for (int s = 0; s < 2; ++s) {
-        const SpinHost& S = ctx->sp[s];
-        b += (size_t)S.N * ctx->M + 1 + 2 * (size_t)S.nh * S.np + (size_t)S.n_str;
-        b += ref_dg_bytes(ctx->M, S.N) / sizeof(double2) + 1;
-        if (ext) b += ctx->ext[s].n2 + ctx->ext[s].n_ext - S.n_str;
-        else if (!fp64_b) b += minor2_count(tables(S, 1));
-        if (ext || !fp64_b) b += (minor2_count(tables(S, 1)) + mark_rows(ctx, s, use)) / 4 + 2;
-        if (ext && cof) b += S.n_str + ctx->ext[s].n_piece;
-        if (fp64_b || want_r) b += S.n_str;
-        if (want_b || cof) b += S.n_str + S.b_per_walker;
-        if (want_b && !fp64_b) b += (S.n_str + 1) / 2;
-        if (ext) b += 1;
+    size_t k = nslot, s = 0;   // complex numbers
+    for (int i = 0; i < 2; ++i) {
+        const SpinHost& S = ctx->sp[i];
+        k += (size_t)S.N * ctx->M + 1 + (size_t)S.nh * S.np;
+        if (fp64_b || want_r) k += S.n_str;
+        if (want_b || cof) k += S.n_str + S.b_per_walker;
+        if (want_b && !fp64_b) k += (S.n_str + 1) / 2;
+        s += (size_t)S.nh * S.np + S.n_str;
+        s += ref_dg_bytes(ctx->M, S.N) / sizeof(double2) + 1;
+        if (ext) s += ctx->ext[i].n2 + ctx->ext[i].n_ext - S.n_str + 1;
+        else if (!fp64_b) s += minor2_count(tables(S, 1));
+        if (ext || !fp64_b) s += (minor2_count(tables(S, 1)) + mark_rows(ctx, i, use)) / 4 + 2;
+        if (ext && cof) s += S.n_str + ctx->ext[i].n_piece;
     }
-    b += nslot;
-    return b * sizeof(double2);
+    return {k * sizeof(double2), s * sizeof(double2)};
 }
 
-int chunk_alloc(msd_ctx* ctx, int cap, StringUse use, int nslot, Chunk& c, bool want_r = false, bool cof = false)
+// piece: walkers that the scratch is for (0: all).
+int chunk_alloc(msd_ctx* ctx, int cap, StringUse use, int nslot, Chunk& c, bool want_r = false, bool cof = false,
+                int piece = 0)
 {
     int rc;
     const bool want_b = use == StringUse::Minors, ext = use_ext(ctx, use);
     const bool fp64_b = want_b && ctx->prec == MSD_FP64;
+    c.cap = cap;
+    c.piece = piece = piece ? piece : cap;
     static const char* names[2][15] = {
         {"Gr_a", "O0_a", "Gact_a", "GactT_a", "m2_a", "rT_a", "r_a", "wts_a", "B_a", "rf_a", "V_a", "Bv_a", "t2_a", "tr_a", "big_a"},
         {"Gr_b", "O0_b", "Gact_b", "GactT_b", "m2_b", "rT_b", "r_b", "wts_b", "B_b", "rf_b", "V_b", "Bv_b", "t2_b", "tr_b", "big_b"}};
     for (int s = 0; s < 2; ++s) {
         const SpinHost& S = ctx->sp[s];
-        const size_t X = std::max(1, S.nh * S.np), w16 = sizeof(double2) * (size_t)cap;
+        const size_t X = std::max(1, S.nh * S.np), w16 = sizeof(double2) * (size_t)cap, p16 = sizeof(double2) * (size_t)piece;
         auto get = [&](int i, size_t bytes, bool wanted, void** out) {
             *out = nullptr;
             return wanted ? arena_get(ctx, names[s][i], bytes, out) : MSD_OK;
@@ -1347,21 +1389,21 @@ int chunk_alloc(msd_ctx* ctx, int cap, StringUse use, int nslot, Chunk& c, bool 
         if ((rc = get(0, w16 * S.N * ctx->M, true, (void**)&c.Gr[s]))) return rc;
         if ((rc = get(1, w16, true, (void**)&c.O0[s]))) return rc;
         if ((rc = get(2, w16 * X, true, (void**)&c.Gact[s]))) return rc;
-        if ((rc = get(3, w16 * X, !ext, (void**)&c.GactT[s]))) return rc;
-        if ((rc = get(4, w16 * minor2_count(tables(S, 1)), !ext && !fp64_b, (void**)&c.m2[s]))) return rc;
-        if ((rc = get(5, w16 * S.n_str, !ext, (void**)&c.rT[s]))) return rc;
+        if ((rc = get(3, p16 * X, !ext, (void**)&c.GactT[s]))) return rc;
+        if ((rc = get(4, p16 * minor2_count(tables(S, 1)), !ext && !fp64_b, (void**)&c.m2[s]))) return rc;
+        if ((rc = get(5, p16 * S.n_str, !ext, (void**)&c.rT[s]))) return rc;
         const ExtTables& g = ctx->ext[s];
-        if ((rc = get(10, w16 * (X + (size_t)g.n2 + g.n_ext), ext, (void**)&c.V[s]))) return rc;
-        if ((rc = get(11, w16 * ((size_t)S.n_str + g.n_piece), ext && cof, (void**)&c.Bv[s]))) return rc;
+        if ((rc = get(10, p16 * (X + (size_t)g.n2 + g.n_ext), ext, (void**)&c.V[s]))) return rc;
+        if ((rc = get(11, p16 * ((size_t)S.n_str + g.n_piece), ext && cof, (void**)&c.Bv[s]))) return rc;
         if (ext) c.GactT[s] = c.V[s];   // the head of V
         const bool marks = ext || !fp64_b;
-        if ((rc = get(12, sizeof(int) * cap * minor2_count(tables(S, 1)), marks, (void**)&c.t2[s]))) return rc;
-        if ((rc = get(13, sizeof(int) * cap * mark_rows(ctx, s, use), marks, (void**)&c.tr[s]))) return rc;
+        if ((rc = get(12, sizeof(int) * piece * minor2_count(tables(S, 1)), marks, (void**)&c.t2[s]))) return rc;
+        if ((rc = get(13, sizeof(int) * piece * mark_rows(ctx, s, use), marks, (void**)&c.tr[s]))) return rc;
         if ((rc = get(6, w16 * S.n_str, fp64_b || want_r, (void**)&c.r[s]))) return rc;
         if ((rc = get(7, w16 * S.n_str, want_b || cof, (void**)&c.wts[s]))) return rc;
         if ((rc = get(8, sizeof(double2) * std::max<long long>(1, cap * S.b_per_walker), want_b || cof, &c.B[s]))) return rc;
         if ((rc = get(9, sizeof(float2) * cap * (size_t)S.n_str, want_b && !fp64_b, (void**)&c.rf[s]))) return rc;
-        if ((rc = get(14, sizeof(int) * cap, ext, (void**)&c.big[s]))) return rc;
+        if ((rc = get(14, sizeof(int) * piece, ext, (void**)&c.big[s]))) return rc;
     }
     void* p;
     if ((rc = arena_get(ctx, "part", sizeof(double2) * cap * std::max(1, nslot), &p))) return rc;
@@ -1373,11 +1415,11 @@ int chunk_alloc(msd_ctx* ctx, int cap, StringUse use, int nslot, Chunk& c, bool 
 
 // Reference inverse of walkers [w0, w0 + nw), both spins: one launch, or alpha
 // first while host beta walkers are still being copied.
-int run_refs(msd_ctx* ctx, const Staged& in, int w0, int nw, int cap, Chunk& c, cudaStream_t st, bool want_act = true)
+int run_refs(msd_ctx* ctx, const Staged& in, int w0, int nw, Chunk& c, cudaStream_t st, bool want_act = true)
 {
     const int M = ctx->M;
     const TimerHook& th = ctx->hook;
-    const SpinTables T[2] = {tables(ctx->sp[0], cap), tables(ctx->sp[1], cap)};
+    const SpinTables T[2] = {tables(ctx->sp[0], c.cap, c.w0), tables(ctx->sp[1], c.cap, c.w0)};
     RefSpinIn r[2];
     static const char* names[2][6] = {{"ref_inv_a", "ref_sa_a", "ref_ea_a", "ref_sb_a", "ref_eb_a", "ref_cs_a"},
                                       {"ref_inv_b", "ref_sa_b", "ref_ea_b", "ref_sb_b", "ref_eb_b", "ref_cs_b"}};
@@ -1390,12 +1432,12 @@ int run_refs(msd_ctx* ctx, const Staged& in, int w0, int nw, int cap, Chunk& c, 
         if (!ref_dg_use(M, N)) continue;
         int rc;
         const size_t rb = dg_row_bytes(2 * N);
-        if ((rc = arena_get(ctx, names[s][0], sizeof(double2) * cap * (size_t)N * N, (void**)&r[s].Sinv))) return rc;
-        if ((rc = arena_get(ctx, names[s][1], rb * cap * (size_t)M, &r[s].sa))) return rc;
-        if ((rc = arena_get(ctx, names[s][2], sizeof(int) * cap * (size_t)M, (void**)&r[s].ea))) return rc;
-        if ((rc = arena_get(ctx, names[s][3], rb * cap * 2 * (size_t)N, &r[s].sb))) return rc;
-        if ((rc = arena_get(ctx, names[s][4], sizeof(int) * cap * 2 * (size_t)N, (void**)&r[s].eb))) return rc;
-        if ((rc = arena_get(ctx, names[s][5], sizeof(double) * cap * (size_t)N, (void**)&r[s].cs))) return rc;
+        if ((rc = arena_get(ctx, names[s][0], sizeof(double2) * c.piece * (size_t)N * N, (void**)&r[s].Sinv))) return rc;
+        if ((rc = arena_get(ctx, names[s][1], rb * c.piece * (size_t)M, &r[s].sa))) return rc;
+        if ((rc = arena_get(ctx, names[s][2], sizeof(int) * c.piece * (size_t)M, (void**)&r[s].ea))) return rc;
+        if ((rc = arena_get(ctx, names[s][3], rb * c.piece * 2 * (size_t)N, &r[s].sb))) return rc;
+        if ((rc = arena_get(ctx, names[s][4], sizeof(int) * c.piece * 2 * (size_t)N, (void**)&r[s].eb))) return rc;
+        if ((rc = arena_get(ctx, names[s][5], sizeof(double) * c.piece * (size_t)N, (void**)&r[s].cs))) return rc;
     }
     th.begin("k_ref", st);
     int g = launch_refs(r, in.b_ready ? 1 : 2, nw, M, ctx->d_err, st);
@@ -1411,11 +1453,11 @@ int run_refs(msd_ctx* ctx, const Staged& in, int w0, int nw, int cap, Chunk& c, 
 
 // String minors, ratios and weights of a chunk whose reference inverse is done.
 // For the overlap alone only the alpha weights' partial sums are formed.
-int run_strings_weights(msd_ctx* ctx, int nw, int cap, Chunk& c, StringUse use, bool fp32_b, cudaStream_t st)
+int run_strings_weights(msd_ctx* ctx, int nw, Chunk& c, StringUse use, bool fp32_b, cudaStream_t st)
 {
     const TimerHook& th = ctx->hook;
     const bool want_b = use == StringUse::Minors;
-    SpinTables T[2] = {tables(ctx->sp[0], cap), tables(ctx->sp[1], cap)};
+    SpinTables T[2] = {tables(ctx->sp[0], c.cap, c.w0), tables(ctx->sp[1], c.cap, c.w0)};
     if (use_ext(ctx, use)) {
         // the ratios are V's last rows
         for (int s = 0; s < 2; ++s) c.rT[s] = c.V[s] + ((size_t)T[s].nh * T[s].np + ctx->ext[s].n2) * nw;
@@ -1446,24 +1488,35 @@ int run_strings_weights(msd_ctx* ctx, int nw, int cap, Chunk& c, StringUse use, 
     return MSD_OK;
 }
 
-// Reference inverse, string minors and weights for walkers [w0, w0 + nw).
-int run_overlap_part(msd_ctx* ctx, const Staged& in, int w0, int nw, int cap, Chunk& c,
-                     StringUse use, bool fp32_b, cudaStream_t st)
-{
-    int rc = run_refs(ctx, in, w0, nw, cap, c, st);
-    return rc ? rc : run_strings_weights(ctx, nw, cap, c, use, fp32_b, st);
-}
-
 // The cofactor matrices of both spins.
-int run_cofactors(msd_ctx* ctx, int nw, int cap, Chunk& c, StringUse use, bool fp32, double2* const Cm[2], cudaStream_t st)
+int run_cofactors(msd_ctx* ctx, int nw, Chunk& c, StringUse use, bool fp32, double2* const Cm[2], cudaStream_t st)
 {
-    const SpinTables T[2] = {tables(ctx->sp[0], cap), tables(ctx->sp[1], cap)};
+    const SpinTables T[2] = {tables(ctx->sp[0], c.cap, c.w0), tables(ctx->sp[1], c.cap, c.w0)};
     ctx->hook.begin("k_cmat", st);
     const bool ext = use_ext(ctx, use);
     if (ext) launch_cofactors(ctx->ext, T[0], T[1], nw, c.V, c.Bv, Cm, st);
     launch_cmat(T[0], T[1], nw, c.wts[0], c.wts[1], c.B[0], c.B[1], fp32, Cm[0], Cm[1], st, ext ? c.big : nullptr);
     ctx->hook.end(st);
     CKLAUNCH();
+    return MSD_OK;
+}
+
+// Reference inverse, string minors and weights, and with Cm the cofactor matrices, for
+// walkers [w0, w0 + nw), in pieces that the scratch is for.
+int run_overlap_part(msd_ctx* ctx, const Staged& in, int w0, int nw, Chunk& c, StringUse use, bool fp32_b, cudaStream_t st,
+                     double2* const* Cm = nullptr)
+{
+    int rc;
+    for (int p = 0; p < nw; p += c.piece) {
+        const int n = std::min(c.piece, nw - p);
+        Chunk q = c.at(ctx, p);
+        if ((rc = run_refs(ctx, in, w0 + p, n, q, st))) return rc;
+        if ((rc = run_strings_weights(ctx, n, q, use, fp32_b, st))) return rc;
+        for (int s = 0; s < 2; ++s) c.rT[s] = q.rT[s];
+        if (!Cm) continue;
+        double2* const cm[2] = {Cm[0] + (size_t)p * ctx->sp[0].nh * ctx->sp[0].np, Cm[1] + (size_t)p * ctx->sp[1].nh * ctx->sp[1].np};
+        if ((rc = run_cofactors(ctx, n, q, use, fp32_b, cm, st))) return rc;
+    }
     return MSD_OK;
 }
 
@@ -1487,7 +1540,7 @@ struct FbWork {
     int ks = 1;
 };
 
-size_t fb_bytes_per_walker(msd_ctx* ctx, bool fp32)
+Bytes fb_bytes_per_walker(msd_ctx* ctx, bool fp32)
 {
     size_t b = sizeof(double2) * (ctx->Kd + 1);
     for (int s = 0; s < 2; ++s) {
@@ -1495,12 +1548,9 @@ size_t fb_bytes_per_walker(msd_ctx* ctx, bool fp32)
         b += sizeof(double2) * (size_t)t.nh * t.np;
     }
     if (fp32) b += sizeof(float) * 2 * 2 * ctx->Kdp + sizeof(float) * 16 * 2 * ctx->n_chol;
-    if (!fp32) {
-        DgScratch d;
-        d.gemm(ctx->n_chol, (int)ctx->Kd, 1);
-        b += d.bytes();
-    }
-    return b;
+    DgScratch d;
+    if (!fp32) d.gemm(ctx->n_chol, (int)ctx->Kd, 1);
+    return {b, d.bytes()};
 }
 
 int fb_alloc(msd_ctx* ctx, int cap, bool fp32, FbWork& f)
@@ -1522,8 +1572,8 @@ int fb_alloc(msd_ctx* ctx, int cap, bool fp32, FbWork& f)
     return MSD_OK;
 }
 
-int fb_chunk(msd_ctx* ctx, Chunk& c, FbWork& f, int w0, int nw, int cap, StringUse use, bool fp32, double2* vb_out,
-             double2* ov_out, cudaStream_t st)
+// (the cofactor matrices are there)
+int fb_chunk(msd_ctx* ctx, Chunk& c, FbWork& f, int w0, int nw, bool fp32, double2* vb_out, double2* ov_out, cudaStream_t st)
 {
     const TimerHook& th = ctx->hook;
     int rc;
@@ -1531,9 +1581,7 @@ int fb_chunk(msd_ctx* ctx, Chunk& c, FbWork& f, int w0, int nw, int cap, StringU
     launch_sum_slots(nw, c.part, c.nslot, 0, c.nR, (double2*)f.Rs, c.O0[0], c.O0[1],
                      ov_out ? ov_out + w0 : nullptr, st);
     th.end(st);
-    double2* const cm[2] = {(double2*)f.Cm[0], (double2*)f.Cm[1]};
-    if ((rc = run_cofactors(ctx, nw, cap, c, use, fp32, cm, st))) return rc;
-    const SpinTables T[2] = {tables(ctx->sp[0], cap), tables(ctx->sp[1], cap)};
+    const SpinTables T[2] = {tables(ctx->sp[0], c.cap), tables(ctx->sp[1], c.cap)};
     const long long off[2] = {0, (long long)(T[0].N + T[0].np) * ctx->M};
     const double2* Cm[2] = {(const double2*)f.Cm[0], (const double2*)f.Cm[1]};
     th.begin("k_gt", st);
@@ -1562,7 +1610,7 @@ int fb_chunk(msd_ctx* ctx, Chunk& c, FbWork& f, int w0, int nw, int cap, StringU
     } else {
         th.begin("k_gemm_vbias", st);
         rc = gemm_zd(ctx, nw, ctx->n_chol, (int)ctx->Kd, (const double2*)f.GT, ctx->Kd, ctx->d_Lcat, ctx->Kd,
-                     ctx->dg_Lcat, out, ctx->n_chol, st);
+                     ctx->dg_Lcat, out, ctx->n_chol, c.piece, st);
         th.end(st);
         if (rc) return rc;
     }
@@ -1613,7 +1661,7 @@ int energy_slots(msd_ctx* ctx)
            (use_pair_y(ctx) ? pair_y_slots(tb) : pair_cross_slots(pair_tables(ctx->pairs), use_runs(ctx)));
 }
 
-size_t en_bytes_per_walker(msd_ctx* ctx, bool fp32)
+Bytes en_bytes_per_walker(msd_ctx* ctx, bool fp32)
 {
     const int G = ctx->n_chol;
     SpinTables T1[2] = {tables(ctx->sp[0], 1), tables(ctx->sp[1], 1)};
@@ -1624,13 +1672,13 @@ size_t en_bytes_per_walker(msd_ctx* ctx, bool fp32)
     for (int s = 0; s < 2; ++s)
         e += (size_t)G * (2 + std::max(2 * X[s], lam_pitch(std::max(1, X[s])))) + 3 * X[s] + 1;
     e += (size_t)X[0] * X[0] + (size_t)X[1] * X[1] + (size_t)X[0] * X[1];
-    size_t b = e * sizeof(double2);
+    size_t b = e * sizeof(double2), scratch = 0;
     if (fp32 && exact_ref_on(ctx)) {
         for (int s = 0; s < 2; ++s)
-            b += (size_t)2 * oz_slices() * oz_k_padded(T1[s].N * (ctx->M - T1[s].N)) * 2 + 2 * sizeof(int);
+            scratch += (size_t)2 * oz_slices() * oz_k_padded(T1[s].N * (ctx->M - T1[s].N)) * 2 + 2 * sizeof(int);
         b += sizeof(float2) * (size_t)G;   // v0w
         for (int s = 0; s < 2; ++s)
-            b += (size_t)2 * oz_parts_for(T1[s].N * (ctx->M - T1[s].N), G) * sizeof(double2) + 2 * sizeof(double) * G;
+            scratch += (size_t)2 * oz_parts_for(T1[s].N * (ctx->M - T1[s].N), G) * sizeof(double2) + 2 * sizeof(double) * G;
     }
     if (fp32 && tensor_gram(ctx)) b += sizeof(float) * 2 * (size_t)(X[0] + X[1]) * G;   // GT
     if (fp32) {
@@ -1649,12 +1697,12 @@ size_t en_bytes_per_walker(msd_ctx* ctx, bool fp32)
             d.gemm((long long)G * NC, ctx->M, T1[s].N);
         }
         if (dg_gram_use(X[0], X[1], G)) d.pair(2 * G, X[0] + X[1], 2 * (size_t)(X[0] + X[1]));
-        b += d.bytes();
+        scratch += d.bytes();
     }
-    return b;
+    return {b, scratch};
 }
 
-int en_alloc(msd_ctx* ctx, int cap, bool fp32, EnWork& E)
+int en_alloc(msd_ctx* ctx, int cap, int piece, bool fp32, EnWork& E)
 {
     const int G = ctx->n_chol;
     SpinTables T1[2] = {tables(ctx->sp[0], 1), tables(ctx->sp[1], 1)};
@@ -1692,7 +1740,7 @@ int en_alloc(msd_ctx* ctx, int cap, bool fp32, EnWork& E)
     if ((rc = arena_get(ctx, "K_ab", sizeof(double2) * cap * std::max(1, X[0] * X[1]), &E.Kab))) return rc;
     if ((rc = arena_get(ctx, "scal", sizeof(double2) * cap * 8, &E.scal))) return rc;
     if (fp32 && exact_ref_on(ctx)) {
-        const int Mpad = oz_rows_padded(2 * cap);
+        const int Mpad = oz_rows_padded(2 * piece);
         static const char* na_[2] = {"oz_A_a", "oz_A_b"};
         static const char* ne_[2] = {"oz_ea_a", "oz_ea_b"};
         static const char* np_[2] = {"oz_part_a", "oz_part_b"};
@@ -1702,7 +1750,7 @@ int en_alloc(msd_ctx* ctx, int cap, bool fp32, EnWork& E)
             if ((rc = arena_get(ctx, na_[s], (size_t)oz_slices() * Mpad * oz_k_padded(NK) * 2, &E.ozA[s]))) return rc;
             if ((rc = arena_get(ctx, ne_[s], sizeof(int) * Mpad, &E.ozE[s]))) return rc;
             if ((rc = arena_get(ctx, np_[s], sizeof(double2) * nparts * Mpad, &E.ozP[s]))) return rc;
-            if ((rc = arena_get(ctx, nt_[s], sizeof(double) * 2 * cap * (size_t)G, &E.ozT[s]))) return rc;
+            if ((rc = arena_get(ctx, nt_[s], sizeof(double) * 2 * piece * (size_t)G, &E.ozT[s]))) return rc;
         }
         if ((rc = arena_get(ctx, "v0w", sizeof(float2) * cap * (size_t)G, &E.v0w))) return rc;
     }
@@ -1763,7 +1811,7 @@ int en_fepi(msd_ctx* ctx, Chunk& c, EnWork& E, int nw, int cap, bool fp32, cudaS
         } else {
             th.begin("k_gemm_F", st);
             const int g = gemm_zd(ctx, nw * N, G * NC[s], M, c.Gr[s], M, ctx->sp[s].d_Lh, M, ctx->dg_Lh[s],
-                                  (double2*)E.F[s], (long long)G * NC[s], st);
+                                  (double2*)E.F[s], (long long)G * NC[s], c.piece * N, st);
             th.end(st);
             if (g) return g;
             th.begin("k_fepi", st);
@@ -1796,27 +1844,32 @@ int en_rest(msd_ctx* ctx, Chunk& c, EnWork& E, int nw, int cap, bool fp32, cudaS
     launch_onebody(T[0], T[1], nw, M, h1, Gr, e1, Lh1, st, hJ);
     th.end(st);
     CKLAUNCH();
-    RefSpin rs[2];
     if (exact) {
         // the reference-determinant sums exactly split on the tensor cores:
         // they replace the FP32 traces in scal[0..2], and their walker parts
         // t1_g of V0_g leave only the small part of sum_g V0_g Lambda_g to
         // the FP32 sum (the reference part C_g is in Lh1, the one-body term
         // of h + J)
-        OzSpin oz[2];
-        for (int s = 0; s < 2; ++s) {
-            const OzConst& K = ctx->oz[s];
-            oz[s] = OzSpin{&K, c.Gr[s], ctx->d_virt[s], E.ozA[s], (int*)E.ozE[s], (double2*)E.ozP[s], (double*)E.ozT[s]};
-            rs[s] = RefSpin{K.N, M, K.Kv, oz_parts(K.NB), oz_rows_padded(2 * nw), c.Gr[s], ctx->d_virt[s],
-                            ctx->d_JJ[s], ctx->d_KK[s], (const double*)E.ozT[s], (const double2*)E.ozP[s],
-                            ctx->oz_x0sum[s]};
+        for (int p = 0; p < nw; p += c.piece) {
+            const int n = std::min(c.piece, nw - p);
+            OzSpin oz[2];
+            RefSpin rs[2];
+            for (int s = 0; s < 2; ++s) {
+                const OzConst& K = ctx->oz[s];
+                const double2* gr = c.Gr[s] + (size_t)p * K.N * M;
+                oz[s] = OzSpin{&K, gr, ctx->d_virt[s], E.ozA[s], (int*)E.ozE[s], (double2*)E.ozP[s], (double*)E.ozT[s]};
+                rs[s] = RefSpin{K.N, M, K.Kv, oz_parts(K.NB), oz_rows_padded(2 * n), gr, ctx->d_virt[s],
+                                ctx->d_JJ[s], ctx->d_KK[s], (const double*)E.ozT[s], (const double2*)E.ozP[s],
+                                ctx->oz_x0sum[s]};
+            }
+            th.begin("tc_ozaki", st);
+            if (oz_both(oz, n, M, ctx->d_err, st)) return fail(ctx, MSD_ERR_CUDA, "exact reference tensor-core launch failed");
+            th.end(st);
+            th.begin("k_ref_reduce", st);
+            launch_ref_reduce(n, G, rs[0], rs[1], ctx->oz_C2sum, (double2*)E.scal + (size_t)p * 8,
+                              (float2*)E.v0w + (size_t)p * G, st);
+            th.end(st);
         }
-        th.begin("tc_ozaki", st);
-        if (oz_both(oz, nw, M, ctx->d_err, st)) return fail(ctx, MSD_ERR_CUDA, "exact reference tensor-core launch failed");
-        th.end(st);
-        th.begin("k_ref_reduce", st);
-        launch_ref_reduce(nw, G, rs[0], rs[1], ctx->oz_C2sum, (double2*)E.scal, (float2*)E.v0w, st);
-        th.end(st);
         CKLAUNCH();
     }
     th.begin("k_gamma_reduce", st);
@@ -1850,7 +1903,7 @@ int en_rest(msd_ctx* ctx, Chunk& c, EnWork& E, int nw, int cap, bool fp32, cudaS
         }
     } else if (dg_gram_use(X[0], X[1], G)) {
         const int g = dg_gram(ctx, nw, X[0], X[1], (double2*)E.La[0], (double2*)E.La[1], (double2*)E.Kaa,
-                              (double2*)E.Kbb, (double2*)E.Kab, st);
+                              (double2*)E.Kbb, (double2*)E.Kab, c.piece, st);
         if (g) return g;
     } else {
         launch_gram(nw, X[0], X[0], G, (double2*)E.La[0], (double2*)E.La[0], E.Kaa, false, st);
@@ -1945,16 +1998,21 @@ int evaluate_impl(msd_ctx* ctx, int n_w, const double* phi_a, const double* phi_
     const int nslot = nR + (want_e ? energy_slots(ctx) : 0);
     StringUse use = StringUse::Overlap;
     if ((want_v || want_e) && (rc = string_use(ctx, want_e, &use))) return rc;
-    size_t per = overlap_bytes_per_walker(ctx, use, nslot, false, want_v);
+    Bytes per = overlap_bytes_per_walker(ctx, use, nslot, false, want_v);
     if (want_v) per += fb_bytes_per_walker(ctx, fp32);
     if (want_e) per += en_bytes_per_walker(ctx, fp32);
-    const int cap = chunk_for(ctx, per, n_w);
+    int cap = chunk_for(ctx, per, n_w), piece = cap;
+    if (defer && cap < n_w && per.keep * n_w <= ctx->ws_limit) {
+        // all walkers in one chunk, the scratch for as many as fit beside them
+        ctx->chunk = cap = n_w;
+        piece = (int)std::max<size_t>(1, std::min<size_t>(n_w, (ctx->ws_limit - per.keep * n_w) / std::max<size_t>(1, per.scratch)));
+    }
     Chunk c;
-    if ((rc = chunk_alloc(ctx, cap, use, nslot, c, false, want_v))) return rc;
+    if ((rc = chunk_alloc(ctx, cap, use, nslot, c, false, want_v, piece))) return rc;
     FbWork f;
     EnWork E;
     if (want_v && (rc = fb_alloc(ctx, cap, fp32, f))) return rc;
-    if (want_e && (rc = en_alloc(ctx, cap, fp32, E))) return rc;
+    if (want_e && (rc = en_alloc(ctx, cap, piece, fp32, E))) return rc;
     if (defer && (cap < n_w || !want_e || in.host_any || o_e.host || o_v.host || o_ov.host))
         return fail(ctx, MSD_ERR_SHAPE, "batched evaluation needs device buffers, the energy output and all "
                                         "walkers in one chunk (%d walkers, %d fit)", n_w, cap);
@@ -1983,10 +2041,11 @@ int evaluate_impl(msd_ctx* ctx, int n_w, const double* phi_a, const double* phi_
         }
         ~Join() { now(); }
     } join;
+    double2* const cm[2] = {(double2*)f.Cm[0], (double2*)f.Cm[1]};
     for (int w0 = 0; w0 < n_w; w0 += cap) {
         const int nw = std::min(cap, n_w - w0);
         if (side) {
-            if ((rc = run_refs(ctx, in, w0, nw, cap, c, st))) return rc;
+            if ((rc = run_refs(ctx, in, w0, nw, c, st))) return rc;
             if ((rc = en_fepi(ctx, c, E, nw, cap, fp32, st))) return rc;
             CK(cudaEventRecord(ctx->ev_fork, st));
             CK(cudaStreamWaitEvent(ctx->side_st, ctx->ev_fork, 0));
@@ -1995,13 +2054,14 @@ int evaluate_impl(msd_ctx* ctx, int n_w, const double* phi_a, const double* phi_
             join.ev = ctx->ev_join;
             if ((rc = en_rest(ctx, c, E, nw, cap, fp32, ctx->side_st))) return rc;
             CK(cudaEventRecord(ctx->ev_rest, ctx->side_st));
-            if ((rc = run_strings_weights(ctx, nw, cap, c, use, fp32, st))) return rc;
+            if ((rc = run_strings_weights(ctx, nw, c, use, fp32, st))) return rc;
             // the force bias (cofactors, G_T, contraction) follows the weights
             // on the second stream, beside the per-determinant terms here
             if (want_v) {
                 CK(cudaEventRecord(ctx->ev_w, st));
                 CK(cudaStreamWaitEvent(ctx->side_st, ctx->ev_w, 0));
-                if ((rc = fb_chunk(ctx, c, f, w0, nw, cap, use, fp32, o_v.dev, nullptr, ctx->side_st))) return rc;
+                if ((rc = run_cofactors(ctx, nw, c, use, fp32, cm, ctx->side_st))) return rc;
+                if ((rc = fb_chunk(ctx, c, f, w0, nw, fp32, o_v.dev, nullptr, ctx->side_st))) return rc;
             }
             CK(cudaStreamWaitEvent(st, ctx->ev_rest, 0));
             if ((rc = en_terms(ctx, c, E, w0, nw, cap, fp32, o_e.dev, o_ov.dev, st))) return rc;
@@ -2009,9 +2069,8 @@ int evaluate_impl(msd_ctx* ctx, int n_w, const double* phi_a, const double* phi_
             CKLAUNCH();
             continue;
         }
-        if ((rc = run_overlap_part(ctx, in, w0, nw, cap, c, use, fp32, st))) return rc;
-        if (want_v && (rc = fb_chunk(ctx, c, f, w0, nw, cap, use, fp32, o_v.dev, want_e ? nullptr : o_ov.dev, st)))
-            return rc;
+        if ((rc = run_overlap_part(ctx, in, w0, nw, c, use, fp32, st, want_v ? cm : nullptr))) return rc;
+        if (want_v && (rc = fb_chunk(ctx, c, f, w0, nw, fp32, o_v.dev, want_e ? nullptr : o_ov.dev, st))) return rc;
         if (want_e && (rc = en_chunk(ctx, c, E, w0, nw, cap, fp32, o_e.dev, o_ov.dev, st, defer != nullptr)))
             return rc;
     }
@@ -2051,7 +2110,9 @@ int rdm1(msd_ctx* ctx, int n_w, const double* phi_a, const double* phi_b, double
     const int nR = weights_blocks(tables(ctx->sp[0], 1));
     StringUse use;
     if ((rc = string_use(ctx, false, &use))) return rc;
-    const int cap = chunk_for(ctx, overlap_bytes_per_walker(ctx, use, nR, false, true) + fb_bytes_per_walker(ctx, false), n_w);
+    Bytes per = overlap_bytes_per_walker(ctx, use, nR, false, true);
+    per += fb_bytes_per_walker(ctx, false);
+    const int cap = chunk_for(ctx, per, n_w);
     Chunk c;
     FbWork f;
     if ((rc = chunk_alloc(ctx, cap, use, nR, c, false, true))) return rc;
@@ -2059,12 +2120,11 @@ int rdm1(msd_ctx* ctx, int n_w, const double* phi_a, const double* phi_b, double
     const TimerHook& th = ctx->hook;
     for (int w0 = 0; w0 < n_w; w0 += cap) {
         const int nw = std::min(cap, n_w - w0);
-        if ((rc = run_overlap_part(ctx, in, w0, nw, cap, c, use, fp32, st))) return rc;
+        double2* const cm[2] = {(double2*)f.Cm[0], (double2*)f.Cm[1]};
+        if ((rc = run_overlap_part(ctx, in, w0, nw, c, use, fp32, st, cm))) return rc;
         th.begin("k_sum_slots", st);
         launch_sum_slots(nw, c.part, c.nslot, 0, c.nR, (double2*)f.Rs, c.O0[0], c.O0[1], nullptr, st);
         th.end(st);
-        double2* const cm[2] = {(double2*)f.Cm[0], (double2*)f.Cm[1]};
-        if ((rc = run_cofactors(ctx, nw, cap, c, use, fp32, cm, st))) return rc;
         const SpinTables T2[2] = {tables(ctx->sp[0], cap), tables(ctx->sp[1], cap)};
         const long long offs[2] = {0, (long long)(T2[0].N + T2[0].np) * M};
         const double2* Cm[2] = {(const double2*)f.Cm[0], (const double2*)f.Cm[1]};
@@ -2120,15 +2180,16 @@ int det_energies(msd_ctx* ctx, int n_w, const double* phi_a, const double* phi_b
     const int nR = weights_blocks(tables(ctx->sp[0], 1));
     StringUse use;
     if ((rc = string_use(ctx, true, &use))) return rc;
-    const size_t per = overlap_bytes_per_walker(ctx, use, nR) + en_bytes_per_walker(ctx, fp32);
+    Bytes per = overlap_bytes_per_walker(ctx, use, nR);
+    per += en_bytes_per_walker(ctx, fp32);
     const int cap = chunk_for(ctx, per, n_w);
     Chunk c;
     EnWork E;
     if ((rc = chunk_alloc(ctx, cap, use, nR, c))) return rc;
-    if ((rc = en_alloc(ctx, cap, fp32, E))) return rc;
+    if ((rc = en_alloc(ctx, cap, cap, fp32, E))) return rc;
     for (int w0 = 0; w0 < n_w; w0 += cap) {
         const int nw = std::min(cap, n_w - w0);
-        if ((rc = run_overlap_part(ctx, in, w0, nw, cap, c, use, fp32, st))) return rc;
+        if ((rc = run_overlap_part(ctx, in, w0, nw, c, use, fp32, st))) return rc;
         if ((rc = en_chunk(ctx, c, E, w0, nw, cap, fp32, nullptr, nullptr, st, true))) return rc;
         launch_det_energy(n_pairs, (const DetRec*)d_rec, w0, nw, tables(ctx->sp[0], cap), tables(ctx->sp[1], cap),
                           c.B[0], c.B[1], E.Kaa, E.Kbb, E.Kab, E.Y[0], E.Y[1], (const double2*)E.scal,
@@ -2315,7 +2376,7 @@ int propagate(msd_ctx* ctx, int n_w, double* phi_a, double* phi_b, double* weigh
         const int nw = std::min(cap, n_w - w0);
         th.begin("k_gemm_V", st);
         rc = gemm_zd(ctx, nw, M * M, G, (const double2*)cf + (size_t)w0 * G, G, ctx->d_Lt, G, ctx->dg_Lt, (double2*)V,
-                     (long long)M * M, st);
+                     (long long)M * M, nw, st);
         th.end(st);
         if (rc) return rc;
         if (tc) {
@@ -2635,7 +2696,7 @@ int msd_overlap(msd_ctx* ctx, int n_w, const double* phi_a, const double* phi_b,
     if ((rc = chunk_alloc(ctx, cap, StringUse::Overlap, nR, c))) return rc;
     for (int w0 = 0; w0 < n_w; w0 += cap) {
         const int nw = std::min(cap, n_w - w0);
-        if ((rc = run_overlap_part(ctx, in, w0, nw, cap, c, StringUse::Overlap, false, st))) return rc;
+        if ((rc = run_overlap_part(ctx, in, w0, nw, c, StringUse::Overlap, false, st))) return rc;
         ctx->hook.begin("k_sum_slots", st);
         launch_sum_slots(nw, c.part, c.nslot, 0, c.nR, o_rs.dev ? o_rs.dev + w0 : nullptr, c.O0[0],
                          c.O0[1], o_ov.dev ? o_ov.dev + w0 : nullptr, st);
@@ -2664,7 +2725,7 @@ int msd_det_ratios(msd_ctx* ctx, int n_w, const double* phi_a, const double* phi
     if ((rc = chunk_alloc(ctx, cap, StringUse::Overlap, nR, c, true))) return rc;
     for (int w0 = 0; w0 < n_w; w0 += cap) {
         const int nw = std::min(cap, n_w - w0);
-        if ((rc = run_overlap_part(ctx, in, w0, nw, cap, c, StringUse::Overlap, false, st))) return rc;
+        if ((rc = run_overlap_part(ctx, in, w0, nw, c, StringUse::Overlap, false, st))) return rc;
         ctx->hook.begin("k_det_ratios", st);
         for (int s = 0; s < 2; ++s) launch_untranspose(ctx->sp[s].n_str, nw, c.rT[s], c.r[s], st);
         launch_det_ratios(pair_tables(ctx->pairs), nw, ctx->sp[0].n_str, ctx->sp[1].n_str, c.r[0],
@@ -2733,7 +2794,7 @@ int msd_features(msd_ctx* ctx, int n_w, const double* phi_a, const double* phi_b
     const int M = ctx->M;
     for (int w0 = 0; w0 < n_w; w0 += cap) {
         const int nw = std::min(cap, n_w - w0);
-        if ((rc = run_refs(ctx, in, w0, nw, cap, c, st, false))) return rc;
+        if ((rc = run_refs(ctx, in, w0, nw, c, st, false))) return rc;
         for (int s = 0; s < 2; ++s) {
             launch_features(nw, M, ctx->n[s], n_core, n_act, ctx->sp[s].d_pos0, c.Gr[s],
                             feat + (size_t)w0 * 2 * 2 * n_act * n_act, s, st);
@@ -2764,7 +2825,7 @@ int msd_features_rows(msd_ctx* ctx, int n_w, const double* phi_a, const double* 
     if (ld > need) CK(cudaMemsetAsync(feat, 0, sizeof(float) * (size_t)n_w * ld, st));
     for (int w0 = 0; w0 < n_w; w0 += cap) {
         const int nw = std::min(cap, n_w - w0);
-        if ((rc = run_refs(ctx, in, w0, nw, cap, c, st, false))) return rc;
+        if ((rc = run_refs(ctx, in, w0, nw, c, st, false))) return rc;
         long long off = 0;
         for (int s = 0; s < 2; ++s) {
             launch_features_rows(nw, M, ctx->n[s], c.Gr[s], feat + (size_t)w0 * ld, ld, off, st);
