@@ -201,7 +201,13 @@ int msd_kernel_stat(msd_ctx* ctx, int index, const char** name, long long* launc
                     double* total_ms);
 
 /* Limit the device workspace (bytes) the context may hold; larger walker
-   batches are processed in chunks. 0 restores the default (16 GiB). */
+   batches are processed in chunks. 0 restores the default (16 GiB). The
+   constants of the Hamiltonian and the trial come on top: the half-rotated
+   Cholesky vectors, their TF32 splits (mixed precision) and, built by the
+   first FP64 call that takes them (with a synchronisation of its stream), 16
+   bytes per entry for the tensor-core forms of the half-rotated and (msd_propagate)
+   the full Cholesky vectors and tables of the trial's minors. A call that
+   cannot have the memory of those last runs without them, many times slower. */
 int msd_set_workspace_limit(msd_ctx* ctx, size_t bytes);
 
 /* With sync = 1 (the default) every call synchronises its stream before

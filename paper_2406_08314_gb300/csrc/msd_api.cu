@@ -8,6 +8,7 @@
 #include <cstdio>
 #include <cstring>
 #include <map>
+#include <new>
 #include <string>
 #include <vector>
 
@@ -99,7 +100,6 @@ struct Buf {
 struct DgConst {
     void* s = nullptr;
     int* e = nullptr;
-    bool tried = false;
 };
 
 }  // namespace
@@ -335,22 +335,19 @@ struct DgScratch {
 };
 
 // Slices of a constant real [rows][K] operand on first use; false where their
-// memory cannot be had (the FP64 kernels run then).
+// memory cannot be had (the FP64 kernels run then, and the next call tries again).
 bool dg_ready(DgConst& c, long long rows, int K, const double* src, long long ld, cudaStream_t st)
 {
-    if (!c.tried) {
-        c.tried = true;
-        if (cudaMalloc(&c.s, dg_row_bytes(K) * (size_t)rows) != cudaSuccess ||
-            cudaMalloc((void**)&c.e, sizeof(int) * (size_t)rows) != cudaSuccess) {
-            cudaGetLastError();
-            free_dg(c);
-            c.tried = true;
-        } else {
-            dg_slice_real(rows, K, src, ld, c.s, c.e, st);
-            cudaStreamSynchronize(st);   // other streams may use the slices next
-        }
+    if (c.s) return true;
+    if (cudaMalloc(&c.s, dg_row_bytes(K) * (size_t)rows) != cudaSuccess ||
+        cudaMalloc((void**)&c.e, sizeof(int) * (size_t)rows) != cudaSuccess) {
+        cudaGetLastError();
+        free_dg(c);
+        return false;
     }
-    return c.s != nullptr;
+    dg_slice_real(rows, K, src, ld, c.s, c.e, st);
+    cudaStreamSynchronize(st);   // other streams may use the slices next
+    return true;
 }
 
 // C[m][n] = sum_k A[m][k] B[n][k] in FP64: A Mr complex rows (walkers), B the
@@ -798,11 +795,10 @@ int minor2_row(const StringKey& q, int a, int b, int c, int d, int nh, int np)
 // entry (i, j) of a string's k x k inverse, the row of V = [G | 2 x 2 minors | ratios] that
 // holds its cofactor (the minor without hole j and particle i), twice, plus 1 where its
 // sign is negative; and the same entries by (hole, particle), in pieces of at most LONG.
-// Trials with far more sub-minors than strings keep the LU path.
-int prepare_ext(msd_ctx* ctx)
+// Trials with far more sub-minors than strings keep the LU path, and calls that cannot
+// have the tables' memory take it (prepare_ext).
+int build_ext(msd_ctx* ctx)
 {
-    if (ctx->ext_ready) return MSD_OK;
-    ctx->ext_ready = true;
     constexpr int LONG = 64;
     Closure C[2];
     std::vector<int> row[2], crow[2], coff[2];
@@ -871,6 +867,22 @@ int prepare_ext(msd_ctx* ctx)
     }
     ctx->ext_ok = true;
     return MSD_OK;
+}
+
+void prepare_ext(msd_ctx* ctx)
+{
+    if (ctx->ext_ready) return;
+    int rc = MSD_ERR_NOMEM;
+    try {
+        rc = build_ext(ctx);
+    } catch (const std::bad_alloc&) {
+    }
+    if (rc) {
+        cudaGetLastError();
+        free_ext(ctx);
+    } else {
+        ctx->ext_ready = true;
+    }
 }
 
 void free_spin(SpinHost& S)
@@ -1328,13 +1340,11 @@ bool use_ext(const msd_ctx* ctx, StringUse use)
 }
 
 // The use of a call that needs the cofactors or inverse minors (energy).
-int string_use(msd_ctx* ctx, bool energy, StringUse* use)
+StringUse string_use(msd_ctx* ctx, bool energy)
 {
-    *use = StringUse::Minors;
-    if (ctx->prec != MSD_FP64) return MSD_OK;
-    const int rc = prepare_ext(ctx);
-    if (!rc && ctx->ext_ok && !energy) *use = StringUse::Cofactors;
-    return rc;
+    if (ctx->prec != MSD_FP64) return StringUse::Minors;
+    prepare_ext(ctx);
+    return ctx->ext_ok && !energy ? StringUse::Cofactors : StringUse::Minors;
 }
 
 // Rows of the minors' marks of spin s (launch_minors, launch_minors_ext).
@@ -1997,7 +2007,7 @@ int evaluate_impl(msd_ctx* ctx, int n_w, const double* phi_a, const double* phi_
     const int nR = weights_blocks(tables(ctx->sp[0], 1));
     const int nslot = nR + (want_e ? energy_slots(ctx) : 0);
     StringUse use = StringUse::Overlap;
-    if ((want_v || want_e) && (rc = string_use(ctx, want_e, &use))) return rc;
+    if (want_v || want_e) use = string_use(ctx, want_e);
     Bytes per = overlap_bytes_per_walker(ctx, use, nslot, false, want_v);
     if (want_v) per += fb_bytes_per_walker(ctx, fp32);
     if (want_e) per += en_bytes_per_walker(ctx, fp32);
@@ -2108,8 +2118,7 @@ int rdm1(msd_ctx* ctx, int n_w, const double* phi_a, const double* phi_b, double
     if ((rc = stage_output(ctx, "out_rdm", rdm, (size_t)n_w * 2 * M * M, o_r))) return rc;
     CK(cudaMemsetAsync(o_r.dev, 0, o_r.bytes, st));
     const int nR = weights_blocks(tables(ctx->sp[0], 1));
-    StringUse use;
-    if ((rc = string_use(ctx, false, &use))) return rc;
+    const StringUse use = string_use(ctx, false);
     Bytes per = overlap_bytes_per_walker(ctx, use, nR, false, true);
     per += fb_bytes_per_walker(ctx, false);
     const int cap = chunk_for(ctx, per, n_w);
@@ -2178,8 +2187,7 @@ int det_energies(msd_ctx* ctx, int n_w, const double* phi_a, const double* phi_b
     if ((rc = arena_get(ctx, "det_rec", sizeof(DetRec) * n_pairs, &d_rec))) return rc;
     CK(cudaMemcpyAsync(d_rec, recs.data(), sizeof(DetRec) * n_pairs, cudaMemcpyHostToDevice, st));
     const int nR = weights_blocks(tables(ctx->sp[0], 1));
-    StringUse use;
-    if ((rc = string_use(ctx, true, &use))) return rc;
+    const StringUse use = string_use(ctx, true);
     Bytes per = overlap_bytes_per_walker(ctx, use, nR);
     per += en_bytes_per_walker(ctx, fp32);
     const int cap = chunk_for(ctx, per, n_w);

@@ -74,3 +74,46 @@ def test_batch_that_fits_its_results(precision):
     batch.close()
     for c in [ref, *ctxs]:
         c.close()
+
+
+def test_constants_are_built_once_their_memory_can_be_had():
+    """A propagation step beside which the tensor-core form of the Cholesky vectors does not
+    fit runs without it; the next one, with memory free again, takes it."""
+    import torch
+
+    from paper_2406_08314_gb300 import msd, synth
+    M, n, G, nw = 64, 6, 1500, 4                 # 64 x 64 rows of 1500: 47 MB, in FP64 form 96 MB
+    s = synth.make_system(4, M, n, n, 2, 8, 20, 3, 1.0, G)
+    w = synth.make_walkers(np.random.default_rng(1), M, n, n, nw)
+    x = torch.from_numpy(np.random.default_rng(2).standard_normal((nw, G))).cuda()
+    ctx = msd.Context(s, "fp64")
+
+    def step():
+        pa, pb = torch.from_numpy(w.phi_a).cuda(), torch.from_numpy(w.phi_b).cuda()
+        wt = torch.ones(nw, dtype=torch.float64, device="cuda")
+        before = msd.launch_count()
+        ctx.propagate(pa, pb, wt, x, 0.01)
+        return msd.launch_count() - before, pa, pb, wt
+
+    step()
+    launches, pa, pb, _ = step()
+    again = msd.Context(s, "fp64")
+    ctx.close()
+    ctx = again
+    # everything a step needs but the propagator's constants
+    ctx.force_bias(pa, pb)
+    ctx.overlap(pa, pb)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    free = torch.cuda.mem_get_info()[0]
+    hog = torch.empty(free - (90 << 20), dtype=torch.uint8, device="cuda")
+    step()                                       # its first launches on the side
+    few = step()
+    del hog
+    torch.cuda.empty_cache()
+    step()
+    many = step()
+    ctx.close()
+    assert few[0] < launches and many[0] == launches
+    for a, b in zip(few[1:], many[1:]):
+        assert torch.allclose(a, b, rtol=1e-10, atol=1e-12)
