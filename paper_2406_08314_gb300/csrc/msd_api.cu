@@ -2500,6 +2500,7 @@ int msd_set_hamiltonian(msd_ctx* ctx, const double* h1, double e0, int n_chol, c
     if (!ctx) return MSD_ERR_ARG;
     if (!h1 || !L || n_chol <= 0) return fail(ctx, MSD_ERR_ARG, "h1, L and n_chol > 0 are required");
     CK(cudaSetDevice(ctx->device));
+    ctx->gen++;   // recorded graphs hold what is freed here, also on an error return
     const int M = ctx->M;
     ctx->h_h1.assign(h1, h1 + (size_t)2 * M * M);
     ctx->h_L.assign(L, L + (size_t)n_chol * M * M);
@@ -2518,6 +2519,7 @@ int msd_set_trial(msd_ctx* ctx, int n_det, const double* coeff, const int32_t* o
     if (!ctx) return MSD_ERR_ARG;
     if (n_det <= 0 || !coeff || !occ_a || !occ_b) return fail(ctx, MSD_ERR_ARG, "empty trial");
     CK(cudaSetDevice(ctx->device));
+    ctx->gen++;   // recorded graphs hold what is freed here, also on an error return
     ctx->have_trial = false;
     free_ext(ctx);
     std::vector<int> sid[2];
