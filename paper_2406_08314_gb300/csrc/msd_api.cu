@@ -334,11 +334,21 @@ struct DgScratch {
     size_t bytes() const { return s + sa + part; }
 };
 
+// Work of a stream that is being captured runs later or not at all: nothing that a context
+// keeps is built then.
+bool capturing(cudaStream_t st)
+{
+    cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &s) != cudaSuccess) { cudaGetLastError(); return true; }
+    return s != cudaStreamCaptureStatusNone;
+}
+
 // Slices of a constant real [rows][K] operand on first use; false where their
 // memory cannot be had (the FP64 kernels run then, and the next call tries again).
 bool dg_ready(DgConst& c, long long rows, int K, const double* src, long long ld, cudaStream_t st)
 {
     if (c.s) return true;
+    if (capturing(st)) return false;
     if (cudaMalloc(&c.s, dg_row_bytes(K) * (size_t)rows) != cudaSuccess ||
         cudaMalloc((void**)&c.e, sizeof(int) * (size_t)rows) != cudaSuccess) {
         cudaGetLastError();
@@ -869,9 +879,9 @@ int build_ext(msd_ctx* ctx)
     return MSD_OK;
 }
 
-void prepare_ext(msd_ctx* ctx)
+void prepare_ext(msd_ctx* ctx, cudaStream_t st)
 {
-    if (ctx->ext_ready) return;
+    if (ctx->ext_ready || capturing(st)) return;
     int rc = MSD_ERR_NOMEM;
     try {
         rc = build_ext(ctx);
@@ -1340,10 +1350,10 @@ bool use_ext(const msd_ctx* ctx, StringUse use)
 }
 
 // The use of a call that needs the cofactors or inverse minors (energy).
-StringUse string_use(msd_ctx* ctx, bool energy)
+StringUse string_use(msd_ctx* ctx, bool energy, cudaStream_t st)
 {
     if (ctx->prec != MSD_FP64) return StringUse::Minors;
-    prepare_ext(ctx);
+    prepare_ext(ctx, st);
     return ctx->ext_ok && !energy ? StringUse::Cofactors : StringUse::Minors;
 }
 
@@ -2007,7 +2017,7 @@ int evaluate_impl(msd_ctx* ctx, int n_w, const double* phi_a, const double* phi_
     const int nR = weights_blocks(tables(ctx->sp[0], 1));
     const int nslot = nR + (want_e ? energy_slots(ctx) : 0);
     StringUse use = StringUse::Overlap;
-    if (want_v || want_e) use = string_use(ctx, want_e);
+    if (want_v || want_e) use = string_use(ctx, want_e, st);
     Bytes per = overlap_bytes_per_walker(ctx, use, nslot, false, want_v);
     if (want_v) per += fb_bytes_per_walker(ctx, fp32);
     if (want_e) per += en_bytes_per_walker(ctx, fp32);
@@ -2118,7 +2128,7 @@ int rdm1(msd_ctx* ctx, int n_w, const double* phi_a, const double* phi_b, double
     if ((rc = stage_output(ctx, "out_rdm", rdm, (size_t)n_w * 2 * M * M, o_r))) return rc;
     CK(cudaMemsetAsync(o_r.dev, 0, o_r.bytes, st));
     const int nR = weights_blocks(tables(ctx->sp[0], 1));
-    const StringUse use = string_use(ctx, false);
+    const StringUse use = string_use(ctx, false, st);
     Bytes per = overlap_bytes_per_walker(ctx, use, nR, false, true);
     per += fb_bytes_per_walker(ctx, false);
     const int cap = chunk_for(ctx, per, n_w);
@@ -2187,7 +2197,7 @@ int det_energies(msd_ctx* ctx, int n_w, const double* phi_a, const double* phi_b
     if ((rc = arena_get(ctx, "det_rec", sizeof(DetRec) * n_pairs, &d_rec))) return rc;
     CK(cudaMemcpyAsync(d_rec, recs.data(), sizeof(DetRec) * n_pairs, cudaMemcpyHostToDevice, st));
     const int nR = weights_blocks(tables(ctx->sp[0], 1));
-    const StringUse use = string_use(ctx, true);
+    const StringUse use = string_use(ctx, true, st);
     Bytes per = overlap_bytes_per_walker(ctx, use, nR);
     per += en_bytes_per_walker(ctx, fp32);
     const int cap = chunk_for(ctx, per, n_w);
