@@ -485,7 +485,7 @@ k_dg_cols(int K, int Kp, int nc, const double2* __restrict__ src, long long ld, 
     __shared__ double2 tile[TK][17];
     __shared__ unsigned top[16][17];
     __shared__ int ex[16];
-    const int z = blockIdx.y, c0 = blockIdx.x * 16, t = threadIdx.x, cl = t & 15, kl = t >> 4;
+    const int z = blockIdx.x, c0 = blockIdx.y * 16, t = threadIdx.x, cl = t & 15, kl = t >> 4;
     const double2* s = src + (size_t)z * src_batch;
     unsigned mx = 0;
     if (c0 + cl < nc)
@@ -590,7 +590,7 @@ void dg_slice_columns(int mode, int K, int nc, int batch, const double2* src, lo
     if (nc <= 0 || batch <= 0) return;
     const int Kp = dg_k_padded(mode == 2 ? K : 2 * K);
     const size_t sa = (size_t)batch * rows * Kp, sb = 2 * sa;
-    const dim3 grid((nc + 15) / 16, batch);
+    const dim3 grid(batch, (nc + 15) / 16);   // x: any number of walkers
     __nv_bfloat16 *a = (__nv_bfloat16*)Sa, *b = (__nv_bfloat16*)Sb;
     if (mode == 0) k_dg_cols<0><<<grid, 256, 0, st>>>(K, Kp, nc, src, ld, src_batch, row0, rows, a, ea, sa, b, eb, sb);
     else if (mode == 1) k_dg_cols<1><<<grid, 256, 0, st>>>(K, Kp, nc, src, ld, src_batch, row0, rows, a, ea, sa, b, eb, sb);
