@@ -33,7 +33,8 @@
 // the per-determinant kernels read.
 //
 // Iron-sulfur trial, 640 walkers (12.5e3 strings per spin): ratios and FP32
-// inverse minors 3.60 (one pivoted LU per string) -> 1.33 ms, weights 1.32 -> 0.89
+// inverse minors 3.60 (one pivoted LU per string) -> 1.48 ms (1.33 without the
+// check of the cancellation and its LUs), weights 1.32 -> 0.89
 // ms; 1e6 determinants, 10 walkers: weights 0.93 -> 0.28 ms.
 #include <algorithm>
 
@@ -291,7 +292,7 @@ struct WeightSpin {
     float2* rf;              // [nw][n_str] r_s in FP32 (may be NULL)
     double2* part;           // [nw][nslot] partial sums over 32 strings (may be NULL)
     double2* wT;             // [n_str][nw] the sums themselves (may be NULL)
-    const int* big;          // [nw] with wT: walkers whose sums go to wT for vanishing ratios only
+    int* big;                // [nw] with wT: walkers (1) whose sums go to wT for vanishing ratios only, 2 if it has any
 };
 struct WeightArgs { WeightSpin s[2]; };
 
@@ -332,7 +333,11 @@ __global__ void __launch_bounds__(256) k_weights(const __grid_constant__ WeightA
                 acc = cz(fma(v.x, c, acc.x), fma(v.y, c, acc.y));
             }
             r = S.self[(size_t)s * nw + w];
-            if (S.wT) S.wT[(size_t)s * nw + w] = S.big[w] && (r.x != 0 || r.y != 0) ? cz(0, 0) : acc;
+            if (S.wT) {
+                const bool zero = r.x == 0 && r.y == 0;
+                if (zero && S.big[w]) S.big[w] = 2;
+                S.wT[(size_t)s * nw + w] = S.big[w] && !zero ? cz(0, 0) : acc;
+            }
             rw = cmul(r, acc);
         }
         tw[sl][wl] = rw;
@@ -490,10 +495,11 @@ __global__ void __launch_bounds__(128) k_inverse_minors(const __grid_constant__ 
 // trial does not hold, appended to its strings): 4 FP64 FMAs per entry and one
 // reciprocal per string, against 8 k^3 / 3 and k reciprocals of an LU with its column
 // solves, which the FP64 unit bounds. The relative error of an entry is that of two
-// division-free minors. Bound by memory now: k^2 gathered rows of the walkers in, k^2
+// minors. Bound by memory now: k^2 gathered rows of the walkers in, k^2
 // entries out per string and walker. A warp takes 32 (string, walker) pairs, walkers
 // fastest, and writes their entries through shared memory, up to 16 (256 bytes) of a
-// pair at a time. 640 copper-oxo walkers, ratios and inverses 3.06 -> 1.28 ms.
+// pair at a time. 640 copper-oxo walkers, ratios and inverses 3.06 -> 1.44 ms.
+// Walkers with large active blocks are done again by LU (k_strings_large in k_wick.cu).
 struct InvRatioSpin {
     int bucket[MSD_KMAX + 2];
     const int* row;
@@ -613,6 +619,7 @@ struct CofSpin {
     const double2* V;
     double2* Bv;
     double2* Cm;             // the sums: [nw][np][nh], entry x = h np + p to p nh + h
+    const int* big;          // [nw] 1: nothing to sum for the walker
     int nh, np;
 };
 struct CofArgs { CofSpin s[2]; };
@@ -624,7 +631,7 @@ __global__ void __launch_bounds__(256) k_cofactors(const __grid_constant__ CofAr
     if (e >= (long long)(S.t1 - S.t0) * nw) return;
     const int t = S.t0 + (int)(e / nw), w = (int)(e % nw);
     double2 acc = cz(0, 0);
-    const int i1 = S.off[t + 1];
+    const int i1 = S.big[w] == 1 ? 0 : S.off[t + 1];
     for (int i = S.off[t]; i < i1; i += 4) {
         double2 a[4], b[4];
 #pragma unroll
@@ -683,7 +690,7 @@ void launch_minors_ext(const ExtTables g[2], const SpinTables& ta, const SpinTab
 }
 
 void launch_cofactors(const ExtTables g[2], const SpinTables& ta, const SpinTables& tb, int nw, double2* const V[2],
-                      double2* const Bv[2], double2* const Cm[2], cudaStream_t st)
+                      double2* const Bv[2], double2* const Cm[2], int* const big[2], cudaStream_t st)
 {
     const SpinTables* T[2] = {&ta, &tb};
     for (int sums = 0; sums < 2; ++sums) {
@@ -691,8 +698,8 @@ void launch_cofactors(const ExtTables g[2], const SpinTables& ta, const SpinTabl
         int n = 0;
         for (int s = 0; s < 2; ++s) {
             const int t0 = sums ? g[s].n_piece : 0, t1 = g[s].n_piece + (sums ? T[s]->nh * T[s]->np : 0);
-            a.s[s] = CofSpin{t0, t1, g[s].cof_row, g[s].cof_off, g[s].cof_ent, V[s], Bv[s], sums ? Cm[s] : nullptr, T[s]->nh,
-                             T[s]->np};
+            a.s[s] = CofSpin{t0, t1, g[s].cof_row, g[s].cof_off, g[s].cof_ent, V[s], Bv[s], sums ? Cm[s] : nullptr, big[s],
+                             T[s]->nh, T[s]->np};
             n = std::max(n, t1 - t0);
         }
         if (n <= 0) continue;

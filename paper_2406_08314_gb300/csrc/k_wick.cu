@@ -2,6 +2,8 @@
 // part of the generalized-Wick evaluation (Sec. III "Implementation":
 // get_dets), plus the cofactor accumulation behind the mixed Green's
 // function (reduce_CI) and its rank-n_p update.
+#include <type_traits>
+
 #include "common.cuh"
 #include "kernels.h"
 
@@ -24,10 +26,10 @@
 // are rounded to 56 bits of a row's largest value over the walker's columns, and G does
 // not depend on the columns' scales: so column k of phi enters as phi_k 2^-e_k, |phi_k|
 // < 2^e_k, and row k of S^-1 as 2^e_k of it (exact; without it columns 1e8 apart left 9
-// digits of G). Reading phi once more for the e_k: k_ref 1.15 -> 1.15 ms as below.
+// digits of G; 0.012 ms of the copper-oxo time below).
 // Measured, both spins: N = 5, 16 walkers 70 -> 21 us; iron-sulfur (N = 30, M = 160)
-// 640 walkers 1.95 -> 1.15 ms, 64 walkers 0.81 -> 0.24 ms; copper-oxo (N = 16, M =
-// 108) 640 walkers 0.73 -> 0.46 ms.
+// 640 walkers 1.95 -> 1.00 ms, 64 walkers 0.81 -> 0.23 ms; copper-oxo (N = 16, M =
+// 108) 640 walkers 0.73 -> 0.37 ms.
 struct RefIn {
     const double2* phi;     // [nw][M][N]
     int N, nh, np;
@@ -393,7 +395,9 @@ __global__ void __launch_bounds__(256) k_large(const __grid_constant__ LargeArgs
 // B G keeps its cancellation; inverse entries as ratios of separately rounded minors do
 // not, and lose the square of the block's magnitude (rank-1 part of 30: density matrix
 // 4e-13 against 3e-14, of 1e4: 4e-8 against 8e-12; entries up to 1: alike). A block takes
-// 128 strings of a level; the blocks of a column share the marked walkers. None marked: 3 us.
+// 128 strings of a level; the blocks of a column share the marked walkers. Levels 1 to 4
+// and 5, 6 apart: 134 and 255 registers. None marked: 3 us a launch; all of 640 copper-oxo
+// walkers marked: density matrix 2.2 -> 6.2 ms (6.3 with an LU for every walker).
 struct StringsLargeArgs {
     SpinTables t[2];
     const double2* Gact[2];
@@ -401,14 +405,15 @@ struct StringsLargeArgs {
     double2 *r[2], *rT[2], *B[2];
     int blk[2][MSD_KMAX + 2];   // first block of each level
 };
+template <int LO, int HI>
 __global__ void __launch_bounds__(128) k_strings_large(const __grid_constant__ StringsLargeArgs a, int nw)
 {
     const int spin = blockIdx.z, t = threadIdx.x;
     const SpinTables& tb = a.t[spin];
-    if ((int)blockIdx.x >= a.blk[spin][MSD_KMAX + 1]) return;
+    if ((int)blockIdx.x >= a.blk[spin][HI + 1]) return;
     __shared__ double2 g[MSD_XMAX];
     __shared__ unsigned marks[32];
-    int k = 1;
+    int k = LO;
     while ((int)blockIdx.x >= a.blk[spin][k + 1]) ++k;
     const int X = tb.nh * tb.np, sl = ((int)blockIdx.x - a.blk[spin][k]) * 128 + t;
     const bool on = sl < tb.bucket[k + 1] - tb.bucket[k];
@@ -429,14 +434,17 @@ __global__ void __launch_bounds__(128) k_strings_large(const __grid_constant__ S
                 for (int e = t; e < X; e += 128) g[e] = a.Gact[spin][(size_t)w * X + e];
                 __syncthreads();
                 if (!on) continue;
-                switch (k) {
-                case 1: string_lu<1>(tb, nw, w, sl, g, a.r[spin], a.rT[spin], a.B[spin]); break;
-                case 2: string_lu<2>(tb, nw, w, sl, g, a.r[spin], a.rT[spin], a.B[spin]); break;
-                case 3: string_lu<3>(tb, nw, w, sl, g, a.r[spin], a.rT[spin], a.B[spin]); break;
-                case 4: string_lu<4>(tb, nw, w, sl, g, a.r[spin], a.rT[spin], a.B[spin]); break;
-                case 5: string_lu<5>(tb, nw, w, sl, g, a.r[spin], a.rT[spin], a.B[spin]); break;
-                default: string_lu<6>(tb, nw, w, sl, g, a.r[spin], a.rT[spin], a.B[spin]); break;
-                }
+                auto lu = [&](auto level) {
+                    constexpr int K = decltype(level)::value;
+                    if constexpr (LO <= K && K <= HI)
+                        if (k == K) string_lu<K>(tb, nw, w, sl, g, a.r[spin], a.rT[spin], a.B[spin]);
+                };
+                lu(std::integral_constant<int, 1>{});
+                lu(std::integral_constant<int, 2>{});
+                lu(std::integral_constant<int, 3>{});
+                lu(std::integral_constant<int, 4>{});
+                lu(std::integral_constant<int, 5>{});
+                lu(std::integral_constant<int, 6>{});
             }
     }
 }
@@ -448,22 +456,29 @@ void launch_strings_large(const SpinTables& ta, const SpinTables& tb, int nw, do
     LargeArgs l;
     StringsLargeArgs a;
     const SpinTables* T[2] = {&ta, &tb};
-    int nb = 0;
     for (int s = 0; s < 2; ++s) {
         l.GT[s] = GT[s]; l.X[s] = T[s]->nh * T[s]->np; l.big[s] = big[s];
         a.t[s] = *T[s]; a.Gact[s] = Gact[s]; a.big[s] = big[s];
         a.r[s] = r[s]; a.rT[s] = rT[s]; a.B[s] = (double2*)B[s];
-        a.blk[s][0] = a.blk[s][1] = 0;
-        for (int k = 1; k <= MSD_KMAX; ++k) a.blk[s][k + 1] = a.blk[s][k] + (T[s]->bucket[k + 1] - T[s]->bucket[k] + 127) / 128;
-        nb = nb > a.blk[s][MSD_KMAX + 1] ? nb : a.blk[s][MSD_KMAX + 1];
     }
     k_large<<<dim3((nw + 31) / 32, 2), 256, 0, st>>>(l, nw);
     msd_note_launch();
-    if (nb <= 0) return;
-    // columns enough to fill the GPU when many walkers are marked
-    const int cols = nb >= 512 ? 4 : nb >= 128 ? 16 : 64;
-    k_strings_large<<<dim3(nb, nw < cols ? nw : cols, 2), 128, 0, st>>>(a, nw);
-    msd_note_launch();
+    auto go = [&](auto kern, int lo, int hi) {
+        int nb = 0;
+        for (int s = 0; s < 2; ++s) {
+            for (int k = 0; k <= lo; ++k) a.blk[s][k] = 0;
+            for (int k = lo; k <= hi; ++k)
+                a.blk[s][k + 1] = a.blk[s][k] + (T[s]->bucket[k + 1] - T[s]->bucket[k] + 127) / 128;
+            nb = nb > a.blk[s][hi + 1] ? nb : a.blk[s][hi + 1];
+        }
+        if (nb <= 0) return;
+        // columns enough to fill the GPU when many walkers are marked
+        const int cols = nb >= 512 ? 4 : nb >= 128 ? 16 : 64;
+        kern<<<dim3(nb, nw < cols ? nw : cols, 2), 128, 0, st>>>(a, nw);
+        msd_note_launch();
+    };
+    go(k_strings_large<1, 4>, 1, 4);
+    go(k_strings_large<5, 6>, 5, 6);
 }
 
 // ------------------------------------------------------------------------

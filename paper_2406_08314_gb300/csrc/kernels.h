@@ -76,7 +76,7 @@ void launch_minors_ext(const ExtTables g[2], const SpinTables& ta, const SpinTab
 void launch_inverse_ratios(const ExtTables g[2], const SpinTables& ta, const SpinTables& tb, int nw,
                            double2* const V[2], void* const B[2], cudaStream_t st);
 void launch_cofactors(const ExtTables g[2], const SpinTables& ta, const SpinTables& tb, int nw, double2* const V[2],
-                      double2* const Bv[2], double2* const Cm[2], cudaStream_t st);
+                      double2* const Bv[2], double2* const Cm[2], int* const big[2], cudaStream_t st);
 void launch_untranspose(int n_str, int nw, const double2* rT, double2* r, cudaStream_t st);
 void launch_det_ratios(const PairTables& pt, int nw, int n_str_a, int n_str_b, const double2* ra,
                        const double2* rb, double2* out, cudaStream_t st);

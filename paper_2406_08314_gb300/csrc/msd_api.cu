@@ -1514,7 +1514,7 @@ int run_cofactors(msd_ctx* ctx, int nw, Chunk& c, StringUse use, bool fp32, doub
     const SpinTables T[2] = {tables(ctx->sp[0], c.cap, c.w0), tables(ctx->sp[1], c.cap, c.w0)};
     ctx->hook.begin("k_cmat", st);
     const bool ext = use_ext(ctx, use);
-    if (ext) launch_cofactors(ctx->ext, T[0], T[1], nw, c.V, c.Bv, Cm, st);
+    if (ext) launch_cofactors(ctx->ext, T[0], T[1], nw, c.V, c.Bv, Cm, c.big, st);
     launch_cmat(T[0], T[1], nw, c.wts[0], c.wts[1], c.B[0], c.B[1], fp32, Cm[0], Cm[1], st, ext ? c.big : nullptr);
     ctx->hook.end(st);
     CKLAUNCH();
@@ -3383,8 +3383,8 @@ int msd_batch_create(msd_batch** out, msd_ctx* const* ctxs, int n_sys)
         b->ctx.push_back(ctxs[i]);
     }
     // the persistent per-determinant kernel implements the per-determinant
-    // opposite-spin form; the systems' own evaluations use the same form, so
-    // batched and per-system results agree
+    // opposite-spin form; the systems' own evaluations use it too, so that batched
+    // and per-system results agree (mixed mode) up to rounding (FP64 mode)
     for (int i = 0; i < n_sys; ++i) msd_set_pair_form(ctxs[i], 0);
     b->device = ctxs[0]->device;
     b->fp32 = ctxs[0]->prec == MSD_MIXED;
