@@ -291,7 +291,8 @@ __host__ __device__ __forceinline__ constexpr int se_pitch(int k) { return (k * 
 // i. The string's limbs are made once, by the group's lanes, in shared memory. A thread
 // per string holds them in registers (254 at level 4: 8 warps per SM, every instruction
 // waiting for the last) and leaves the SM idle where strings are few (one level-6 string
-// in 640 walkers: 0.66 ms). 640 copper-oxo walkers, levels 3 to 6: 2.94 -> 1.31 ms.
+// in 640 walkers: 0.66 ms). 640 copper-oxo walkers, levels 3 to 6: 2.94 -> 1.42 ms
+// (1.31 without the rule below).
 //
 // The b_ml of z_ij carry 54 bits of the string's largest entry b_ab, and the term is of
 // the size of the largest product b_ij b_ml, i != m, j != l: of

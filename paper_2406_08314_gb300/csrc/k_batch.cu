@@ -3,9 +3,13 @@
 // excitation levels) in one launch. Work items are (system, walker, kind,
 // spin or opposite-spin level pair, block of strings or determinants); a
 // resident grid of CTAs takes items from a global counter (atomicAdd, no
-// waiting), so small and large systems share the machine. Each item computes
-// exactly what one block of k_string_energy / k_pair_cross computes and
-// writes the same partial-sum slot, so batched and per-system results agree.
+// waiting), so small and large systems share the machine. Each item covers the
+// strings or determinants of one block of k_string_energy / k_pair_cross and
+// writes the same partial-sum slot. In mixed mode it computes what that block
+// computes. In FP64 mode the opposite-spin term has other forms here (a thread per
+// determinant in fixed point up to ka + kb = 6, the general FP64 form above; the
+// per-system kernels give a determinant a group of lanes up to 8) and sums in
+// another order: batched and per-system energies agree to rounding.
 #include "common.cuh"
 #include "det_block.cuh"
 #include "kernels.h"

@@ -15,9 +15,11 @@
 // 64-bit integers, and rounds once to FP64 at the end.
 //
 // Error: the operands' rounding (2^-57 of the row maximum) and the dropped
-// products c >= 10 (below 2^-63 K^1/2 of the two row maxima). For rows without
-// a dynamic range beyond a few thousand that is less than what an FP64 FMA
-// chain accumulates (about 2^-53 (K / 8)^1/2 of the result).
+// products c >= 10 (below 2^-63 K^1/2 of the two row maxima): small against the
+// rounding of an FP64 FMA chain (about 2^-53 (K / 8)^1/2 of the result) where the
+// row maxima meet, less accurate than it where a row's largest entries meet only
+// small ones, by their ratio. Rows whose entries differ by scales of their own are
+// for the caller to scale: the reference product does (k_ref).
 //
 // Tile 128 x 64: eight accumulators of 64 columns are the whole TMEM (512
 // columns). An MMA of N = 64 reads 6 KB of shared memory for 32 tensor clocks,
@@ -27,7 +29,7 @@
 // Structure (persistent, one CTA per SM, 10 warps):
 //   warp 0    TMA producer: k-blocks of 32 BF16 (64-byte swizzle) of all
 //             slices of A and B into a two-stage ring (96 KB a stage);
-//   warp 1    TMEM owner; lane 0 issues the MMAs;
+//   warp 1    TMEM owner; one elected lane issues the MMAs;
 //   warps 2-9 epilogue: lane quarter (warp % 4), column half; each drains the
 //             accumulators in the order c = 2..9 and releases every one as soon
 //             as it is read, so the next tile's products start while this

@@ -22,7 +22,7 @@
 // Structure (persistent, one CTA per SM, 14 warps):
 //   warp 0      TMA producer: A and B k-blocks of 16 FP32 (64-byte swizzle),
 //               TF32 hi and lo parts, into a two-stage shared-memory ring;
-//   warp 1      TMEM owner; lane 0 issues tcgen05.mma into one of two TMEM
+//   warp 1      TMEM owner; one elected lane issues tcgen05.mma into one of two TMEM
 //               accumulators (the next tile's products overlap this tile's
 //               epilogue);
 //   warps 2-13  epilogue, three sets of four warps (one per lane quarter)

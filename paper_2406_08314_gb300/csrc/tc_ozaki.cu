@@ -32,7 +32,7 @@
 // Structure (one CTA per 128 x 96 output tile, 10 warps):
 //   warp 0    TMA producer: k-blocks of 32 BF16 (64-byte swizzle) of all S
 //             slices of A and B into a three-stage shared-memory ring;
-//   warp 1    TMEM owner; lane 0 issues tcgen05.mma kind::f16 (15 products
+//   warp 1    TMEM owner; one elected lane issues tcgen05.mma kind::f16 (15 products
 //             per 16-element K step) into the S accumulators;
 //   warps 2-9 epilogue: lane quarter (warp % 4), column half ((warp - 2) / 4);
 //             each drains its 48 columns of the S accumulators after every
