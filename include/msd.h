@@ -272,7 +272,7 @@ int msd_set_tensor_gram(msd_ctx* ctx, int on);
    concurrently with the string minors and weights (bound by FP64
    arithmetic) on the caller's stream; then the force bias runs on the
    second stream, concurrently with the per-determinant terms, which wait for
-   the energy sums. On the iron-sulfur shape: 19.15 against 19.94 ms per
+   the energy sums. On the iron-sulfur shape: 19.41 against 20.09 ms per
    step. The call stays ordered on the caller's stream: the second stream
    waits for the caller's stream at each fork, and the caller's stream waits
    for the second stream before the per-determinant terms (energy sums) and
