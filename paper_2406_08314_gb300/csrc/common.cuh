@@ -196,6 +196,13 @@ __device__ __forceinline__ double int_to_fp64(long long v, int s)
     return __longlong_as_double((long long)((((unsigned long long)(ex - 1)) << 52) + m) | (v & (long long)(1ull << 63)));
 }
 
+// GELU of the control-variate network and its derivative.
+__device__ __forceinline__ float net_gelu(float z) { return 0.5f * z * (1.f + erff(z * 0.70710678118654752f)); }
+__device__ __forceinline__ float net_gelu_d(float z)
+{
+    return 0.5f * (1.f + erff(z * 0.70710678118654752f)) + z * 0.39894228040143268f * expf(-0.5f * z * z);
+}
+
 // Sum of n partial sums by one warp (every lane returns it).
 __device__ __forceinline__ double2 warp_sum_slots(const double2* __restrict__ p, int n, int lane)
 {

@@ -24,11 +24,6 @@ typedef __nv_bfloat16 bf16;
 
 namespace {
 
-__device__ __forceinline__ float gelu_d(float z)
-{
-    return 0.5f * (1.f + erff(z * 0.70710678118654752f)) + z * 0.39894228040143268f * expf(-0.5f * z * z);
-}
-
 int grid_of(long long n)
 {
     const long long cap = 32ll * msd_sm_count();
@@ -103,7 +98,7 @@ __global__ void k_out_back_dz(int B, int Bp, int n, const float* __restrict__ dy
         bf16 vb = __float2bfloat16(0.f);
         if (b < B && j < n) {
             const size_t e = (size_t)b * n + j;
-            const float v = dy[b] * w[j] * gelu_d(z[e]);
+            const float v = dy[b] * w[j] * net_gelu_d(z[e]);
             dzf[e] = v;
             vb = __float2bfloat16(v);
             dz[e] = vb;

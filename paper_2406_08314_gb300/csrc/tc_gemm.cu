@@ -24,15 +24,10 @@
 namespace {
 
 using namespace tcx;
+
 // SPLIT: 3xTF32 (hi/lo operands, three products per K step) or a single
 // BF16 product. One k-block is 128 bytes of K per row in both cases
 // (32 FP32 or 64 BF16 elements); one MMA covers 32 bytes of K.
-__device__ __forceinline__ float net_gelu(float z) { return 0.5f * z * (1.f + erff(z * 0.70710678118654752f)); }
-__device__ __forceinline__ float net_gelu_d(float z)
-{
-    return 0.5f * (1.f + erff(z * 0.70710678118654752f)) + z * 0.39894228040143268f * expf(-0.5f * z * z);
-}
-
 template <int BN, bool SPLIT>
 struct TcCfg {
     static constexpr int BM = 128;
