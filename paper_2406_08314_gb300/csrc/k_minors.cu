@@ -227,7 +227,7 @@ __device__ __forceinline__ double2 lu_minor(const uint4 rec, int np, const doubl
 // pairs from string s0 on and then its threads take those marked (few: one in a warp
 // would occupy all of it). No marks (tr NULL): all of them. The marks are 4 bytes a pair:
 // 64 MB, 20 us, at 640 iron-sulfur walkers.
-#define LU_PAIRS 2048
+#define LU_PAIRS 4096
 #define LU_THREADS 128
 __global__ void __launch_bounds__(LU_THREADS) k_minor_lu(const __grid_constant__ MinorArgs a, int level0, int nw)
 {
