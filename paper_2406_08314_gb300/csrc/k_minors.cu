@@ -225,8 +225,8 @@ __device__ __forceinline__ double2 lu_minor(const uint4 rec, int np, const doubl
 
 // The minors that k_minors marked, by LU: a block looks through LU_PAIRS (string, walker)
 // pairs from string s0 on and then its threads take those marked (few: one in a warp
-// would occupy all of it). No marks (tr NULL): all of them. The marks are 4 bytes a pair:
-// 64 MB, 20 us, at 640 iron-sulfur walkers.
+// would occupy all of it). No marks (tr NULL): all of them. 0.106 of the 0.78 ms that the
+// ratios of 640 iron-sulfur walkers take; 12 us for 16 small ones, the latency of one LU.
 #define LU_PAIRS 4096
 #define LU_THREADS 128
 __global__ void __launch_bounds__(LU_THREADS) k_minor_lu(const __grid_constant__ MinorArgs a, int level0, int nw)
