@@ -40,6 +40,7 @@
 
 #include "common.cuh"
 #include "kernels.h"
+#include "minor_lu.cuh"
 
 namespace {
 
@@ -55,6 +56,8 @@ struct MinorSpin {
     double2* rT;             // [n_str][nw]
     int* t2;                 // as m2: log2 of the larger product (log_mag)
     int* tr;                 // from string bucket[3] on, as rT: log2 of the largest product; odd: evaluate by LU
+    double2* B;              // inverse minors of the trial's strings to write with the LU, or NULL
+    long long b_off[MSD_KMAX + 2];
 };
 // Both spins of a launch (indexed by the block, in constant memory).
 struct MinorArgs { MinorSpin s[2]; };
@@ -185,50 +188,16 @@ k_minors(const __grid_constant__ MinorArgs a, int k0, int k1, bool subs, int nw)
     tr[(size_t)(s - S.bucket[3]) * nw] = (top & ~1) | (lu ? 1 : 0);
 }
 
-// sign * det A of one string by an LU with partial pivoting (by the larger of |Re|, |Im|).
-template <int K>
-__device__ __forceinline__ double2 lu_minor(const uint4 rec, int np, const double2* __restrict__ g, int nw, double sign)
-{
-    double2 a[K][K];
-#pragma unroll
-    for (int i = 0; i < K; ++i)
-#pragma unroll
-        for (int j = 0; j < K; ++j) a[i][j] = g[(size_t)(rec_h(rec, i) * np + rec_p(rec, j)) * nw];
-    double2 det = cz(sign, 0);
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-        int p = k, best = mag_key(a[k][k]);
-#pragma unroll
-        for (int i = k + 1; i < K; ++i) {
-            const int v = mag_key(a[i][k]);
-            if (v > best) { best = v; p = i; }
-        }
-#pragma unroll
-        for (int i = k + 1; i < K; ++i)
-            if (i == p) {
-#pragma unroll
-                for (int j = k; j < K; ++j) { const double2 t = a[k][j]; a[k][j] = a[i][j]; a[i][j] = t; }
-                det = cz(-det.x, -det.y);
-            }
-        const double2 v = a[k][k];
-        det = cmul(det, v);
-        const double2 inv = v.x == 0.0 && v.y == 0.0 ? cz(0, 0) : crecip(v);
-#pragma unroll
-        for (int i = k + 1; i < K; ++i) {
-            const double2 f = cmul(a[i][k], inv);
-#pragma unroll
-            for (int j = k + 1; j < K; ++j) a[i][j] = cfms(f, a[k][j], a[i][j]);
-        }
-    }
-    return det;
-}
-
 // The minors that k_minors marked, by LU: a block looks through LU_PAIRS (string, walker)
 // pairs from string s0 on and then its threads take those marked (few: one in a warp
-// would occupy all of it). No marks (tr NULL): all of them. 0.106 of the 0.78 ms that the
+// would occupy all of it). With B their inverse minors too: entries as ratios of separately
+// rounded minors are accurate one by one, but the string's energy cancels between them where
+// the minor is close to low rank (entries below 1, rank 1 to 1e-4: energies off by 4e-9
+// rms against 8e-13). No marks (tr NULL): all of them. 0.106 of the 0.78 ms that the
 // ratios of 640 iron-sulfur walkers take; 12 us for 16 small ones, the latency of one LU.
 #define LU_PAIRS 4096
 #define LU_THREADS 128
+template <bool INVERSE>
 __global__ void __launch_bounds__(LU_THREADS) k_minor_lu(const __grid_constant__ MinorArgs a, int level0, int nw)
 {
     const MinorSpin& S = a.s[blockIdx.y];
@@ -266,15 +235,19 @@ __global__ void __launch_bounds__(LU_THREADS) k_minor_lu(const __grid_constant__
         const uint4 rec = S.str_hp[s];
         const double2* g = S.GT + w;
         const double sg = S.str_sign[s];
+        auto G = [&](int i, int j) { return g[(size_t)(rec_h(rec, i) * S.np + rec_p(rec, j)) * nw]; };
+        double2* B = nullptr;
+        if (INVERSE && s < S.n_str)
+            B = S.B + S.b_off[k] + ((size_t)w * (S.bucket[k + 1] - S.bucket[k]) + s - S.bucket[k]) * b_stride(k);
         double2 r = cz(1, 0);
         switch (k) {
         case 0: break;
-        case 1: r = lu_minor<1>(rec, S.np, g, nw, sg); break;
-        case 2: r = lu_minor<2>(rec, S.np, g, nw, sg); break;
-        case 3: r = lu_minor<3>(rec, S.np, g, nw, sg); break;
-        case 4: r = lu_minor<4>(rec, S.np, g, nw, sg); break;
-        case 5: r = lu_minor<5>(rec, S.np, g, nw, sg); break;
-        default: r = lu_minor<6>(rec, S.np, g, nw, sg); break;
+        case 1: r = minor_lu<1>(sg, G, INVERSE ? B : nullptr); break;
+        case 2: r = minor_lu<2>(sg, G, INVERSE ? B : nullptr); break;
+        case 3: r = minor_lu<3>(sg, G, INVERSE ? B : nullptr); break;
+        case 4: r = minor_lu<4>(sg, G, INVERSE ? B : nullptr); break;
+        case 5: r = minor_lu<5>(sg, G, INVERSE ? B : nullptr); break;
+        default: r = minor_lu<6>(sg, G, INVERSE ? B : nullptr); break;
         }
         S.rT[(size_t)s * nw + w] = r;
     }
@@ -508,6 +481,7 @@ struct InvRatioSpin {
     const double2* r;        // [string][nw], within V
     double2* B;
     long long b_off[MSD_KMAX + 2];
+    const int* tr;           // from level 3 on: marked ones have theirs (k_minor_lu)
     int blk[MSD_KMAX + 2];   // first block of each level
 };
 struct InvRatioArgs { InvRatioSpin s[2]; };
@@ -537,6 +511,8 @@ __device__ __forceinline__ void inverse_ratios(const InvRatioSpin& S, int nw, do
     const double2* V = S.V + w;
     const long long base = ((long long)w * ns + sl) * KST;
     double2* B = S.B + S.b_off[K];
+    const bool mine = on && !(K >= 3 && (S.tr[(size_t)(S.bucket[K] - S.bucket[3] + sl) * nw + w] & 1));
+    const unsigned write = __ballot_sync(0xffffffffu, mine);
 #pragma unroll 1
     for (int p = 0; p < KST; p += IR_E) {
         const int n = KST < IR_E ? KST : min(IR_E, KST - p);
@@ -555,7 +531,7 @@ __device__ __forceinline__ void inverse_ratios(const InvRatioSpin& S, int nw, do
         for (int i = 0; i < n; ++i) {
             const int f = i * 32 + lane, it = f / n;   // pair, entry
             const long long b = __shfl_sync(0xffffffffu, base, it);
-            if (e0 + it < items) B[b + p + f - it * n] = tile[it][f - it * n];
+            if (write >> it & 1) B[b + p + f - it * n] = tile[it][f - it * n];
         }
         __syncwarp();
     }
@@ -586,6 +562,8 @@ MinorSpin minor_spin(const SpinTables& t, const double2* GT, double2* m2, double
     for (int k = 0; k < MSD_KMAX + 2; ++k) { s.bucket[k] = t.bucket[k]; s.vbucket[k] = 0; }
     s.str_hp = t.str_hp; s.str_sign = t.str_sign; s.sub = t.sub;
     s.GT = GT; s.m2 = m2; s.rT = rT; s.t2 = t2; s.tr = tr;
+    s.B = nullptr;
+    for (int k = 0; k < MSD_KMAX + 2; ++k) s.b_off[k] = t.b_off[k];
     return s;
 }
 
@@ -596,7 +574,9 @@ void launch_lu(const MinorArgs& a, int nw, cudaStream_t st)
     long long n = 0;
     for (const MinorSpin& s : a.s) n = std::max(n, (long long)std::max(s.n_str, s.vbucket[MSD_KMAX + 1]) - s.bucket[level0]);
     if (n <= 0) return;
-    k_minor_lu<<<dim3((unsigned)((n * nw + LU_PAIRS - 1) / LU_PAIRS), 2), LU_THREADS, 0, st>>>(a, level0, nw);
+    const dim3 grid((unsigned)((n * nw + LU_PAIRS - 1) / LU_PAIRS), 2);
+    if (a.s[0].B) k_minor_lu<true><<<grid, LU_THREADS, 0, st>>>(a, level0, nw);
+    else k_minor_lu<false><<<grid, LU_THREADS, 0, st>>>(a, level0, nw);
     msd_note_launch();
 }
 
@@ -662,13 +642,14 @@ __global__ void __launch_bounds__(256) k_cofactors(const __grid_constant__ CofAr
 
 // Ratios of the trial's strings and of the sub-minors outside it.
 void launch_minors_ext(const ExtTables g[2], const SpinTables& ta, const SpinTables& tb, int nw, double2* const V[2],
-                       int* const t2[2], int* const tr[2], cudaStream_t st)
+                       int* const t2[2], int* const tr[2], void* const B[2], cudaStream_t st)
 {
     MinorArgs a;
     const SpinTables* T[2] = {&ta, &tb};
     for (int s = 0; s < 2; ++s) {
         double2* m2 = V[s] + (size_t)T[s]->nh * T[s]->np * nw;
         a.s[s] = minor_spin(*T[s], V[s], m2, m2 + (size_t)g[s].n2 * nw, t2[s], tr[s]);
+        a.s[s].B = B ? (double2*)B[s] : nullptr;
         a.s[s].str_hp = g[s].str_hp; a.s[s].str_sign = g[s].str_sign; a.s[s].sub = g[s].sub;
         for (int k = 0; k < MSD_KMAX + 2; ++k) a.s[s].vbucket[k] = g[s].vbucket[k];
     }
@@ -763,14 +744,14 @@ void launch_inverse_minors(const SpinTables& ta, const SpinTables& tb, int nw, d
 }
 
 void launch_inverse_ratios(const ExtTables g[2], const SpinTables& ta, const SpinTables& tb, int nw,
-                           double2* const V[2], void* const B[2], cudaStream_t st)
+                           double2* const V[2], int* const tr[2], void* const B[2], cudaStream_t st)
 {
     InvRatioArgs args;
     const SpinTables* t[2] = {&ta, &tb};
     int nb = 0;
     for (int i = 0; i < 2; ++i) {
         InvRatioSpin& s = args.s[i];
-        s.row = g[i].row; s.V = V[i]; s.B = (double2*)B[i];
+        s.row = g[i].row; s.V = V[i]; s.B = (double2*)B[i]; s.tr = tr[i];
         s.r = V[i] + ((size_t)t[i]->nh * t[i]->np + g[i].n2) * nw;
         s.blk[0] = s.blk[1] = 0;
         for (int k = 0; k < MSD_KMAX + 2; ++k) {

@@ -6,6 +6,7 @@
 
 #include "common.cuh"
 #include "kernels.h"
+#include "minor_lu.cuh"
 
 // ------------------------------------------------------------------------
 // Reference determinant per (walker, spin): S = D0^dag phi = phi[occ0, :]
@@ -226,97 +227,21 @@ int launch_refs(const RefSpinIn* in, int n_spin, int nw, int M, unsigned* err, c
 // Excitation strings of level K for one spin with their FP64 inverse minors
 // by an LU of its own, for FP64 energies and force bias of trials whose sub-minors are
 // far more than their strings (all else: k_minors.cu):
-// A[i][j] = G[h_i][p_j] (a K x K minor of G). LU with partial pivoting in
-// FP64 gives r = sign * det A, the overlap ratio <D_s|phi>/<D_0|phi> of the
-// string's spin sector, and B = A^-1 from its factors, K*K entries
-// contiguous (B[i][j] at i*K + j), for the Green's-function and energy
-// terms. One thread per (walker, string); the walker's active block lives in
+// A[i][j] = G[h_i][p_j] (a K x K minor of G); r = sign * det A, the overlap ratio
+// <D_s|phi>/<D_0|phi> of the string's spin sector, and B = A^-1 for the Green's-function
+// and energy terms. One thread per (walker, string); the walker's active block lives in
 // shared memory.
-//
-// FP64 issue rate is the bound here (a few FP64 operations per clock per
-// SM), so the LU spends FP64 operations on the elimination and the
-// determinant only: the pivot search compares integer magnitude keys (the
-// larger high word of |Re|, |Im|: partial pivoting by the max-norm), the row
-// swaps count parity in an integer, and the pivot reciprocals are
-// Newton-Raphson iterations from an FP32 seed.
-
-// String s = bucket[K] + sl of walker w, its active block in shared memory (g).
+// String s = bucket[K] + sl of walker w, its active block in shared memory (gs).
 template <int K>
-__device__ __forceinline__ void string_lu(const SpinTables& tb, int nw, int w, int sl, const double2* g, double2* r,
+__device__ __forceinline__ void string_lu(const SpinTables& tb, int nw, int w, int sl, const double2* gs, double2* r,
                                           double2* rT, double2* Bout)
 {
     const int ns = tb.bucket[K + 1] - tb.bucket[K], s = tb.bucket[K] + sl;
     const uint4 rec = tb.str_hp[s];
-    double2 a[K][K];
-#pragma unroll
-    for (int i = 0; i < K; ++i)
-#pragma unroll
-        for (int j = 0; j < K; ++j) a[i][j] = g[rec_h(rec, i) * tb.np + rec_p(rec, j)];
-    int perm[K];
-#pragma unroll
-    for (int i = 0; i < K; ++i) perm[i] = i;
-    double2 det = cz(tb.str_sign[s], 0);
-    double2 dinv[K];
-    bool sing = false;
-    int odd = 0;
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-        int p = k, best = mag_key(a[k][k]);
-        double2 pv = a[k][k];
-#pragma unroll
-        for (int i = k + 1; i < K; ++i) {
-            const int v = mag_key(a[i][k]);
-            if (v > best) { best = v; p = i; pv = a[i][k]; }
-        }
-        if (pv.x == 0.0 && pv.y == 0.0) sing = true;
-#pragma unroll
-        for (int i = k + 1; i < K; ++i) {
-            if (i == p) {
-#pragma unroll
-                for (int j = 0; j < K; ++j) { double2 tt = a[k][j]; a[k][j] = a[i][j]; a[i][j] = tt; }
-                int tp = perm[k]; perm[k] = perm[i]; perm[i] = tp;
-                odd ^= 1;
-            }
-        }
-        det = cmul(det, a[k][k]);
-        const double m2 = fma(a[k][k].x, a[k][k].x, a[k][k].y * a[k][k].y);
-        const double im2 = sing ? 0.0 : recip_nr(m2);
-        dinv[k] = cz(a[k][k].x * im2, -a[k][k].y * im2);
-        if (k + 1 < K) {
-#pragma unroll
-            for (int i = k + 1; i < K; ++i) {
-                const double2 f = cmul(a[i][k], dinv[k]);
-                a[i][k] = f;
-#pragma unroll
-                for (int j = k + 1; j < K; ++j) a[i][j] = cfms(f, a[k][j], a[i][j]);
-            }
-        }
-    }
-    if (odd) det = cz(-det.x, -det.y);
-    if (sing) det = cz(0, 0);
+    const double2 det = minor_lu<K>(tb.str_sign[s], [&](int i, int j) { return gs[rec_h(rec, i) * tb.np + rec_p(rec, j)]; },
+                                    Bout + (size_t)tb.b_off[K] + ((size_t)w * ns + sl) * b_stride(K));
     if (r) r[(size_t)w * tb.n_str + s] = det;
     rT[(size_t)s * nw + w] = det;
-    // B = A^-1 from P A = L U: column c solves L U x = P e_c
-    double2* B = Bout + (size_t)tb.b_off[K] + ((size_t)w * ns + sl) * b_stride(K);
-    if (K & 1) B[K * K] = cz(0, 0);   // the pad entry
-#pragma unroll
-    for (int c = 0; c < K; ++c) {
-        double2 x[K];
-#pragma unroll
-        for (int i = 0; i < K; ++i) x[i] = cz(perm[i] == c ? 1 : 0, 0);
-#pragma unroll
-        for (int i = 0; i < K; ++i)
-#pragma unroll
-            for (int k = 0; k < i; ++k) x[i] = cfms(a[i][k], x[k], x[i]);
-#pragma unroll
-        for (int i = K - 1; i >= 0; --i) {
-#pragma unroll
-            for (int k = i + 1; k < K; ++k) x[i] = cfms(a[i][k], x[k], x[i]);
-            x[i] = cmul(x[i], dinv[i]);
-        }
-#pragma unroll
-        for (int i = 0; i < K; ++i) B[i * K + c] = x[i];
-    }
 }
 
 template <int K>

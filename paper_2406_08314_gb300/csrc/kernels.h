@@ -69,12 +69,13 @@ struct ExtTables {
     int *cof_row = nullptr, *cof_off = nullptr;
     int2* cof_ent = nullptr;
 };
-// t2 [n2][nw], tr [n_ext - bucket[3]][nw]: scratch.
+// t2 [n2][nw], tr [n_ext - bucket[3]][nw]: scratch. B (may be NULL): the inverse minors of
+// the strings whose ratios take the LU.
 void launch_minors_ext(const ExtTables g[2], const SpinTables& ta, const SpinTables& tb, int nw, double2* const V[2],
-                       int* const t2[2], int* const tr[2], cudaStream_t st);
-// FP64 inverse minors from V as launch_minors_ext left it.
+                       int* const t2[2], int* const tr[2], void* const B[2], cudaStream_t st);
+// The other FP64 inverse minors from V and tr as launch_minors_ext left them.
 void launch_inverse_ratios(const ExtTables g[2], const SpinTables& ta, const SpinTables& tb, int nw,
-                           double2* const V[2], void* const B[2], cudaStream_t st);
+                           double2* const V[2], int* const tr[2], void* const B[2], cudaStream_t st);
 void launch_cofactors(const ExtTables g[2], const SpinTables& ta, const SpinTables& tb, int nw, double2* const V[2],
                       double2* const Bv[2], double2* const Cm[2], int* const big[2], cudaStream_t st);
 void launch_untranspose(int n_str, int nw, const double2* rT, double2* r, cudaStream_t st);

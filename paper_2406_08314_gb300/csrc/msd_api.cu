@@ -1482,9 +1482,9 @@ int run_strings_weights(msd_ctx* ctx, int nw, Chunk& c, StringUse use, bool fp32
         // the ratios are V's last rows
         for (int s = 0; s < 2; ++s) c.rT[s] = c.V[s] + ((size_t)T[s].nh * T[s].np + ctx->ext[s].n2) * nw;
         th.begin("k_strings", st);
-        launch_minors_ext(ctx->ext, T[0], T[1], nw, c.V, c.t2, c.tr, st);
+        launch_minors_ext(ctx->ext, T[0], T[1], nw, c.V, c.t2, c.tr, want_b ? c.B : nullptr, st);
         if (want_b) {
-            launch_inverse_ratios(ctx->ext, T[0], T[1], nw, c.V, c.B, st);
+            launch_inverse_ratios(ctx->ext, T[0], T[1], nw, c.V, c.tr, c.B, st);
             for (int s = 0; s < 2; ++s) launch_untranspose(T[s].n_str, nw, c.rT[s], c.r[s], st);
         }
         launch_strings_large(T[0], T[1], nw, c.GactT, c.Gact, c.big, c.r, c.rT, c.B, st);

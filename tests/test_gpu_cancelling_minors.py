@@ -109,3 +109,31 @@ def test_observables(rank, size):
         assert np.all(np.abs(x - ref["vbias"]).max(1) <= tol_g * lam)
     assert np.all(np.abs(e - ref["e_loc"]) <= tol_e)
     ctx.close()
+
+
+@pytest.mark.parametrize("size", [1e-2, 1e-4, 1e-6])
+def test_energy_of_blocks_near_rank_one(size):
+    """Active blocks with entries below 1, of rank one but for a part of 0.1 size: minors from
+    level 2 on are small, inverse minors large."""
+    import torch
+
+    from paper_2406_08314_gb300 import msd
+    s, n_w = _system(2, False), 4
+    rng = np.random.default_rng(5)
+
+    def c(*shape):
+        return rng.standard_normal(shape) + 1j * rng.standard_normal(shape)
+
+    walkers = []
+    for _ in (0, 1):
+        t = c(n_w, N_ACT + 1 - N, 1) @ c(n_w, 1, N)
+        t *= 0.9 / np.maximum(np.abs(t.real), np.abs(t.imag)).max((1, 2), keepdims=True)
+        t += 0.1 * size * c(*t.shape)
+        walkers.append(np.ascontiguousarray(np.concatenate([np.broadcast_to(np.eye(N), (n_w, N, N)), t], 1)))
+    ref = exact_msd.msd(s, *walkers)
+    ctx = msd.Context(s, "fp64")
+    e = ctx.local_energy(*[torch.from_numpy(x).cuda() for x in walkers]).cpu().numpy()
+    ctx.close()
+    # an inverse of condition k = 10 / size is off by u k of its entries, and a string's energy is
+    # ratio x inverse x inverse, of the size of k for level 2 and its sums of up to 64 terms
+    assert np.all(np.abs(e - ref["e_loc"]) <= 64 * 2.0 ** -53 * 10 / size * np.abs(ref["e_loc"]))
