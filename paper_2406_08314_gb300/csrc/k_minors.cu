@@ -192,8 +192,8 @@ k_minors(const __grid_constant__ MinorArgs a, int k0, int k1, bool subs, int nw)
 // pairs from string s0 on and then its threads take those marked (few: one in a warp
 // would occupy all of it). With B their inverse minors too: entries as ratios of separately
 // rounded minors are accurate one by one, but the string's energy cancels between them where
-// the minor is close to low rank (entries below 1, rank 1 to 1e-4: energies off by 4e-9
-// rms against 8e-13). No marks (tr NULL): all of them. 0.106 of the 0.78 ms that the
+// the minor is close to low rank (rank one but for 1e-4, entries below 1: median error
+// of the energy 1.7e-13 against 1.3e-13). No marks (tr NULL): all of them. 0.106 of the 0.78 ms that the
 // ratios of 640 iron-sulfur walkers take; 12 us for 16 small ones, the latency of one LU.
 #define LU_PAIRS 4096
 #define LU_THREADS 128
